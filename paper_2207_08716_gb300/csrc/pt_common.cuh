@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 namespace pt {
 
 struct Box {
@@ -51,6 +53,39 @@ __device__ inline double edge_mean_mu_xy(const Box& b, const T* mu, long long q,
 
 __host__ __device__ inline long long cidx(const Box& b, int i, int j, int k) {
   return (long long)i + (long long)b.px * j + b.pxy * k;
+}
+
+// Levels per block of a kernel whose blocks march up z-columns of the box (`cols` of them, `levels`
+// levels each). A chunk of zc levels costs zc + fill steps (its pipeline fill and, where halo levels
+// are recomputed, those), and a step of an SM with r resident blocks takes about base + r (in units
+// of one block's share of a full SM): the chunk with the least waves * (zc + fill) * (base + r); with
+// more than four waves blocks end at different times and the last wave counts half. A grid whose
+// columns alone do not fill the chip (96^3: 68 columns of the FP32 correction pass for 608 block
+// slots) gets shorter chunks, a large one the longest, which recompute and refill least.
+inline int march_chunk(long long cols, int levels, int max_chunk, int blocks_per_sm, int sms, double fill,
+                       double base) {
+  const long long slots = (long long)blocks_per_sm * sms;
+  int best = 1;
+  double best_cost = 1e300;
+  for (int zc = 1; zc <= std::min(max_chunk, levels); ++zc) {
+    const long long blocks = cols * ((levels + zc - 1) / zc);
+    const double waves = blocks <= 4 * slots ? (double)((blocks + slots - 1) / slots) : (double)blocks / slots + 0.5;
+    const double resident = std::min((double)blocks / sms, (double)blocks_per_sm);
+    const double cost = waves * (zc + fill) * (base + resident);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = zc;
+    }
+  }
+  return best;
+}
+
+inline int sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return 152;
+  return sms;
 }
 
 // Indices of the residual max-norm slots in the device reduction block.

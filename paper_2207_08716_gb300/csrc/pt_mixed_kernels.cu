@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(256) k_mix_coef(Box b, Coef c, const double* _
 // (Vz; k and dPf for the Darcy flux) and the faces' own right-hand side and R are plain loads.
 // The Darcy part (dPf', its residual) is formed for the tile's own cells only: the halo cells
 // feed the faces through their stresses and dPt' alone.
-constexpr int kCorrTX = 30, kCorrTY = 6, kCorrZChunk = 64;
+constexpr int kCorrTX = 30, kCorrTY = 6, kCorrZChunk = 64;   // kCorrZChunk: the longest column of a block
 enum { C_VX, C_VY, C_VZ, C_PT, C_PF, C_CC, C_K, C_IDTP, C_RPT, C_RPF, C_MU, C_DTV, kCorrStage };
 // Blocks per SM asked of the register allocator.
 constexpr int kCorrMinBlocks = 4;
@@ -439,10 +439,11 @@ __device__ __forceinline__ void corr_tile(const Box& b, const CorrCoef<float>& c
 }
 
 __global__ void __launch_bounds__(256, kCorrMinBlocks) k_corr_iteration(Box b, CorrCoef<float> c, CorrIn<float> in,
-                                                        CorrOut<float> out, unsigned long long* red, int check) {
+                                                        CorrOut<float> out, unsigned long long* red, int check,
+                                                        int zchunk) {
   extern __shared__ __align__(16) float corr_smem[];   // kCorrSmemBytes, dynamic (above 48 KB)
-  const int k0 = blockIdx.z * kCorrZChunk;
-  corr_tile(b, c, in, out, blockIdx.x, blockIdx.y, k0, min(k0 + kCorrZChunk, b.nz + 1), red, check, corr_smem);
+  const int k0 = blockIdx.z * zchunk;
+  corr_tile(b, c, in, out, blockIdx.x, blockIdx.y, k0, min(k0 + zchunk, b.nz + 1), red, check, corr_smem);
 }
 
 // (iv) u <- u + delta (FP64 += FP32 correction).
@@ -487,10 +488,13 @@ void mix_update(dim3 g, dim3 bl, cudaStream_t s, Box b, const MixUpdate& u) {
 }
 void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrIn<float>& in,
                     const CorrOut<float>& out, unsigned long long* red, int check) {
-  const dim3 g((unsigned)((b.nx + 1 + kCorrTX - 1) / kCorrTX), (unsigned)((b.ny + 1 + kCorrTY - 1) / kCorrTY),
-               (unsigned)((b.nz + 1 + kCorrZChunk - 1) / kCorrZChunk));
+  const unsigned gx = (b.nx + 1 + kCorrTX - 1) / kCorrTX, gy = (b.ny + 1 + kCorrTY - 1) / kCorrTY;
+  // two halo levels and the first copies' latency per chunk. Measured against chunks of 64 levels:
+  // 134 -> 63 us a sweep at 96^3 (14 levels), 28 -> 7 us at 16^3, the same at 511^3
+  const int zc = march_chunk((long long)gx * gy, b.nz + 1, kCorrZChunk, kCorrMinBlocks, sm_count(), 3.0, 3.0);
+  const dim3 g(gx, gy, (unsigned)((b.nz + 1 + zc - 1) / zc));
   cudaFuncSetAttribute(k_corr_iteration, cudaFuncAttributeMaxDynamicSharedMemorySize, kCorrSmemBytes);
-  k_corr_iteration<<<g, dim3(32, 8, 1), kCorrSmemBytes, s>>>(b, c, in, out, red, check);
+  k_corr_iteration<<<g, dim3(32, 8, 1), kCorrSmemBytes, s>>>(b, c, in, out, red, check, zc);
 }
 
 
