@@ -1287,11 +1287,11 @@ struct pt_batch {
   MixBatchStatus* d_mst;
   MixBatchStatus* h_mst;
   unsigned long long* d_ired;
-  int zchunk, minb, mult;   // correction tile depth, CTAs per SM of the correction kernel, rounds per replay
+  int zchunk, mult;         // correction tile depth, rounds per replay
   int groups;               // members split into this many contiguous groups, each a parallel graph branch
   long long nptiles, nctiles;
   int pgrid, cgrid;
-  int exec_zchunk, exec_minb, exec_mult, exec_groups;
+  int exec_zchunk, exec_mult, exec_groups;
   std::vector<int> gm;                  // group g = members [gm[g], gm[g + 1])
   std::vector<cudaStream_t> gstream;    // capture streams of the branches
   std::vector<cudaEvent_t> gevent;      // fork (0) and one join per branch
@@ -1453,9 +1453,9 @@ void fill_mix_inst(pt_batch* B, int m, long long base, long long cbase) {
   I.max_iter = c->num.max_iter;
   I.gx = (c->box.nx + 1 + 31) / 32;
   I.gy = (c->box.ny + 1 + 7) / 8;
-  I.cgx = (c->box.nx + 1 + corr_tile_x() - 1) / corr_tile_x();
-  I.cgy = (c->box.ny + 1 + corr_tile_y() - 1) / corr_tile_y();
-  I.cgz = (c->box.nz + 1 + B->zchunk - 1) / B->zchunk;
+  I.cgx = (c->box.nx + corr_tile_x() - 1) / corr_tile_x();
+  I.cgy = (c->box.ny + corr_tile_y() - 1) / corr_tile_y();
+  I.cgz = (c->box.nz + B->zchunk - 1) / B->zchunk;
   I.tile_base = base;
   I.ctile_base = cbase;
 }
@@ -1474,7 +1474,7 @@ cudaError_t upload_mix(pt_batch* B) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   B->pgrid = std::max(1, sms * mb_points_blocks_per_sm());
-  B->cgrid = std::max(1, sms * mb_corr_blocks_per_sm(B->minb));
+  B->cgrid = std::max(1, sms * mb_corr_blocks_per_sm());
   return cudaMemcpyAsync(B->d_minst, B->h_minst.data(), sizeof(MixBatchInst) * B->ninst, cudaMemcpyHostToDevice,
                          B->stream);
 }
@@ -1509,7 +1509,7 @@ void record_mix_group(pt_batch* B, int g, cudaStream_t s) {
     mb_points(B->pgrid, s, MB_PH_FACES, inst, st, n, p0, p1);
     mb_decide_outer(s, inst, st, n);
     mb_points(B->pgrid, s, MB_PH_INIT, inst, st, n, p0, p1);
-    for (int k = 1; k <= B->nup; ++k) mb_corr(B->cgrid, B->minb, s, inst, st, n, c0, c1, k, B->nup, B->zchunk);
+    for (int k = 1; k <= B->nup; ++k) mb_corr(B->cgrid, s, inst, st, n, c0, c1, k, B->nup, B->zchunk);
     mb_decide_inner(s, inst, st, n, B->nup);
     mb_points(B->pgrid, s, MB_PH_UPDATE, inst, st, n, p0, p1);
     mb_points(B->pgrid, s, MB_PH_POROSITY, inst, st, n, p0, p1);
@@ -1536,7 +1536,7 @@ void record_mix_rounds(pt_batch* B) {
 }
 
 int build_mix_graph(pt_batch* B) {
-  if (B->exec && B->exec_zchunk == B->zchunk && B->exec_minb == B->minb && B->exec_mult == B->mult &&
+  if (B->exec && B->exec_zchunk == B->zchunk && B->exec_mult == B->mult &&
       B->exec_groups == B->groups)
     return PT_OK;
   if (B->exec) {
@@ -1554,7 +1554,6 @@ int build_mix_graph(pt_batch* B) {
     return PT_ECUDA;
   }
   B->exec_zchunk = B->zchunk;
-  B->exec_minb = B->minb;
   B->exec_mult = B->mult;
   B->exec_groups = B->groups;
   return PT_OK;
@@ -1583,7 +1582,7 @@ struct TunerEvents {
 
 // FP32 ensemble step: every member's step begin (host, as pt_step), then graph replays until
 // every member is done; the first step times one replay of each candidate configuration
-// (correction tile depth, CTAs per SM, rounds per replay) and keeps the fastest per round.
+// (correction tile depth, member groups) and keeps the fastest per round.
 int batch_step_mixed(pt_batch* B, pt_report* reps, double* ttc_ms) {
   int rc = PT_OK;
   int cap = 0;
@@ -1598,19 +1597,17 @@ int batch_step_mixed(pt_batch* B, pt_report* reps, double* ttc_ms) {
   // every round advances each member that is not done: an outer iteration takes at least one
   // round and at least min(nup, budget) correction iterations, so this many rounds end every member
   const long long max_rounds = 2LL * ((long long)cap / B->nup + 2) + 4;
-  struct Cfg { int zchunk, minb, mult, groups; };
-  const Cfg cands[] = {{64, 4, 1, 1}, {64, 3, 1, 4}, {64, 4, 1, 4}, {64, 3, 1, 8}, {64, 3, 1, 16}, {32, 3, 1, 8},
-                       {64, 3, 2, 8}};
+  struct Cfg { int zchunk, mult, groups; };
+  const Cfg cands[] = {{64, 1, 1}, {32, 1, 1}, {64, 1, 4}, {32, 1, 4}, {32, 1, 8}, {64, 1, 8}, {64, 1, 16}};
   const int ncand = B->tuned ? 0 : (int)(sizeof cands / sizeof cands[0]);
   float best_ms = 1e30f;
-  Cfg best = {B->zchunk, B->minb, B->mult, B->groups};
+  Cfg best = {B->zchunk, B->mult, B->groups};
   long long rounds = 0;
   int nactive = B->ninst;
   TunerEvents ev;
   if (ncand && !ev.create()) return PT_ECUDA;
   for (int t = 0; t < ncand && nactive > 0 && rounds < max_rounds; ++t) {
     B->zchunk = cands[t].zchunk;
-    B->minb = cands[t].minb;
     B->mult = cands[t].mult;
     B->groups = cands[t].groups;
     if (upload_mix(B) != cudaSuccess) return PT_ECUDA;
@@ -1631,7 +1628,6 @@ int batch_step_mixed(pt_batch* B, pt_report* reps, double* ttc_ms) {
   }
   if (ncand) {
     B->zchunk = best.zchunk;
-    B->minb = best.minb;
     B->mult = best.mult;
     B->groups = best.groups;
     B->tuned = true;
@@ -1725,10 +1721,9 @@ int pt_batch_init(pt_batch** out, int32_t ninst, const pt_grid* grids, const pt_
   B->h_inst.resize(ninst);
   B->mixed = fp32;
   B->zchunk = 64;
-  B->minb = 4;
   B->mult = 1;
   B->groups = 1;
-  B->exec_zchunk = B->exec_minb = B->exec_mult = B->exec_groups = 0;
+  B->exec_zchunk = B->exec_mult = B->exec_groups = 0;
   B->h_st = nullptr;
   B->h_mst = nullptr;
   if (fp32) B->h_minst.resize(ninst);
@@ -1891,7 +1886,7 @@ int pt_batch_config(const pt_batch* B, int32_t* tile_x, int32_t* tile_y, int32_t
 int pt_batch_config_fp32(const pt_batch* B, int32_t* tile_z, int32_t* blocks_per_sm, int32_t* groups) {
   if (!B || !B->mixed) return PT_EINVAL;
   if (tile_z) *tile_z = B->zchunk;
-  if (blocks_per_sm) *blocks_per_sm = B->minb;
+  if (blocks_per_sm) *blocks_per_sm = mb_corr_blocks_per_sm();
   if (groups) *groups = std::max(1, std::min(B->groups, B->ninst));
   return PT_OK;
 }

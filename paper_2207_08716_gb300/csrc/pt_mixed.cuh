@@ -176,9 +176,8 @@ struct MixBatchStatus {
 void mb_points(int grid, cudaStream_t s, int phase, const MixBatchInst* inst, const MixBatchStatus* st, int ninst,
                long long t0, long long t1);
 // Correction iteration number inner + step (1-based) of every member in MB_INNER within its budget;
-// minb (3 or 4): the CTAs per SM the kernel's registers are budgeted for. Sets the kernel's
-// shared-memory attribute first (mb_corr_blocks_per_sm, before any capture).
-void mb_corr(int grid, int minb, cudaStream_t s, const MixBatchInst* inst, const MixBatchStatus* st, int ninst,
+// mb_corr_blocks_per_sm sets the kernel's shared-memory attribute (before any capture).
+void mb_corr(int grid, cudaStream_t s, const MixBatchInst* inst, const MixBatchStatus* st, int ninst,
              long long t0, long long t1, int step, int nup, int zchunk);
 void mb_decide_outer(cudaStream_t s, const MixBatchInst* inst, MixBatchStatus* st, int ninst);
 void mb_decide_inner(cudaStream_t s, const MixBatchInst* inst, MixBatchStatus* st, int ninst, int nup);
@@ -186,7 +185,7 @@ void mb_finish(cudaStream_t s, const MixBatchInst* inst, MixBatchStatus* st, int
 void mb_start(cudaStream_t s, const MixBatchInst* inst, MixBatchStatus* st, int ninst);
 // Resident CTAs per SM of the point and correction kernels.
 int mb_points_blocks_per_sm();
-int mb_corr_blocks_per_sm(int minb);
+int mb_corr_blocks_per_sm();
 // Correction tile extents in x and y (faces per tile).
 int corr_tile_x();
 int corr_tile_y();

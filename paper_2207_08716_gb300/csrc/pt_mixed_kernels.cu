@@ -18,6 +18,8 @@
 #include "pt_lean_body.cuh"
 #include "../../include/porowave_pt.h"
 
+#include <type_traits>
+
 namespace pt {
 
 namespace {
@@ -187,263 +189,350 @@ __global__ void __launch_bounds__(256) k_mix_coef(Box b, Coef c, const double* _
 // The iteration's two halves depend on each other across neighbours: the faces (momentum,
 // damped R, dV) of level k read the cells' stresses and new dPt at k and k-1 (own cell, x- and
 // y-neighbours below) and the edge stresses at k and k+1 (own edge, x- and y-neighbours above).
-// A 32 x 8 block owns a tile of 30 x 6 faces and cells and marches up a column of face levels:
+// A block of 32 x rows threads owns a tile of 30 x (rows - 2) faces and cells and marches up a column of face levels:
 // at level L every thread computes the cell and the three lower edges at its index for the tile
 // plus a one-cell halo on each side (the halo is recomputed by the neighbouring tiles' blocks from
-// the same inputs, bit for bit), into rings in shared memory; after a barrier the tile's threads
-// compute the faces of level L-1 from the rings. Stresses and the new dPt never go to global
-// memory: per cell the pass reads dV, dPt, dPf, R, the right-hand sides and the frozen cc, k,
-// 1/dtau_Pt, mu, dtau_V (18 arrays) and writes dV', dPt', dPf', R (8 arrays): 104 B per cell
-// against 200 B for a cells kernel plus a faces kernel. dV is read from one buffer and written to
-// another (other blocks' halos still read the old dV). The pseudo-step of dPf (largest neighbour
-// k), the local-implicit denominators, 2 mu/(1+xi) at centres and edges (mean of the four
-// centres' mu) and the face pseudo-steps (mean of the two centres') are formed here.
+// the same inputs, bit for bit). Stresses and the new dPt never go to global memory: per cell the
+// pass reads dV, dPt, dPf, R, the right-hand sides and the frozen cc, k, 1/dtau_Pt, mu, dtau_V (18
+// arrays) and writes dV', dPt', dPf', R (8 arrays): 104 B per cell. dV is read from one buffer and
+// written to another (other blocks' halos still read the old dV). The pseudo-step of dPf (largest
+// neighbour k), the local-implicit denominators, 2 mu/(1+xi) at centres and edges (mean of the
+// four centres' mu) and the face pseudo-steps (mean of the two centres') are formed here.
 //
-// Staging: the 12 arrays read at a point's own index go into a three-slot shared-memory ring by
-// cp.async, one level ahead (levels L-1 and L resident while L+1 is in flight), so every x-, y-
-// and z-1 neighbour a point reads comes from shared memory; only the three z+1 values of a cell
-// (Vz; k and dPf for the Darcy flux) and the faces' own right-hand side and R are plain loads.
-// The Darcy part (dPf', its residual) is formed for the tile's own cells only: the halo cells
-// feed the faces through their stresses and dPt' alone.
-constexpr int kCorrTX = 30, kCorrTY = 6, kCorrZChunk = 64;   // kCorrZChunk: the longest column of a block
-enum { C_VX, C_VY, C_VZ, C_PT, C_PF, C_CC, C_K, C_IDTP, C_RPT, C_RPF, C_MU, C_DTV, kCorrStage };
-// Blocks per SM asked of the register allocator.
-constexpr int kCorrMinBlocks = 4;
-// rings: cells (4 values) over three levels, edges (3) over two, staged inputs over three
-constexpr int kCorrSmemBytes = (3 * 4 + 2 * 3 + 3 * kCorrStage) * 8 * 32 * (int)sizeof(float);
+// What bounds it is instruction issue and the latency between block barriers, not DRAM, so:
+//   * one barrier per level: in the interval of level L a thread computes the faces of level L - 2
+//     and then the cell and edges of level L, which no thread reads before the next barrier;
+//   * a point's own values of the levels below (stresses, dV, the Darcy flux through the lower z
+//     face) are carried in registers, x-neighbours of the stresses come by warp shuffle (a warp is a
+//     row of the tile), so that only tyy, dPt' and the xy and yz edge stresses, which the row above
+//     or below reads, go through shared memory (rings of three levels);
+//   * the 12 arrays read at a point's own index and its x- and y-neighbours' are staged by 16-byte
+//     cp.async one level ahead: a row of a tile is 9 aligned vectors, so that a level takes 4 copies of
+//     27 lanes per warp instead of 12 of 32. dVz, dPf and k run one level further ahead (the cell of
+//     level L reads them at L + 1), dtau_V two levels behind (the faces' level);
+//   * the faces' own R and right-hand side are loaded an interval before their use;
+//   * every ring has three slots and the loop takes three levels per turn, so that slots are constants
+//     and the carried values change names instead of registers;
+//   * tiles that touch no wall in x and y (INNER) take no wall tests; the z tests are uniform. A sweep
+//     without damping neither reads nor keeps R (nothing reads it before an evaluation writes it).
+// Measured at 511^3: 4.83 ms a sweep with two barriers a level, every neighbour from shared memory and
+// 32 x 8 blocks; 3.08 ms in this form (4.5 TB/s of its 104 B per cell, 0.67 of the copy peak; at
+// 239^3 546 thread instructions per cell against 791, issue slots 58 % busy).
+constexpr int kCorrTX = 30;
+constexpr int kCorrZChunk = 64; // the longest column of a block
+constexpr int kCorrW = 36;      // floats of a staged row: 32 points and up to 3 in front (16-byte alignment)
+// Staged arrays, in units of one level's tile (rows of kCorrW), three slots each: a level's
+// slot is its distance from the column's first level modulo 3 (DTV: the slot of the level above).
+enum { C_VX = 0, C_VY = 3, C_PT = 6, C_CC = 9, C_IDTP = 12, C_RPT = 15, C_RPF = 18, C_DTV = 21, C_MU = 24, C_VZ = 27,
+       C_K = 30, C_PF = 33, kCorrStage = 36 };
+enum { R_TYY, R_P, R_XY, R_YZ, kCorrRing };   // values the neighbouring rows read, three levels each
+// ROWS: rows (warps) of a block, the tile's and a halo row on each side; BLOCKS per SM asked of the
+// register allocator.
+template <int ROWS, int BLOCKS>
+struct CorrShape {
+  static constexpr int rows = ROWS, blocks = BLOCKS, threads = 32 * ROWS, ty = ROWS - 2;
+  static constexpr int smem = (kCorrStage * kCorrW + 3 * kCorrRing * 32) * ROWS * (int)sizeof(float);
+};
+// A step of 60 sweeps at 511^3 and one of 240 at 96^3: 10 rows, 2 blocks of 96 registers 340 and 12.2 ms;
+// 8 rows, 3 blocks (80 registers) 343 and 13.8; 12 rows, 2 blocks 352 and 12.9; 10 rows, 3 blocks
+// (64 registers, spilling) 460 and 18.1. The ensemble engine's tile is part of its interface (30 x 6).
+using CorrSingle = CorrShape<10, 2>;
+using CorrBatch = CorrShape<8, 3>;
 
-__device__ __forceinline__ void corr_cp4(float* smem, const float* gmem) {
+__device__ __forceinline__ void corr_cp16(float* smem, const float* gmem) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gmem) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem) : "memory");
 }
 
+// a / b for b far inside the normal range: the hardware's approximate reciprocal (1 ulp) times a
+__device__ __forceinline__ float corr_div(float a, float b) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  return a * r;
+}
+// 2 m / (1 + m / (G dtS)) of the viscosity m, and of the mean of four given their sum
 __device__ __forceinline__ float corr_modulus(const CorrCoef<float>& c, float m) {
-  return __fdividef(2.0f * m, 1.0f + m * c.rG);
+  return corr_div(2.0f * m, fmaf(m, c.rG, 1.0f));
+}
+__device__ __forceinline__ float corr_modulus4(const CorrCoef<float>& c, float sum) {
+  return corr_div(0.5f * sum, fmaf(sum, 0.25f * c.rG, 1.0f));
 }
 
 // One tile of the iteration: faces and cells of columns [tbx kCorrTX, +kCorrTX) x [tby kCorrTY,
-// +kCorrTY) and face levels [k0, k1), by a 32 x 8 block whose dynamic shared memory (kCorrSmemBytes)
-// starts at corr_smem. Leaves no copy in flight: the block may start another tile after a barrier.
-__device__ __forceinline__ void corr_tile(const Box& b, const CorrCoef<float>& c, const CorrIn<float>& in,
-                                          const CorrOut<float>& out, int tbx, int tby, int k0, int k1,
-                                          unsigned long long* red, int check, float* corr_smem) {
+// +kCorrTY) and face levels [k0, ke), ke <= nz (the level nz holds walls only), by a 32 x SH::rows
+// block whose dynamic shared memory (SH::smem) starts at corr_smem. Leaves no copy in flight:
+// the block may start another tile after a barrier.
+template <class SH, bool INNER>
+__device__ __forceinline__ void corr_tile_run(const Box& b, const CorrCoef<float>& c, const CorrIn<float>& in,
+                                              const CorrOut<float>& out, int tbx, int tby, int k0, int ke,
+                                              unsigned long long* red, int check, float* corr_smem) {
   using T = float;
-  T(*s_cell)[4][8][32] = reinterpret_cast<T(*)[4][8][32]>(corr_smem);                 // txx, tyy, tzz, dPt'
-  T(*s_edge)[3][8][32] = reinterpret_cast<T(*)[3][8][32]>(corr_smem + 3 * 4 * 8 * 32);  // txy, txz, tyz
-  T(*s_in)[kCorrStage][8][32] = reinterpret_cast<T(*)[kCorrStage][8][32]>(corr_smem + (3 * 4 + 2 * 3) * 8 * 32);
+  constexpr int kCorrTY = SH::ty;
+  constexpr int AR = SH::rows * kCorrW;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int i = tbx * kCorrTX - 1 + tx;
+  const int i0 = tbx * kCorrTX - 1;
+  const int i = i0 + tx;
   const int j = tby * kCorrTY - 1 + ty;
-  const bool own = tx >= 1 && tx <= kCorrTX && ty >= 1 && ty <= kCorrTY;
-  const int ipx = b.px, ipxy = (int)b.pxy;   // the host keeps the box below 2^31 elements
-  // residual norms as bit patterns of non-negative doubles: a NaN (largest pattern) stays in them
-  unsigned long long r_pt = 0ull, r_pf = 0ull, r_v = 0ull;
-  auto keep_max = [](unsigned long long& m, float x) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong((double)fabsf(x));
-    m = u > m ? u : m;
-  };
-  auto slot = [](int L) { return (L + 6) % 3; };     // L >= -2
-  const bool in_box = i >= 0 && j >= 0 && i <= b.nx && j <= b.ny;
-  auto stage = [&](int L) {   // own-index values of level L (inside the box) into its ring slot
-    if (in_box && L >= 0 && L <= b.nz) {
-      const int q = i + ipx * j + ipxy * L;
-      float(*st)[8][32] = s_in[slot(L)];
-      corr_cp4(&st[C_VX][ty][tx], in.Vx + q);
-      corr_cp4(&st[C_VY][ty][tx], in.Vy + q);
-      corr_cp4(&st[C_VZ][ty][tx], in.Vz + q);
-      corr_cp4(&st[C_PT][ty][tx], in.Pt + q);
-      corr_cp4(&st[C_PF][ty][tx], in.Pf + q);
-      corr_cp4(&st[C_CC][ty][tx], in.cc + q);
-      corr_cp4(&st[C_K][ty][tx], in.perm + q);
-      corr_cp4(&st[C_IDTP][ty][tx], in.idtp + q);
-      corr_cp4(&st[C_RPT][ty][tx], in.r_pt + q);
-      corr_cp4(&st[C_RPF][ty][tx], in.r_pf + q);
-      corr_cp4(&st[C_MU][ty][tx], in.mu + q);
-      corr_cp4(&st[C_DTV][ty][tx], in.dtvc + q);
+  const int ga = i0 & ~3;                       // first staged column (a multiple of 4; -4 for the first tile)
+  const int ipx = b.px, ipxy = (int)b.pxy;      // the host keeps the box below 2^31 elements
+  const bool row_own = ty >= 1 && ty <= kCorrTY;           // uniform over a warp
+  const bool own = row_own && tx >= 1 && tx <= kCorrTX && (INNER || (i < b.nx && j < b.ny));
+  // this thread's place in a staged tile and in a ring level
+  const float* const st = corr_smem + ty * kCorrW + (i0 - ga) + tx;
+  float* const ring = corr_smem + kCorrStage * AR + ty * 32 + tx;
+  constexpr int RA = SH::rows * 32, RL = kCorrRing * RA;   // one ring array, one level of the rings
+
+  // ---- staging: lanes 0-26 copy three arrays' rows of 9 vectors in each of four rounds
+  const int sub = tx / 9, vec = tx - 9 * sub;
+  const int col = ga + 4 * vec;
+  const bool cp_ok = tx < 27 && j >= 0 && j <= b.ny && col >= 0 && col < b.px;
+  const int cq = col + ipx * j;
+  const float* const g0 = (sub == 0 ? in.Vx : sub == 1 ? in.Vy : in.Pt) + cq;
+  const float* const g1 = (sub == 0 ? in.cc : sub == 1 ? in.idtp : in.r_pt) + cq;
+  const float* const g2 = (sub == 0 ? in.r_pf : sub == 1 ? in.dtvc : in.mu) + cq;
+  const float* const g3 = (sub == 0 ? in.Vz : sub == 1 ? in.perm : in.Pf) + cq;
+  float* const sdst = corr_smem + 3 * sub * AR + ty * kCorrW + 4 * vec;
+  static_assert(C_VY == 3 && C_PT == 6 && C_CC == 9 && C_RPF == 18 && C_VZ == 27, "a round's three arrays in order");
+  const int lag2 = sub == 1 ? 2 : 0;            // DTV is staged two levels behind
+  // level L of every array but VZ, K, PF (and DTV at L - 2) into slot s; level L of VZ, K, PF
+  auto stage_a = [&](int s, int L) {
+    if (!cp_ok) return;
+    if (L >= 0 && L <= b.nz) {
+      corr_cp16(sdst + (C_VX + s) * AR, g0 + ipxy * L);
+      corr_cp16(sdst + (C_CC + s) * AR, g1 + ipxy * L);
     }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    const int M = L - lag2;
+    if (M >= 0 && M <= b.nz) corr_cp16(sdst + (C_RPF + s) * AR, g2 + ipxy * M);
   };
-  T dtv_zm = T(0);   // dtau_V at (i, j, F - 1) for the z-face of level F (carried up the column)
-  stage(k0 - 2);
-  stage(k0 - 1);
-  for (int L = k0 - 1; L <= k1; ++L) {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");   // this thread's copies of level L landed
-    // every thread's copies are visible (points read their neighbours' staged values), and every
-    // thread is done with the previous level: its faces' ring slots and the stage slot L - 2
+  auto stage_b = [&](int s, int L) {
+    if (cp_ok && L >= 0 && L <= b.nz) corr_cp16(sdst + (C_VZ + s) * AR, g3 + ipxy * L);
+  };
+
+  unsigned r_pt = 0u, r_pf = 0u, r_v = 0u;      // norms as bit patterns of |x|: a NaN stays the largest
+  auto keep_max = [](unsigned& m, float x) { m = max(m, __float_as_uint(fabsf(x))); };
+
+  // ---- carried up the column
+  T vx1 = T(0), vy1 = T(0), vz1 = T(0), vx2 = T(0), vy2 = T(0), vz2 = T(0);   // dV at L - 1, L - 2
+  T mux1 = T(0), muy1 = T(0);                   // mu of this cell plus its x- / y-neighbour's at L - 1
+  T k1 = T(0), fz1 = T(0);                      // k at L - 1; Darcy flux term through the face L - 1/2
+  T txx1 = T(0), tyy1 = T(0), tzz1 = T(0), P1 = T(0), exy1 = T(0), exz1 = T(0), eyz1 = T(0);   // level L - 1
+  T txx2 = T(0), tyy2 = T(0), tzz2 = T(0), P2 = T(0), exy2 = T(0), exz2 = T(0), eyz2 = T(0);   // level L - 2
+  T tzz3 = T(0), P3 = T(0), dtv_zm = T(0);      // level L - 3
+  T rfx = T(0), rfy = T(0), rfz = T(0), Rx0 = T(0), Ry0 = T(0), Rz0 = T(0);   // the faces of level L - 2
+  const bool own_fx = own && (INNER || i > 0), own_fy = own && (INNER || j > 0);
+  const bool damped = c.damp_x != T(0) || c.damp_y != T(0) || c.damp_z != T(0);
+  const bool keep_R = damped || out.eval;
+
+  stage_a(0, k0 - 1);
+  stage_b(0, k0 - 1);
+  stage_b(1, k0);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+
+  // the interval of level L, whose slot is s = (L - k0 + 1) mod 3
+  auto level = [&](auto slot, int L) {
+    constexpr int s = decltype(slot)::value, sp = (s + 1) % 3, sm = (s + 2) % 3;   // slots of L, L + 1, L + 2
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");   // this thread's copies have landed
+    // every thread's copies and ring values are visible, and every thread is done with the interval
+    // before: the slots refilled below
     __syncthreads();
-    stage(L + 1);                                             // in flight while this level computes
-    const float(*S)[8][32] = s_in[slot(L)];
-    const float(*Sm)[8][32] = s_in[slot(L - 1)];
-    const int sl = slot(L), se = L & 1;
-    // the faces of level L - 1 read these after the cell phase: their loads go out first
-    const int F = L - 1;
-    const bool face_here = own && F >= k0 && F < k1 && in_box && F <= b.nz;
-    T rfx = T(0), rfy = T(0), rfz = T(0), Rx0 = T(0), Ry0 = T(0), Rz0 = T(0);
-    const bool fx = face_here && i > 0 && i < b.nx && j < b.ny && F < b.nz;
-    const bool fy = face_here && j > 0 && j < b.ny && i < b.nx && F < b.nz;
-    const bool fz = face_here && F > 0 && F < b.nz && i < b.nx && j < b.ny;
-    if (face_here) {
+    if (L <= ke) stage_a(sp, L + 1);
+    if (L + 2 <= ke) stage_b(sm, L + 2);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+
+    // ---------------- faces of level F = L - 2
+    const int F = L - 2;
+    const float* const dv = st + (C_DTV + s) * AR;
+    const T dtv_c = dv[0];
+    if (F >= k0 && row_own) {
+      const float* const rg = ring + sp * RL;       // ring level F
+      const T txx_l = __shfl_up_sync(0xffffffffu, txx2, 1), P_l = __shfl_up_sync(0xffffffffu, P2, 1);
+      const T exy_r = __shfl_down_sync(0xffffffffu, exy2, 1), exz_r = __shfl_down_sync(0xffffffffu, exz2, 1);
+      const T exy_u = rg[R_XY * RA + 32], eyz_u = rg[R_YZ * RA + 32];
+      const T tyy_d = rg[R_TYY * RA - 32], P_d = rg[R_P * RA - 32];
       const int q = i + ipx * j + ipxy * F;
-      if (fx) { rfx = in.rfx[q]; Rx0 = out.Rx[q]; }
-      if (fy) { rfy = in.rfy[q]; Ry0 = out.Ry[q]; }
-      if (fz) { rfz = in.rfz[q]; Rz0 = out.Rz[q]; }
+      if (own_fx) {
+        const T Fx = rfx + (txx2 - txx_l) * c.rdx + (exy_u - exy2) * c.rdy + (exz1 - exz2) * c.rdz - (P2 - P_l) * c.rdx;
+        const T R1 = Fx * c.rrho_i + c.damp_x * Rx0;
+        if (keep_R) out.Rx[q] = R1;
+        if (!out.eval) out.Vx[q] = vx2 + T(0.5) * (dv[-1] + dtv_c) * R1;
+        if (check) keep_max(r_v, Fx);
+      }
+      if (own_fy) {
+        const T Fy = rfy + (exy_r - exy2) * c.rdx + (tyy2 - tyy_d) * c.rdy + (eyz1 - eyz2) * c.rdz - (P2 - P_d) * c.rdy;
+        const T R1 = Fy * c.rrho_i + c.damp_y * Ry0;
+        if (keep_R) out.Ry[q] = R1;
+        if (!out.eval) out.Vy[q] = vy2 + T(0.5) * (dv[-kCorrW] + dtv_c) * R1;
+        if (check) keep_max(r_v, Fy);
+      }
+      if (own && F > 0) {
+        const T Fz = rfz + (exz_r - exz2) * c.rdx + (eyz_u - eyz2) * c.rdy + (tzz2 - tzz3) * c.rdz - (P2 - P3) * c.rdz;
+        const T R1 = Fz * c.rrho_i + c.damp_z * Rz0;
+        if (keep_R) out.Rz[q] = R1;
+        if (!out.eval) out.Vz[q] = vz2 + T(0.5) * (dtv_zm + dtv_c) * R1;
+        if (check) keep_max(r_v, Fz);
+      }
     }
-    // ---------------- cell and lower edges at (i, j, L). Cells are needed for the tile and its
-    // left / lower halo (tx <= 30, ty <= 6), edges for the tile and its right / upper halo
-    // (tx >= 1, ty >= 1); x-, y- and z-1 neighbours come from the stage ring.
-    T txx = T(0), tyy = T(0), tzz = T(0), P1 = T(0), exy = T(0), exz = T(0), eyz = T(0);
-    if (in_box && L >= 0 && L <= b.nz) {
-      const int q = i + ipx * j + ipxy * L;
-      const T mu_c = S[C_MU][ty][tx], vx_c = S[C_VX][ty][tx], vy_c = S[C_VY][ty][tx], vz_c = S[C_VZ][ty][tx];
-      if (tx >= 1 && ty >= 1) {
-        if (L < b.nz && i > 0 && i < b.nx && j > 0 && j < b.ny) {
-          const T m = T(0.25) * (S[C_MU][ty - 1][tx - 1] + S[C_MU][ty - 1][tx] + S[C_MU][ty][tx - 1] + mu_c);
-          exy = corr_modulus(c, m) * ((vx_c - S[C_VX][ty - 1][tx]) * c.hrdy + (vy_c - S[C_VY][ty][tx - 1]) * c.hrdx);
-        }
-        if (j < b.ny && i > 0 && i < b.nx && L > 0 && L < b.nz) {
-          const T m = T(0.25) * (Sm[C_MU][ty][tx - 1] + Sm[C_MU][ty][tx] + S[C_MU][ty][tx - 1] + mu_c);
-          exz = corr_modulus(c, m) * ((vx_c - Sm[C_VX][ty][tx]) * c.hrdz + (vz_c - S[C_VZ][ty][tx - 1]) * c.hrdx);
-        }
-        if (i < b.nx && j > 0 && j < b.ny && L > 0 && L < b.nz) {
-          const T m = T(0.25) * (Sm[C_MU][ty - 1][tx] + Sm[C_MU][ty][tx] + S[C_MU][ty - 1][tx] + mu_c);
-          eyz = corr_modulus(c, m) * ((vy_c - Sm[C_VY][ty][tx]) * c.hrdz + (vz_c - S[C_VZ][ty - 1][tx]) * c.hrdy);
+    dtv_zm = dtv_c;
+    // the next interval's faces (level L - 1): their own R and right-hand side
+    if (L - 1 >= k0 && L - 1 < ke) {
+      const int q = i + ipx * j + ipxy * (L - 1);
+      if (own_fx) rfx = in.rfx[q];
+      if (own_fy) rfy = in.rfy[q];
+      if (own && L - 1 > 0) rfz = in.rfz[q];
+      if (damped) {
+        if (own_fx) Rx0 = out.Rx[q];
+        if (own_fy) Ry0 = out.Ry[q];
+        if (own && L - 1 > 0) Rz0 = out.Rz[q];
+      }
+    }
+    if (L > ke) return;                             // (uniform) nothing above is needed
+
+    // ---------------- cell and lower edges at (i, j, L). The lowest row needs cells only, the highest
+    // edges only; the lanes of the other side's halo compute values nobody reads.
+    T txx = T(0), tyy = T(0), tzz = T(0), P = T(0), exy = T(0), exz = T(0), eyz = T(0);
+    T vx_c = T(0), vy_c = T(0), vz_c = T(0), mux = T(0), muy = T(0), k_c = T(0), fz = T(0);
+    if (L >= 0 && L < b.nz) {
+      const float* const S = st + s * AR;
+      const float* const Sp = st + sp * AR;
+      vx_c = S[C_VX * AR];
+      vy_c = S[C_VY * AR];
+      vz_c = S[C_VZ * AR];
+      const T mu_c = S[C_MU * AR];
+      if (ty >= 1) {
+        const T mu_l = S[C_MU * AR - 1], mu_d = S[C_MU * AR - kCorrW];
+        mux = mu_l + mu_c;
+        muy = mu_d + mu_c;
+        if (L >= k0) {
+          if (INNER || (i > 0 && i < b.nx && j > 0 && j < b.ny))
+            exy = corr_modulus4(c, (S[C_MU * AR - kCorrW - 1] + mu_d) + mux) *
+                  ((vx_c - S[C_VX * AR - kCorrW]) * c.hrdy + (vy_c - S[C_VY * AR - 1]) * c.hrdx);
+          if (L > 0) {
+            if (INNER || (i > 0 && i < b.nx && j < b.ny))
+              exz = corr_modulus4(c, mux1 + mux) * ((vx_c - vx1) * c.hrdz + (vz_c - S[C_VZ * AR - 1]) * c.hrdx);
+            if (INNER || (i < b.nx && j > 0 && j < b.ny))
+              eyz = corr_modulus4(c, muy1 + muy) * ((vy_c - vy1) * c.hrdz + (vz_c - S[C_VZ * AR - kCorrW]) * c.hrdy);
+          }
         }
       }
-      if (tx <= kCorrTX && ty <= kCorrTY && i < b.nx && j < b.ny && L < b.nz) {
-        const T dPt = S[C_PT][ty][tx], dPf = S[C_PF][ty][tx], cc = S[C_CC][ty][tx];
-        const T rpt = S[C_RPT][ty][tx];
-        const T gx = (S[C_VX][ty][tx + 1] - vx_c) * c.rdx, gy = (S[C_VY][ty + 1][tx] - vy_c) * c.rdy;
-        const T gz = (in.Vz[q + ipxy] - vz_c) * c.rdz;
+      if (L < ke && ty <= kCorrTY && (INNER || (i >= 0 && j >= 0 && i < b.nx && j < b.ny))) {
+        const T dPt = S[C_PT * AR], dPf = S[C_PF * AR], cc = S[C_CC * AR];
+        const T rpt = S[C_RPT * AR];
+        const T gx = (S[C_VX * AR + 1] - vx_c) * c.rdx, gy = (S[C_VY * AR + kCorrW] - vy_c) * c.rdy;
+        const T gz = (Sp[C_VZ * AR] - vz_c) * c.rdz;
         const T divV = gx + gy + gz;
         const T cpl = c.bd_rdt_a + cc;                 // beta_d alpha / dt + cc
         const T rho_pt = rpt + divV + (c.bd_rdt + cc) * dPt - cpl * dPf;
         // dP' = dP - dtau rho(dP', ...) solved for dP' (local terms implicit; the quotient only
         // scales the pseudo-step, so the fast reciprocal does)
-        const T idtp = S[C_IDTP][ty][tx];
-        const T dPt1 = __fdividef(dPt * idtp - (rpt + divV - cpl * dPf), idtp + c.bd_rdt + cc);
+        const T idtp = S[C_IDTP * AR];
+        const T dPt1 = corr_div(dPt * idtp - (rpt + divV - cpl * dPf), idtp + c.bd_rdt + cc);
         const T third = divV * T(1.0 / 3.0);
         const T bn = c.beta_n * (rho_pt - rpt);
         const T cm2 = corr_modulus(c, mu_c);
         txx = cm2 * (gx - third + bn);
         tyy = cm2 * (gy - third + bn);
         tzz = cm2 * (gz - third + bn);
-        P1 = out.eval ? dPt : dPt1;
-        if (own && L >= k0 && L < k1) {
-          // Darcy flux divergence, the largest neighbour k and dPf' (the tile's own cells)
-          const T rpf = S[C_RPF][ty][tx], kc = S[C_K][ty][tx];
-          T kmax = kc, sx = T(0), sy = T(0), sz = T(0);
-          if (i > 0) {
-            const T kn = S[C_K][ty][tx - 1];
-            kmax = fmaxf(kmax, kn);
-            sx -= (kn + kc) * (dPf - S[C_PF][ty][tx - 1]);
-          }
-          if (i < b.nx - 1) {
-            const T kn = S[C_K][ty][tx + 1];
-            kmax = fmaxf(kmax, kn);
-            sx += (kc + kn) * (S[C_PF][ty][tx + 1] - dPf);
-          }
-          if (j > 0) {
-            const T kn = S[C_K][ty - 1][tx];
-            kmax = fmaxf(kmax, kn);
-            sy -= (kn + kc) * (dPf - S[C_PF][ty - 1][tx]);
-          }
-          if (j < b.ny - 1) {
-            const T kn = S[C_K][ty + 1][tx];
-            kmax = fmaxf(kmax, kn);
-            sy += (kc + kn) * (S[C_PF][ty + 1][tx] - dPf);
-          }
-          if (L > 0) {
-            const T kn = Sm[C_K][ty][tx];
-            kmax = fmaxf(kmax, kn);
-            sz -= (kn + kc) * (dPf - Sm[C_PF][ty][tx]);
-          }
+        P = out.eval ? dPt : dPt1;
+        if (row_own) {
+          // Darcy flux divergence, the largest neighbour k and dPf' (the tile's own cells; the flux
+          // through the lower z face is the level below's upper one)
+          k_c = S[C_K * AR];
+          T kzp = T(0), sz = -fz1;
           if (L < b.nz - 1) {
-            const T kn = in.perm[q + ipxy];
-            kmax = fmaxf(kmax, kn);
-            sz += (kc + kn) * (in.Pf[q + ipxy] - dPf);
+            kzp = Sp[C_K * AR];
+            const T kf = k_c + kzp, dn = Sp[C_PF * AR] - dPf;
+            fz = kf * dn;
+            sz = fmaf(kf, dn, -fz1);
           }
-          const T divq = -(sx * c.hrdx2 + sy * c.hrdy2 + sz * c.hrdz2);
-          const T rho_pf = rpf + divq + (c.bda_B_rdt + cc) * dPf - cpl * dPt;
-          const T idtf = kmax * c.ifac_pf;
-          const T dPf1 = __fdividef(dPf * idtf - (rpf + divq - cpl * dPt), idtf + c.bda_B_rdt + cc);
-          if (!out.eval) {
-            out.Pt[q] = dPt1;
-            out.Pf[q] = dPf1;
-          }
-          if (out.res_pt) {
-            out.res_pt[q] = rho_pt;
-            out.res_pf[q] = rho_pf;
-          }
-          if (check) {
-            keep_max(r_pt, rho_pt);
-            keep_max(r_pf, rho_pf);
+          if (L >= k0 && own) {
+            const T rpf = S[C_RPF * AR];
+            T kmax = fmaxf(k_c, fmaxf(k1, kzp)), sx = T(0), sy = T(0);
+            if (INNER || i > 0) {
+              const T kn = S[C_K * AR - 1];
+              kmax = fmaxf(kmax, kn);
+              sx -= (kn + k_c) * (dPf - S[C_PF * AR - 1]);
+            }
+            if (INNER || i < b.nx - 1) {
+              const T kn = S[C_K * AR + 1];
+              kmax = fmaxf(kmax, kn);
+              sx += (k_c + kn) * (S[C_PF * AR + 1] - dPf);
+            }
+            if (INNER || j > 0) {
+              const T kn = S[C_K * AR - kCorrW];
+              kmax = fmaxf(kmax, kn);
+              sy -= (kn + k_c) * (dPf - S[C_PF * AR - kCorrW]);
+            }
+            if (INNER || j < b.ny - 1) {
+              const T kn = S[C_K * AR + kCorrW];
+              kmax = fmaxf(kmax, kn);
+              sy += (k_c + kn) * (S[C_PF * AR + kCorrW] - dPf);
+            }
+            const T divq = -(sx * c.hrdx2 + sy * c.hrdy2 + sz * c.hrdz2);
+            const T rho_pf = rpf + divq + (c.bda_B_rdt + cc) * dPf - cpl * dPt;
+            const T idtf = kmax * c.ifac_pf;
+            const T dPf1 = corr_div(dPf * idtf - (rpf + divq - cpl * dPt), idtf + c.bda_B_rdt + cc);
+            const int q = i + ipx * j + ipxy * L;
+            if (!out.eval) {
+              out.Pt[q] = dPt1;
+              out.Pf[q] = dPf1;
+            }
+            if (out.res_pt) {
+              out.res_pt[q] = rho_pt;
+              out.res_pf[q] = rho_pf;
+            }
+            if (check) {
+              keep_max(r_pt, rho_pt);
+              keep_max(r_pf, rho_pf);
+            }
           }
         }
       }
     }
-    s_cell[sl][0][ty][tx] = txx;
-    s_cell[sl][1][ty][tx] = tyy;
-    s_cell[sl][2][ty][tx] = tzz;
-    s_cell[sl][3][ty][tx] = P1;
-    s_edge[se][0][ty][tx] = exy;
-    s_edge[se][1][ty][tx] = exz;
-    s_edge[se][2][ty][tx] = eyz;
-    __syncthreads();
-    // ---------------- faces of level F = L - 1 (cells at F and F-1, edges at F and L = F+1;
-    // V and dtau_V at F from the stage slot of F, dtau_V at F - 1 carried from the level below)
-    if (face_here) {
-      const int sf = slot(F), sb = slot(F - 1), ef = F & 1, eu = se;
-      const int q = i + ipx * j + ipxy * F;
-      const T Pc = s_cell[sf][3][ty][tx];
-      const T dtv_c = Sm[C_DTV][ty][tx];
-      T Fx = T(0), Fy = T(0), Fz = T(0);
-      if (fx) {
-        Fx = rfx + (s_cell[sf][0][ty][tx] - s_cell[sf][0][ty][tx - 1]) * c.rdx +
-             (s_edge[ef][0][ty + 1][tx] - s_edge[ef][0][ty][tx]) * c.rdy +
-             (s_edge[eu][1][ty][tx] - s_edge[ef][1][ty][tx]) * c.rdz - (Pc - s_cell[sf][3][ty][tx - 1]) * c.rdx;
-        const T R1 = Fx * c.rrho_i + c.damp_x * Rx0;
-        out.Rx[q] = R1;
-        if (!out.eval) out.Vx[q] = Sm[C_VX][ty][tx] + T(0.5) * (Sm[C_DTV][ty][tx - 1] + dtv_c) * R1;
-      }
-      if (fy) {
-        Fy = rfy + (s_edge[ef][0][ty][tx + 1] - s_edge[ef][0][ty][tx]) * c.rdx +
-             (s_cell[sf][1][ty][tx] - s_cell[sf][1][ty - 1][tx]) * c.rdy +
-             (s_edge[eu][2][ty][tx] - s_edge[ef][2][ty][tx]) * c.rdz - (Pc - s_cell[sf][3][ty - 1][tx]) * c.rdy;
-        const T R1 = Fy * c.rrho_i + c.damp_y * Ry0;
-        out.Ry[q] = R1;
-        if (!out.eval) out.Vy[q] = Sm[C_VY][ty][tx] + T(0.5) * (Sm[C_DTV][ty - 1][tx] + dtv_c) * R1;
-      }
-      if (fz) {
-        Fz = rfz + (s_edge[ef][1][ty][tx + 1] - s_edge[ef][1][ty][tx]) * c.rdx +
-             (s_edge[ef][2][ty + 1][tx] - s_edge[ef][2][ty][tx]) * c.rdy +
-             (s_cell[sf][2][ty][tx] - s_cell[sb][2][ty][tx]) * c.rdz - (Pc - s_cell[sb][3][ty][tx]) * c.rdz;
-        const T R1 = Fz * c.rrho_i + c.damp_z * Rz0;
-        out.Rz[q] = R1;
-        if (!out.eval) out.Vz[q] = Sm[C_VZ][ty][tx] + T(0.5) * (dtv_zm + dtv_c) * R1;
-      }
-      if (check) {
-        keep_max(r_v, Fx);
-        keep_max(r_v, Fy);
-        keep_max(r_v, Fz);
-      }
-    }
-    // dtau_V at (i, j, L - 1), the z-face of the next level's lower pseudo-step
-    dtv_zm = (in_box && L >= 1 && L - 1 <= b.nz) ? Sm[C_DTV][ty][tx] : T(0);
+    float* const rw = ring + s * RL;
+    rw[R_TYY * RA] = tyy;
+    rw[R_P * RA] = P;
+    rw[R_XY * RA] = exy;
+    rw[R_YZ * RA] = eyz;
+    // one level up
+    tzz3 = tzz2; P3 = P2;
+    txx2 = txx1; tyy2 = tyy1; tzz2 = tzz1; P2 = P1; exy2 = exy1; exz2 = exz1; eyz2 = eyz1;
+    txx1 = txx; tyy1 = tyy; tzz1 = tzz; P1 = P; exy1 = exy; exz1 = exz; eyz1 = eyz;
+    vx2 = vx1; vy2 = vy1; vz2 = vz1;
+    vx1 = vx_c; vy1 = vy_c; vz1 = vz_c;
+    mux1 = mux; muy1 = muy; k1 = k_c; fz1 = fz;
+  };
+  for (int L = k0 - 1;; L += 3) {
+    level(std::integral_constant<int, 0>{}, L);
+    if (L + 1 > ke + 1) break;
+    level(std::integral_constant<int, 1>{}, L + 1);
+    if (L + 2 > ke + 1) break;
+    level(std::integral_constant<int, 2>{}, L + 2);
+    if (L + 3 > ke + 1) break;
   }
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");   // the last level's look-ahead copies
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");   // the last look-ahead copies
   if (check) {
-    block_max_atomic(__longlong_as_double((long long)r_pt), red + RED_PT);
-    block_max_atomic(__longlong_as_double((long long)r_pf), red + RED_PF);
-    block_max_atomic(__longlong_as_double((long long)r_v), red + RED_V);
+    block_max_atomic((double)__uint_as_float(r_pt), red + RED_PT);
+    block_max_atomic((double)__uint_as_float(r_pf), red + RED_PF);
+    block_max_atomic((double)__uint_as_float(r_v), red + RED_V);
   }
 }
 
-__global__ void __launch_bounds__(256, kCorrMinBlocks) k_corr_iteration(Box b, CorrCoef<float> c, CorrIn<float> in,
+template <class SH>
+__device__ __forceinline__ void corr_tile(const Box& b, const CorrCoef<float>& c, const CorrIn<float>& in,
+                                          const CorrOut<float>& out, int tbx, int tby, int k0, int ke,
+                                          unsigned long long* red, int check, float* corr_smem) {
+  // every point the tile computes or stages has its x- and y-neighbours inside the grid
+  const bool inner = tbx > 0 && tby > 0 && (tbx + 1) * kCorrTX + 1 < b.nx && (tby + 1) * SH::ty + 1 < b.ny;
+  if (inner) corr_tile_run<SH, true>(b, c, in, out, tbx, tby, k0, ke, red, check, corr_smem);
+  else corr_tile_run<SH, false>(b, c, in, out, tbx, tby, k0, ke, red, check, corr_smem);
+}
+
+__global__ void __launch_bounds__(CorrSingle::threads, CorrSingle::blocks) k_corr_iteration(Box b, CorrCoef<float> c, CorrIn<float> in,
                                                         CorrOut<float> out, unsigned long long* red, int check,
                                                         int zchunk) {
-  extern __shared__ __align__(16) float corr_smem[];   // kCorrSmemBytes, dynamic (above 48 KB)
+  extern __shared__ __align__(16) float corr_smem[];   // CorrSingle::smem, dynamic (above 48 KB)
   const int k0 = blockIdx.z * zchunk;
-  corr_tile(b, c, in, out, blockIdx.x, blockIdx.y, k0, min(k0 + zchunk, b.nz + 1), red, check, corr_smem);
+  corr_tile<CorrSingle>(b, c, in, out, blockIdx.x, blockIdx.y, k0, min(k0 + zchunk, b.nz), red, check, corr_smem);
 }
 
 // (iv) u <- u + delta (FP64 += FP32 correction).
@@ -488,13 +577,12 @@ void mix_update(dim3 g, dim3 bl, cudaStream_t s, Box b, const MixUpdate& u) {
 }
 void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrIn<float>& in,
                     const CorrOut<float>& out, unsigned long long* red, int check) {
-  const unsigned gx = (b.nx + 1 + kCorrTX - 1) / kCorrTX, gy = (b.ny + 1 + kCorrTY - 1) / kCorrTY;
-  // two halo levels and the first copies' latency per chunk. Measured against chunks of 64 levels:
-  // 134 -> 63 us a sweep at 96^3 (14 levels), 28 -> 7 us at 16^3, the same at 511^3
-  const int zc = march_chunk((long long)gx * gy, b.nz + 1, kCorrZChunk, kCorrMinBlocks, sm_count(), 3.0, 3.0);
-  const dim3 g(gx, gy, (unsigned)((b.nz + 1 + zc - 1) / zc));
-  cudaFuncSetAttribute(k_corr_iteration, cudaFuncAttributeMaxDynamicSharedMemorySize, kCorrSmemBytes);
-  k_corr_iteration<<<g, dim3(32, 8, 1), kCorrSmemBytes, s>>>(b, c, in, out, red, check, zc);
+  // the faces i = nx, j = ny, k = nz are walls: tiles cover the cells and their lower faces
+  const unsigned gx = (b.nx + kCorrTX - 1) / kCorrTX, gy = (b.ny + CorrSingle::ty - 1) / CorrSingle::ty;
+  const int zc = march_chunk((long long)gx * gy, b.nz, kCorrZChunk, CorrSingle::blocks, sm_count(), 3.0, 1.0);
+  const dim3 g(gx, gy, (unsigned)((b.nz + zc - 1) / zc));
+  cudaFuncSetAttribute(k_corr_iteration, cudaFuncAttributeMaxDynamicSharedMemorySize, CorrSingle::smem);
+  k_corr_iteration<<<g, dim3(32, CorrSingle::rows, 1), CorrSingle::smem, s>>>(b, c, in, out, red, check, zc);
 }
 
 
@@ -781,8 +869,7 @@ __global__ void __launch_bounds__(kMbBX * kMbBY) k_mb_points(const MixBatchInst*
 
 // Correction iteration number inner + step of the members in MB_INNER (within their budget),
 // one corr_tile per work item; the block's shared memory is reused from tile to tile.
-template <int MINB>
-__global__ void __launch_bounds__(256, MINB) k_mb_corr(const MixBatchInst* __restrict__ inst,
+__global__ void __launch_bounds__(CorrBatch::threads, CorrBatch::blocks) k_mb_corr(const MixBatchInst* __restrict__ inst,
                                                        const MixBatchStatus* __restrict__ st, int ninst,
                                                        long long t0, long long t1, int step, int nup,
                                                        int zchunk) {
@@ -817,7 +904,7 @@ __global__ void __launch_bounds__(256, MINB) k_mb_corr(const MixBatchInst* __res
     const Box b = I.b;
     unsigned long long* const ired = I.ired;
     __syncthreads();   // s_cc written
-    corr_tile(b, s_cc, ci, co, tbx, tby, k0, min(k0 + zchunk, b.nz + 1), ired, step == nup, corr_smem);
+    corr_tile<CorrBatch>(b, s_cc, ci, co, tbx, tby, k0, min(k0 + zchunk, b.nz), ired, step == nup, corr_smem);
     __syncthreads();   // the next tile's stage and rings overwrite this one's
   }
 }
@@ -953,13 +1040,9 @@ void mb_points(int grid, cudaStream_t s, int phase, const MixBatchInst* inst, co
   }
 }
 
-void mb_corr(int grid, int minb, cudaStream_t s, const MixBatchInst* inst, const MixBatchStatus* st, int ninst,
+void mb_corr(int grid, cudaStream_t s, const MixBatchInst* inst, const MixBatchStatus* st, int ninst,
              long long t0, long long t1, int step, int nup, int zchunk) {
-  if (minb == 3) {
-    k_mb_corr<3><<<grid, dim3(32, 8, 1), kCorrSmemBytes, s>>>(inst, st, ninst, t0, t1, step, nup, zchunk);
-  } else {
-    k_mb_corr<4><<<grid, dim3(32, 8, 1), kCorrSmemBytes, s>>>(inst, st, ninst, t0, t1, step, nup, zchunk);
-  }
+  k_mb_corr<<<grid, dim3(32, CorrBatch::rows, 1), CorrBatch::smem, s>>>(inst, st, ninst, t0, t1, step, nup, zchunk);
 }
 
 void mb_decide_outer(cudaStream_t s, const MixBatchInst* inst, MixBatchStatus* st, int ninst) {
@@ -982,20 +1065,14 @@ int mb_points_blocks_per_sm() {
   return (e == cudaSuccess && n > 0) ? n : 1;
 }
 
-int mb_corr_blocks_per_sm(int minb) {
+int mb_corr_blocks_per_sm() {
   int n = 0;
-  cudaError_t e;
-  if (minb == 3) {
-    cudaFuncSetAttribute(k_mb_corr<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCorrSmemBytes);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mb_corr<3>, 256, kCorrSmemBytes);
-  } else {
-    cudaFuncSetAttribute(k_mb_corr<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCorrSmemBytes);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mb_corr<4>, 256, kCorrSmemBytes);
-  }
+  cudaFuncSetAttribute(k_mb_corr, cudaFuncAttributeMaxDynamicSharedMemorySize, CorrBatch::smem);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_mb_corr, CorrBatch::threads, CorrBatch::smem);
   return (e == cudaSuccess && n > 0) ? n : 1;
 }
 
 int corr_tile_x() { return kCorrTX; }
-int corr_tile_y() { return kCorrTY; }
+int corr_tile_y() { return CorrBatch::ty; }
 
 }  // namespace pt

@@ -1,0 +1,43 @@
+"""The kernels' tile shapes, chunks and index maps at the sizes where they can go wrong (one cell more
+or less than a tile, single-cell tiles, columns shorter than a chunk, every wall): fixed-count steps of
+the solver against a plain 64-bit restatement of the same iteration on whole arrays (perf/cases.py)."""
+import os
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _cases():
+    sys.path.insert(0, os.path.join(ROOT, "perf"))
+    try:
+        import cases
+    finally:
+        sys.path.pop(0)
+    return cases
+
+
+def _worst(case, seed=3):
+    import torch
+    C = _cases()
+    got = C.run(C.prepare(case, seed))
+    torch.cuda.synchronize()
+    want = C.exact(case, seed)
+    off = {k: float((got[k].double() - want[k]).norm() / want[k].norm().clamp_min(1e-300)) for k in got}
+    return max(off.values()), off
+
+
+# tiles of 30 x 8 columns, three-slot rings, chunks chosen by size: n = 30 m + {0, 1, 2}, n < 30,
+# rows 8 m + {0, 1, 7}, depths of 1-3 levels and beyond one chunk
+@pytest.mark.parametrize("nx,ny,nz", [(3, 2, 1), (29, 7, 2), (30, 8, 3), (31, 9, 13), (61, 17, 4), (62, 24, 40),
+                                      (90, 25, 67), (121, 33, 130)])
+def test_fp32_correction_tiles(nx, ny, nz):
+    """Two rounds of 20 FP32 iterations. Bound: each iteration rounds a value some 8 times in a row
+    (2^-24 each), the iteration does not amplify them, and the update adds them once a round:
+    2 * 20 * 8 * 2^-24 = 1.9e-5."""
+    case = dict(kind="corr", nx=nx, ny=ny, nz=nz, rounds=2, iters=20, mg=0, logk=True)
+    worst, off = _worst(case)
+    assert worst < 2 * 20 * 8 * 2.0 ** -24, off
