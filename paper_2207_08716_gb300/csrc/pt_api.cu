@@ -192,8 +192,8 @@ dim3 grid_dims(const Box& b) {
 void fill_lean_coef(pt_ctx* c);
 void fill_corr_coef(pt_ctx* c);
 
-// m when the Picard relaxation weight is 1/m (2 <= m <= 64, to rounding), else 0: the
-// double-float path takes x^(1/m) by Newton's m-th root instead of exp(rel log x).
+// m when the Picard relaxation weight is 1/m (2 <= m <= 64, to rounding), else 0: x^(1/m) is then
+// taken as an m-th root instead of exp(rel log x).
 int relax_root(double rel) {
   if (!(rel > 0.0) || !std::isfinite(rel)) return 0;
   const double m = std::nearbyint(1.0 / rel);
@@ -211,7 +211,7 @@ LeanCoef<df64> lean_coef_df64(const LeanCoef<double>& L) {
   PT_DF(rphi0); PT_DF(k0); PT_DF(phi0); PT_DF(drho_g); PT_DF(ifac_pf); PT_DF(rrho_i);
   PT_DF(damp_x); PT_DF(damp_y); PT_DF(damp_z); PT_DF(rdx_r); PT_DF(rdy_r); PT_DF(rdz_r);
   PT_DF(drho_g_r); PT_DF(rho_i); PT_DF(ebg); PT_DF(mu0); PT_DF(eta0); PT_DF(R_weak);
-  PT_DF(rtau0_2); PT_DF(rGdtS); PT_DF(dtaupt_fac); PT_DF(dtauv_fac);
+  PT_DF(rtau0_2); PT_DF(rmu0); PT_DF(rGdtS); PT_DF(dtaupt_fac); PT_DF(dtauv_fac);
 #undef PT_DF
   F.compaction_on = L.compaction_on;
   F.powerlaw_on = L.powerlaw_on;
@@ -222,6 +222,8 @@ LeanCoef<df64> lean_coef_df64(const LeanCoef<double>& L) {
   F.rel_eta = L.rel_eta;
   F.root_mu = L.root_mu;
   F.root_eta = L.root_eta;
+  F.series_mu = L.series_mu;
+  F.series_eta = L.series_eta;
   return F;
 }
 
@@ -271,6 +273,9 @@ void fill_lean_coef(pt_ctx* c) {
   L.dtauv_fac = k.dtauv_fac;
   L.root_mu = relax_root(k.rel_mu);
   L.root_eta = relax_root(k.rel_eta);
+  L.rmu0 = 1.0 / k.mu0;
+  L.series_mu = root_series(L.root_mu);
+  L.series_eta = root_series(L.root_eta);
   c->fcoef = lean_coef_df64(L);
 }
 

@@ -8,6 +8,15 @@
 
 namespace pt {
 
+// The coefficients of (1 - t)^(-1/m) = 1 + t (a + t (b + t c) ...) (root_full)
+struct RootSeries {
+  double a, b, c;   // 1/m, (m + 1) / (2 m^2), (m + 1) (2 m + 1) / (6 m^3)
+};
+__host__ __device__ inline RootSeries root_series(int m) {
+  const double r = m > 0 ? 1.0 / m : 0.0;
+  return RootSeries{r, 0.5 * r * (1.0 + r), r * (1.0 + r) * (1.0 + 0.5 * r) / 3.0};
+}
+
 // Per-step scalars in the field type, pre-folded so each kernel multiplies instead of divides.
 template <class T>
 struct LeanCoef {
@@ -32,7 +41,9 @@ struct LeanCoef {
   T rtau0_2;                    // 1 / tau0^2
   T rGdtS, dtaupt_fac, dtauv_fac;
   double tau0, n_pow, rel_mu, rel_eta;
-  int root_mu, root_eta;        // m when rel = 1/m (2 <= m <= 64), else 0 (double-float roots)
+  T rmu0;                       // 1 / mu0
+  int root_mu, root_eta;        // m when rel = 1/m (2 <= m <= 64), else 0
+  RootSeries series_mu, series_eta;   // of (1 - t)^(-1/m) (pt_lean_body.cuh)
 };
 
 template <class T>

@@ -68,13 +68,49 @@ __device__ inline double rcp_pseudo(double x) {
 }
 __device__ inline float rcp_pseudo(float x) { return __frcp_rn(x); }
 
-// 1 / x to rounding accuracy for the coefficients that set the fixed point (x > 0, normal):
-// two Newton steps r' = r + r (1 - x r) on the hardware's approximate reciprocal.
+// 1 / x to rounding accuracy for the coefficients that set the fixed point (x > 0, normal): one
+// third-order step r (1 + e + e^2), e = 1 - x r, on the hardware's approximate reciprocal r (good to
+// about 2^-20, so e^3 is below the rounding): three FP64 instructions, where two Newton steps take four.
 __device__ inline double rcp_full(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// sqrt(x), x > 0 and normal, from the hardware's approximate reciprocal root r: s = x r,
+// e = 1 - x r^2, sqrt(x) = s (1 - e)^(-1/2) = s (1 + e/2 + 3 e^2 / 8 + ...): five FP64 instructions.
+__device__ inline double sqrt_full(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double s = x * r, e = fma(-s, r, 1.0);
+  return fma(s * e, fma(0.375, e, 0.5), s);
+}
+
+// x^(1/m) for 3 <= m <= 64 with rx = 1/x: from the FP32 root y (|t| <= 64 2^-20 for
+// t = (x - y^m) / x) by the series above; the first dropped term is below 2^-57. y^m by square and
+// multiply, m is uniform. For m = 10 13 FP64 instructions, where exp(log x / 10) takes some 45.
+// x far from 1 (never near a solution) falls back to the library functions, a NaN stays one.
+__device__ inline double root_full(double x, double rx, int m, const RootSeries& k) {
+  const int e2 = (__double2hiint(x) >> 20) - 1023;      // a negative x falls outside too
+  if (e2 < -60 || e2 > 60) return exp(k.a * log(x));
+  float lg, y0;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"((float)x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(lg * (float)k.a));
+  const double y = (double)y0;
+  int e = m;
+  double b = y;
+  while (!(e & 1)) {
+    b *= b;
+    e >>= 1;
+  }
+  double ym = b;
+  for (e >>= 1; e; e >>= 1) {
+    b *= b;
+    if (e & 1) ym *= b;
+  }
+  const double t = (x - ym) * rx;
+  return fma(y, t * fma(t, fma(t, k.c, k.b), k.a), y);
 }
 
 // ---- the same operations in double-float (PT_DF64): one Newton step from the FP32 seed
@@ -120,21 +156,27 @@ __device__ inline T from_d(double x) { return T(x); }
 __device__ inline double tdiv(double a, double b) { return a / b; }
 __device__ inline df64 tdiv(df64 a, df64 b) { return a * df_rcp(b); }
 
-__device__ inline double tmax(double a, double b) { return fmax(a, b); }
-__device__ inline df64 tmax(df64 a, df64 b) { return a < b ? b : a; }
-
-// x^rel of the log-space Picard relaxation (x > 0). FP64: sqrt for rel = 1/2, else
-// exp(rel log x). Double-float: the square root for rel = 1/2, Newton's m-th root for
-// rel = 1/m (root = m, set on the host), else exp(rel log x) in FP64.
-__device__ inline double relax_pow(double x, double rel, int /*root*/) {
-  return rel == 0.5 ? sqrt(x) : exp(rel * log(x));
+// x^rel of the log-space Picard relaxation (x > 0, rx = 1/x): the square root for rel = 1/2, the
+// m-th root for rel = 1/m (root = m, set on the host), else exp(rel log x) in FP64.
+__device__ inline double relax_pow(double x, double rx, double rel, int root, const RootSeries& k) {
+  if (root == 2) return sqrt_full(x);
+  if (root > 2) return root_full(x, rx, root, k);
+  return exp(rel * log(x));
 }
-__device__ inline df64 relax_pow(df64 x, double rel, int root) {
+__device__ inline df64 relax_pow(df64 x, df64 /*rx*/, double rel, int root, const RootSeries& /*k*/) {
   if (root == 2) return df_sqrt(x);
   if (root > 2) return df_root(x, root);
   return df64(exp(rel * log((double)x)));
 }
 
+// max of |values| whose NaN is the largest, through bit patterns (off the FP64 pipe)
+__device__ inline double abs_max(double a, double b) {
+  const unsigned long long m = 0x7fffffffffffffffull;
+  const unsigned long long ia = (unsigned long long)__double_as_longlong(a) & m;
+  const unsigned long long ib = (unsigned long long)__double_as_longlong(b) & m;
+  return __longlong_as_double((long long)(ia > ib ? ia : ib));
+}
+__device__ inline df64 abs_max(df64 a, df64 b) { return a < b ? b : a; }   // positive values; drops a NaN
 
 }  // namespace lean_detail
 
@@ -422,15 +464,18 @@ __device__ __forceinline__ void lean_picard_point(const Box& b, const LeanCoef<T
       den = p == 2.0 ? T(1.0) + x2 : from_d<T>(1.0 + exp(0.5 * p * log(to_d(x2))));
     }
     const T mu_old = mu[q], eta_old = eta[q];
-    const T x_mu = tdiv(c.mu0, den * mu_old);                        // mu* / mu
-    const T mu_new = mu_old * relax_pow(x_mu, c.rel_mu, c.root_mu);
+    const T D = den * mu_old;
+    const T x_mu = c.mu0 * rcp_full(D), rx_mu = D * c.rmu0;          // mu* / mu and its inverse
+    const T mu_new = mu_old * relax_pow(x_mu, rx_mu, c.rel_mu, c.root_mu, c.series_mu);
     const T R = (in.Pf1[q] > in.Pt1[q]) ? c.R_weak : T(1.0);
     // Eq. 26: eta* = eta0 mu / phi R (with the relaxed mu), relaxed the same way
-    const T x_eta = tdiv(c.eta0 * mu_new * R, in.phi1[q] * eta_old);
-    m = to_d(tmax(tmax(x_mu, rcp_full(x_mu)), tmax(x_eta, rcp_full(x_eta))));
-    if (!(x_mu == x_mu && x_eta == x_eta)) m = to_d(x_mu) + to_d(x_eta);   // NaN stays NaN (fmax drops it)
+    const T x_eta = c.eta0 * mu_new * R * rcp_full(in.phi1[q] * eta_old), rx_eta = rcp_full(x_eta);
+    m = to_d(abs_max(abs_max(x_mu, rx_mu), abs_max(x_eta, rx_eta)));
+    if constexpr (LeanRecompute<T>::value) {
+      if (!(x_mu == x_mu && x_eta == x_eta)) m = to_d(x_mu) + to_d(x_eta);   // NaN stays NaN
+    }
     mu[q] = mu_new;
-    eta[q] = eta_old * relax_pow(x_eta, c.rel_eta, c.root_eta);
+    eta[q] = eta_old * relax_pow(x_eta, rx_eta, c.rel_eta, c.root_eta, c.series_eta);
   }
 }
 
