@@ -129,22 +129,22 @@ namespace {
 
 enum KernelId { K_PERM, K_CENTRES, K_EDGES, K_POROSITY, K_FACES, K_PICARD, K_BEGIN, K_INIT_VISC,
                 K_RESIDUAL_FACES, K_LEAN_CELLS, K_LEAN_FACES, K_LEAN_PICARD, K_LEAN_COEF, K_LEAN_BEGIN,
-                K_LEAN_K0, K_MIX_PREP, K_MIX_FACES, K_MIX_COEF, K_CORR_ITER,
+                K_LEAN_K0, K_MIX_PREP, K_MIX_FACES, K_STRESSES, K_CORR_ITER,
                 K_MIX_UPDATE, K_ADJ_PREP, K_ADJ_CELLS, K_ADJ_FACES, K_ADJ_CARRY, K_DF_CELLS, K_DF_FACES,
                 K_DF_PICARD, K_DF_COEF, K_DF_BEGIN, K_DF_K0, K_DF_CONVERT, K_ADJ_EDGES_PL, K_ADJ_CELLS_PL,
-                K_ADJ_FACES_PL, K_MG_FINE, K_MG_COARSE, K_MG_TRANSFER, K_MIX_EDGES, K_MIX_POROSITY, K_COUNT };
+                K_ADJ_FACES_PL, K_MG_FINE, K_MG_COARSE, K_MG_TRANSFER, K_MIX_POROSITY, K_COUNT };
 const char* const kKernelNames[K_COUNT] = {"k_perm", "k_centres", "k_edges", "k_porosity", "k_faces",
                                            "k_picard", "k_begin_step", "k_init_visc",
                                            "k_residual_faces", "k_lean_cells", "k_lean_faces",
                                            "k_lean_picard", "k_lean_coef", "k_lean_begin", "k_lean_k0",
-                                           "k_mix_prepare", "k_mix_res_faces", "k_mix_coef",
+                                           "k_mix_prepare", "k_mix_faces", "k_lean_stresses",
                                            "k_corr_iteration", "k_mix_update",
                                            "k_adj_prep", "k_adj_cells", "k_adj_faces", "k_adj_carry",
                                            "k_lean_cells_df64", "k_lean_faces_df64", "k_lean_picard_df64",
                                            "k_lean_coef_df64", "k_lean_begin_df64", "k_lean_k0_df64",
                                            "k_df64_convert", "k_adj_edges_pl", "k_adj_cells_pl",
                                            "k_adj_faces_pl", "k_corr_iteration_mg_fine",
-                                           "k_corr_iteration_mg_coarse", "k_mg_transfer", "k_mix_edges",
+                                           "k_corr_iteration_mg_coarse", "k_mg_transfer",
                                            "k_mix_porosity"};
 
 cudaEvent_t pooled_event(pt_ctx* c) {
@@ -208,7 +208,7 @@ LeanCoef<df64> lean_coef_df64(const LeanCoef<double>& L) {
   PT_DF(rdx); PT_DF(rdy); PT_DF(rdz); PT_DF(hrdx); PT_DF(hrdy); PT_DF(hrdz);
   PT_DF(hrdx2); PT_DF(hrdy2); PT_DF(hrdz2); PT_DF(buoy_dz); PT_DF(bd_rdt); PT_DF(bda_B_rdt);
   PT_DF(alpha); PT_DF(alpha_B); PT_DF(bd_rdt_a); PT_DF(beta_n); PT_DF(beta_phi); PT_DF(dt);
-  PT_DF(rphi0); PT_DF(k0); PT_DF(phi0); PT_DF(drho_g); PT_DF(ifac_pf); PT_DF(rrho_i);
+  PT_DF(rphi0); PT_DF(k0); PT_DF(k0r3); PT_DF(phi0); PT_DF(drho_g); PT_DF(ifac_pf); PT_DF(rrho_i);
   PT_DF(damp_x); PT_DF(damp_y); PT_DF(damp_z); PT_DF(rdx_r); PT_DF(rdy_r); PT_DF(rdz_r);
   PT_DF(drho_g_r); PT_DF(rho_i); PT_DF(ebg); PT_DF(mu0); PT_DF(eta0); PT_DF(R_weak);
   PT_DF(rtau0_2); PT_DF(rmu0); PT_DF(rGdtS); PT_DF(dtaupt_fac); PT_DF(dtauv_fac);
@@ -255,6 +255,7 @@ void fill_lean_coef(pt_ctx* c) {
   L.dt = k.dt;
   L.rphi0 = k.rphi0;
   L.k0 = k.k0;
+  L.k0r3 = k.k0 * k.rphi0 * k.rphi0 * k.rphi0;
   L.phi0 = k.phi0;
   L.drho_g = p.rhof_g - p.rhos_g;
   L.ifac_pf = 1.0 / k.dtaupf_fac;
@@ -676,6 +677,16 @@ void mg_vcycle(pt_ctx* c, int l) {
   for (int s = 0; s < kMgNu2; ++s) mg_sweep(c, l, c->mg_smooth[l], 0, 0);
 }
 
+// Zeroes `count` arrays of `bytes` bytes, `stride` bytes apart: one launch where the stride is a
+// pitch the runtime takes (below 2 GiB), else one per array.
+void zero_arrays(void* first, size_t stride, size_t bytes, int count, cudaStream_t s) {
+  if (stride < ((size_t)1 << 31) - 1) {
+    cudaMemset2DAsync(first, stride, 0, bytes, count, s);
+    return;
+  }
+  for (int i = 0; i < count; ++i) cudaMemsetAsync((char*)first + i * stride, 0, bytes, s);
+}
+
 // One outer iteration of the mixed-precision path (see pt_mixed_kernels.cu): FP64 residuals
 // and Picard update at u, then up to n_in FP32 PT iterations on the correction (stopping early
 // at a relative drop kInnerRtol when early_exit), u <- u + delta, FP64 porosity update.
@@ -683,27 +694,24 @@ void mg_vcycle(pt_ctx* c, int l) {
 // (then no correction is run).
 int mixed_outer(pt_ctx* c, int n_in, bool early_exit, pt_report* outer, bool* converged, int* inner_done) {
   const Box& b = c->box;
-  const Coef& k = c->coef;
   const dim3 bl = block_dims(), gr = grid_dims(b);
   const int a = c->cur;
   *converged = false;
   *inner_done = 0;
   cudaMemsetAsync(c->red, 0, RED_N * sizeof(unsigned long long), c->stream);
-  // (i) FP64 residuals at u, frozen coefficients of the correction problem
-  PT_LAUNCH(c, K_PERM, k_perm<<<gr, bl, 0, c->stream>>>(b, k, c->phi[a], c->logk, c->perm, c->rog));
-  MixPrepIn pin{c->Vx, c->Vy, c->Vz, c->Pt[a], c->Pf[a], c->phi[a], c->mu, c->eta, c->perm, c->Pto,
-                c->Pfo, c->txxo, c->tyyo, c->tzzo};
-  MixPrepOut pout{c->s_txx, c->s_tyy, c->s_tzz, c->m_rpt, c->m_rpf, c->m_cc, c->m_perm, c->m_idtp};
+  // (i) FP64 residuals at u, frozen coefficients of the correction problem; (ii) Picard update
+  const LeanCoef<double>& k = c->lcoef;
+  PT_LAUNCH(c, K_PERM, mix_perm(gr, bl, c->stream, b, k, c->phi[a], c->logk, c->perm));
+  const MixPrepIn pin{StressIn{c->Vx, c->Vy, c->Vz, c->mu, c->txxo, c->tyyo, c->tzzo, c->txyo, c->txzo, c->tyzo},
+                      c->Pt[a], c->Pf[a], c->phi[a], c->eta, c->perm, c->Pto, c->Pfo};
+  const MixPrepOut pout{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz,
+                        c->m_rpt, c->m_rpf, c->m_cc, c->m_perm, c->m_idtp};
   PT_LAUNCH(c, K_MIX_PREP, mix_prepare(gr, bl, c->stream, b, k, pin, pout, c->red));
-  EdgeIn ei{c->Vx, c->Vy, c->Vz, c->mu, c->txyo, c->txzo, c->tyzo};
-  EdgeOut eo{c->s_txy, c->s_txz, c->s_tyz};
-  PT_LAUNCH(c, K_MIX_EDGES, mix_edges(gr, bl, c->stream, b, k, ei, eo));
-  MixFaceIn fin{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz, c->Pt[a], c->phi[a]};
-  PT_LAUNCH(c, K_MIX_FACES, mix_res_faces(gr, bl, c->stream, b, k, fin, c->m_rfx, c->m_rfy, c->m_rfz, c->red));
-  // (ii) Picard update of mu, eta from the stresses at u
-  LeanPicardIn<double> pi{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz, c->phi[a],
-                          c->Pt[a], c->Pf[a]};
-  PT_LAUNCH(c, K_LEAN_PICARD, lean_picard<double>(gr, bl, c->stream, b, c->lcoef, pi, c->mu, c->eta, c->red));
+  const MixFaceIn fin{LeanPicardIn<double>{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz, c->phi[a],
+                                           c->Pt[a], c->Pf[a]},
+                      c->mu, c->eta};
+  const MixFaceOut fout{c->m_rfx, c->m_rfy, c->m_rfz, c->m_mu, c->m_dtvc};
+  PT_LAUNCH(c, K_MIX_FACES, mix_faces(gr, bl, c->stream, b, k, fin, fout, c->red));
   if (cudaGetLastError() != cudaSuccess) return PT_ECUDA;
   int rc = read_report(c, outer);
   if (rc != PT_OK) return rc;
@@ -723,14 +731,12 @@ int mixed_outer(pt_ctx* c, int n_in, bool early_exit, pt_report* outer, bool* co
     c->mix_prev = r;
   }
   const double target = (c->num.inner_rtol > 0 ? c->num.inner_rtol : kInnerRtol) * report_max(outer);
-  // (iii) FP32 PT on the correction, from delta = 0, R = 0
-  MixCoefOut mco{c->m_mu, c->m_dtvc};
-  PT_LAUNCH(c, K_MIX_COEF, mix_coef(gr, bl, c->stream, b, k, c->mu, mco));
-  const size_t fb = (size_t)b.n * sizeof(float);
-  // both correction-velocity buffers: the wall faces, never written by the iteration, stay zero
-  float* zero[] = {c->m_dVx[0], c->m_dVy[0], c->m_dVz[0], c->m_dVx[1], c->m_dVy[1], c->m_dVz[1],
-                   c->m_dPt[0], c->m_dPf[0], c->m_Rx, c->m_Ry, c->m_Rz};
-  for (float* z : zero) cudaMemsetAsync(z, 0, fb, c->stream);
+  // (iii) FP32 PT on the correction, from delta = 0 in buffer 0 (slots 10, 12, .. 18 of the FP32
+  // arrays; the wall faces of either buffer are never written and stay zero) and R = 0 (undamped
+  // V-cycle sweeps do not read R)
+  const size_t fb = (size_t)b.n * sizeof(float), fs = (size_t)(c->m_dVx[1] - c->m_dVx[0]) * sizeof(float);
+  zero_arrays(c->m_dVx[0], 2 * fs, fb, 5, c->stream);
+  if (c->mg_L < 2) zero_arrays(c->m_Rx, fs, fb, 3, c->stream);
   int d = 0;
   const int nup = c->num.nup;
   if (c->mg_L >= 2) {
@@ -773,17 +779,15 @@ int mixed_outer(pt_ctx* c, int n_in, bool early_exit, pt_report* outer, bool* co
     }
   }
   // (iv) u <- u + delta in FP64, then the FP64 porosity time integration (Eq. 22, log space)
-  MixUpdate mu{c->Vx, c->Vy, c->Vz, c->Pt[a], c->Pf[a], c->m_dVx[d], c->m_dVy[d], c->m_dVz[d], c->m_dPt[d], c->m_dPf[d],
+  const int n = 1 - a;   // the new pressures and porosity go to the other buffers
+  MixUpdate mu{c->Vx, c->Vy, c->Vz, c->Pt[a], c->Pf[a], c->Pt[n], c->Pf[n], c->m_dVx[d], c->m_dVy[d], c->m_dVz[d], c->m_dPt[d], c->m_dPf[d],
                c->mix_omega};
   PT_LAUNCH(c, K_MIX_UPDATE, mix_update(gr, bl, c->stream, b, mu));
   PT_LAUNCH(c, K_MIX_POROSITY,
             mix_porosity(gr, bl, c->stream, b, k,
-                         MixPorosity{c->Vx, c->Vy, c->Vz, c->phi[a], c->Pt[a], c->Pf[a], c->Pto, c->Pfo, c->Lo,
-                                     c->eta, c->phi[1 - a]}));
-  // Pt, Pf stay in buffer a; phi moves to 1 - a: copy the pressures along so cur stays paired
-  cudaMemcpyAsync(c->Pt[1 - a], c->Pt[a], (size_t)b.n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
-  cudaMemcpyAsync(c->Pf[1 - a], c->Pf[a], (size_t)b.n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
-  c->cur = 1 - a;
+                         MixPorosity{c->Vx, c->Vy, c->Vz, c->phi[a], c->Pt[n], c->Pf[n], c->Pto, c->Pfo, c->Lo,
+                                     c->eta, c->phi[n]}));
+  c->cur = n;
   return cuda_status(cudaGetLastError());
 }
 
@@ -809,6 +813,9 @@ int step_begin_launch(pt_ctx* c) {
     LeanBeginIn<double> bi{c->Pt[0], c->Pf[0], c->phi[0], c->mu, c->logk ? c->K0 : nullptr};
     LeanBeginOut<double> bo{c->Pto, c->Pfo, c->phio, c->Eo, c->iEo, c->lw[0], c->lperm[0]};
     PT_LAUNCH(c, K_LEAN_BEGIN, lean_begin<double>(grid_dims(b), block_dims(), c->stream, b, c->lcoef, bi, bo, c->red));
+  } else if (c->mixed) {   // Lo holds the old porosity (its integration needs no logarithm)
+    PT_LAUNCH(c, K_BEGIN, mix_begin(grid_dims(b), block_dims(), c->stream, b, c->Pt[0], c->Pf[0], c->phi[0], c->mu,
+                                    c->Pto, c->Pfo, c->Lo, c->red));
   } else {
     PT_LAUNCH(c, K_BEGIN, k_begin_step<<<grid_dims(b), block_dims(), 0, c->stream>>>(
                                b, c->Pt[0], c->Pf[0], c->phi[0], c->mu, c->Pto, c->Pfo, c->Lo, c->red));
@@ -1108,6 +1115,15 @@ int pt_step_end(pt_ctx* c) {
   int rc = sync_current_to_caller(c);
   if (rc != PT_OK) return rc;
   const Box& b = c->box;
+  if (c->lean || c->mixed) {
+    const StressIn si{c->Vx, c->Vy, c->Vz, c->mu, c->txxo, c->tyyo, c->tzzo, c->txyo, c->txzo, c->tyzo};
+    PT_LAUNCH(c, K_STRESSES,
+              lean_stresses(grid_dims(b), block_dims(), c->stream, b, c->lcoef, si,
+                            StressCentre{c->Pt[0], c->Pf[0], c->Pto, c->Pfo, c->phi[0], c->eta},
+                            StressOut{c->txx, c->tyy, c->tzz, c->txy, c->txz, c->tyz}));
+    c->dt_cum += c->num.dt;
+    return cuda_status(cudaGetLastError());
+  }
   CentreIn ci{c->Vx, c->Vy, c->Vz, c->Pt[0], c->Pf[0], c->phi[0], c->mu, c->eta, c->perm,
               c->Pto, c->Pfo, c->txxo, c->tyyo, c->tzzo};
   CentreOut co{nullptr, nullptr, c->txx, c->tyy, c->tzz};
@@ -1426,7 +1442,6 @@ void fill_mix_inst(pt_batch* B, int m, long long base, long long cbase) {
   pt_ctx* c = B->ctx[m];
   MixBatchInst& I = B->h_minst[m];
   I.b = c->box;
-  I.k = c->coef;
   I.lc = c->lcoef;
   I.cc = c->ccoef;
   I.Vx = c->Vx; I.Vy = c->Vy; I.Vz = c->Vz;
@@ -1435,7 +1450,7 @@ void fill_mix_inst(pt_batch* B, int m, long long base, long long cbase) {
     I.dVx[a] = c->m_dVx[a]; I.dVy[a] = c->m_dVy[a]; I.dVz[a] = c->m_dVz[a];
     I.dPt[a] = c->m_dPt[a]; I.dPf[a] = c->m_dPf[a];
   }
-  I.mu = c->mu; I.eta = c->eta; I.perm = c->perm; I.rog = c->rog; I.Pto = c->Pto; I.Pfo = c->Pfo; I.Lo = c->Lo;
+  I.mu = c->mu; I.eta = c->eta; I.perm = c->perm; I.Pto = c->Pto; I.Pfo = c->Pfo; I.Lo = c->Lo;
   I.logk = c->logk;
   I.txxo = c->txxo; I.tyyo = c->tyyo; I.tzzo = c->tzzo; I.txyo = c->txyo; I.txzo = c->txzo; I.tyzo = c->tyzo;
   I.s_txx = c->s_txx; I.s_tyy = c->s_tyy; I.s_tzz = c->s_tzz; I.s_txy = c->s_txy; I.s_txz = c->s_txz;

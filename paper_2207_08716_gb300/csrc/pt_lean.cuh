@@ -29,6 +29,7 @@ struct LeanCoef {
   T bd_rdt_a;                   // beta_d alpha / dt
   T beta_n, beta_phi, dt;
   T rphi0, k0, phi0, drho_g;    // 1 / phi0, k0, phi0, (rho_f - rho_s) g
+  T k0r3;                       // k0 / phi0^3
   T ifac_pf;                    // 1 / (cfl_pf h^2 (1 + beta_d B / alpha)): 1/dtau_Pf = kmax * ifac_pf
   T rrho_i, damp_x, damp_y, damp_z;
   T rdx_r, rdy_r, rdz_r, drho_g_r;  // 1/(d rho_i), (rho_f - rho_s) g / rho_i: the momentum residual over rho_i
@@ -79,6 +80,17 @@ struct LeanCoefOut {
   T *em2_xy, *em2_xz, *em2_yz, *eb_xy, *eb_xz, *eb_yz, *toa_xy, *toa_xz, *toa_yz;
   T *dtv_x, *dtv_y, *dtv_z;
 };
+// End-of-step stresses and the FP32 form's outer phases: velocities, mu and the old stresses; the
+// centre fields enter through the numerical divergence of Eq. 17 when beta_n != 0.
+struct StressIn {
+  const double *Vx, *Vy, *Vz, *mu, *txxo, *tyyo, *tzzo, *txyo, *txzo, *tyzo;
+};
+struct StressCentre {
+  const double *Pt, *Pf, *Pto, *Pfo, *phi, *eta;
+};
+struct StressOut {
+  double *txx, *tyy, *tzz, *txy, *txz, *tyz;
+};
 template <class T>
 struct LeanBeginIn {
   const T *Pt, *Pf, *phi, *mu, *K0;
@@ -104,6 +116,9 @@ void lean_coef(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, c
 template <class T>
 void lean_begin(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanBeginIn<T>& in,
                 const LeanBeginOut<T>& out, unsigned long long* red);
+// The stresses of the current state (Eq. 21), centres and edges (end of a step).
+void lean_stresses(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c, const StressIn& in,
+                   const StressCentre& ce, const StressOut& out);
 template <class T>
 void lean_k0(dim3 gr, dim3 bl, cudaStream_t st, Box b, double k0, const double* logk, T* K0);
 

@@ -492,6 +492,58 @@ __device__ inline T lean_edge_mean_mu_xy(const Box& b, const T* mu, long long q,
   return s * T(n == 4 ? 0.25 : (n == 2 ? 0.5 : 1.0));
 }
 
+// Maxwell stress (Eq. 21) of viscosity m, xi = m rG: tau = tau_o a + M edot with a = xi / (1 + xi),
+// M = 2 m / (1 + xi); for an edge m is given as the sum of its four centres' mu.
+struct Maxwell {
+  double a, M;
+};
+__device__ __forceinline__ Maxwell maxwell(double m, double rG) {
+  const double s = lean_detail::rcp_full(fma(m, rG, 1.0));
+  return Maxwell{1.0 - s, 2.0 * m * s};
+}
+__device__ __forceinline__ Maxwell maxwell4(double sum, double rG) {
+  const double s = lean_detail::rcp_full(fma(sum, 0.25 * rG, 1.0));
+  return Maxwell{1.0 - s, 0.5 * sum * s};
+}
+
+// Shear stresses on the three lower edges of (i, j, k), zero on boundary edges unless a background
+// shear is applied (Eqs. 32-33).
+__device__ __forceinline__ void stress_edges_point(const Box& b, const LeanCoef<double>& c, const StressIn& in,
+                                                   double* __restrict__ txy, double* __restrict__ txz,
+                                                   double* __restrict__ tyz, int i, int j, int k) {
+  if (i > b.nx || j > b.ny || k > b.nz) return;
+  const long long q = cidx(b, i, j, k);
+  const long long px = b.px, pxy = b.pxy;
+  if (k < b.nz) {
+    double t = 0.0;
+    if (i > 0 && i < b.nx && j > 0 && j < b.ny) {
+      const Maxwell m = maxwell4((in.mu[q - 1 - px] + in.mu[q - px]) + (in.mu[q - 1] + in.mu[q]), c.rGdtS);
+      const double e = fma(in.Vx[q] - in.Vx[q - px], c.hrdy, fma(in.Vy[q] - in.Vy[q - 1], c.hrdx, c.ebg));
+      t = fma(in.txyo[q], m.a, m.M * e);
+    } else if (c.bg_on) {   // wall edge: background part only
+      const Maxwell m = maxwell(lean_edge_mean_mu_xy(b, in.mu, q, i, j), c.rGdtS);
+      t = fma(in.txyo[q], m.a, m.M * c.ebg);
+    }
+    txy[q] = t;
+  }
+  if (j < b.ny) {
+    double t = 0.0;
+    if (i > 0 && i < b.nx && k > 0 && k < b.nz) {
+      const Maxwell m = maxwell4((in.mu[q - 1 - pxy] + in.mu[q - pxy]) + (in.mu[q - 1] + in.mu[q]), c.rGdtS);
+      t = fma(in.txzo[q], m.a, m.M * fma(in.Vx[q] - in.Vx[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - 1]) * c.hrdx));
+    }
+    txz[q] = t;
+  }
+  if (i < b.nx) {
+    double t = 0.0;
+    if (j > 0 && j < b.ny && k > 0 && k < b.nz) {
+      const Maxwell m = maxwell4((in.mu[q - px - pxy] + in.mu[q - pxy]) + (in.mu[q - px] + in.mu[q]), c.rGdtS);
+      t = fma(in.tyzo[q], m.a, m.M * fma(in.Vy[q] - in.Vy[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - px]) * c.hrdy));
+    }
+    tyz[q] = t;
+  }
+}
+
 // Coefficient refresh at box index (i, j, k).
 template <class T>
 __device__ __forceinline__ void lean_coef_point(const Box& b, const LeanCoef<T>& c, const LeanCoefIn<T>& in,

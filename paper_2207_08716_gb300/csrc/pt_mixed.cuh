@@ -8,25 +8,30 @@
 namespace pt {
 
 struct MixPrepIn {
-  const double *Vx, *Vy, *Vz, *Pt, *Pf, *phi, *mu, *eta, *perm, *Pto, *Pfo, *txxo, *tyyo, *tzzo;
+  StressIn s;
+  const double *Pt, *Pf, *phi, *eta, *perm, *Pto, *Pfo;
 };
 struct MixPrepOut {
-  double *txx, *tyy, *tzz;                                  // FP64 stresses at u
+  double *txx, *tyy, *tzz, *txy, *txz, *tyz;                // FP64 stresses at u
   float *r_pt, *r_pf, *cc, *perm, *idtp;
 };
 struct MixFaceIn {
-  const double *txx, *tyy, *tzz, *txy, *txz, *tyz, *Pt, *phi;
+  LeanPicardIn<double> s;                                   // stresses, phi, Pt, Pf at u
+  double *mu, *eta;                                         // updated in place
 };
-struct MixCoefOut {
+struct MixFaceOut {
+  float *rfx, *rfy, *rfz;
   float *mu;                                                // mu at centres (FP32)
   float *dtvc;                                              // velocity pseudo-step fac / mu at centres
 };
 struct MixPorosity {       // the porosity integration of Eq. 22 at the corrected state
-  const double *Vx, *Vy, *Vz, *phi, *Pt1, *Pf1, *Pto, *Pfo, *Lo, *eta;
+  const double *Vx, *Vy, *Vz, *phi, *Pt1, *Pf1, *Pto, *Pfo, *phio, *eta;
   double* phi1;
 };
 struct MixUpdate {
-  double *Vx, *Vy, *Vz, *Pt, *Pf;
+  double *Vx, *Vy, *Vz;
+  const double *Pt, *Pf;
+  double *Pt1, *Pf1;        // the pressures' other buffer
   const float *dVx, *dVy, *dVz, *dPt, *dPf;
   double omega;             // u <- u + omega delta
 };
@@ -84,13 +89,16 @@ struct MgLevel {
   float *res_pt, *res_pf;                          // cell residuals of an evaluation sweep
 };
 
-void mix_prepare(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const MixPrepIn& in,
+// Step start: Pto, Pfo, phio and max(mu).
+void mix_begin(dim3 g, dim3 bl, cudaStream_t s, Box b, const double* Pt, const double* Pf, const double* phi,
+               const double* mu, double* Pto, double* Pfo, double* phio, unsigned long long* red);
+void mix_perm(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk,
+              double* perm);
+void mix_prepare(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in,
                  const MixPrepOut& out, unsigned long long* red);
-void mix_res_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const MixFaceIn& in, float* rfx,
-                   float* rfy, float* rfz, unsigned long long* red);
-void mix_coef(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const double* mu, const MixCoefOut& out);
-void mix_edges(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const EdgeIn& in, const EdgeOut& out);
-void mix_porosity(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const MixPorosity& p);
+void mix_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in,
+               const MixFaceOut& out, unsigned long long* red);
+void mix_porosity(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p);
 void mix_update(dim3 g, dim3 bl, cudaStream_t s, Box b, const MixUpdate& u);
 // One fused FP32 correction iteration over the whole grid (z-marching tiles, see the kernel).
 void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrIn<float>& in,
@@ -132,10 +140,9 @@ enum { MB_PH_PERM = 0, MB_PH_PREP = 1, MB_PH_FACES = 2, MB_PH_INIT = 3, MB_PH_UP
 
 struct MixBatchInst {
   Box b;
-  Coef k;                                   // FP64 residuals, porosity update
-  LeanCoef<double> lc;                      // Picard update
+  LeanCoef<double> lc;                      // FP64 outer phases
   CorrCoef<float> cc;                       // FP32 correction iteration
-  double *Vx, *Vy, *Vz, *Pt[2], *Pf[2], *phi[2], *mu, *eta, *perm, *rog, *Pto, *Pfo, *Lo;
+  double *Vx, *Vy, *Vz, *Pt[2], *Pf[2], *phi[2], *mu, *eta, *perm, *Pto, *Pfo, *Lo;   // Lo: phi of the old step
   const double* logk;
   double *txxo, *tyyo, *tzzo, *txyo, *txzo, *tyzo;
   double *s_txx, *s_tyy, *s_tzz, *s_txy, *s_txz, *s_tyz;

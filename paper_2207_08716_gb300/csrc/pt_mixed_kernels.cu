@@ -4,8 +4,8 @@
 // One outer iteration at the FP64 state u = (V, Pt, Pf, phi; mu, eta):
 //   (i)   FP64 residuals of Eqs. 17-19 at u: r_Pt (numerical div V), r_Pf (fluid pressure),
 //         r_F (momentum) — stored in FP32 as the right-hand side of the correction problem —
-//         and their max-norms (k_mix_prepare, k_edges, k_mix_res_faces);
-//   (ii)  FP64 Picard update of mu, eta (Eqs. 24-26) from the stresses at u;
+//         and their max-norms (k_mix_perm, k_mix_prepare, k_mix_faces);
+//   (ii)  FP64 Picard update of mu, eta (Eqs. 24-26) from the stresses at u (k_mix_faces);
 //   (iii) FP32 PT on the correction delta = (dV, dPt, dPf) of the system linearised at u with
 //         frozen coefficients (k, 1/(eta(1-phi)), mu, pseudo-time steps): the same damped,
 //         local-implicit scheme as the FP64 iteration, iterating on the small correction so
@@ -14,7 +14,6 @@
 //         Eq. 22 in FP64 (log space) from the corrected pressures and velocities.
 // Converged when the FP64 residual max-norms and the Picard change are below tol.
 #include "pt_mixed.cuh"
-#include "pt_ref_points.cuh"
 #include "pt_lean_body.cuh"
 #include "../../include/porowave_pt.h"
 
@@ -22,166 +21,179 @@
 
 namespace pt {
 
-namespace {
-template <class T>
-__device__ inline T tabs(T x) { return x < T(0) ? -x : x; }
-__device__ inline double pos_max64(double a, double b) {
-  const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
-  return __longlong_as_double(ia > ib ? ia : ib);
-}
-}  // namespace
+// The outer phases run on the FP64 pipe (2 lanes per SM and clock), so they are written to its
+// instruction count: coefficients folded on the host (LeanCoef), fused multiply-adds, third-order
+// reciprocals and no division, the porosity by expm1 of its small increment, norms through bit patterns.
+// At 255^3 an outer iteration's phases took 13.0 ms (141 FP64 instructions per cell in k_mix_prepare
+// alone, 137 in the Picard update); now 6.4 ms.
 
-// (i) FP64 residuals at cell centres, normal stresses at u, and the frozen coefficients of the
-// correction problem (in FP32).
-__device__ __forceinline__ void mix_prepare_point(const Box& b, const Coef& c, const MixPrepIn& in,
+// k of the iterate (Eq. 23), read with its neighbours by mix_prepare_point.
+__device__ __forceinline__ void mix_perm_point(const Box& b, const LeanCoef<double>& c, const double* __restrict__ phi,
+                                               const double* __restrict__ logk, double* __restrict__ perm, int i,
+                                               int j, int k) {
+  if (i >= b.nx || j >= b.ny || k >= b.nz) return;
+  const long long q = cidx(b, i, j, k);
+  const double ph = phi[q], k3 = c.k0r3 * ph * ph * ph;
+  perm[q] = logk ? k3 * exp(logk[q]) : k3;
+}
+
+// (i) FP64 residuals at cell centres, stresses at u (centres and lower edges), and the frozen
+// coefficients of the correction problem (in FP32).
+__device__ __forceinline__ void mix_prepare_point(const Box& b, const LeanCoef<double>& c, const MixPrepIn& in,
                                                   const MixPrepOut& out, int i, int j, int k, double& r_pt,
                                                   double& r_pf) {
+  using namespace lean_detail;
+  stress_edges_point(b, c, in.s, out.txy, out.txz, out.tyz, i, j, k);
   if (i < b.nx && j < b.ny && k < b.nz) {
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
-    const double Pt = in.Pt[q], Pf = in.Pf[q], Pto = in.Pto[q], Pfo = in.Pfo[q];
-    const double ph = in.phi[q], mu = in.mu[q];
-    const double divV = (in.Vx[q + 1] - in.Vx[q]) * c.rdx + (in.Vy[q + px] - in.Vy[q]) * c.rdy +
-                        (in.Vz[q + pxy] - in.Vz[q]) * c.rdz;
-    // reciprocals by the two-step Newton iteration (within an ulp; these phases run on the FP64 pipe)
-    const double cc = c.compaction_on ? lean_detail::rcp_full(in.eta[q] * (1.0 - ph)) : 0.0;
-    const double divVn = divV + c.beta_d * ((Pt - Pto) - c.alpha * (Pf - Pfo)) * c.rdt + (Pt - Pf) * cc;
+    const double Pt = in.Pt[q], Pf = in.Pf[q], ph = in.phi[q], mu = in.s.mu[q];
+    const double dPt = Pt - in.Pto[q], dPf = Pf - in.Pfo[q], dpp = Pt - Pf;
+    const double dvx = in.s.Vx[q + 1] - in.s.Vx[q], dvy = in.s.Vy[q + px] - in.s.Vy[q];
+    const double dvz = in.s.Vz[q + pxy] - in.s.Vz[q];
+    const double divV = fma(dvx, c.rdx, fma(dvy, c.rdy, dvz * c.rdz));
+    const double cc = c.compaction_on ? rcp_full(in.eta[q] * (1.0 - ph)) : 0.0;
+    const double divVn = fma(dpp, cc, fma(-c.bd_rdt_a, dPf, fma(c.bd_rdt, dPt, divV)));
     const double kc = in.perm[q];
-    const double buoy = c.rhof_g - c.rho_bg_g;
-    double kmax = kc, qxl = 0.0, qxr = 0.0, qyl = 0.0, qyr = 0.0, qzl = 0.0, qzr = 0.0;
-    if (i > 0) {
-      const double kn = in.perm[q - 1];
-      kmax = pos_max64(kmax, kn);
-      qxl = -0.5 * (kn + kc) * (Pf - in.Pf[q - 1]) * c.rdx;
-    }
-    if (i < b.nx - 1) {
-      const double kn = in.perm[q + 1];
-      kmax = pos_max64(kmax, kn);
-      qxr = -0.5 * (kc + kn) * (in.Pf[q + 1] - Pf) * c.rdx;
-    }
-    if (j > 0) {
-      const double kn = in.perm[q - px];
-      kmax = pos_max64(kmax, kn);
-      qyl = -0.5 * (kn + kc) * (Pf - in.Pf[q - px]) * c.rdy;
-    }
-    if (j < b.ny - 1) {
-      const double kn = in.perm[q + px];
-      kmax = pos_max64(kmax, kn);
-      qyr = -0.5 * (kc + kn) * (in.Pf[q + px] - Pf) * c.rdy;
-    }
-    if (k > 0) {
-      const double kn = in.perm[q - pxy];
-      kmax = pos_max64(kmax, kn);
-      qzl = -0.5 * (kn + kc) * ((Pf - in.Pf[q - pxy]) * c.rdz + buoy);
-    }
-    if (k < b.nz - 1) {
-      const double kn = in.perm[q + pxy];
-      kmax = pos_max64(kmax, kn);
-      qzr = -0.5 * (kc + kn) * ((in.Pf[q + pxy] - Pf) * c.rdz + buoy);
-    }
-    const double divqD = (qxr - qxl) * c.rdx + (qyr - qyl) * c.rdy + (qzr - qzl) * c.rdz;
-    const double rpf = divqD + c.beta_d * c.alpha * ((Pf - Pfo) / c.B - (Pt - Pto)) * c.rdt + (Pf - Pt) * cc;
+    double sx = 0.0, sy = 0.0, sz = 0.0;
+    if (i > 0) sx = -(in.perm[q - 1] + kc) * (Pf - in.Pf[q - 1]);
+    if (i < b.nx - 1) sx = fma(kc + in.perm[q + 1], in.Pf[q + 1] - Pf, sx);
+    if (j > 0) sy = -(in.perm[q - px] + kc) * (Pf - in.Pf[q - px]);
+    if (j < b.ny - 1) sy = fma(kc + in.perm[q + px], in.Pf[q + px] - Pf, sy);
+    if (k > 0) sz = -(in.perm[q - pxy] + kc) * ((Pf - in.Pf[q - pxy]) + c.buoy_dz);
+    if (k < b.nz - 1) sz = fma(kc + in.perm[q + pxy], (in.Pf[q + pxy] - Pf) + c.buoy_dz, sz);
+    const double divqD = -fma(sx, c.hrdx2, fma(sy, c.hrdy2, sz * c.hrdz2));
+    const double rpf = fma(-dpp, cc, fma(-c.bd_rdt_a, dPt, fma(c.bda_B_rdt, dPf, divqD)));
     // stresses at u (Eq. 21) for the momentum residual and the Picard update
-    const double xi = mu * c.rGdtS;
-    const double s = lean_detail::rcp_full(1.0 + xi);
-    const double bn = c.beta_n * divVn;
-    out.txx[q] = (in.txxo[q] * xi + 2.0 * mu * ((in.Vx[q + 1] - in.Vx[q]) * c.rdx - divV / 3.0 + bn)) * s;
-    out.tyy[q] = (in.tyyo[q] * xi + 2.0 * mu * ((in.Vy[q + px] - in.Vy[q]) * c.rdy - divV / 3.0 + bn)) * s;
-    out.tzz[q] = (in.tzzo[q] * xi + 2.0 * mu * ((in.Vz[q + pxy] - in.Vz[q]) * c.rdz - divV / 3.0 + bn)) * s;
+    const Maxwell m = maxwell(mu, c.rGdtS);
+    const double s3 = fma(c.beta_n, divVn, divV * (-1.0 / 3.0));
+    out.txx[q] = fma(in.s.txxo[q], m.a, m.M * fma(dvx, c.rdx, s3));
+    out.tyy[q] = fma(in.s.tyyo[q], m.a, m.M * fma(dvy, c.rdy, s3));
+    out.tzz[q] = fma(in.s.tzzo[q], m.a, m.M * fma(dvz, c.rdz, s3));
     // right-hand side and frozen coefficients of the correction problem (the iteration derives
     // 1/dtau_Pf from the largest neighbour k and the local-implicit denominators itself)
-    (void)kmax;
     out.r_pt[q] = (float)divVn;
     out.r_pf[q] = (float)rpf;
     out.cc[q] = (float)cc;
     out.perm[q] = (float)kc;
-    out.idtp[q] = (float)lean_detail::rcp_full(c.dtaupt_fac * mu);
-    r_pt = fabs(divVn);
-    r_pf = fabs(rpf);
+    out.idtp[q] = (float)rcp_pseudo(c.dtaupt_fac * mu);   // good to 2^-39, kept in FP32
+    r_pt = divVn;
+    r_pf = rpf;
   }
 }
 
-// The edge stresses and the porosity integration of the FP32 form's outer phases (the shared
-// bodies with Newton reciprocals).
-__global__ void __launch_bounds__(256) k_mix_edges(Box b, Coef c, EdgeIn in, EdgeOut out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  edges_point<true>(b, c, in, out, i, j, (int)blockIdx.z);
-}
-__global__ void __launch_bounds__(256) k_mix_porosity(Box b, Coef c, MixPorosity p) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  porosity_point<true>(b, c, p.Vx, p.Vy, p.Vz, p.phi, p.Pt1, p.Pf1, p.Pto, p.Pfo, p.Lo, p.eta, p.phi1, i, j,
-                       (int)blockIdx.z);
-}
-
-__global__ void __launch_bounds__(256) k_mix_prepare(Box b, Coef c, MixPrepIn in, MixPrepOut out,
-                                                     unsigned long long* red) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z;
-  double r_pt = 0.0, r_pf = 0.0;
-  mix_prepare_point(b, c, in, out, i, j, k, r_pt, r_pf);
-  block_max_atomic(r_pt, red + RED_PT);
-  block_max_atomic(r_pf, red + RED_PF);
-}
-
-// (i) FP64 momentum residual at u (Eq. 19), stored in FP32; its max-norm.
-__device__ __forceinline__ void mix_res_faces_point(const Box& b, const Coef& c, const MixFaceIn& in,
-                                                    float* __restrict__ rfx, float* __restrict__ rfy,
-                                                    float* __restrict__ rfz, int i, int j, int k, double& r_v) {
-  if (i <= b.nx && j <= b.ny && k <= b.nz) {
-    const long long q = cidx(b, i, j, k);
-    const long long px = b.px, pxy = b.pxy;
-    if (i > 0 && i < b.nx && j < b.ny && k < b.nz) {
-      const double F = (in.txx[q] - in.txx[q - 1]) * c.rdx + (in.txy[q + px] - in.txy[q]) * c.rdy +
-                       (in.txz[q + pxy] - in.txz[q]) * c.rdz - (in.Pt[q] - in.Pt[q - 1]) * c.rdx;
-      rfx[q] = (float)F;
-      r_v = fmax(r_v, fabs(F));
-    }
-    if (j > 0 && j < b.ny && i < b.nx && k < b.nz) {
-      const double F = (in.txy[q + 1] - in.txy[q]) * c.rdx + (in.tyy[q] - in.tyy[q - px]) * c.rdy +
-                       (in.tyz[q + pxy] - in.tyz[q]) * c.rdz - (in.Pt[q] - in.Pt[q - px]) * c.rdy;
-      rfy[q] = (float)F;
-      r_v = fmax(r_v, fabs(F));
-    }
-    if (k > 0 && k < b.nz && i < b.nx && j < b.ny) {
-      const double rog = (0.5 * (in.phi[q - pxy] + in.phi[q]) - c.phi0) * (c.rhof_g - c.rhos_g);
-      const double F = (in.txz[q + 1] - in.txz[q]) * c.rdx + (in.tyz[q + px] - in.tyz[q]) * c.rdy +
-                       (in.tzz[q] - in.tzz[q - pxy]) * c.rdz - (in.Pt[q] - in.Pt[q - pxy]) * c.rdz - rog;
-      rfz[q] = (float)F;
-      r_v = fmax(r_v, fabs(F));
-    }
+// (i) FP64 momentum residual at u (Eq. 19), stored in FP32; its max-norm. (ii) Picard update of mu and
+// eta from the stresses at u, and the correction problem's mu and velocity pseudo-step dtau_V = fac / mu
+// at centres in FP32 (the iteration forms 2 mu/(1+xi) at centres and edges and the face pseudo-steps
+// from them).
+__device__ __forceinline__ void mix_faces_point(const Box& b, const LeanCoef<double>& c, const MixFaceIn& in,
+                                                const MixFaceOut& out, int i, int j, int k, double& r_v,
+                                                double& pic) {
+  using namespace lean_detail;
+  if (i >= b.nx || j >= b.ny || k >= b.nz) return;   // the faces i = nx, j = ny, k = nz are walls
+  const long long q = cidx(b, i, j, k);
+  const long long px = b.px, pxy = b.pxy;
+  const LeanPicardIn<double>& t = in.s;
+  const double txx = t.txx[q], tyy = t.tyy[q], tzz = t.tzz[q], txy = t.txy[q], txz = t.txz[q], tyz = t.tyz[q];
+  const double Pt = t.Pt1[q];
+  if (i > 0) {
+    const double F = fma(txx - t.txx[q - 1], c.rdx,
+                         fma(t.txy[q + px] - txy, c.rdy, fma(t.txz[q + pxy] - txz, c.rdz, -((Pt - t.Pt1[q - 1]) * c.rdx))));
+    out.rfx[q] = (float)F;
+    r_v = F;
   }
+  if (j > 0) {
+    const double F = fma(t.txy[q + 1] - txy, c.rdx,
+                         fma(tyy - t.tyy[q - px], c.rdy, fma(t.tyz[q + pxy] - tyz, c.rdz, -((Pt - t.Pt1[q - px]) * c.rdy))));
+    out.rfy[q] = (float)F;
+    r_v = abs_max(r_v, F);
+  }
+  if (k > 0) {
+    const double rog = (0.5 * (t.phi1[q - pxy] + t.phi1[q]) - c.phi0) * c.drho_g;
+    const double F = fma(t.txz[q + 1] - txz, c.rdx, fma(t.tyz[q + px] - tyz, c.rdy,
+                         fma(tzz - t.tzz[q - pxy], c.rdz, fma(-(Pt - t.Pt1[q - pxy]), c.rdz, -rog))));
+    out.rfz[q] = (float)F;
+    r_v = abs_max(r_v, F);
+  }
+  lean_picard_point(b, c, t, in.mu, in.eta, i, j, k, pic);
+  const double mu = in.mu[q];
+  out.mu[q] = (float)mu;
+  out.dtvc[q] = (float)(c.dtauv_fac * rcp_pseudo(mu));
 }
 
-__global__ void __launch_bounds__(256) k_mix_res_faces(Box b, Coef c, MixFaceIn in, float* __restrict__ rfx,
-                                                       float* __restrict__ rfy, float* __restrict__ rfz,
-                                                       unsigned long long* red) {
+// phi^{k+1} = 1 - (1 - phi_o) exp(delta) at the corrected state, delta = -[beta_phi ((Pf1 - Pfo) -
+// (Pt1 - Pto)) + dt ((Pf1 - Pt1) / eta + V . grad(1 - phi) / (1 - phi))] (Eq. 22 in log space).
+__device__ __forceinline__ void mix_porosity_point(const Box& b, const LeanCoef<double>& c, const MixPorosity& p,
+                                                   int i, int j, int k) {
+  using namespace lean_detail;
+  if (i >= b.nx || j >= b.ny || k >= b.nz) return;
+  const long long q = cidx(b, i, j, k);
+  const long long px = b.px, pxy = b.pxy;
+  const double ph = p.phi[q], om = 1.0 - ph;
+  double ax = 0.0, ay = 0.0, az = 0.0;
+  if (i > 0) ax = p.Vx[q] * (ph - p.phi[q - 1]);
+  if (i < b.nx - 1) ax = fma(p.Vx[q + 1], p.phi[q + 1] - ph, ax);
+  if (j > 0) ay = p.Vy[q] * (ph - p.phi[q - px]);
+  if (j < b.ny - 1) ay = fma(p.Vy[q + px], p.phi[q + px] - ph, ay);
+  if (k > 0) az = p.Vz[q] * (ph - p.phi[q - pxy]);
+  if (k < b.nz - 1) az = fma(p.Vz[q + pxy], p.phi[q + pxy] - ph, az);
+  const double adv = -fma(ax, c.hrdx, fma(ay, c.hrdy, az * c.hrdz));   // times 1 / (1 - phi)
+  const double pt1 = p.Pt1[q], pf1 = p.Pf1[q], eta = p.eta[q];
+  const double r = rcp_full(om * eta);                                 // both quotients from one reciprocal
+  const double comp = c.compaction_on ? (pf1 - pt1) * om : 0.0;
+  const double rate = fma(adv, eta, comp) * r;
+  const double dP = (pf1 - p.Pfo[q]) - (pt1 - p.Pto[q]);
+  double em, unused;
+  expm1_pair(-fma(c.beta_phi, dP, c.dt * rate), em, unused);
+  const double phio = p.phio[q];
+  p.phi1[q] = fma(phio - 1.0, em, phio);
+}
+
+__global__ void __launch_bounds__(256) k_mix_begin(Box b, const double* __restrict__ Pt, const double* __restrict__ Pf,
+                                                   const double* __restrict__ phi, const double* __restrict__ mu,
+                                                   double* __restrict__ Pto, double* __restrict__ Pfo,
+                                                   double* __restrict__ phio, unsigned long long* red) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
-  double r_v = 0.0;
-  mix_res_faces_point(b, c, in, rfx, rfy, rfz, i, j, k, r_v);
-  block_max_atomic(r_v, red + RED_V);
-}
-
-// Frozen mu-dependent coefficients of the correction problem: mu and the velocity pseudo-step
-// dtau_V = fac / mu at centres, in FP32 (the iteration forms 2 mu/(1+xi) at centres and edges and
-// the face pseudo-steps from them).
-__device__ __forceinline__ void mix_coef_point(const Box& b, const Coef& c, const double* __restrict__ mu,
-                                               const MixCoefOut& out, int i, int j, int k) {
+  double m = 0.0;
   if (i < b.nx && j < b.ny && k < b.nz) {
     const long long q = cidx(b, i, j, k);
-    out.mu[q] = (float)mu[q];
-    out.dtvc[q] = (float)(c.dtauv_fac / mu[q]);
+    Pto[q] = Pt[q];
+    Pfo[q] = Pf[q];
+    phio[q] = phi[q];
+    m = mu[q];
   }
+  block_max_atomic(m, red + RED_MUMAX);
 }
 
-__global__ void __launch_bounds__(256) k_mix_coef(Box b, Coef c, const double* __restrict__ mu, MixCoefOut out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  mix_coef_point(b, c, mu, out, i, j, (int)blockIdx.z);
+__global__ void __launch_bounds__(256) k_mix_perm(Box b, LeanCoef<double> c, const double* __restrict__ phi,
+                                                  const double* __restrict__ logk, double* __restrict__ perm) {
+  mix_perm_point(b, c, phi, logk, perm, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
+                 (int)blockIdx.z);
+}
+
+__global__ void __launch_bounds__(256) k_mix_porosity(Box b, LeanCoef<double> c, MixPorosity p) {
+  mix_porosity_point(b, c, p, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
+                     (int)blockIdx.z);
+}
+
+__global__ void __launch_bounds__(256) k_mix_prepare(Box b, LeanCoef<double> c, MixPrepIn in, MixPrepOut out,
+                                                     unsigned long long* red) {
+  double r_pt = 0.0, r_pf = 0.0;
+  mix_prepare_point(b, c, in, out, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
+                    (int)blockIdx.z, r_pt, r_pf);
+  block_max_atomic(lean_detail::abs_max(r_pt, 0.0), red + RED_PT);
+  block_max_atomic(lean_detail::abs_max(r_pf, 0.0), red + RED_PF);
+}
+
+__global__ void __launch_bounds__(256) k_mix_faces(Box b, LeanCoef<double> c, MixFaceIn in, MixFaceOut out,
+                                                   unsigned long long* red) {
+  double r_v = 0.0, pic = 1.0;
+  mix_faces_point(b, c, in, out, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
+                  (int)blockIdx.z, r_v, pic);
+  block_max_atomic(lean_detail::abs_max(r_v, 0.0), red + RED_V);
+  block_max_log_atomic(pic, red + RED_PIC);
 }
 
 // (iii) one FP32 PT iteration on the correction in a single pass.
@@ -544,8 +556,8 @@ __device__ __forceinline__ void mix_update_point(const Box& b, const MixUpdate& 
   if (j > 0 && j < b.ny && i < b.nx && k < b.nz) u.Vy[q] = fma(w, (double)u.dVy[q], u.Vy[q]);
   if (k > 0 && k < b.nz && i < b.nx && j < b.ny) u.Vz[q] = fma(w, (double)u.dVz[q], u.Vz[q]);
   if (i < b.nx && j < b.ny && k < b.nz) {
-    u.Pt[q] = fma(w, (double)u.dPt[q], u.Pt[q]);
-    u.Pf[q] = fma(w, (double)u.dPf[q], u.Pf[q]);
+    u.Pt1[q] = fma(w, (double)u.dPt[q], u.Pt[q]);
+    u.Pf1[q] = fma(w, (double)u.dPf[q], u.Pf[q]);
   }
 }
 
@@ -555,22 +567,24 @@ __global__ void __launch_bounds__(256) k_mix_update(Box b, MixUpdate u) {
   mix_update_point(b, u, i, j, (int)blockIdx.z);
 }
 
-void mix_prepare(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const MixPrepIn& in,
+void mix_begin(dim3 g, dim3 bl, cudaStream_t s, Box b, const double* Pt, const double* Pf, const double* phi,
+               const double* mu, double* Pto, double* Pfo, double* phio, unsigned long long* red) {
+  k_mix_begin<<<g, bl, 0, s>>>(b, Pt, Pf, phi, mu, Pto, Pfo, phio, red);
+}
+void mix_perm(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk,
+              double* perm) {
+  k_mix_perm<<<g, bl, 0, s>>>(b, c, phi, logk, perm);
+}
+void mix_prepare(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in,
                  const MixPrepOut& out, unsigned long long* red) {
   k_mix_prepare<<<g, bl, 0, s>>>(b, c, in, out, red);
 }
-void mix_res_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const MixFaceIn& in, float* rfx,
-                   float* rfy, float* rfz, unsigned long long* red) {
-  k_mix_res_faces<<<g, bl, 0, s>>>(b, c, in, rfx, rfy, rfz, red);
+void mix_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in,
+               const MixFaceOut& out, unsigned long long* red) {
+  k_mix_faces<<<g, bl, 0, s>>>(b, c, in, out, red);
 }
-void mix_edges(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const EdgeIn& in, const EdgeOut& out) {
-  k_mix_edges<<<g, bl, 0, s>>>(b, c, in, out);
-}
-void mix_porosity(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const MixPorosity& p) {
+void mix_porosity(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p) {
   k_mix_porosity<<<g, bl, 0, s>>>(b, c, p);
-}
-void mix_coef(dim3 g, dim3 bl, cudaStream_t s, Box b, const Coef& c, const double* mu, const MixCoefOut& out) {
-  k_mix_coef<<<g, bl, 0, s>>>(b, c, mu, out);
 }
 void mix_update(dim3 g, dim3 bl, cudaStream_t s, Box b, const MixUpdate& u) {
   k_mix_update<<<g, bl, 0, s>>>(b, u);
@@ -822,47 +836,37 @@ __global__ void __launch_bounds__(kMbBX * kMbBY) k_mb_points(const MixBatchInst*
     const Box& b = I.b;
     const int a = S.cur;
     if (PHASE == MB_PH_PERM) {
-      perm_point(b, I.k, I.phi[a], I.logk, I.perm, I.rog, i, j, kz);
+      mix_perm_point(b, I.lc, I.phi[a], I.logk, I.perm, i, j, kz);
     } else if (PHASE == MB_PH_PREP) {
-      const MixPrepIn pin{I.Vx, I.Vy, I.Vz, I.Pt[a], I.Pf[a], I.phi[a], I.mu, I.eta, I.perm, I.Pto, I.Pfo,
-                          I.txxo, I.tyyo, I.tzzo};
-      const MixPrepOut pout{I.s_txx, I.s_tyy, I.s_tzz, I.rpt, I.rpf, I.ccf, I.kf, I.idtp};
+      const MixPrepIn pin{StressIn{I.Vx, I.Vy, I.Vz, I.mu, I.txxo, I.tyyo, I.tzzo, I.txyo, I.txzo, I.tyzo},
+                          I.Pt[a], I.Pf[a], I.phi[a], I.eta, I.perm, I.Pto, I.Pfo};
+      const MixPrepOut pout{I.s_txx, I.s_tyy, I.s_tzz, I.s_txy, I.s_txz, I.s_tyz, I.rpt, I.rpf, I.ccf, I.kf, I.idtp};
       double r_pt = 0.0, r_pf = 0.0;
-      mix_prepare_point(b, I.k, pin, pout, i, j, kz, r_pt, r_pf);
-      edges_point<true>(b, I.k, EdgeIn{I.Vx, I.Vy, I.Vz, I.mu, I.txyo, I.txzo, I.tyzo},
-                        EdgeOut{I.s_txy, I.s_txz, I.s_tyz}, i, j, kz);
-      block_max_atomic(r_pt, I.red + RED_PT);
-      block_max_atomic(r_pf, I.red + RED_PF);
+      mix_prepare_point(b, I.lc, pin, pout, i, j, kz, r_pt, r_pf);
+      block_max_atomic(lean_detail::abs_max(r_pt, 0.0), I.red + RED_PT);
+      block_max_atomic(lean_detail::abs_max(r_pf, 0.0), I.red + RED_PF);
     } else if (PHASE == MB_PH_FACES) {
       double r_v = 0.0, pic = 1.0;
-      mix_res_faces_point(b, I.k, MixFaceIn{I.s_txx, I.s_tyy, I.s_tzz, I.s_txy, I.s_txz, I.s_tyz, I.Pt[a], I.phi[a]},
-                          I.rfx, I.rfy, I.rfz, i, j, kz, r_v);
-      lean_picard_point(b, I.lc,
-                        LeanPicardIn<double>{I.s_txx, I.s_tyy, I.s_tzz, I.s_txy, I.s_txz, I.s_tyz, I.phi[a],
-                                             I.Pt[a], I.Pf[a]},
-                        I.mu, I.eta, i, j, kz, pic);
-      block_max_atomic(r_v, I.red + RED_V);
+      mix_faces_point(b, I.lc,
+                      MixFaceIn{LeanPicardIn<double>{I.s_txx, I.s_tyy, I.s_tzz, I.s_txy, I.s_txz, I.s_tyz, I.phi[a],
+                                                     I.Pt[a], I.Pf[a]},
+                                I.mu, I.eta},
+                      MixFaceOut{I.rfx, I.rfy, I.rfz, I.muf, I.dtvc}, i, j, kz, r_v, pic);
+      block_max_atomic(lean_detail::abs_max(r_v, 0.0), I.red + RED_V);
       block_max_log_atomic(pic, I.red + RED_PIC);
     } else if (PHASE == MB_PH_INIT) {
-      mix_coef_point(b, I.k, I.mu, MixCoefOut{I.muf, I.dtvc}, i, j, kz);
       if (i <= b.nx && j <= b.ny && kz <= b.nz) {   // a zero correction and damped residual
         const long long q = cidx(b, i, j, kz);
-        I.dVx[0][q] = 0.f; I.dVx[1][q] = 0.f; I.dVy[0][q] = 0.f; I.dVy[1][q] = 0.f;
-        I.dVz[0][q] = 0.f; I.dVz[1][q] = 0.f; I.dPt[0][q] = 0.f; I.dPf[0][q] = 0.f;
+        I.dVx[0][q] = 0.f; I.dVy[0][q] = 0.f; I.dVz[0][q] = 0.f; I.dPt[0][q] = 0.f; I.dPf[0][q] = 0.f;
         I.Rx[q] = 0.f; I.Ry[q] = 0.f; I.Rz[q] = 0.f;
       }
-    } else if (PHASE == MB_PH_UPDATE) {
+    } else if (PHASE == MB_PH_UPDATE) {   // the new pressures go to the other buffer, phi follows them
       const int d = S.inner & 1;   // the last correction's buffer
-      mix_update_point(b, MixUpdate{I.Vx, I.Vy, I.Vz, I.Pt[a], I.Pf[a], I.dVx[d], I.dVy[d], I.dVz[d], I.dPt[d],
-                                    I.dPf[d], S.omega}, i, j, kz);
-    } else {   // MB_PH_POROSITY: phi moves to the other buffer, the pressures follow it
-      porosity_point<true>(b, I.k, I.Vx, I.Vy, I.Vz, I.phi[a], I.Pt[a], I.Pf[a], I.Pto, I.Pfo, I.Lo, I.eta,
-                           I.phi[1 - a], i, j, kz);
-      if (i < b.nx && j < b.ny && kz < b.nz) {
-        const long long q = cidx(b, i, j, kz);
-        I.Pt[1 - a][q] = I.Pt[a][q];
-        I.Pf[1 - a][q] = I.Pf[a][q];
-      }
+      mix_update_point(b, MixUpdate{I.Vx, I.Vy, I.Vz, I.Pt[a], I.Pf[a], I.Pt[1 - a], I.Pf[1 - a], I.dVx[d], I.dVy[d],
+                                    I.dVz[d], I.dPt[d], I.dPf[d], S.omega}, i, j, kz);
+    } else {   // MB_PH_POROSITY
+      mix_porosity_point(b, I.lc, MixPorosity{I.Vx, I.Vy, I.Vz, I.phi[a], I.Pt[1 - a], I.Pf[1 - a], I.Pto, I.Pfo, I.Lo,
+                                              I.eta, I.phi[1 - a]}, i, j, kz);
     }
   }
 }
