@@ -1027,8 +1027,8 @@ int pt_init(pt_ctx** ctx, const pt_grid* grid, const pt_phys* phys, const pt_num
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(tb.first, tb.second.data(), tb.second.size() * 4, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess && c->dfm && c->logk) {
-    PT_LAUNCH(c, K_DF_K0, lean_k0<df64>(grid_dims(c->box), block_dims(), c->stream, c->box, c->phys.k0, c->logk,
-                                        D(c->K0)));
+    PT_LAUNCH(c, K_DF_K0, lean_k0<df64>(grid_dims(c->box), block_dims(), c->stream, c->box, c->lcoef.k0r3,
+                                        c->logk, D(c->K0)));
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && c->lean && c->logk) {

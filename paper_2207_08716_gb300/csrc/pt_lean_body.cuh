@@ -121,29 +121,31 @@ __device__ inline df64 rcp_full(df64 x) { return df_rcp(x); }
 
 __device__ inline df64 pos_max(df64 a, df64 b) { return a < b ? b : a; }
 
-// Same tiers as the FP64 pair (the truncation stays below 2^-60 |d|, far under the format's
-// 2^-48); outside them the library expm1 in FP64.
-__device__ inline void expm1_pair(df64 d, df64& em_pos, df64& em_neg) {
+// exp(d) - 1 with the tiers of the FP64 pair: for |d| <= 2^-20 d + d^2/2 + d^3/6 with d^2 exact to the
+// pair and the cubic term (below 2^-42 |d|) in FP32; up to 2^-6 the split series; outside them the library
+// expm1 in FP64.
+__device__ inline df64 df_expm1(df64 d) {
   const float ad = fabsf(d.hi);
   if (ad <= 0x1p-20f) {
-    const df64 d2 = d * d;
-    const df64 E = scale2(d2, 0.5f);
-    const df64 O = d * fma(d2, df64(1.0 / 6.0), df64(1.0));
-    em_pos = E + O;
-    em_neg = E - O;
-  } else if (ad <= 0.015625f) {
+    const float p = __fmul_rn(d.hi, d.hi);
+    const float e = __fmaf_rn(2.0f * d.hi, d.lo, __fmaf_rn(d.hi, d.hi, -p));   // d^2 = p + e
+    float s, t;
+    dfd::fast_two_sum(d.hi, 0.5f * p, s, t);
+    return dfd::renorm(s, __fadd_rn(t, __fmaf_rn(p * d.hi, 1.0f / 6.0f, __fmaf_rn(0.5f, e, d.lo))));
+  }
+  if (ad <= 0.015625f) {
     const df64 d2 = d * d;
     const df64 E = d2 * fma(d2, fma(d2, fma(d2, df64(1.0 / 40320.0), df64(1.0 / 720.0)), df64(1.0 / 24.0)),
                             df64(0.5));
     const df64 O = d * fma(d2, fma(d2, fma(d2, fma(d2, df64(1.0 / 362880.0), df64(1.0 / 5040.0)),
                                            df64(1.0 / 120.0)), df64(1.0 / 6.0)), df64(1.0));
-    em_pos = E + O;
-    em_neg = E - O;
-  } else {
-    const double x = (double)d;
-    em_pos = df64(expm1(x));
-    em_neg = df64(expm1(-x));
+    return E + O;
   }
+  return df64(expm1((double)d));
+}
+__device__ inline void expm1_pair(df64 d, df64& em_pos, df64& em_neg) {
+  em_pos = df_expm1(d);
+  em_neg = df_expm1(-d);
 }
 
 // conversions between the field type and FP64 (identity for FP64)
@@ -182,36 +184,25 @@ __device__ inline df64 abs_max(df64 a, df64 b) { return a < b ? b : a; }   // po
 
 // Which arrays a form stores. The FP64 form is bound by the FP64 pipe and stores everything that
 // changes less often than every iteration (1/(1-phi) and k travelling with phi, 1 - phi_o and its
-// reciprocal, edge moduli pre-multiplied by both spacings, three face pseudo-steps). Double-float
-// arithmetic is cheap and the double-float form is bound by HBM and instruction issue, so it
-// recomputes 1/(1-phi), 1 - phi_o and its reciprocal, keeps one modulus per edge (em2_* hold
-// 2 mu/(1+xi); eb_* unused) and one velocity pseudo-step per centre (dtv_x = dtv_y = dtv_z hold
-// fac / mu, averaged to each face): 56 fewer bytes per cell and iteration.
+// reciprocal, edge moduli pre-multiplied by both spacings, three face pseudo-steps). The double-float
+// form is bound by HBM and instruction issue, so it recomputes 1/(1-phi), 1 - phi_o and its reciprocal,
+// keeps one modulus per edge (em2_* hold 2 mu/(1+xi); eb_* unused) and one velocity pseudo-step per
+// centre (dtv_x = dtv_y = dtv_z hold half of fac / mu; a face adds its two): 56 fewer bytes per cell and
+// iteration. k(phi) travels with phi in both (recomputing it for the cell and its six neighbours costs
+// more issue slots than its 16 bytes).
 template <class T>
 struct LeanRecompute { static constexpr bool value = false; };
 template <>
 struct LeanRecompute<df64> { static constexpr bool value = true; };
-// k(phi) travels with phi (written by the cells kernel for the next iteration) in both forms:
-// recomputing it for the cell and its six neighbours costs more issue slots than its 16 bytes
-template <class T>
-struct LeanStoreK { static constexpr bool value = true; };
 
-// Where the cells body reads the arrays it needs only at its own index q ("pointwise"): straight
-// from global memory, or from a shared-memory stage that cp.async filled ahead (slot order below).
+// Shared-memory stage of the double-float cells kernel (pointwise arrays, slot order).
 enum { S_PTO, S_PFO, S_PHIO, S_IETA, S_IDTP, S_CM2, S_TXX, S_TYY, S_TZZ, S_EXY, S_EXZ, S_EYZ, S_TXY, S_TXZ,
-       S_TYZ, kStageSlots,
-       // own-index values of the neighbour arrays (staged too when the whole level is staged)
-       S_VX = kStageSlots, S_VY, S_VZ, S_PT, S_PF, S_PHI, S_K, kStageSlotsAll };
-struct DirectPoint {
-  template <class T>
-  __device__ __forceinline__ T operator()(const T* a, long long q, int) const { return a[q]; }
-};
+       S_TYZ, kStageSlots };
 
-// Cells, stresses of the three lower edges, pressures, porosity at box index (i, j, k).
-template <class T, class PP = DirectPoint>
-__device__ __forceinline__ void lean_cell_point(const Box& b, const LeanCoef<T>& c, const LeanCellIn<T>& in,
-                                                const LeanCellOut<T>& out, int i, int j, int k, int check,
-                                                double& r_pt, double& r_pf, const PP& pp = PP()) {
+// Cells, stresses of the three lower edges, pressures, porosity at box index (i, j, k) in FP64.
+__device__ __forceinline__ void lean_cell_point(const Box& b, const LeanCoef<double>& c,
+                                                const LeanCellIn<double>& in, const LeanCellOut<double>& out, int i,
+                                                int j, int k, int check, double& r_pt, double& r_pf) {
   using namespace lean_detail;
   if (i <= b.nx && j <= b.ny && k <= b.nz) {
     const long long q = cidx(b, i, j, k);
@@ -219,146 +210,94 @@ __device__ __forceinline__ void lean_cell_point(const Box& b, const LeanCoef<T>&
     const bool cell = i < b.nx && j < b.ny && k < b.nz;
     // ---- edges owned by this index: xy (i, j, k), xz (i, j, k), yz (i, j, k); stored at the end
     // with the cell's outputs, after every load (the arrays are not declared non-aliasing)
-    constexpr bool RC = LeanRecompute<T>::value;
-    constexpr bool KS = LeanStoreK<T>::value;
-    T t_xy = T(0), t_xz = T(0), t_yz = T(0);
+    double t_xy = 0.0, t_xz = 0.0, t_yz = 0.0;
     if (k < b.nz && i > 0 && i < b.nx && j > 0 && j < b.ny) {   // toa_xy holds the background part too
-      if constexpr (RC)
-        t_xy = fma(pp(in.em2_xy, q, S_EXY), fma(pp(in.Vy, q, S_VY) - in.Vy[q - 1], c.hrdx,
-                                                (pp(in.Vx, q, S_VX) - in.Vx[q - px]) * c.hrdy),
-                   pp(in.toa_xy, q, S_TXY));
-      else
-        t_xy = fma(in.eb_xy[q], in.Vy[q] - in.Vy[q - 1], fma(pp(in.em2_xy, q, S_EXY), in.Vx[q] - in.Vx[q - px],
-                                                             pp(in.toa_xy, q, S_TXY)));
+      t_xy = fma(in.eb_xy[q], in.Vy[q] - in.Vy[q - 1], fma(in.em2_xy[q], in.Vx[q] - in.Vx[q - px], in.toa_xy[q]));
     } else if (k < b.nz && c.bg_on) {   // wall xy-edge under background shear (Eqs. 32-33)
-      t_xy = pp(in.toa_xy, q, S_TXY);
+      t_xy = in.toa_xy[q];
     }
-    if (j < b.ny && i > 0 && i < b.nx && k > 0 && k < b.nz) {
-      if constexpr (RC)
-        t_xz = fma(pp(in.em2_xz, q, S_EXZ), fma(pp(in.Vz, q, S_VZ) - in.Vz[q - 1], c.hrdx,
-                                                (pp(in.Vx, q, S_VX) - in.Vx[q - pxy]) * c.hrdz),
-                   pp(in.toa_xz, q, S_TXZ));
-      else
-        t_xz = fma(in.eb_xz[q], in.Vz[q] - in.Vz[q - 1], fma(pp(in.em2_xz, q, S_EXZ), in.Vx[q] - in.Vx[q - pxy],
-                                                             pp(in.toa_xz, q, S_TXZ)));
-    }
-    if (i < b.nx && j > 0 && j < b.ny && k > 0 && k < b.nz) {
-      if constexpr (RC)
-        t_yz = fma(pp(in.em2_yz, q, S_EYZ), fma(pp(in.Vz, q, S_VZ) - in.Vz[q - px], c.hrdy,
-                                                (pp(in.Vy, q, S_VY) - in.Vy[q - pxy]) * c.hrdz),
-                   pp(in.toa_yz, q, S_TYZ));
-      else
-        t_yz = fma(in.eb_yz[q], in.Vz[q] - in.Vz[q - px], fma(pp(in.em2_yz, q, S_EYZ), in.Vy[q] - in.Vy[q - pxy],
-                                                              pp(in.toa_yz, q, S_TYZ)));
-    }
+    if (j < b.ny && i > 0 && i < b.nx && k > 0 && k < b.nz)
+      t_xz = fma(in.eb_xz[q], in.Vz[q] - in.Vz[q - 1], fma(in.em2_xz[q], in.Vx[q] - in.Vx[q - pxy], in.toa_xz[q]));
+    if (i < b.nx && j > 0 && j < b.ny && k > 0 && k < b.nz)
+      t_yz = fma(in.eb_yz[q], in.Vz[q] - in.Vz[q - px], fma(in.em2_yz[q], in.Vy[q] - in.Vy[q - pxy], in.toa_yz[q]));
     if (cell) {
-      const T Pt = pp(in.Pt, q, S_PT), Pf = pp(in.Pf, q, S_PF), Pto = pp(in.Pto, q, S_PTO), Pfo = pp(in.Pfo, q, S_PFO);
-      const T ph = pp(in.phi, q, S_PHI), ieta = pp(in.ieta, q, S_IETA);
-      // k = K0 (phi / phi0)^3 (Eq. 23) at box index e with porosity p (recomputing forms)
-      auto kperm = [&](T p, long long e) {
-        const T r = p * c.rphi0;
-        return (in.K0 ? in.K0[e] : c.k0) * r * r * r;
-      };
-      T w;
-      if constexpr (RC) w = rcp_full(T(1.0) - ph);
-      else w = in.w[q];
-      const T vxl = pp(in.Vx, q, S_VX), vxr = in.Vx[q + 1], vyl = pp(in.Vy, q, S_VY), vyr = in.Vy[q + px];
-      const T vzl = pp(in.Vz, q, S_VZ), vzr = in.Vz[q + pxy];
-      const T gx = (vxr - vxl) * c.rdx, gy = (vyr - vyl) * c.rdy, gz = (vzr - vzl) * c.rdz;
-      const T divV = gx + gy + gz;
-      const T cc = c.compaction_on ? ieta * w : T(0);
-      const T dPt = Pt - Pto, dPf = Pf - Pfo, dpp = Pt - Pf;
+      const double Pt = in.Pt[q], Pf = in.Pf[q], Pto = in.Pto[q], Pfo = in.Pfo[q];
+      const double ph = in.phi[q], ieta = in.ieta[q], w = in.w[q];
+      const double vxl = in.Vx[q], vxr = in.Vx[q + 1], vyl = in.Vy[q], vyr = in.Vy[q + px];
+      const double vzl = in.Vz[q], vzr = in.Vz[q + pxy];
+      const double gx = (vxr - vxl) * c.rdx, gy = (vyr - vyl) * c.rdy, gz = (vzr - vzl) * c.rdz;
+      const double divV = gx + gy + gz;
+      const double cc = c.compaction_on ? ieta * w : 0.0;
+      const double dPt = Pt - Pto, dPf = Pf - Pfo, dpp = Pt - Pf;
       // explicit fused multiply-adds: the same rounding in every kernel that inlines this body
-      const T divVn = fma(dpp, cc, fma(-c.bd_rdt_a, dPf, fma(c.bd_rdt, dPt, divV)));
+      const double divVn = fma(dpp, cc, fma(-c.bd_rdt_a, dPf, fma(c.bd_rdt, dPt, divV)));
       // Darcy flux through the six faces (zero on the boundary) and the largest neighbour k
-      T kc;
-      if constexpr (!KS) kc = kperm(ph, q);
-      else kc = pp(in.perm, q, S_K);
-      T kmax = kc, sx = T(0), sy = T(0), sz = T(0);
+      const double kc = in.perm[q];
+      double kmax = kc, sx = 0.0, sy = 0.0, sz = 0.0;
       if (i > 0) {
-        T kn;
-        if constexpr (!KS) kn = kperm(in.phi[q - 1], q - 1);
-        else kn = in.perm[q - 1];
+        const double kn = in.perm[q - 1];
         kmax = pos_max(kmax, kn);
         sx -= (kn + kc) * (Pf - in.Pf[q - 1]);
       }
       if (i < b.nx - 1) {
-        T kn;
-        if constexpr (!KS) kn = kperm(in.phi[q + 1], q + 1);
-        else kn = in.perm[q + 1];
+        const double kn = in.perm[q + 1];
         kmax = pos_max(kmax, kn);
         sx += (kc + kn) * (in.Pf[q + 1] - Pf);
       }
       if (j > 0) {
-        T kn;
-        if constexpr (!KS) kn = kperm(in.phi[q - px], q - px);
-        else kn = in.perm[q - px];
+        const double kn = in.perm[q - px];
         kmax = pos_max(kmax, kn);
         sy -= (kn + kc) * (Pf - in.Pf[q - px]);
       }
       if (j < b.ny - 1) {
-        T kn;
-        if constexpr (!KS) kn = kperm(in.phi[q + px], q + px);
-        else kn = in.perm[q + px];
+        const double kn = in.perm[q + px];
         kmax = pos_max(kmax, kn);
         sy += (kc + kn) * (in.Pf[q + px] - Pf);
       }
       if (k > 0) {
-        T kn;
-        if constexpr (!KS) kn = kperm(in.phi[q - pxy], q - pxy);
-        else kn = in.perm[q - pxy];
+        const double kn = in.perm[q - pxy];
         kmax = pos_max(kmax, kn);
         sz -= (kn + kc) * ((Pf - in.Pf[q - pxy]) + c.buoy_dz);
       }
       if (k < b.nz - 1) {
-        T kn;
-        if constexpr (!KS) kn = kperm(in.phi[q + pxy], q + pxy);
-        else kn = in.perm[q + pxy];
+        const double kn = in.perm[q + pxy];
         kmax = pos_max(kmax, kn);
         sz += (kc + kn) * ((in.Pf[q + pxy] - Pf) + c.buoy_dz);
       }
       // div qD = -1/2 sum_d rd^2 [(k + k_r)(Pf_r - Pf) - (k_l + k)(Pf - Pf_l)]
-      const T divqD = -(sx * c.hrdx2 + sy * c.hrdy2 + sz * c.hrdz2);
+      const double divqD = -(sx * c.hrdx2 + sy * c.hrdy2 + sz * c.hrdz2);
       // local-implicit pressure updates, Eqs. 17-18: P1 = P - res / (1/dtau + d res/dP), the
       // residuals being divVn (row Pt) and resF (row Pf)
-      const T resF = fma(-dpp, cc, fma(-c.bd_rdt_a, dPt, fma(c.bda_B_rdt, dPf, divqD)));
-      const T Pt1 = Pt - rcp_pseudo(pp(in.idtp, q, S_IDTP) + cc) * divVn;   // idtp holds 1/dtau_Pt + beta_d/dt
-      const T Pf1 = Pf - rcp_pseudo(kmax * c.ifac_pf + c.bda_B_rdt + cc) * resF;
+      const double resF = fma(-dpp, cc, fma(-c.bd_rdt_a, dPt, fma(c.bda_B_rdt, dPf, divqD)));
+      const double Pt1 = Pt - rcp_pseudo(in.idtp[q] + cc) * divVn;   // idtp holds 1/dtau_Pt + beta_d/dt
+      const double Pf1 = Pf - rcp_pseudo(kmax * c.ifac_pf + c.bda_B_rdt + cc) * resF;
       // normal deviatoric stresses (Eq. 21): tau = tau_o xi/(1+xi) + 2 mu/(1+xi) (edot + beta_n divVn)
-      const T s3 = fma(c.beta_n, divVn, -(divV * T(1.0 / 3.0)));
-      const T cm2 = pp(in.cm2, q, S_CM2);
-      const T sxx = fma(cm2, gx + s3, pp(in.toa_xx, q, S_TXX));
-      const T syy = fma(cm2, gy + s3, pp(in.toa_yy, q, S_TYY));
-      const T szz = fma(cm2, gz + s3, pp(in.toa_zz, q, S_TZZ));
+      const double s3 = fma(c.beta_n, divVn, -(divV * (1.0 / 3.0)));
+      const double cm2 = in.cm2[q];
+      const double sxx = fma(cm2, gx + s3, in.toa_xx[q]);
+      const double syy = fma(cm2, gy + s3, in.toa_yy[q]);
+      const double szz = fma(cm2, gz + s3, in.toa_zz[q]);
       // porosity in log space (Eq. 22): L = Lo + delta,
       // delta = -[beta_phi ((Pf1 - Pfo) - (Pt1 - Pto)) + dt (Pf1 - Pt1) / eta + dt V.grad(1-phi)/(1-phi)]
       // V.grad(1-phi)/(1-phi) = -(w/2) sum_d rd [v_r (phi_r - phi) + v_l (phi - phi_l)]
       //                      = -w [sum_d hrd (v_r phi_r - v_l phi_l) - phi divV / 2]
       // (the velocities of wall faces are zero, so the divergence term is div V exactly)
-      T ax = T(0), ay = T(0), az = T(0);
+      double ax = 0.0, ay = 0.0, az = 0.0;
       if (i > 0) ax = -vxl * in.phi[q - 1];
       if (i < b.nx - 1) ax = fma(vxr, in.phi[q + 1], ax);
       if (j > 0) ay = -vyl * in.phi[q - px];
       if (j < b.ny - 1) ay = fma(vyr, in.phi[q + px], ay);
       if (k > 0) az = -vzl * in.phi[q - pxy];
       if (k < b.nz - 1) az = fma(vzr, in.phi[q + pxy], az);
-      const T adv = -w * fma(T(-0.5) * ph, divV, fma(ax, c.hrdx, fma(ay, c.hrdy, az * c.hrdz)));
-      const T comp = c.compaction_on ? (Pf1 - Pt1) * ieta : T(0);
-      const T delta = -(c.beta_phi * ((Pf1 - Pfo) - (Pt1 - Pto)) + c.dt * (comp + adv));
-      T em_p, em_n;
+      const double adv = -w * fma(-0.5 * ph, divV, fma(ax, c.hrdx, fma(ay, c.hrdy, az * c.hrdz)));
+      const double comp = c.compaction_on ? (Pf1 - Pt1) * ieta : 0.0;
+      const double delta = -(c.beta_phi * ((Pf1 - Pfo) - (Pt1 - Pto)) + c.dt * (comp + adv));
+      double em_p, em_n;
       expm1_pair(delta, em_p, em_n);
-      const T phio = pp(in.phio, q, S_PHIO);
-      T Eo, iEo;
-      if constexpr (RC) {
-        Eo = T(1.0) - phio;
-        iEo = T(0.0);   // not needed: 1/(1-phi) is recomputed from phi
-      } else {
-        Eo = in.Eo[q];
-        iEo = in.iEo[q];
-      }
-      const T K0 = in.K0 ? in.K0[q] : c.k0;
-      const T ph1 = phio - Eo * em_p;
-      const T r = ph1 * c.rphi0;
+      const double phio = in.phio[q], Eo = in.Eo[q], iEo = in.iEo[q];
+      const double K0 = in.K0 ? in.K0[q] : c.k0;
+      const double ph1 = phio - Eo * em_p;
+      const double r = ph1 * c.rphi0;
       // every load above precedes the stores (the arrays are not declared non-aliasing)
       out.Pt[q] = Pt1;
       out.Pf[q] = Pf1;
@@ -366,11 +305,11 @@ __device__ __forceinline__ void lean_cell_point(const Box& b, const LeanCoef<T>&
       out.tyy[q] = syy;
       out.tzz[q] = szz;
       out.phi[q] = ph1;
-      if constexpr (!RC) out.w[q] = iEo + iEo * em_n;
-      if constexpr (KS) out.perm[q] = K0 * r * r * r;
+      out.w[q] = iEo + iEo * em_n;
+      out.perm[q] = K0 * r * r * r;
       if (check) {
-        r_pt = to_d(tabs(divVn));
-        r_pf = to_d(tabs(resF));
+        r_pt = fabs(divVn);
+        r_pf = fabs(resF);
       }
     }
     if (k < b.nz) out.txy[q] = t_xy;
@@ -379,15 +318,13 @@ __device__ __forceinline__ void lean_cell_point(const Box& b, const LeanCoef<T>&
   }
 }
 
-// Momentum residual, damped R and velocity update of the three lower faces of (i, j, k); bit d
+// Momentum residual, damped R and velocity update of the three lower faces of (i, j, k) in FP64; bit d
 // of `mask` includes the face normal to direction d in the residual norm r_v.
-template <class T>
-__device__ __forceinline__ void lean_face_point(const Box& b, const LeanCoef<T>& c, const LeanFaceIn<T>& in,
-                                                T* __restrict__ Vx, T* __restrict__ Vy, T* __restrict__ Vz,
-                                                T* __restrict__ Rx, T* __restrict__ Ry, T* __restrict__ Rz,
-                                                int i, int j, int k, int check, double& r_v, int mask = 7) {
-  using namespace lean_detail;
-  constexpr bool RC = LeanRecompute<T>::value;
+__device__ __forceinline__ void lean_face_point(const Box& b, const LeanCoef<double>& c, const LeanFaceIn<double>& in,
+                                                double* __restrict__ Vx, double* __restrict__ Vy,
+                                                double* __restrict__ Vz, double* __restrict__ Rx,
+                                                double* __restrict__ Ry, double* __restrict__ Rz, int i, int j, int k,
+                                                int check, double& r_v, int mask = 7) {
   if (i <= b.nx && j <= b.ny && k <= b.nz) {
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
@@ -395,44 +332,35 @@ __device__ __forceinline__ void lean_face_point(const Box& b, const LeanCoef<T>&
     const bool fy = j > 0 && j < b.ny && i < b.nx && k < b.nz;
     const bool fz = k > 0 && k < b.nz && i < b.nx && j < b.ny;
     // all loads before the first store (the arrays are not declared non-aliasing)
-    T Fx = T(0), Fy = T(0), Fz = T(0), Rx1 = T(0), Ry1 = T(0), Rz1 = T(0), Vx1 = T(0), Vy1 = T(0), Vz1 = T(0);
+    double Fx = 0.0, Fy = 0.0, Fz = 0.0, Rx1 = 0.0, Ry1 = 0.0, Rz1 = 0.0, Vx1 = 0.0, Vy1 = 0.0, Vz1 = 0.0;
     // F / rho_i directly (the spacings carry 1/rho_i); the norm takes |F| = rho_i |F / rho_i|
     if (fx) {
       Fx = (in.txx[q] - in.txx[q - 1]) * c.rdx_r + (in.txy[q + px] - in.txy[q]) * c.rdy_r +
            (in.txz[q + pxy] - in.txz[q]) * c.rdz_r - (in.Pt1[q] - in.Pt1[q - 1]) * c.rdx_r;
       Rx1 = fma(c.damp_x, Rx[q], Fx);
-      T dtv;
-      if constexpr (RC) dtv = T(0.5) * (in.dtv_x[q - 1] + in.dtv_x[q]);
-      else dtv = in.dtv_x[q];
-      Vx1 = fma(dtv, Rx1, Vx[q]);
+      Vx1 = fma(in.dtv_x[q], Rx1, Vx[q]);
     }
     if (fy) {
       Fy = (in.txy[q + 1] - in.txy[q]) * c.rdx_r + (in.tyy[q] - in.tyy[q - px]) * c.rdy_r +
            (in.tyz[q + pxy] - in.tyz[q]) * c.rdz_r - (in.Pt1[q] - in.Pt1[q - px]) * c.rdy_r;
       Ry1 = fma(c.damp_y, Ry[q], Fy);
-      T dtv;
-      if constexpr (RC) dtv = T(0.5) * (in.dtv_y[q - px] + in.dtv_y[q]);
-      else dtv = in.dtv_y[q];
-      Vy1 = fma(dtv, Ry1, Vy[q]);
+      Vy1 = fma(in.dtv_y[q], Ry1, Vy[q]);
     }
     if (fz) {
       // buoyancy -(rho g - rho_BG g) averaged to the face, rho g - rho_BG g = (phi - phi0) drho_g
-      const T rog = (T(0.5) * (in.phi[q - pxy] + in.phi[q]) - c.phi0) * c.drho_g_r;
+      const double rog = (0.5 * (in.phi[q - pxy] + in.phi[q]) - c.phi0) * c.drho_g_r;
       Fz = (in.txz[q + 1] - in.txz[q]) * c.rdx_r + (in.tyz[q + px] - in.tyz[q]) * c.rdy_r +
            (in.tzz[q] - in.tzz[q - pxy]) * c.rdz_r - (in.Pt1[q] - in.Pt1[q - pxy]) * c.rdz_r - rog;
       Rz1 = fma(c.damp_z, Rz[q], Fz);
-      T dtv;
-      if constexpr (RC) dtv = T(0.5) * (in.dtv_z[q - pxy] + in.dtv_z[q]);
-      else dtv = in.dtv_z[q];
-      Vz1 = fma(dtv, Rz1, Vz[q]);
+      Vz1 = fma(in.dtv_z[q], Rz1, Vz[q]);
     }
     if (fx) { Rx[q] = Rx1; Vx[q] = Vx1; }
     if (fy) { Ry[q] = Ry1; Vy[q] = Vy1; }
     if (fz) { Rz[q] = Rz1; Vz[q] = Vz1; }
     if (check) {
-      if (fx && (mask & 1)) r_v = fmax(r_v, to_d(tabs(Fx)) * to_d(c.rho_i));
-      if (fy && (mask & 2)) r_v = fmax(r_v, to_d(tabs(Fy)) * to_d(c.rho_i));
-      if (fz && (mask & 4)) r_v = fmax(r_v, to_d(tabs(Fz)) * to_d(c.rho_i));
+      if (fx && (mask & 1)) r_v = fmax(r_v, fabs(Fx) * c.rho_i);
+      if (fy && (mask & 2)) r_v = fmax(r_v, fabs(Fy) * c.rho_i);
+      if (fz && (mask & 4)) r_v = fmax(r_v, fabs(Fz) * c.rho_i);
     }
   }
 }
@@ -605,9 +533,9 @@ __device__ __forceinline__ void lean_coef_point(const Box& b, const LeanCoef<T>&
     out.toa_yz[q] = in.tyzo[q] * (one - s);
   }
   // pseudo-time steps of the velocities, mean of the two centres' dtau_V = fac / mu (the
-  // recomputing forms store the centre values and average them in the faces kernel)
+  // recomputing forms store half the centre values and add two in the faces kernel)
   if constexpr (RC) {
-    if (i < b.nx && j < b.ny && k < b.nz) out.dtv_x[q] = c.dtauv_fac * rcp_full(in.mu[q]);
+    if (i < b.nx && j < b.ny && k < b.nz) out.dtv_x[q] = T(0.5) * c.dtauv_fac * rcp_full(in.mu[q]);
     return;
   }
   const T imu = (i < b.nx && j < b.ny && k < b.nz) ? rcp_full(in.mu[q]) : T(0.0);

@@ -22,6 +22,7 @@
 // local-implicit Pt, Pf (Eqs. 17-18), stresses at centres and the cell's three lower edges
 // (Eq. 21), porosity (Eq. 22). k_lean_faces: momentum residual (Eq. 19) with Pt^{k+1},
 // damped R, V^{k+1}. k_lean_picard: Picard targets (Eqs. 24-26) with log-space relaxation.
+#include "pt_df_body.cuh"
 #include "pt_lean_body.cuh"
 
 #include <algorithm>
@@ -29,10 +30,8 @@
 namespace pt {
 
 // ------------------------------------------------------------------------------ cells
-template <class T>
-__global__ void __launch_bounds__(256, 3) k_lean_cells(Box b, LeanCoef<T> c, LeanCellIn<T> in,
-                                                    LeanCellOut<T> out, unsigned long long* red,
-                                                    int check) {
+__global__ void __launch_bounds__(256, 3) k_lean_cells(Box b, LeanCoef<double> c, LeanCellIn<double> in,
+                                                       LeanCellOut<double> out, unsigned long long* red, int check) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -44,110 +43,160 @@ __global__ void __launch_bounds__(256, 3) k_lean_cells(Box b, LeanCoef<T> c, Lea
   }
 }
 
-// ------------------------------------------------- cells, z-marching with staged inputs
-// The double-float cells kernel is limited by memory latency: with 80 registers a thread cannot
-// hold all of its ~30 loads in flight, so memory time and issue time add up. Here each 32 x 8
-// block marches through kLeanZChunk z-levels of its column; the 15 arrays read only at the
-// thread's own index (kStageSlots, pointwise) of level k+1 are copied into a shared-memory stage
-// by cp.async while level k computes (two stages, 61,440 B per block), so those loads take no
-// registers and overlap the arithmetic. The neighbour arrays (V, Pt, Pf, phi, k) are loaded
-// directly (z-neighbours of consecutive levels hit L1 / L2).
-constexpr int kLeanZChunk = 16;
-constexpr int kStageThreads = 256;
-// stage the own-index values of the neighbour arrays too (22 slots, 102 registers, 2 blocks per
-// SM: 10.4 ms per 511^3 launch) or only the pointwise arrays (15 slots, 80 registers, 3 blocks
-// per SM: 9.9 ms)
-constexpr bool kStageAll = false;
-constexpr int kSlots = kStageAll ? (int)kStageSlotsAll : (int)kStageSlots;
-constexpr int kZmarchBlocks = kStageAll ? 2 : 3;
+// ------------------------------------------------- double-float cells, z-marching
+// Each 32 x 8 block marches up a chunk of z-levels (march_chunk) of its column. Every array a level reads
+// is copied by 16-byte cp.async into a shared-memory stage one level ahead (Pf, phi, k, Vz two, since
+// level k reads them at k + 1), rows by warps: two arrays' 16 vectors of a row at a time, the row ends
+// of all six neighbour arrays in one instruction, the halo rows above and below by six of the warps. So
+// no load from global memory is waited for inside a level, neighbours come from shared memory by
+// constant offsets, and one barrier per level separates a slot's readers from its refill. The Darcy
+// flux through a z face is formed once and carried up. 111,616 B per block, 2 blocks per SM. At 239^3:
+// 1.05 ms a launch when the neighbours were read from global memory (1929 instructions per cell, 55 % of
+// the issue slots), 0.67 ms in this form (5.2 TB/s of its 256 B per cell, 0.77 of the copy peak).
+constexpr int kLeanZChunk = 16;   // the longest chunk (32: the same at 383^3, 14.0 against 13.0 ms at 127^3)
+constexpr int kZmarchBlocks = 2;
 
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gmem) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// Reads a staged slot from this level's stage (kSlots x kStageThreads values); slots outside the
-// staged set are read from global memory (the stage holds nothing for them).
-template <class T>
-struct StagedPoint {
-  const T* s;
-  int tid;
-  __device__ __forceinline__ T operator()(const T* a, long long q, int slot) const {
-    return slot < kSlots ? s[slot * kStageThreads + tid] : a[q];
-  }
+// The copies of one thread: pointers at level 0 (its row or halo row and column), places in the stage.
+struct DfStager {
+  const df64 *h3a, *h3b, *h2, *pw[kDfPoint / 2];   // pairs: the lower half-warp's array or the upper's
+  const df64 *edge, *halo;
+  int d_row, d_pw, d_edge, d_halo;                 // offsets into the stage
+  bool ok_row, ok_edge, ok_halo, edge3, halo3;     // edge3, halo3: an array of three slots
 };
 
-template <class T>
-__device__ __forceinline__ void stage_level(T* dst, const LeanCellIn<T>& in, long long q) {
-  cp_async8(dst + S_PTO * kStageThreads, in.Pto + q);
-  cp_async8(dst + S_PFO * kStageThreads, in.Pfo + q);
-  cp_async8(dst + S_PHIO * kStageThreads, in.phio + q);
-  cp_async8(dst + S_IETA * kStageThreads, in.ieta + q);
-  cp_async8(dst + S_IDTP * kStageThreads, in.idtp + q);
-  cp_async8(dst + S_CM2 * kStageThreads, in.cm2 + q);
-  cp_async8(dst + S_TXX * kStageThreads, in.toa_xx + q);
-  cp_async8(dst + S_TYY * kStageThreads, in.toa_yy + q);
-  cp_async8(dst + S_TZZ * kStageThreads, in.toa_zz + q);
-  cp_async8(dst + S_EXY * kStageThreads, in.em2_xy + q);
-  cp_async8(dst + S_EXZ * kStageThreads, in.em2_xz + q);
-  cp_async8(dst + S_EYZ * kStageThreads, in.em2_yz + q);
-  cp_async8(dst + S_TXY * kStageThreads, in.toa_xy + q);
-  cp_async8(dst + S_TXZ * kStageThreads, in.toa_xz + q);
-  cp_async8(dst + S_TYZ * kStageThreads, in.toa_yz + q);
-  if constexpr (kStageAll) {
-    cp_async8(dst + S_VX * kStageThreads, in.Vx + q);
-    cp_async8(dst + S_VY * kStageThreads, in.Vy + q);
-    cp_async8(dst + S_VZ * kStageThreads, in.Vz + q);
-    cp_async8(dst + S_PT * kStageThreads, in.Pt + q);
-    cp_async8(dst + S_PF * kStageThreads, in.Pf + q);
-    cp_async8(dst + S_PHI * kStageThreads, in.phi + q);
-    cp_async8(dst + S_K * kStageThreads, in.perm + q);
+__device__ __forceinline__ DfStager df_stager(const Box& b, const LeanCellIn<df64>& in, int i0, int j0) {
+  const int lane = threadIdx.x, w = threadIdx.y, hi = lane >> 4, v = lane & 15;
+  DfStager s;
+  const int j = j0 + w, col = i0 + 2 * v;
+  s.ok_row = j <= b.ny && col < b.px;
+  const long long q = (long long)col + (long long)b.px * j;
+  s.h3a = (hi ? in.phi : in.Pf) + q;
+  s.h3b = (hi ? in.Vz : in.perm) + q;
+  s.h2 = (hi ? in.Vy : in.Vx) + q;
+  const df64* const p[kDfPoint] = {in.Pto, in.Pfo, in.phio, in.ieta, in.idtp, in.cm2, in.toa_xx, in.toa_yy,
+                                   in.toa_zz, in.em2_xy, in.em2_xz, in.em2_yz, in.toa_xy, in.toa_xz, in.toa_yz,
+                                   in.Pt};          // the order of the S_ slots
+#pragma unroll
+  for (int n = 0; n < kDfPoint / 2; ++n) s.pw[n] = (hi ? p[2 * n + 1] : p[2 * n]) + q;
+  s.d_row = (w + 1) * kDfW + 2 + 2 * v;
+  s.d_pw = kDfPW + hi * 256 + 32 * w + 2 * v;
+  // row ends: lanes 0-11, array lane / 2, the vector left (even lanes) or right of the row
+  const int a = lane >> 1, ec = (lane & 1) ? i0 + 32 : i0 - 2;
+  s.edge3 = a < kDfHalo3;
+  s.ok_edge = lane < 12 && j <= b.ny && ec >= 0 && ec < b.px;
+  s.edge = (a == 0 ? in.Pf : a == 1 ? in.phi : a == 2 ? in.perm : a == 3 ? in.Vz : a == 4 ? in.Vx : in.Vy) + ec +
+           (long long)b.px * j;
+  s.d_edge = (s.edge3 ? a * 3 * kDfAR : kDfH2 + (a - kDfHalo3) * 2 * kDfAR) + (w + 1) * kDfW + ((lane & 1) ? 34 : 0);
+  // halo rows: warps 0-5, one array each, the row below (lower half-warp) and above
+  const int hj = hi ? j0 + 8 : j0 - 1;
+  s.halo3 = w < kDfHalo3;
+  s.ok_halo = w < 6 && hj >= 0 && hj <= b.ny && col < b.px;
+  s.halo = (w == 0 ? in.Pf : w == 1 ? in.phi : w == 2 ? in.perm : w == 3 ? in.Vz : w == 4 ? in.Vx : in.Vy) + col +
+           (long long)b.px * hj;
+  s.d_halo = (s.halo3 ? w * 3 * kDfAR : kDfH2 + (w - kDfHalo3) * 2 * kDfAR) + (hi ? 9 * kDfW : 0) + 2 + 2 * v;
+  return s;
+}
+
+// Level L of Pf, phi, k, Vz into slot m3 of three.
+__device__ __forceinline__ void df_stage3(df64* st, const DfStager& s, long long pxy, int L, int m3) {
+  const long long o = pxy * L;
+  const int t = m3 * kDfAR, hi = threadIdx.x >> 4;
+  if (s.ok_row) {
+    cp_async16(st + t + hi * 3 * kDfAR + s.d_row, s.h3a + o);
+    cp_async16(st + t + (2 + hi) * 3 * kDfAR + s.d_row, s.h3b + o);
+  }
+  if (s.ok_edge && s.edge3) cp_async16(st + t + s.d_edge, s.edge + o);
+  if (s.ok_halo && s.halo3) cp_async16(st + t + s.d_halo, s.halo + o);
+}
+// Level L of Vx, Vy and the pointwise arrays into slot m2 of two.
+__device__ __forceinline__ void df_stage2(df64* st, const DfStager& s, long long pxy, int L, int m2) {
+  const long long o = pxy * L;
+  const int t = m2 * kDfAR, hi = threadIdx.x >> 4;
+  if (s.ok_row) {
+    cp_async16(st + t + kDfH2 + hi * 2 * kDfAR + s.d_row, s.h2 + o);
+#pragma unroll
+    for (int n = 0; n < kDfPoint / 2; ++n) cp_async16(st + m2 * kDfPWSlot + n * 512 + s.d_pw, s.pw[n] + o);
+  }
+  if (s.ok_edge && !s.edge3) cp_async16(st + t + s.d_edge, s.edge + o);
+  if (s.ok_halo && !s.halo3) cp_async16(st + t + s.d_halo, s.halo + o);
+}
+
+template <bool INNER>
+__device__ __forceinline__ void df_cells_run(const Box& b, const LeanCoef<df64>& c, const LeanCellIn<df64>& in,
+                                             const LeanCellOut<df64>& out, int i, int j, int k0, int k1, int check,
+                                             df64* st, unsigned long long& m_pt, unsigned long long& m_pf) {
+  const DfStager s = df_stager(b, in, i - (int)threadIdx.x, j - (int)threadIdx.y);
+  df_stage3(st, s, b.pxy, k0, 0);
+  df_stage3(st, s, b.pxy, k0 + 1, 1);
+  df_stage2(st, s, b.pxy, k0, 0);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  DfColumn col;
+  col.phi_d = col.k_d = col.vx_d = col.vy_d = col.fz = df64(0.0f, 0.0f);
+  if (k0 > 0 && (INNER || (i <= b.nx && j <= b.ny))) {
+    const long long q = cidx(b, i, j, k0), d = q - b.pxy;
+    col.phi_d = in.phi[d];
+    col.k_d = in.perm[d];
+    col.vx_d = in.Vx[d];
+    col.vy_d = in.Vy[d];
+    col.fz = dfu::mul(dfu::add(col.k_d, in.perm[q]), dfu::add(dfu::sub(in.Pf[q], in.Pf[d]), c.buoy_dz));
+  }
+  const df64* const t3 = st + (threadIdx.y + 1) * kDfW + threadIdx.x + 2;
+  const df64* const tp = st + kDfPW + 32 * threadIdx.y + threadIdx.x;
+  int m3 = 0;                                       // slot of level k in the rings of three
+  for (int k = k0; k < k1; ++k) {
+    const int m2 = (k - k0) & 1, m3p = m3 == 2 ? 0 : m3 + 1, m3n = m3p == 2 ? 0 : m3p + 1;
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();   // level k's copies are visible, and every thread is done with level k - 1
+    if (k + 1 < k1) {
+      df_stage2(st, s, b.pxy, k + 1, m2 ^ 1);
+      df_stage3(st, s, b.pxy, k + 2, m3n);          // k + 2 <= nz: a level of the box
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    df_cell_level<INNER>(b, c, in.K0, out, i, j, k, check, col, m_pt, m_pf, t3 + m3 * kDfAR, t3 + m3p * kDfAR,
+                         t3 + kDfH2 + m2 * kDfAR, tp + m2 * kDfPWSlot);
+    m3 = m3p;
   }
 }
 
-template <class T>
-__global__ void __launch_bounds__(kStageThreads, kZmarchBlocks) k_lean_cells_zmarch(Box b, LeanCoef<T> c, LeanCellIn<T> in,
-                                                                       LeanCellOut<T> out,
-                                                                       unsigned long long* red, int check) {
+__global__ void __launch_bounds__(256, kZmarchBlocks) k_df_cells(Box b, LeanCoef<df64> c, LeanCellIn<df64> in,
+                                                                 LeanCellOut<df64> out, unsigned long long* red,
+                                                                 int check, int zchunk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* stage = reinterpret_cast<T*>(smem_raw);   // [2][kSlots][kStageThreads]
-  const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k0 = blockIdx.z * kLeanZChunk;
-  const int k1 = min(k0 + kLeanZChunk, b.nz + 1);   // levels [k0, k1), all inside the box
-  const bool active = i <= b.nx && j <= b.ny;      // the body's own index range
-  constexpr int stage_elems = kSlots * kStageThreads;
-  if (active) stage_level(stage + tid, in, cidx(b, i, j, k0));
-  cp_async_commit();
+  df64* const st = reinterpret_cast<df64*>(smem_raw);
+  const int i = blockIdx.x * 32 + threadIdx.x;
+  const int j = blockIdx.y * 8 + threadIdx.y;
+  const int k0 = blockIdx.z * zchunk;
+  const int k1 = min(k0 + zchunk, b.nz);
+  const bool inner = blockIdx.x > 0 && blockIdx.y > 0 && (int)blockIdx.x * 32 + 32 < b.nx && (int)blockIdx.y * 8 + 8 < b.ny;
   unsigned long long m_pt = 0ull, m_pf = 0ull;     // norms as bit patterns: a NaN stays the largest
-  for (int k = k0; k < k1; ++k) {
-    const int buf = (k - k0) & 1;
-    if (active && k + 1 < k1) stage_level(stage + (buf ^ 1) * stage_elems + tid, in, cidx(b, i, j, k + 1));
-    cp_async_commit();
-    cp_async_wait_1();                              // this level's copies have landed
-    double r_pt = 0.0, r_pf = 0.0;
-    lean_cell_point(b, c, in, out, i, j, k, check, r_pt, r_pf, StagedPoint<T>{stage + buf * stage_elems, tid});
-    const unsigned long long a = (unsigned long long)__double_as_longlong(r_pt);
-    const unsigned long long d = (unsigned long long)__double_as_longlong(r_pf);
-    m_pt = a > m_pt ? a : m_pt;
-    m_pf = d > m_pf ? d : m_pf;
-    __syncthreads();                                // every read of this stage precedes its refill
-  }
+  if (inner) df_cells_run<true>(b, c, in, out, i, j, k0, k1, check, st, m_pt, m_pf);
+  else df_cells_run<false>(b, c, in, out, i, j, k0, k1, check, st, m_pt, m_pf);
   if (check) {
     block_max_atomic(__longlong_as_double((long long)m_pt), red + RED_PT);
     block_max_atomic(__longlong_as_double((long long)m_pf), red + RED_PF);
   }
 }
 
+__global__ void __launch_bounds__(256) k_df_faces(Box b, LeanCoef<df64> c, LeanFaceIn<df64> in, df64* __restrict__ Vx,
+                                                  df64* __restrict__ Vy, df64* __restrict__ Vz, df64* __restrict__ Rx,
+                                                  df64* __restrict__ Ry, df64* __restrict__ Rz,
+                                                  unsigned long long* red, int check) {
+  double r_v = 0.0;
+  df_face_point(b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, blockIdx.x * 32 + threadIdx.x, blockIdx.y * 8 + threadIdx.y,
+                blockIdx.z, check, r_v);
+  if (check) block_max_atomic(r_v, red + RED_V);
+}
+
 // ------------------------------------------------------------------------------ faces
-template <class T>
-__global__ void __launch_bounds__(256) k_lean_faces(Box b, LeanCoef<T> c, LeanFaceIn<T> in,
-                                                    T* __restrict__ Vx, T* __restrict__ Vy,
-                                                    T* __restrict__ Vz, T* __restrict__ Rx,
-                                                    T* __restrict__ Ry, T* __restrict__ Rz,
+__global__ void __launch_bounds__(256) k_lean_faces(Box b, LeanCoef<double> c, LeanFaceIn<double> in,
+                                                    double* __restrict__ Vx, double* __restrict__ Vy,
+                                                    double* __restrict__ Vz, double* __restrict__ Rx,
+                                                    double* __restrict__ Ry, double* __restrict__ Rz,
                                                     unsigned long long* red, int check) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -235,7 +284,9 @@ __global__ void __launch_bounds__(256) k_lean_begin(Box b, LeanCoef<T> c, LeanBe
       out.iEo[q] = iEo;
       out.w[q] = iEo;
     }
-    if constexpr (LeanStoreK<T>::value) {
+    if constexpr (LeanRecompute<T>::value) {   // K0 = k0 e^logk / phi0^3
+      out.perm[q] = (in.K0 ? in.K0[q] : c.k0r3) * ph * ph * ph;
+    } else {
       const T r = ph * c.rphi0;
       out.perm[q] = (in.K0 ? in.K0[q] : c.k0) * r * r * r;
     }
@@ -244,7 +295,7 @@ __global__ void __launch_bounds__(256) k_lean_begin(Box b, LeanCoef<T> c, LeanBe
   block_max_atomic(m, red + RED_MUMAX);
 }
 
-// K0 = k0 e^logk / phi0^3 is folded into k = K0 phi^3; here K0 = k0 e^logk (phi0 via rphi0).
+// K0 = k0 e^logk (k0 / phi0^3 in the double-float form, whose k is K0 phi^3).
 template <class T>
 __global__ void k_lean_k0(Box b, double k0, const double* __restrict__ logk, T* __restrict__ K0) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -319,24 +370,33 @@ void math_check(cudaStream_t st, int fn, const double* a, const double* b, doubl
   k_math_check<<<g, 256, 0, st>>>(fn, a, b, out, n);
 }
 
-template <class T>
-void lean_cells(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanCellIn<T>& in,
-                const LeanCellOut<T>& out, unsigned long long* red, int check) {
-  k_lean_cells<T><<<gr, bl, 0, st>>>(b, c, in, out, red, check);
-}
-// The double-float form's cells launch: the z-marching staged kernel (the block shape stays 32 x 8).
 template <>
-void lean_cells<df64>(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<df64>& c, const LeanCellIn<df64>& in,
-                      const LeanCellOut<df64>& out, unsigned long long* red, int check) {
-  const int smem = 2 * kSlots * kStageThreads * (int)sizeof(df64);
-  cudaFuncSetAttribute(k_lean_cells_zmarch<df64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  const dim3 g(gr.x, gr.y, (unsigned)((b.nz + 1 + kLeanZChunk - 1) / kLeanZChunk));
-  k_lean_cells_zmarch<df64><<<g, dim3(32, 8, 1), smem, st>>>(b, c, in, out, red, check);
+void lean_cells<double>(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c,
+                        const LeanCellIn<double>& in, const LeanCellOut<double>& out, unsigned long long* red,
+                        int check) {
+  k_lean_cells<<<gr, bl, 0, st>>>(b, c, in, out, red, check);
 }
-template <class T>
-void lean_faces(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanFaceIn<T>& in,
-                T* Vx, T* Vy, T* Vz, T* Rx, T* Ry, T* Rz, unsigned long long* red, int check) {
-  k_lean_faces<T><<<gr, bl, 0, st>>>(b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, red, check);
+// The double-float form: the wall indices i = nx, j = ny carry stress under a background shear only.
+template <>
+void lean_cells<df64>(dim3, dim3, cudaStream_t st, Box b, const LeanCoef<df64>& c, const LeanCellIn<df64>& in,
+                      const LeanCellOut<df64>& out, unsigned long long* red, int check) {
+  const int smem = kDfStageElems * (int)sizeof(df64), w = c.bg_on ? 1 : 0;
+  cudaFuncSetAttribute(k_df_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const unsigned gx = (b.nx + w + 31) / 32, gy = (b.ny + w + 7) / 8;
+  const int zc = march_chunk((long long)gx * gy, b.nz, kLeanZChunk, kZmarchBlocks, sm_count(), 1.0, 1.6);
+  k_df_cells<<<dim3(gx, gy, (unsigned)((b.nz + zc - 1) / zc)), dim3(32, 8, 1), smem, st>>>(b, c, in, out, red, check, zc);
+}
+template <>
+void lean_faces<df64>(dim3, dim3, cudaStream_t st, Box b, const LeanCoef<df64>& c, const LeanFaceIn<df64>& in, df64* Vx,
+                      df64* Vy, df64* Vz, df64* Rx, df64* Ry, df64* Rz, unsigned long long* red, int check) {
+  const dim3 g((unsigned)((b.nx + 31) / 32), (unsigned)((b.ny + 7) / 8), (unsigned)b.nz);
+  k_df_faces<<<g, dim3(32, 8, 1), 0, st>>>(b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, red, check);
+}
+template <>
+void lean_faces<double>(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c,
+                        const LeanFaceIn<double>& in, double* Vx, double* Vy, double* Vz, double* Rx, double* Ry,
+                        double* Rz, unsigned long long* red, int check) {
+  k_lean_faces<<<gr, bl, 0, st>>>(b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, red, check);
 }
 template <class T>
 void lean_picard(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanPicardIn<T>& in,
@@ -358,10 +418,6 @@ void lean_k0(dim3 gr, dim3 bl, cudaStream_t st, Box b, double k0, const double* 
   k_lean_k0<T><<<gr, bl, 0, st>>>(b, k0, logk, K0);
 }
 
-template void lean_cells<double>(dim3, dim3, cudaStream_t, Box, const LeanCoef<double>&, const LeanCellIn<double>&,
-                                 const LeanCellOut<double>&, unsigned long long*, int);
-template void lean_faces<double>(dim3, dim3, cudaStream_t, Box, const LeanCoef<double>&, const LeanFaceIn<double>&,
-                                 double*, double*, double*, double*, double*, double*, unsigned long long*, int);
 template void lean_picard<double>(dim3, dim3, cudaStream_t, Box, const LeanCoef<double>&, const LeanPicardIn<double>&,
                                   double*, double*, unsigned long long*);
 template void lean_coef<double>(dim3, dim3, cudaStream_t, Box, const LeanCoef<double>&, const LeanCoefIn<double>&,
@@ -370,8 +426,6 @@ template void lean_begin<double>(dim3, dim3, cudaStream_t, Box, const LeanCoef<d
                                  const LeanBeginOut<double>&, unsigned long long*);
 template void lean_k0<double>(dim3, dim3, cudaStream_t, Box, double, const double*, double*);
 
-template void lean_faces<df64>(dim3, dim3, cudaStream_t, Box, const LeanCoef<df64>&, const LeanFaceIn<df64>&,
-                                 df64*, df64*, df64*, df64*, df64*, df64*, unsigned long long*, int);
 template void lean_picard<df64>(dim3, dim3, cudaStream_t, Box, const LeanCoef<df64>&, const LeanPicardIn<df64>&,
                                   df64*, df64*, unsigned long long*);
 template void lean_coef<df64>(dim3, dim3, cudaStream_t, Box, const LeanCoef<df64>&, const LeanCoefIn<df64>&,

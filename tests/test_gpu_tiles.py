@@ -41,3 +41,16 @@ def test_fp32_correction_tiles(nx, ny, nz):
     case = dict(kind="corr", nx=nx, ny=ny, nz=nz, rounds=2, iters=20, mg=0, logk=True)
     worst, off = _worst(case)
     assert worst < 2 * 20 * 8 * 2.0 ** -24, off
+
+
+# 32 x 8 column blocks in chunks of levels, and index maps over the planes' points
+@pytest.mark.parametrize("form", ["df64", "fp64"])
+@pytest.mark.parametrize("nx,ny,nz,shear,logk", [(3, 2, 1, False, False), (31, 7, 5, True, False),
+                                                 (32, 8, 17, False, True), (33, 9, 16, True, True),
+                                                 (64, 15, 33, False, False), (97, 26, 40, True, False),
+                                                 (130, 50, 21, False, True)])
+def test_fixed_count_steps(form, nx, ny, nz, shear, logk):
+    """Three Picard intervals of PT iterations; the FP64-class bar of the oracle comparisons, 1e-10."""
+    case = dict(kind="step", form=form, nx=nx, ny=ny, nz=nz, iters=45, shear=shear, logk=logk)
+    worst, off = _worst(case)
+    assert worst < 1e-10, off
