@@ -17,7 +17,7 @@ struct AdjCoef {
   double bd_rdt, bd_rdt_a, bda_B_rdt, beta_phi, dt, dt_r;   // dt_r = dt / (eta0 mu0)
   double idtp;                          // 1 / dtau_Pt
   double ifac_pf;                       // dtau_Pf = 1 / (kmax ifac_pf)
-  double rphi0, k0;
+  double k0;                            // k0 / phi0^3: k = k0 phi^3 (or K0 phi^3)
   double buoy;                          // (rho_f - rho_BG) g
   double hdrho_g;                       // (rho_f - rho_s) g / 2
   double hdt_rdx, hdt_rdy, hdt_rdz;     // dt / 2 / d_i (advection)

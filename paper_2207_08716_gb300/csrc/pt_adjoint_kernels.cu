@@ -29,8 +29,7 @@ __device__ inline double pos_max_d(double a, double b) {
   return __longlong_as_double(ia > ib ? ia : ib);
 }
 __device__ inline double kperm(const AdjCoef& c, const double* K0, long long q, double ph) {
-  const double r = ph * c.rphi0;
-  return (K0 ? K0[q] : c.k0) * r * r * r;
+  return (K0 ? K0[q] : c.k0) * ph * ph * ph;
 }
 }  // namespace
 

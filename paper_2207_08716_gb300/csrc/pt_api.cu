@@ -500,7 +500,7 @@ void launch_lean_coef(pt_ctx* c) {
                          c->em2_xz, c->em2_yz, c->eb_xy, c->eb_xz, c->eb_yz, c->toa_xy, c->toa_xz, c->toa_yz,
                          c->dtv_x, c->dtv_y,
                          c->dtv_z};
-  PT_LAUNCH(c, K_LEAN_COEF, lean_coef<double>(grid_dims(b), block_dims(), c->stream, b, c->lcoef, ci, co));
+  PT_LAUNCH(c, K_LEAN_COEF, lean_coef<double>(c->stream, b, c->lcoef, ci, co));
 }
 
 // One PT iteration of the FP64-lean form: cells (pressures, stresses, porosity), faces
@@ -517,15 +517,15 @@ void launch_iteration_lean(pt_ctx* c, int check) {
                         c->toa_xy, c->toa_xz, c->toa_yz, c->logk ? c->K0 : nullptr};
   LeanCellOut<double> co{c->Pt[n], c->Pf[n], c->phi[n], c->lw[n], c->lperm[n], c->s_txx, c->s_tyy,
                          c->s_tzz, c->s_txy, c->s_txz, c->s_tyz};
-  PT_LAUNCH(c, K_LEAN_CELLS, lean_cells<double>(gr, bl, c->stream, b, c->lcoef, ci, co, c->red, check));
+  PT_LAUNCH(c, K_LEAN_CELLS, lean_cells<double>(c->stream, b, c->lcoef, ci, co, c->red, check));
   LeanFaceIn<double> fi{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz, c->Pt[n],
                         c->phi[a], c->dtv_x, c->dtv_y, c->dtv_z};
-  PT_LAUNCH(c, K_LEAN_FACES, lean_faces<double>(gr, bl, c->stream, b, c->lcoef, fi, c->Vx, c->Vy, c->Vz, c->Rx,
+  PT_LAUNCH(c, K_LEAN_FACES, lean_faces<double>(c->stream, b, c->lcoef, fi, c->Vx, c->Vy, c->Vz, c->Rx,
                                                    c->Ry, c->Rz, c->red, check));
   if (check) {
     LeanPicardIn<double> pi{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz, c->phi[n],
                             c->Pt[n], c->Pf[n]};
-    PT_LAUNCH(c, K_LEAN_PICARD, lean_picard<double>(gr, bl, c->stream, b, c->lcoef, pi, c->mu, c->eta, c->red));
+    PT_LAUNCH(c, K_LEAN_PICARD, lean_picard<double>(c->stream, b, c->lcoef, pi, c->mu, c->eta, c->red));
     launch_lean_coef(c);
   }
   c->cur = n;
@@ -572,7 +572,7 @@ void launch_df_coef(pt_ctx* c) {
                        D(c->em2_xy), D(c->em2_xz), D(c->em2_yz), D(c->eb_xy), D(c->eb_xz), D(c->eb_yz),
                        D(c->toa_xy), D(c->toa_xz), D(c->toa_yz), D(c->dtv_x), D(c->dtv_x), D(c->dtv_x)};
   // (double-float form: em2_* hold the raw edge moduli, dtv_x the per-centre velocity pseudo-step)
-  PT_LAUNCH(c, K_DF_COEF, lean_coef<df64>(grid_dims(b), block_dims(), c->stream, b, c->fcoef, ci, co));
+  PT_LAUNCH(c, K_DF_COEF, lean_coef<df64>(c->stream, b, c->fcoef, ci, co));
 }
 
 // The cells kernel's inputs at double-float iterate a, outputs into buffer n.
@@ -585,7 +585,7 @@ void df_cells(pt_ctx* c, int a, int n, int check) {
                       c->logk ? D(c->K0) : nullptr};
   LeanCellOut<df64> co{c->fPt[n], c->fPf[n], c->fphi[n], D(c->lw[n]), D(c->lperm[n]), c->fs_txx, c->fs_tyy,
                        c->fs_tzz, c->fs_txy, c->fs_txz, c->fs_tyz};
-  PT_LAUNCH(c, K_DF_CELLS, lean_cells<df64>(grid_dims(b), block_dims(), c->stream, b, c->fcoef, ci, co, c->red, check));
+  PT_LAUNCH(c, K_DF_CELLS, lean_cells<df64>(c->stream, b, c->fcoef, ci, co, c->red, check));
 }
 
 // One PT iteration in double-float: the lean form's kernels on the df64 iterate.
@@ -597,12 +597,12 @@ void launch_iteration_df(pt_ctx* c, int check) {
   df_cells(c, a, n, check);
   LeanFaceIn<df64> fi{c->fs_txx, c->fs_tyy, c->fs_tzz, c->fs_txy, c->fs_txz, c->fs_tyz, c->fPt[n],
                       c->fphi[a], D(c->dtv_x), D(c->dtv_x), D(c->dtv_x)};
-  PT_LAUNCH(c, K_DF_FACES, lean_faces<df64>(gr, bl, c->stream, b, c->fcoef, fi, c->fVx, c->fVy, c->fVz, c->fRx,
+  PT_LAUNCH(c, K_DF_FACES, lean_faces<df64>(c->stream, b, c->fcoef, fi, c->fVx, c->fVy, c->fVz, c->fRx,
                                             c->fRy, c->fRz, c->red, check));
   if (check) {
     LeanPicardIn<df64> pi{c->fs_txx, c->fs_tyy, c->fs_tzz, c->fs_txy, c->fs_txz, c->fs_tyz, c->fphi[n],
                           c->fPt[n], c->fPf[n]};
-    PT_LAUNCH(c, K_DF_PICARD, lean_picard<df64>(gr, bl, c->stream, b, c->fcoef, pi, c->fmu, c->feta, c->red));
+    PT_LAUNCH(c, K_DF_PICARD, lean_picard<df64>(c->stream, b, c->fcoef, pi, c->fmu, c->feta, c->red));
     launch_df_coef(c);
   }
   c->fcur = n;
@@ -701,17 +701,17 @@ int mixed_outer(pt_ctx* c, int n_in, bool early_exit, pt_report* outer, bool* co
   cudaMemsetAsync(c->red, 0, RED_N * sizeof(unsigned long long), c->stream);
   // (i) FP64 residuals at u, frozen coefficients of the correction problem; (ii) Picard update
   const LeanCoef<double>& k = c->lcoef;
-  PT_LAUNCH(c, K_PERM, mix_perm(gr, bl, c->stream, b, k, c->phi[a], c->logk, c->perm));
+  PT_LAUNCH(c, K_PERM, mix_perm(c->stream, b, k, c->phi[a], c->logk, c->perm));
   const MixPrepIn pin{StressIn{c->Vx, c->Vy, c->Vz, c->mu, c->txxo, c->tyyo, c->tzzo, c->txyo, c->txzo, c->tyzo},
                       c->Pt[a], c->Pf[a], c->phi[a], c->eta, c->perm, c->Pto, c->Pfo};
   const MixPrepOut pout{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz,
                         c->m_rpt, c->m_rpf, c->m_cc, c->m_perm, c->m_idtp};
-  PT_LAUNCH(c, K_MIX_PREP, mix_prepare(gr, bl, c->stream, b, k, pin, pout, c->red));
+  PT_LAUNCH(c, K_MIX_PREP, mix_prepare(c->stream, b, k, pin, pout, c->red));
   const MixFaceIn fin{LeanPicardIn<double>{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz, c->phi[a],
                                            c->Pt[a], c->Pf[a]},
                       c->mu, c->eta};
   const MixFaceOut fout{c->m_rfx, c->m_rfy, c->m_rfz, c->m_mu, c->m_dtvc};
-  PT_LAUNCH(c, K_MIX_FACES, mix_faces(gr, bl, c->stream, b, k, fin, fout, c->red));
+  PT_LAUNCH(c, K_MIX_FACES, mix_faces(c->stream, b, k, fin, fout, c->red));
   if (cudaGetLastError() != cudaSuccess) return PT_ECUDA;
   int rc = read_report(c, outer);
   if (rc != PT_OK) return rc;
@@ -782,9 +782,9 @@ int mixed_outer(pt_ctx* c, int n_in, bool early_exit, pt_report* outer, bool* co
   const int n = 1 - a;   // the new pressures and porosity go to the other buffers
   MixUpdate mu{c->Vx, c->Vy, c->Vz, c->Pt[a], c->Pf[a], c->Pt[n], c->Pf[n], c->m_dVx[d], c->m_dVy[d], c->m_dVz[d], c->m_dPt[d], c->m_dPf[d],
                c->mix_omega};
-  PT_LAUNCH(c, K_MIX_UPDATE, mix_update(gr, bl, c->stream, b, mu));
+  PT_LAUNCH(c, K_MIX_UPDATE, mix_update(c->stream, b, mu));
   PT_LAUNCH(c, K_MIX_POROSITY,
-            mix_porosity(gr, bl, c->stream, b, k,
+            mix_porosity(c->stream, b, k,
                          MixPorosity{c->Vx, c->Vy, c->Vz, c->phi[a], c->Pt[n], c->Pf[n], c->Pto, c->Pfo, c->Lo,
                                      c->eta, c->phi[n]}));
   c->cur = n;
@@ -814,7 +814,7 @@ int step_begin_launch(pt_ctx* c) {
     LeanBeginOut<double> bo{c->Pto, c->Pfo, c->phio, c->Eo, c->iEo, c->lw[0], c->lperm[0]};
     PT_LAUNCH(c, K_LEAN_BEGIN, lean_begin<double>(grid_dims(b), block_dims(), c->stream, b, c->lcoef, bi, bo, c->red));
   } else if (c->mixed) {   // Lo holds the old porosity (its integration needs no logarithm)
-    PT_LAUNCH(c, K_BEGIN, mix_begin(grid_dims(b), block_dims(), c->stream, b, c->Pt[0], c->Pf[0], c->phi[0], c->mu,
+    PT_LAUNCH(c, K_BEGIN, mix_begin(c->stream, b, c->Pt[0], c->Pf[0], c->phi[0], c->mu,
                                     c->Pto, c->Pfo, c->Lo, c->red));
   } else {
     PT_LAUNCH(c, K_BEGIN, k_begin_step<<<grid_dims(b), block_dims(), 0, c->stream>>>(
@@ -1032,8 +1032,8 @@ int pt_init(pt_ctx** ctx, const pt_grid* grid, const pt_phys* phys, const pt_num
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && c->lean && c->logk) {
-    PT_LAUNCH(c, K_LEAN_K0, lean_k0<double>(grid_dims(c->box), block_dims(), c->stream, c->box, c->phys.k0, c->logk,
-                                            c->K0));
+    PT_LAUNCH(c, K_LEAN_K0, lean_k0<double>(grid_dims(c->box), block_dims(), c->stream, c->box, c->lcoef.k0r3,
+                                            c->logk, c->K0));
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && !keep_visc) {
@@ -1363,8 +1363,9 @@ void fill_batch_inst(pt_batch* B, int m, long long base) {
   }
   I.tol = c->num.tol;
   I.max_iter = c->num.max_iter;
-  I.gx = (c->box.nx + 1 + B->bx - 1) / B->bx;
-  I.gy = (c->box.ny + 1 + B->by - 1) / B->by;
+  const int wall = c->lcoef.bg_on ? 1 : 0;   // i = nx, j = ny carry stress under a background shear only
+  I.gx = (c->box.nx + wall + B->bx - 1) / B->bx;
+  I.gy = (c->box.ny + wall + B->by - 1) / B->by;
   I.tile_base = base;
 }
 
@@ -1373,7 +1374,7 @@ cudaError_t upload_batch(pt_batch* B) {
   long long base = 0;
   for (int m = 0; m < B->ninst; ++m) {
     fill_batch_inst(B, m, base);
-    base += (long long)B->h_inst[m].gx * B->h_inst[m].gy * (B->ctx[m]->box.nz + 1);
+    base += (long long)B->h_inst[m].gx * B->h_inst[m].gy * B->ctx[m]->box.nz;
   }
   B->ntiles = base;
   const int dev_blocks = batch_blocks_per_sm(B->bx, B->by);
@@ -1471,8 +1472,9 @@ void fill_mix_inst(pt_batch* B, int m, long long base, long long cbase) {
   I.tol = c->num.tol;
   I.rtol = c->num.inner_rtol > 0 ? c->num.inner_rtol : kInnerRtol;
   I.max_iter = c->num.max_iter;
-  I.gx = (c->box.nx + 1 + 31) / 32;
-  I.gy = (c->box.ny + 1 + 7) / 8;
+  const int wall = c->lcoef.bg_on ? 1 : 0;
+  I.gx = (c->box.nx + wall + 31) / 32;
+  I.gy = (c->box.ny + wall + 7) / 8;
   I.cgx = (c->box.nx + corr_tile_x() - 1) / corr_tile_x();
   I.cgy = (c->box.ny + corr_tile_y() - 1) / corr_tile_y();
   I.cgz = (c->box.nz + B->zchunk - 1) / B->zchunk;
@@ -1485,7 +1487,7 @@ cudaError_t upload_mix(pt_batch* B) {
   for (int m = 0; m < B->ninst; ++m) {
     fill_mix_inst(B, m, base, cbase);
     const MixBatchInst& I = B->h_minst[m];
-    base += (long long)I.gx * I.gy * (I.b.nz + 1);
+    base += (long long)I.gx * I.gy * I.b.nz;
     cbase += (long long)I.cgx * I.cgy * I.cgz;
   }
   B->nptiles = base;
@@ -2038,8 +2040,7 @@ AdjCoef adjoint_coef(const pt_ctx* c) {
   ac.dt_r = k.dt * ac.r_eta0mu0;
   ac.idtp = 1.0 / (k.dtaupt_fac * c->phys.mu0);
   ac.ifac_pf = 1.0 / k.dtaupf_fac;
-  ac.rphi0 = k.rphi0;
-  ac.k0 = k.k0;
+  ac.k0 = c->lcoef.k0r3;
   ac.buoy = k.rhof_g - k.rho_bg_g;
   ac.hdrho_g = 0.5 * (c->phys.rhof_g - c->phys.rhos_g);
   ac.hdt_rdx = 0.5 * k.dt * k.rdx; ac.hdt_rdy = 0.5 * k.dt * k.rdy; ac.hdt_rdz = 0.5 * k.dt * k.rdz;

@@ -59,7 +59,11 @@ __global__ void __launch_bounds__(BX * BY) k_batch_phase(const BatchInst* __rest
     const bool own = ox && oy && oz;
     if (PHASE == BATCH_CELLS) {
       double r_pt = 0.0, r_pf = 0.0;
-      lean_cell_point(I.b, I.c, I.cin[a], I.cout[a], i, j, k, check, r_pt, r_pf);
+      const int wall = I.c.bg_on ? 1 : 0;
+      if (i < I.b.nx + wall && j < I.b.ny + wall) {
+        LeanColumn col = lean_column(I.b, I.c, I.cin[a], i, j, k);
+        lean_cell_level(I.b, I.c, I.cin[a], I.cout[a], i, j, k, check, col, r_pt, r_pf);
+      }
       if (check) {
         block_max_atomic(own ? r_pt : 0.0, I.red + RED_PT);
         block_max_atomic(own ? r_pf : 0.0, I.red + RED_PF);

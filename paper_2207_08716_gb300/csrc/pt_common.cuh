@@ -10,6 +10,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 
 namespace pt {
 
@@ -57,21 +58,23 @@ __host__ __device__ inline long long cidx(const Box& b, int i, int j, int k) {
 
 // Levels per block of a kernel whose blocks march up z-columns of the box (`cols` of them, `levels`
 // levels each). A chunk of zc levels costs zc + fill steps (its pipeline fill and, where halo levels
-// are recomputed, those), and a step of an SM with r resident blocks takes about base + r (in units
-// of one block's share of a full SM): the chunk with the least waves * (zc + fill) * (base + r); with
-// more than four waves blocks end at different times and the last wave counts half. A grid whose
-// columns alone do not fill the chip (96^3: 68 columns of the FP32 correction pass for 608 block
-// slots) gets shorter chunks, a large one the longest, which recompute and refill least.
+// are recomputed, those); the steps of an SM's blocks share its issue slots or pipes, and every wave adds
+// base of a step's latency that they do not hide: the chunk with the least (zc + fill) *
+// (ceil(blocks / SMs) + base * waves), without the rounding beyond four waves, where blocks end at
+// different times. A grid whose columns alone do not fill the chip (96^3: 48 columns of the FP32
+// correction pass for 304 block slots) gets shorter chunks, a large one the longest, which recompute and
+// refill least.
 inline int march_chunk(long long cols, int levels, int max_chunk, int blocks_per_sm, int sms, double fill,
                        double base) {
-  const long long slots = (long long)blocks_per_sm * sms;
+  const double slots = (double)blocks_per_sm * sms;
   int best = 1;
   double best_cost = 1e300;
   for (int zc = 1; zc <= std::min(max_chunk, levels); ++zc) {
-    const long long blocks = cols * ((levels + zc - 1) / zc);
-    const double waves = blocks <= 4 * slots ? (double)((blocks + slots - 1) / slots) : (double)blocks / slots + 0.5;
-    const double resident = std::min((double)blocks / sms, (double)blocks_per_sm);
-    const double cost = waves * (zc + fill) * (base + resident);
+    const double blocks = (double)(cols * ((levels + zc - 1) / zc));
+    const bool few = blocks <= 4 * slots;
+    const double share = few ? std::ceil(blocks / sms) : blocks / sms + 0.5 * blocks_per_sm;
+    const double waves = few ? std::ceil(blocks / slots) : blocks / slots;
+    const double cost = (zc + fill) * (share + base * waves);
     if (cost < best_cost) {
       best_cost = cost;
       best = zc;
@@ -86,6 +89,40 @@ inline int sm_count() {
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return 152;
   return sms;
+}
+
+// Point kernels of the FP64 pipe run 128 threads per block, which spreads a small grid over the SMs, on a
+// tile of 32 x 4 points of a plane or, where rows leave much of their last tile empty, on 128 points of
+// the plane in linear order (x fastest): a warp instruction with one lane costs the FP64 pipe the same 16
+// cycles as a full one (33 x 33 points fill 52 % of their tiles), but a warp that straddles rows reads two
+// lines per load. Extents: the cells, or the
+// box where wall indices carry values.
+constexpr int kPlaneThreads = 128;
+struct Plane {
+  int nxe, n;
+  int tiles_x;   // tiles per row of tiles, 0: linear order
+};
+__device__ __forceinline__ bool plane_point(const Plane& p, int& i, int& j) {
+  if (p.tiles_x) {
+    const int by = (int)(blockIdx.x / (unsigned)p.tiles_x), bx = (int)blockIdx.x - by * p.tiles_x;
+    i = bx * 32 + (int)(threadIdx.x & 31);
+    j = by * 4 + (int)(threadIdx.x >> 5);
+    return i < p.nxe && j * p.nxe < p.n;
+  }
+  const unsigned t = blockIdx.x * kPlaneThreads + threadIdx.x;
+  j = (int)(t / (unsigned)p.nxe);
+  i = (int)(t - (unsigned)j * (unsigned)p.nxe);
+  return t < (unsigned)p.n;
+}
+inline Plane plane_of(const Box& b, int wall) {
+  const int nx = b.nx + wall, ny = b.ny + wall, tiles_x = (nx + 31) / 32;
+  const bool tiles = (long long)nx * ny >= 9LL * (tiles_x * 32) * ((ny + 3) / 4 * 4) / 10;   // at least 90 % full
+  return Plane{nx, nx * ny, tiles ? tiles_x : 0};
+}
+inline dim3 plane_grid(const Plane& p, int levels) {
+  const int rows = p.n / p.nxe;
+  return dim3((unsigned)(p.tiles_x ? p.tiles_x * ((rows + 3) / 4) : (p.n + kPlaneThreads - 1) / kPlaneThreads),
+              (unsigned)levels, 1);
 }
 
 // Indices of the residual max-norm slots in the device reduction block.

@@ -169,7 +169,7 @@ __device__ __forceinline__ void df_cell_level(const Box& b, const LeanCoef<df64>
     const df64 sxx = fma(cm2, norm(add(gx, s3n)), PW(S_TXX));
     const df64 syy = fma(cm2, norm(add(gy, s3n)), PW(S_TYY));
     const df64 szz = fma(cm2, norm(add(gz, s3n)), PW(S_TZZ));
-    // porosity in log space (Eq. 22): L = Lo + delta (see lean_cell_point)
+    // porosity in log space (Eq. 22): L = Lo + delta (see lean_cell_level)
     const df64 adv = mul(-w, mad(half(-ph), divV, mad(ax, c.hrdx, mad(ay, c.hrdy, mul(az, c.hrdz)))));
     const df64 dp1 = sub(Pf1, Pt1);
     const df64 rate = c.compaction_on ? mad(dp1, ieta, adv) : adv;

@@ -55,7 +55,7 @@ struct LeanCellIn {
   // edge moduli 2 mu/(1+xi) pre-multiplied by the two half inverse spacings of each edge's strain
   // rate: em2_xy = m hrdy, eb_xy = m hrdx; em2_xz = m hrdz, eb_xz = m hrdx; em2_yz = m hrdz, eb_yz = m hrdy
   const T *em2_xy, *em2_xz, *em2_yz, *eb_xy, *eb_xz, *eb_yz, *toa_xy, *toa_xz, *toa_yz;
-  const T *K0;  // k0 e^logk per cell, or null (scalar k0)
+  const T *K0;  // k0 e^logk / phi0^3 per cell, or null (scalar k0r3)
 };
 template <class T>
 struct LeanCellOut {
@@ -102,16 +102,16 @@ struct LeanBeginOut {
 
 // Host-side launchers (the kernels are templates and are launched from their own TU).
 template <class T>
-void lean_cells(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanCellIn<T>& in,
+void lean_cells(cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanCellIn<T>& in,
                 const LeanCellOut<T>& out, unsigned long long* red, int check);
 template <class T>
-void lean_faces(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanFaceIn<T>& in,
+void lean_faces(cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanFaceIn<T>& in,
                 T* Vx, T* Vy, T* Vz, T* Rx, T* Ry, T* Rz, unsigned long long* red, int check);
 template <class T>
-void lean_picard(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanPicardIn<T>& in,
+void lean_picard(cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanPicardIn<T>& in,
                  T* mu, T* eta, unsigned long long* red);
 template <class T>
-void lean_coef(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanCoefIn<T>& in,
+void lean_coef(cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanCoefIn<T>& in,
                const LeanCoefOut<T>& out);
 template <class T>
 void lean_begin(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanBeginIn<T>& in,
@@ -120,7 +120,7 @@ void lean_begin(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, 
 void lean_stresses(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c, const StressIn& in,
                    const StressCentre& ce, const StressOut& out);
 template <class T>
-void lean_k0(dim3 gr, dim3 bl, cudaStream_t st, Box b, double k0, const double* logk, T* K0);
+void lean_k0(dim3 gr, dim3 bl, cudaStream_t st, Box b, double k0r3, const double* logk, T* K0);
 
 // Up to 16 arrays converted in one launch between FP64 (d) and double-float (f), whole boxes.
 struct DfCopy {

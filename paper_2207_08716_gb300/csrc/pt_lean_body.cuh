@@ -13,13 +13,13 @@ namespace lean_detail {
 // |d| <= 2^-20 and after d^9 / d^8 for |d| <= 2^-6: in both cases the first dropped term is
 // below 2^-60 |d|). expm1(d) = E + O, expm1(-d) = E - O.
 __device__ inline void expm1_pair(double d, double& em_pos, double& em_neg) {
-  if (fabs(d) <= 0x1p-20) {
+  const int ad = __double2hiint(d) & 0x7fffffff;      // |d|'s upper word: the tiers off the FP64 pipe
+  if (ad < 0x3eb00000) {                              // |d| < 2^-20
     const double d2 = d * d;
-    const double E = 0.5 * d2;
     const double O = d * fma(d2, 1.0 / 6.0, 1.0);
-    em_pos = E + O;
-    em_neg = E - O;
-  } else if (fabs(d) <= 0.015625) {
+    em_pos = fma(0.5, d2, O);
+    em_neg = fma(0.5, d2, -O);
+  } else if (ad < 0x3f900000) {                       // |d| < 2^-6
     const double d2 = d * d;
     const double E = d2 * fma(d2, fma(d2, fma(d2, 1.0 / 40320.0, 1.0 / 720.0), 1.0 / 24.0), 0.5);
     const double O = d * fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 362880.0, 1.0 / 5040.0), 1.0 / 120.0), 1.0 / 6.0), 1.0);
@@ -28,18 +28,6 @@ __device__ inline void expm1_pair(double d, double& em_pos, double& em_neg) {
   } else {
     em_pos = expm1(d);
     em_neg = expm1(-d);
-  }
-}
-__device__ inline void expm1_pair(float d, float& em_pos, float& em_neg) {
-  if (fabsf(d) <= 0.0625f) {
-    const float d2 = d * d;
-    const float E = d2 * fmaf(d2, fmaf(d2, 1.0f / 720.0f, 1.0f / 24.0f), 0.5f);
-    const float O = d * fmaf(d2, fmaf(d2, 1.0f / 120.0f, 1.0f / 6.0f), 1.0f);
-    em_pos = E + O;
-    em_neg = E - O;
-  } else {
-    em_pos = expm1f(d);
-    em_neg = expm1f(-d);
   }
 }
 
@@ -171,11 +159,15 @@ __device__ inline df64 relax_pow(df64 x, df64 /*rx*/, double rel, int root, cons
   return df64(exp(rel * log((double)x)));
 }
 
-// max of |values| whose NaN is the largest, through bit patterns (off the FP64 pipe)
+// max of |values| whose NaN is the largest, through bit patterns. The sign is cleared in assembly: the
+// compiler takes a mask of it for fabs, an addition on the FP64 pipe.
+__device__ inline unsigned long long abs_bits(double x) {
+  unsigned long long u;
+  asm("and.b64 %0, %1, 0x7fffffffffffffff;" : "=l"(u) : "l"(__double_as_longlong(x)));
+  return u;
+}
 __device__ inline double abs_max(double a, double b) {
-  const unsigned long long m = 0x7fffffffffffffffull;
-  const unsigned long long ia = (unsigned long long)__double_as_longlong(a) & m;
-  const unsigned long long ib = (unsigned long long)__double_as_longlong(b) & m;
+  const unsigned long long ia = abs_bits(a), ib = abs_bits(b);
   return __longlong_as_double((long long)(ia > ib ? ia : ib));
 }
 __device__ inline df64 abs_max(df64 a, df64 b) { return a < b ? b : a; }   // positive values; drops a NaN
@@ -199,123 +191,153 @@ struct LeanRecompute<df64> { static constexpr bool value = true; };
 enum { S_PTO, S_PFO, S_PHIO, S_IETA, S_IDTP, S_CM2, S_TXX, S_TYY, S_TZZ, S_EXY, S_EXZ, S_EYZ, S_TXY, S_TXZ,
        S_TYZ, kStageSlots };
 
-// Cells, stresses of the three lower edges, pressures, porosity at box index (i, j, k) in FP64.
-__device__ __forceinline__ void lean_cell_point(const Box& b, const LeanCoef<double>& c,
-                                                const LeanCellIn<double>& in, const LeanCellOut<double>& out, int i,
-                                                int j, int k, int check, double& r_pt, double& r_pf) {
-  using namespace lean_detail;
-  if (i <= b.nx && j <= b.ny && k <= b.nz) {
-    const long long q = cidx(b, i, j, k);
-    const long long px = b.px, pxy = b.pxy;
-    const bool cell = i < b.nx && j < b.ny && k < b.nz;
-    // ---- edges owned by this index: xy (i, j, k), xz (i, j, k), yz (i, j, k); stored at the end
-    // with the cell's outputs, after every load (the arrays are not declared non-aliasing)
-    double t_xy = 0.0, t_xz = 0.0, t_yz = 0.0;
-    if (k < b.nz && i > 0 && i < b.nx && j > 0 && j < b.ny) {   // toa_xy holds the background part too
-      t_xy = fma(in.eb_xy[q], in.Vy[q] - in.Vy[q - 1], fma(in.em2_xy[q], in.Vx[q] - in.Vx[q - px], in.toa_xy[q]));
-    } else if (k < b.nz && c.bg_on) {   // wall xy-edge under background shear (Eqs. 32-33)
-      t_xy = in.toa_xy[q];
-    }
-    if (j < b.ny && i > 0 && i < b.nx && k > 0 && k < b.nz)
-      t_xz = fma(in.eb_xz[q], in.Vz[q] - in.Vz[q - 1], fma(in.em2_xz[q], in.Vx[q] - in.Vx[q - pxy], in.toa_xz[q]));
-    if (i < b.nx && j > 0 && j < b.ny && k > 0 && k < b.nz)
-      t_yz = fma(in.eb_yz[q], in.Vz[q] - in.Vz[q - px], fma(in.em2_yz[q], in.Vy[q] - in.Vy[q - pxy], in.toa_yz[q]));
-    if (cell) {
-      const double Pt = in.Pt[q], Pf = in.Pf[q], Pto = in.Pto[q], Pfo = in.Pfo[q];
-      const double ph = in.phi[q], ieta = in.ieta[q], w = in.w[q];
-      const double vxl = in.Vx[q], vxr = in.Vx[q + 1], vyl = in.Vy[q], vyr = in.Vy[q + px];
-      const double vzl = in.Vz[q], vzr = in.Vz[q + pxy];
-      const double gx = (vxr - vxl) * c.rdx, gy = (vyr - vyl) * c.rdy, gz = (vzr - vzl) * c.rdz;
-      const double divV = gx + gy + gz;
-      const double cc = c.compaction_on ? ieta * w : 0.0;
-      const double dPt = Pt - Pto, dPf = Pf - Pfo, dpp = Pt - Pf;
-      // explicit fused multiply-adds: the same rounding in every kernel that inlines this body
-      const double divVn = fma(dpp, cc, fma(-c.bd_rdt_a, dPf, fma(c.bd_rdt, dPt, divV)));
-      // Darcy flux through the six faces (zero on the boundary) and the largest neighbour k
-      const double kc = in.perm[q];
-      double kmax = kc, sx = 0.0, sy = 0.0, sz = 0.0;
-      if (i > 0) {
-        const double kn = in.perm[q - 1];
-        kmax = pos_max(kmax, kn);
-        sx -= (kn + kc) * (Pf - in.Pf[q - 1]);
-      }
-      if (i < b.nx - 1) {
-        const double kn = in.perm[q + 1];
-        kmax = pos_max(kmax, kn);
-        sx += (kc + kn) * (in.Pf[q + 1] - Pf);
-      }
-      if (j > 0) {
-        const double kn = in.perm[q - px];
-        kmax = pos_max(kmax, kn);
-        sy -= (kn + kc) * (Pf - in.Pf[q - px]);
-      }
-      if (j < b.ny - 1) {
-        const double kn = in.perm[q + px];
-        kmax = pos_max(kmax, kn);
-        sy += (kc + kn) * (in.Pf[q + px] - Pf);
-      }
-      if (k > 0) {
-        const double kn = in.perm[q - pxy];
-        kmax = pos_max(kmax, kn);
-        sz -= (kn + kc) * ((Pf - in.Pf[q - pxy]) + c.buoy_dz);
-      }
-      if (k < b.nz - 1) {
-        const double kn = in.perm[q + pxy];
-        kmax = pos_max(kmax, kn);
-        sz += (kc + kn) * ((in.Pf[q + pxy] - Pf) + c.buoy_dz);
-      }
-      // div qD = -1/2 sum_d rd^2 [(k + k_r)(Pf_r - Pf) - (k_l + k)(Pf - Pf_l)]
-      const double divqD = -(sx * c.hrdx2 + sy * c.hrdy2 + sz * c.hrdz2);
-      // local-implicit pressure updates, Eqs. 17-18: P1 = P - res / (1/dtau + d res/dP), the
-      // residuals being divVn (row Pt) and resF (row Pf)
-      const double resF = fma(-dpp, cc, fma(-c.bd_rdt_a, dPt, fma(c.bda_B_rdt, dPf, divqD)));
-      const double Pt1 = Pt - rcp_pseudo(in.idtp[q] + cc) * divVn;   // idtp holds 1/dtau_Pt + beta_d/dt
-      const double Pf1 = Pf - rcp_pseudo(kmax * c.ifac_pf + c.bda_B_rdt + cc) * resF;
-      // normal deviatoric stresses (Eq. 21): tau = tau_o xi/(1+xi) + 2 mu/(1+xi) (edot + beta_n divVn)
-      const double s3 = fma(c.beta_n, divVn, -(divV * (1.0 / 3.0)));
-      const double cm2 = in.cm2[q];
-      const double sxx = fma(cm2, gx + s3, in.toa_xx[q]);
-      const double syy = fma(cm2, gy + s3, in.toa_yy[q]);
-      const double szz = fma(cm2, gz + s3, in.toa_zz[q]);
-      // porosity in log space (Eq. 22): L = Lo + delta,
-      // delta = -[beta_phi ((Pf1 - Pfo) - (Pt1 - Pto)) + dt (Pf1 - Pt1) / eta + dt V.grad(1-phi)/(1-phi)]
-      // V.grad(1-phi)/(1-phi) = -(w/2) sum_d rd [v_r (phi_r - phi) + v_l (phi - phi_l)]
-      //                      = -w [sum_d hrd (v_r phi_r - v_l phi_l) - phi divV / 2]
-      // (the velocities of wall faces are zero, so the divergence term is div V exactly)
-      double ax = 0.0, ay = 0.0, az = 0.0;
-      if (i > 0) ax = -vxl * in.phi[q - 1];
-      if (i < b.nx - 1) ax = fma(vxr, in.phi[q + 1], ax);
-      if (j > 0) ay = -vyl * in.phi[q - px];
-      if (j < b.ny - 1) ay = fma(vyr, in.phi[q + px], ay);
-      if (k > 0) az = -vzl * in.phi[q - pxy];
-      if (k < b.nz - 1) az = fma(vzr, in.phi[q + pxy], az);
-      const double adv = -w * fma(-0.5 * ph, divV, fma(ax, c.hrdx, fma(ay, c.hrdy, az * c.hrdz)));
-      const double comp = c.compaction_on ? (Pf1 - Pt1) * ieta : 0.0;
-      const double delta = -(c.beta_phi * ((Pf1 - Pfo) - (Pt1 - Pto)) + c.dt * (comp + adv));
-      double em_p, em_n;
-      expm1_pair(delta, em_p, em_n);
-      const double phio = in.phio[q], Eo = in.Eo[q], iEo = in.iEo[q];
-      const double K0 = in.K0 ? in.K0[q] : c.k0;
-      const double ph1 = phio - Eo * em_p;
-      const double r = ph1 * c.rphi0;
-      // every load above precedes the stores (the arrays are not declared non-aliasing)
-      out.Pt[q] = Pt1;
-      out.Pf[q] = Pf1;
-      out.txx[q] = sxx;
-      out.tyy[q] = syy;
-      out.tzz[q] = szz;
-      out.phi[q] = ph1;
-      out.w[q] = iEo + iEo * em_n;
-      out.perm[q] = K0 * r * r * r;
-      if (check) {
-        r_pt = fabs(divVn);
-        r_pf = fabs(resF);
-      }
-    }
-    if (k < b.nz) out.txy[q] = t_xy;
-    if (j < b.ny) out.txz[q] = t_xz;
-    if (i < b.nx) out.tyz[q] = t_yz;
+// Cells of a column in FP64, level by level: pressures, porosity, k, 1/(1-phi), stresses of the centre and
+// of its three lower edges. The form is bound by the FP64 pipe, so what the level below has formed or
+// loaded is carried: the Darcy term through the lower z face, and the z-neighbours' values.
+struct LeanColumn {
+  double Pf, kk, phi, vz;          // own values at the current level
+  double k_d, phi_d, vx_d, vy_d;   // one level below
+  double fz;                       // (k_d + k) (Pf - Pf_d + buoyancy), 0 at the floor
+};
+
+__device__ __forceinline__ LeanColumn lean_column(const Box& b, const LeanCoef<double>& c,
+                                                  const LeanCellIn<double>& in, int i, int j, int k) {
+  const long long q = cidx(b, i, j, k);
+  LeanColumn s;
+  s.Pf = in.Pf[q];
+  s.kk = in.perm[q];
+  s.phi = in.phi[q];
+  s.vz = in.Vz[q];
+  s.k_d = s.phi_d = s.vx_d = s.vy_d = s.fz = 0.0;
+  if (k > 0) {
+    const long long d = q - b.pxy;
+    s.k_d = in.perm[d];
+    s.phi_d = in.phi[d];
+    s.vx_d = in.Vx[d];
+    s.vy_d = in.Vy[d];
+    s.fz = (s.k_d + s.kk) * ((s.Pf - in.Pf[d]) + c.buoy_dz);
   }
+  return s;
+}
+
+// Level k in [0, nz) (the level nz holds walls only) at i <= nx, j <= ny; leaves the column at k + 1.
+__device__ __forceinline__ void lean_cell_level(const Box& b, const LeanCoef<double>& c,
+                                                const LeanCellIn<double>& in, const LeanCellOut<double>& out, int i,
+                                                int j, int k, int check, LeanColumn& col, double& r_pt, double& r_pf) {
+  using namespace lean_detail;
+  const long long q = cidx(b, i, j, k);
+  const long long px = b.px, pxy = b.pxy;
+  const double vx = in.Vx[q], vy = in.Vy[q], vz = col.vz, vz_u = in.Vz[q + pxy];
+  const bool up = k < b.nz - 1;
+  double Pf_u = 0.0, k_u = 0.0, phi_u = 0.0;
+  if (up) {
+    Pf_u = in.Pf[q + pxy];
+    k_u = in.perm[q + pxy];
+    phi_u = in.phi[q + pxy];
+  }
+  // ---- edges owned by this index, stored at the end with the cell's outputs, after every load (the
+  // arrays are not declared non-aliasing); toa_xy holds the background part too
+  double t_xy = 0.0, t_xz = 0.0, t_yz = 0.0;
+  const bool ix = i > 0 && i < b.nx, jy = j > 0 && j < b.ny;
+  if (ix && jy) {
+    t_xy = fma(in.eb_xy[q], vy - in.Vy[q - 1], fma(in.em2_xy[q], vx - in.Vx[q - px], in.toa_xy[q]));
+  } else if (c.bg_on) {   // wall xy-edge under background shear (Eqs. 32-33)
+    t_xy = in.toa_xy[q];
+  }
+  if (k > 0) {
+    if (ix && j < b.ny)
+      t_xz = fma(in.eb_xz[q], vz - in.Vz[q - 1], fma(in.em2_xz[q], vx - col.vx_d, in.toa_xz[q]));
+    if (i < b.nx && jy)
+      t_yz = fma(in.eb_yz[q], vz - in.Vz[q - px], fma(in.em2_yz[q], vy - col.vy_d, in.toa_yz[q]));
+  }
+  double fz_u = 0.0;
+  if (i < b.nx && j < b.ny) {
+    const double Pt = in.Pt[q], Pf = col.Pf, Pto = in.Pto[q], Pfo = in.Pfo[q], ph = col.phi, kc = col.kk;
+    const double ieta = in.ieta[q], w = in.w[q];
+    const double vxr = in.Vx[q + 1], vyr = in.Vy[q + px];
+    const double dvx = vxr - vx, dvy = vyr - vy, dvz = vz_u - vz;
+    const double divV = fma(dvx, c.rdx, fma(dvy, c.rdy, dvz * c.rdz));
+    const double cc = c.compaction_on ? ieta * w : 0.0;
+    const double dPt = Pt - Pto, dPf = Pf - Pfo, dpp = Pt - Pf;
+    // explicit fused multiply-adds: the same rounding in every kernel that inlines this body
+    const double divVn = fma(dpp, cc, fma(-c.bd_rdt_a, dPf, fma(c.bd_rdt, dPt, divV)));
+    // Darcy flux through the six faces (zero on the boundary), the largest neighbour k, and the
+    // advection sums v_r phi_r - v_l phi_l over the same faces (wall velocities are zero)
+    double kmax = pos_max(kc, col.k_d), sx = 0.0, sy = 0.0, ax = 0.0, ay = 0.0, az = -vz * col.phi_d;
+    if (i > 0) {
+      const double kn = in.perm[q - 1];
+      kmax = pos_max(kmax, kn);
+      sx = (kn + kc) * (in.Pf[q - 1] - Pf);
+      ax = -vx * in.phi[q - 1];
+    }
+    if (i < b.nx - 1) {
+      const double kn = in.perm[q + 1];
+      kmax = pos_max(kmax, kn);
+      sx = fma(kc + kn, in.Pf[q + 1] - Pf, sx);
+      ax = fma(vxr, in.phi[q + 1], ax);
+    }
+    if (j > 0) {
+      const double kn = in.perm[q - px];
+      kmax = pos_max(kmax, kn);
+      sy = (kn + kc) * (in.Pf[q - px] - Pf);
+      ay = -vy * in.phi[q - px];
+    }
+    if (j < b.ny - 1) {
+      const double kn = in.perm[q + px];
+      kmax = pos_max(kmax, kn);
+      sy = fma(kc + kn, in.Pf[q + px] - Pf, sy);
+      ay = fma(vyr, in.phi[q + px], ay);
+    }
+    if (up) {
+      kmax = pos_max(kmax, k_u);
+      fz_u = (kc + k_u) * ((Pf_u - Pf) + c.buoy_dz);
+      az = fma(vz_u, phi_u, az);
+    }
+    // div qD = -1/2 sum_d rd^2 [(k + k_r)(Pf_r - Pf) - (k_l + k)(Pf - Pf_l)]
+    const double divqD = -fma(sx, c.hrdx2, fma(sy, c.hrdy2, (fz_u - col.fz) * c.hrdz2));
+    // local-implicit pressure updates, Eqs. 17-18: P1 = P - res / (1/dtau + d res/dP), the
+    // residuals being divVn (row Pt) and resF (row Pf)
+    const double resF = fma(-dpp, cc, fma(-c.bd_rdt_a, dPt, fma(c.bda_B_rdt, dPf, divqD)));
+    const double Pt1 = fma(-rcp_pseudo(in.idtp[q] + cc), divVn, Pt);   // idtp holds 1/dtau_Pt + beta_d/dt
+    const double Pf1 = fma(-rcp_pseudo(fma(kmax, c.ifac_pf, c.bda_B_rdt) + cc), resF, Pf);
+    // normal deviatoric stresses (Eq. 21): tau = tau_o xi/(1+xi) + 2 mu/(1+xi) (edot + beta_n divVn)
+    const double s3 = fma(c.beta_n, divVn, divV * (-1.0 / 3.0));
+    const double cm2 = in.cm2[q];
+    const double sxx = fma(cm2, fma(dvx, c.rdx, s3), in.toa_xx[q]);
+    const double syy = fma(cm2, fma(dvy, c.rdy, s3), in.toa_yy[q]);
+    const double szz = fma(cm2, fma(dvz, c.rdz, s3), in.toa_zz[q]);
+    // porosity in log space (Eq. 22): L = Lo + delta,
+    // delta = -[beta_phi ((Pf1 - Pfo) - (Pt1 - Pto)) + dt (Pf1 - Pt1) / eta + dt V.grad(1-phi)/(1-phi)]
+    // V.grad(1-phi)/(1-phi) = -(w/2) sum_d rd [v_r (phi_r - phi) + v_l (phi - phi_l)]
+    //                      = -w [sum_d hrd (v_r phi_r - v_l phi_l) - phi divV / 2]
+    const double adv = -w * fma(ph, -0.5 * divV, fma(ax, c.hrdx, fma(ay, c.hrdy, az * c.hrdz)));
+    const double dp1 = Pf1 - Pt1;
+    const double rate = c.compaction_on ? fma(dp1, ieta, adv) : adv;
+    const double delta = -fma(c.beta_phi, dp1 - (Pfo - Pto), c.dt * rate);
+    double em_p, em_n;
+    expm1_pair(delta, em_p, em_n);
+    const double phio = in.phio[q], Eo = in.Eo[q], iEo = in.iEo[q];
+    const double K = in.K0 ? in.K0[q] : c.k0r3;
+    const double ph1 = fma(-Eo, em_p, phio);
+    // every load above precedes the stores (the arrays are not declared non-aliasing)
+    out.Pt[q] = Pt1;
+    out.Pf[q] = Pf1;
+    out.txx[q] = sxx;
+    out.tyy[q] = syy;
+    out.tzz[q] = szz;
+    out.phi[q] = ph1;
+    out.w[q] = fma(iEo, em_n, iEo);
+    out.perm[q] = K * ph1 * ph1 * ph1;
+    if (check) {   // of the column: a NaN stays the largest
+      r_pt = abs_max(r_pt, divVn);
+      r_pf = abs_max(r_pf, resF);
+    }
+  }
+  out.txy[q] = t_xy;
+  if (j < b.ny) out.txz[q] = t_xz;
+  if (i < b.nx) out.tyz[q] = t_yz;
+  col.k_d = col.kk; col.phi_d = col.phi; col.vx_d = vx; col.vy_d = vy; col.fz = fz_u;
+  col.Pf = Pf_u; col.kk = k_u; col.phi = phi_u; col.vz = vz_u;
 }
 
 // Momentum residual, damped R and velocity update of the three lower faces of (i, j, k) in FP64; bit d
@@ -325,12 +347,10 @@ __device__ __forceinline__ void lean_face_point(const Box& b, const LeanCoef<dou
                                                 double* __restrict__ Vz, double* __restrict__ Rx,
                                                 double* __restrict__ Ry, double* __restrict__ Rz, int i, int j, int k,
                                                 int check, double& r_v, int mask = 7) {
-  if (i <= b.nx && j <= b.ny && k <= b.nz) {
+  if (i < b.nx && j < b.ny && k < b.nz) {   // the faces i = nx, j = ny, k = nz are walls
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
-    const bool fx = i > 0 && i < b.nx && j < b.ny && k < b.nz;
-    const bool fy = j > 0 && j < b.ny && i < b.nx && k < b.nz;
-    const bool fz = k > 0 && k < b.nz && i < b.nx && j < b.ny;
+    const bool fx = i > 0, fy = j > 0, fz = k > 0;
     // all loads before the first store (the arrays are not declared non-aliasing)
     double Fx = 0.0, Fy = 0.0, Fz = 0.0, Rx1 = 0.0, Ry1 = 0.0, Rz1 = 0.0, Vx1 = 0.0, Vy1 = 0.0, Vz1 = 0.0;
     // F / rho_i directly (the spacings carry 1/rho_i); the norm takes |F| = rho_i |F / rho_i|
@@ -358,9 +378,11 @@ __device__ __forceinline__ void lean_face_point(const Box& b, const LeanCoef<dou
     if (fy) { Ry[q] = Ry1; Vy[q] = Vy1; }
     if (fz) { Rz[q] = Rz1; Vz[q] = Vz1; }
     if (check) {
-      if (fx && (mask & 1)) r_v = fmax(r_v, fabs(Fx) * c.rho_i);
-      if (fy && (mask & 2)) r_v = fmax(r_v, fabs(Fy) * c.rho_i);
-      if (fz && (mask & 4)) r_v = fmax(r_v, fabs(Fz) * c.rho_i);
+      double m = 0.0;
+      if (mask & 1) m = Fx;
+      if (mask & 2) m = lean_detail::abs_max(m, Fy);
+      if (mask & 4) m = lean_detail::abs_max(m, Fz);
+      r_v = lean_detail::abs_max(m, 0.0) * c.rho_i;
     }
   }
 }

@@ -90,16 +90,15 @@ struct MgLevel {
 };
 
 // Step start: Pto, Pfo, phio and max(mu).
-void mix_begin(dim3 g, dim3 bl, cudaStream_t s, Box b, const double* Pt, const double* Pf, const double* phi,
-               const double* mu, double* Pto, double* Pfo, double* phio, unsigned long long* red);
-void mix_perm(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk,
-              double* perm);
-void mix_prepare(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in,
-                 const MixPrepOut& out, unsigned long long* red);
-void mix_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in,
-               const MixFaceOut& out, unsigned long long* red);
-void mix_porosity(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p);
-void mix_update(dim3 g, dim3 bl, cudaStream_t s, Box b, const MixUpdate& u);
+void mix_begin(cudaStream_t s, Box b, const double* Pt, const double* Pf, const double* phi, const double* mu,
+               double* Pto, double* Pfo, double* phio, unsigned long long* red);
+void mix_perm(cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk, double* perm);
+void mix_prepare(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in, const MixPrepOut& out,
+                 unsigned long long* red);
+void mix_faces(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in, const MixFaceOut& out,
+               unsigned long long* red);
+void mix_porosity(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p);
+void mix_update(cudaStream_t s, Box b, const MixUpdate& u);
 // One fused FP32 correction iteration over the whole grid (z-marching tiles, see the kernel).
 void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrIn<float>& in,
                     const CorrOut<float>& out, unsigned long long* red, int check);

@@ -25,7 +25,8 @@ namespace pt {
 // instruction count: coefficients folded on the host (LeanCoef), fused multiply-adds, third-order
 // reciprocals and no division, the porosity by expm1 of its small increment, norms through bit patterns.
 // At 255^3 an outer iteration's phases took 13.0 ms (141 FP64 instructions per cell in k_mix_prepare
-// alone, 137 in the Picard update); now 6.4 ms.
+// alone, 137 in the Picard update, 67 at the edges); now 9.3 ms: 118 in k_mix_prepare with the edges, 86 in
+// k_mix_faces with the Picard update, 36 in k_mix_porosity, the pipe at 85 %.
 
 // k of the iterate (Eq. 23), read with its neighbours by mix_prepare_point.
 __device__ __forceinline__ void mix_perm_point(const Box& b, const LeanCoef<double>& c, const double* __restrict__ phi,
@@ -149,16 +150,16 @@ __device__ __forceinline__ void mix_porosity_point(const Box& b, const LeanCoef<
   p.phi1[q] = fma(phio - 1.0, em, phio);
 }
 
-__global__ void __launch_bounds__(256) k_mix_begin(Box b, const double* __restrict__ Pt, const double* __restrict__ Pf,
-                                                   const double* __restrict__ phi, const double* __restrict__ mu,
-                                                   double* __restrict__ Pto, double* __restrict__ Pfo,
-                                                   double* __restrict__ phio, unsigned long long* red) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z;
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_begin(Box b, const double* __restrict__ Pt,
+                                                             const double* __restrict__ Pf,
+                                                             const double* __restrict__ phi,
+                                                             const double* __restrict__ mu, double* __restrict__ Pto,
+                                                             double* __restrict__ Pfo, double* __restrict__ phio,
+                                                             unsigned long long* red, Plane pl) {
+  int i, j;
   double m = 0.0;
-  if (i < b.nx && j < b.ny && k < b.nz) {
-    const long long q = cidx(b, i, j, k);
+  if (plane_point(pl, i, j)) {
+    const long long q = cidx(b, i, j, (int)blockIdx.y);
     Pto[q] = Pt[q];
     Pfo[q] = Pf[q];
     phio[q] = phi[q];
@@ -167,31 +168,32 @@ __global__ void __launch_bounds__(256) k_mix_begin(Box b, const double* __restri
   block_max_atomic(m, red + RED_MUMAX);
 }
 
-__global__ void __launch_bounds__(256) k_mix_perm(Box b, LeanCoef<double> c, const double* __restrict__ phi,
-                                                  const double* __restrict__ logk, double* __restrict__ perm) {
-  mix_perm_point(b, c, phi, logk, perm, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
-                 (int)blockIdx.z);
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_perm(Box b, LeanCoef<double> c, const double* __restrict__ phi,
+                                                            const double* __restrict__ logk,
+                                                            double* __restrict__ perm, Plane pl) {
+  int i, j;
+  if (plane_point(pl, i, j)) mix_perm_point(b, c, phi, logk, perm, i, j, (int)blockIdx.y);
 }
 
-__global__ void __launch_bounds__(256) k_mix_porosity(Box b, LeanCoef<double> c, MixPorosity p) {
-  mix_porosity_point(b, c, p, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
-                     (int)blockIdx.z);
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_porosity(Box b, LeanCoef<double> c, MixPorosity p, Plane pl) {
+  int i, j;
+  if (plane_point(pl, i, j)) mix_porosity_point(b, c, p, i, j, (int)blockIdx.y);
 }
 
-__global__ void __launch_bounds__(256) k_mix_prepare(Box b, LeanCoef<double> c, MixPrepIn in, MixPrepOut out,
-                                                     unsigned long long* red) {
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_prepare(Box b, LeanCoef<double> c, MixPrepIn in,
+                                                               MixPrepOut out, unsigned long long* red, Plane pl) {
+  int i, j;
   double r_pt = 0.0, r_pf = 0.0;
-  mix_prepare_point(b, c, in, out, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
-                    (int)blockIdx.z, r_pt, r_pf);
+  if (plane_point(pl, i, j)) mix_prepare_point(b, c, in, out, i, j, (int)blockIdx.y, r_pt, r_pf);
   block_max_atomic(lean_detail::abs_max(r_pt, 0.0), red + RED_PT);
   block_max_atomic(lean_detail::abs_max(r_pf, 0.0), red + RED_PF);
 }
 
-__global__ void __launch_bounds__(256) k_mix_faces(Box b, LeanCoef<double> c, MixFaceIn in, MixFaceOut out,
-                                                   unsigned long long* red) {
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_faces(Box b, LeanCoef<double> c, MixFaceIn in, MixFaceOut out,
+                                                             unsigned long long* red, Plane pl) {
+  int i, j;
   double r_v = 0.0, pic = 1.0;
-  mix_faces_point(b, c, in, out, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
-                  (int)blockIdx.z, r_v, pic);
+  if (plane_point(pl, i, j)) mix_faces_point(b, c, in, out, i, j, (int)blockIdx.y, r_v, pic);
   block_max_atomic(lean_detail::abs_max(r_v, 0.0), red + RED_V);
   block_max_log_atomic(pic, red + RED_PIC);
 }
@@ -561,33 +563,37 @@ __device__ __forceinline__ void mix_update_point(const Box& b, const MixUpdate& 
   }
 }
 
-__global__ void __launch_bounds__(256) k_mix_update(Box b, MixUpdate u) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  mix_update_point(b, u, i, j, (int)blockIdx.z);
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_update(Box b, MixUpdate u, Plane pl) {
+  int i, j;
+  if (plane_point(pl, i, j)) mix_update_point(b, u, i, j, (int)blockIdx.y);
 }
 
-void mix_begin(dim3 g, dim3 bl, cudaStream_t s, Box b, const double* Pt, const double* Pf, const double* phi,
-               const double* mu, double* Pto, double* Pfo, double* phio, unsigned long long* red) {
-  k_mix_begin<<<g, bl, 0, s>>>(b, Pt, Pf, phi, mu, Pto, Pfo, phio, red);
+void mix_begin(cudaStream_t s, Box b, const double* Pt, const double* Pf, const double* phi, const double* mu,
+               double* Pto, double* Pfo, double* phio, unsigned long long* red) {
+  const Plane pl = plane_of(b, 0);
+  k_mix_begin<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, Pt, Pf, phi, mu, Pto, Pfo, phio, red, pl);
 }
-void mix_perm(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk,
-              double* perm) {
-  k_mix_perm<<<g, bl, 0, s>>>(b, c, phi, logk, perm);
+void mix_perm(cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk, double* perm) {
+  const Plane pl = plane_of(b, 0);
+  k_mix_perm<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, phi, logk, perm, pl);
 }
-void mix_prepare(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in,
-                 const MixPrepOut& out, unsigned long long* red) {
-  k_mix_prepare<<<g, bl, 0, s>>>(b, c, in, out, red);
+void mix_prepare(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in, const MixPrepOut& out,
+                 unsigned long long* red) {
+  const Plane pl = plane_of(b, c.bg_on ? 1 : 0);   // wall edges carry stress under a background shear only
+  k_mix_prepare<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, in, out, red, pl);
 }
-void mix_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in,
-               const MixFaceOut& out, unsigned long long* red) {
-  k_mix_faces<<<g, bl, 0, s>>>(b, c, in, out, red);
+void mix_faces(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in, const MixFaceOut& out,
+               unsigned long long* red) {
+  const Plane pl = plane_of(b, 0);
+  k_mix_faces<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, in, out, red, pl);
 }
-void mix_porosity(dim3 g, dim3 bl, cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p) {
-  k_mix_porosity<<<g, bl, 0, s>>>(b, c, p);
+void mix_porosity(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p) {
+  const Plane pl = plane_of(b, 0);
+  k_mix_porosity<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, p, pl);
 }
-void mix_update(dim3 g, dim3 bl, cudaStream_t s, Box b, const MixUpdate& u) {
-  k_mix_update<<<g, bl, 0, s>>>(b, u);
+void mix_update(cudaStream_t s, Box b, const MixUpdate& u) {
+  const Plane pl = plane_of(b, 0);
+  k_mix_update<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, u, pl);
 }
 void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrIn<float>& in,
                     const CorrOut<float>& out, unsigned long long* red, int check) {
