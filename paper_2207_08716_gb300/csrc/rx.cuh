@@ -111,6 +111,13 @@ struct MgCorr {
 template <class T>
 void mg_smooth(cudaStream_t s, Box b, const RxCoef<T>& c, double omega, const RxIn<T>& in, const MgSrc<T>* fas,
                const RxOut<T>& out, const MgE<T>* laste, unsigned long long* red, int check);
+// The sweeps of a visit of a coarsest grid small enough for one block (mg_coarsest_fits), from buffer 0
+// (in0, out0) and ping-ponging with buffer 1; the last writes e = u' - u0 over u0.
+template <class T>
+bool mg_coarsest_fits(const Box& b);
+template <class T>
+void mg_coarsest(cudaStream_t s, Box b, const RxCoef<T>& c, double omega, const RxIn<T>& in0, const RxIn<T>& in1,
+                 const MgSrc<T>& fas, const RxOut<T>& out0, const RxOut<T>& out1, const MgE<T>& e0, int sweeps);
 // fine residual and iterate -> coarse iterate, u0 and (restricted residual) sources
 template <class T>
 void mg_restrict(cudaStream_t s, Box fine, Box coarse, const RxCoef<T>& c, const RxIn<T>& in, const MgSrc<T>* fas,

@@ -271,6 +271,21 @@ void vcycle(rx_ctx* c, int l) {
   const rx_mg& m = c->mg;
   MgLevel& L = c->lv[l];
   if (l == m.levels - 1) {
+    if (l > 0 && mg_coarsest_fits<T>(L.b)) {
+      RxIn<T> in[2];
+      RxOut<T> out[2];
+      for (int d = 0; d < 2; ++d) {
+        in[d] = RxIn<T>{(const T*)L.Pf[d],   (const T*)L.phi[d],   (const T*)L.Xs[d],
+                        (const T*)L.Pf_o, (const T*)L.phi_o, (const T*)L.Xs_o};
+        out[d] = RxOut<T>{(T*)L.Pf[d], (T*)L.phi[d], (T*)L.Xs[d], nullptr};
+      }
+      const int d = L.cur;
+      mg_coarsest<T>(c->stream, L.b, lcoef<T>(L), m.omega, in[d], in[1 - d],
+                     MgSrc<T>{(const T*)L.fP, (const T*)L.fphi, (const T*)L.fX}, out[d], out[1 - d],
+                     MgE<T>{(T*)L.Pf0, (T*)L.phi0, (T*)L.Xs0}, m.nu_coarse);
+      ++c->launches;
+      return;
+    }
     for (int s = 0; s < m.nu_coarse; ++s) mg_sweep<T>(c, l, s == m.nu_coarse - 1);
     return;
   }

@@ -54,3 +54,27 @@ def test_fixed_count_steps(form, nx, ny, nz, shear, logk):
     case = dict(kind="step", form=form, nx=nx, ny=ny, nz=nz, iters=45, shear=shear, logk=logk)
     worst, off = _worst(case)
     assert worst < 1e-10, off
+
+
+# one cell per thread on small grids; beyond 300 k cells four: rows of 4 m + {0, 1, 3} cells, single cells and
+# rows, chunks of up to 16 levels
+@pytest.mark.parametrize("nx,ny,nz", [(1, 3, 5), (33, 31, 17), (1, 701, 431), (3, 2, 60001), (32, 5, 1901),
+                                      (33, 31, 297), (127, 129, 19)])
+def test_reactive_rows_fp32(nx, ny, nz):
+    """20 FP32 iterations of some 16 roundings (2^-24 each) in a row: 20 * 16 * 2^-24 = 1.9e-5."""
+    worst, off = _worst(dict(kind="rx", form="fp32", nx=nx, ny=ny, nz=nz, iters=20))
+    assert worst < 20 * 16 * 2.0 ** -24, off
+
+
+# coarse rows of one, odd and even numbers of cells; a coarsest grid of one block and larger ones; one cell
+# per thread, four on the finest grid, four on the next one too
+@pytest.mark.parametrize("nx,ny,nz", [(4, 12, 8), (20, 8, 40), (36, 28, 72), (4, 300, 256), (20, 100, 152),
+                                      (132, 132, 140)])
+def test_reactive_cycles_fp32(nx, ny, nz):
+    """Two V-cycles on three levels against the FP64 form, which has one cell per thread: some 40 sweeps a
+    cycle (30 of them coarsest) of 8 roundings in a row, 2 * 40 * 8 * 2^-24 = 3.8e-5."""
+    C = _cases()
+    case = dict(kind="rxmg", nx=nx, ny=ny, nz=nz, levels=3, cycles=2)
+    got, want = (C.run(C.prepare(dict(case, form=f), 3)) for f in ("fp32", "fp64"))
+    off = {k: float((got[k].double() - want[k]).norm() / want[k].norm().clamp_min(1e-300)) for k in got}
+    assert max(off.values()) < 2 * 40 * 8 * 2.0 ** -24, off
