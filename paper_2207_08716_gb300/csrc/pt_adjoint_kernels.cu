@@ -34,8 +34,9 @@ __device__ inline double kperm(const AdjCoef& c, const double* K0, long long q, 
 }  // namespace
 
 // Per-step coefficients from the converged state u (cells i < nx ... and their lower faces).
-__global__ void __launch_bounds__(256) k_adj_prep(Box b, AdjCoef c, AdjState u, const double* __restrict__ K0,
+__global__ void __launch_bounds__(256) k_adj_prep(Box b, AdjCoef c, AdjState u, const double* K0,
                                                   AdjPrep o) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(256) k_adj_prep(Box b, AdjCoef c, AdjState u, 
 // updates of lambda_P, lambda_F, lambda_L.
 __global__ void __launch_bounds__(256) k_adj_cells(Box b, AdjCoef c, AdjState u, AdjCellIn in, AdjCellOut out,
                                                    unsigned long long* red, int check) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(256) k_adj_cells(Box b, AdjCoef c, AdjState u,
 __global__ void __launch_bounds__(256) k_adj_faces(Box b, AdjCoef c, AdjFaceIn in, double* Lx, double* Ly,
                                                    double* Lz, double* Rx, double* Ry, double* Rz,
                                                    unsigned long long* red, int check) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -333,6 +336,7 @@ __device__ inline double dmodulus(double m, double Gdt) {
 // Pass 1: edge moduli, P_e and the state's edge stresses (scratch), for the edges owned by the index.
 __global__ void __launch_bounds__(256) k_adj_prep_pl_edges(Box b, AdjCoef c, AdjState u, AdjPrepPL pl,
                                                            double* tau_xy, double* tau_xz, double* tau_yz) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -375,10 +379,11 @@ __global__ void __launch_bounds__(256) k_adj_prep_pl_edges(Box b, AdjCoef c, Adj
 }
 
 // Pass 2: the coefficients of k_adj_prep with mu per cell, and the power-law arrays.
-__global__ void __launch_bounds__(256) k_adj_prep_pl(Box b, AdjCoef c, AdjState u, const double* __restrict__ K0,
-                                                     AdjPrep o, AdjPrepPL pl, const double* __restrict__ tau_xy,
-                                                     const double* __restrict__ tau_xz,
-                                                     const double* __restrict__ tau_yz) {
+__global__ void __launch_bounds__(256) k_adj_prep_pl(Box b, AdjCoef c, AdjState u, const double* K0,
+                                                     AdjPrep o, AdjPrepPL pl, const double* tau_xy,
+                                                     const double* tau_xz,
+                                                     const double* tau_yz) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -488,6 +493,7 @@ __global__ void __launch_bounds__(256) k_adj_prep_pl(Box b, AdjCoef c, AdjState 
 // Edges of one iteration: sigma_e from lambda_mu, adjoint edge stress m_e (eps_e(lambda_V) - sigma_e/2),
 // Z_e = sigma_e - 2 eps_e(lambda_V); zero on wall edges.
 __global__ void __launch_bounds__(256) k_adj_edges_pl(Box b, AdjCoef c, AdjEdgeIn in, AdjEdgeOut out) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -534,6 +540,7 @@ __global__ void __launch_bounds__(256) k_adj_edges_pl(Box b, AdjCoef c, AdjEdgeI
 __global__ void __launch_bounds__(256) k_adj_cells_pl(Box b, AdjCoef c, AdjState u, AdjCellIn in, AdjCellOut out,
                                                       AdjPrepPL pl, AdjMuIn mi, unsigned long long* red,
                                                       int check) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -638,10 +645,11 @@ __global__ void __launch_bounds__(256) k_adj_cells_pl(Box b, AdjCoef c, AdjState
 
 // d(lambda . F)/d(G dtS): the moduli depend on Gdt through xi = mu / Gdt; summed over the grid.
 __global__ void __launch_bounds__(256) k_adj_dgdt_pl(Box b, AdjCoef c, AdjState u, AdjPrepPL pl,
-                                                     const double* __restrict__ Lx, const double* __restrict__ Ly,
-                                                     const double* __restrict__ Lz, const double* __restrict__ lM,
-                                                     const double* __restrict__ Zxy, const double* __restrict__ Zxz,
-                                                     const double* __restrict__ Zyz, double* acc) {
+                                                     const double* Lx, const double* Ly,
+                                                     const double* Lz, const double* lM,
+                                                     const double* Zxy, const double* Zxz,
+                                                     const double* Zyz, double* acc) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -682,7 +690,8 @@ __global__ void __launch_bounds__(256) k_adj_dgdt_pl(Box b, AdjCoef c, AdjState 
   }
 }
 
-__global__ void __launch_bounds__(256) k_adj_mumax(Box b, const double* __restrict__ mu, unsigned long long* red) {
+__global__ void __launch_bounds__(256) k_adj_mumax(Box b, const double* mu, unsigned long long* red) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -690,7 +699,8 @@ __global__ void __launch_bounds__(256) k_adj_mumax(Box b, const double* __restri
   if (i < b.nx && j < b.ny && k < b.nz) m = mu[cidx(b, i, j, k)];
   block_max_atomic(m, red + RED_MUMAX);
 }
-__global__ void __launch_bounds__(256) k_adj_argmax(Box b, const double* __restrict__ mu, unsigned long long* red) {
+__global__ void __launch_bounds__(256) k_adj_argmax(Box b, const double* mu, unsigned long long* red) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -701,49 +711,50 @@ __global__ void __launch_bounds__(256) k_adj_argmax(Box b, const double* __restr
 }
 __global__ void k_adj_add_at(double* gM, long long n, const unsigned long long* red, const double* acc,
                              double scale) {
+  chain_begin();
   const unsigned long long q = red[RED_ARG];
   if (threadIdx.x == 0 && blockIdx.x == 0 && q < (unsigned long long)n) gM[q] += scale * (*acc);
 }
 
 void adj_prep_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const double* K0,
                  const AdjPrep& out, const AdjPrepPL& pl, double* tau_xy, double* tau_xz, double* tau_yz) {
-  k_adj_prep_pl_edges<<<g, bl, 0, s>>>(b, c, u, pl, tau_xy, tau_xz, tau_yz);
-  k_adj_prep_pl<<<g, bl, 0, s>>>(b, c, u, K0, out, pl, tau_xy, tau_xz, tau_yz);
+  launch_chained(k_adj_prep_pl_edges, g, bl, 0, s, b, c, u, pl, tau_xy, tau_xz, tau_yz);
+  launch_chained(k_adj_prep_pl, g, bl, 0, s, b, c, u, K0, out, pl, tau_xy, tau_xz, tau_yz);
 }
 void adj_edges_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjEdgeIn& in,
                   const AdjEdgeOut& out) {
-  k_adj_edges_pl<<<g, bl, 0, s>>>(b, c, in, out);
+  launch_chained(k_adj_edges_pl, g, bl, 0, s, b, c, in, out);
 }
 void adj_cells_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const AdjCellIn& in,
                   const AdjCellOut& out, const AdjPrepPL& pl, const AdjMuIn& mu, unsigned long long* red,
                   int check) {
-  k_adj_cells_pl<<<g, bl, 0, s>>>(b, c, u, in, out, pl, mu, red, check);
+  launch_chained(k_adj_cells_pl, g, bl, 0, s, b, c, u, in, out, pl, mu, red, check);
 }
 void adj_dgdt_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u,
                  const AdjPrepPL& pl, const double* Lx, const double* Ly, const double* Lz, const double* lM,
                  const double* Zxy, const double* Zxz, const double* Zyz, double* acc) {
-  k_adj_dgdt_pl<<<g, bl, 0, s>>>(b, c, u, pl, Lx, Ly, Lz, lM, Zxy, Zxz, Zyz, acc);
+  launch_chained(k_adj_dgdt_pl, g, bl, 0, s, b, c, u, pl, Lx, Ly, Lz, lM, Zxy, Zxz, Zyz, acc);
 }
 void adj_argmax(dim3 g, dim3 bl, cudaStream_t s, Box b, const double* mu, unsigned long long* red) {
-  k_adj_mumax<<<g, bl, 0, s>>>(b, mu, red);
-  k_adj_argmax<<<g, bl, 0, s>>>(b, mu, red);
+  launch_chained(k_adj_mumax, g, bl, 0, s, b, mu, red);
+  launch_chained(k_adj_argmax, g, bl, 0, s, b, mu, red);
 }
 void adj_add_at(cudaStream_t s, Box b, double* gM, const unsigned long long* red, const double* acc,
                 double scale) {
-  k_adj_add_at<<<1, 32, 0, s>>>(gM, b.n, red, acc, scale);
+  launch_chained(k_adj_add_at, 1, 32, 0, s, gM, b.n, red, acc, scale);
 }
 
 void adj_prep(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const double* K0,
               const AdjPrep& out) {
-  k_adj_prep<<<g, bl, 0, s>>>(b, c, u, K0, out);
+  launch_chained(k_adj_prep, g, bl, 0, s, b, c, u, K0, out);
 }
 void adj_cells(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const AdjCellIn& in,
                const AdjCellOut& out, unsigned long long* red, int check) {
-  k_adj_cells<<<g, bl, 0, s>>>(b, c, u, in, out, red, check);
+  launch_chained(k_adj_cells, g, bl, 0, s, b, c, u, in, out, red, check);
 }
 void adj_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjFaceIn& in, double* Lx,
                double* Ly, double* Lz, double* Rx, double* Ry, double* Rz, unsigned long long* red, int check) {
-  k_adj_faces<<<g, bl, 0, s>>>(b, c, in, Lx, Ly, Lz, Rx, Ry, Rz, red, check);
+  launch_chained(k_adj_faces, g, bl, 0, s, b, c, in, Lx, Ly, Lz, Rx, Ry, Rz, red, check);
 }
 void adj_carry(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjCarry& a) {
   k_adj_carry<<<g, bl, 0, s>>>(b, c, a);

@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(kPlaneThreads, kLeanCellBlocks) k_lean_cells(B
                                                                                LeanCellOut<double> out,
                                                                                unsigned long long* red, int check,
                                                                                Plane pl, int zchunk) {
+  chain_begin();
   int i, j;
   double r_pt = 0.0, r_pf = 0.0;
   if (plane_point(pl, i, j)) {
@@ -175,6 +176,7 @@ __device__ __forceinline__ void df_cells_run(const Box& b, const LeanCoef<df64>&
 __global__ void __launch_bounds__(256, kZmarchBlocks) k_df_cells(Box b, LeanCoef<df64> c, LeanCellIn<df64> in,
                                                                  LeanCellOut<df64> out, unsigned long long* red,
                                                                  int check, int zchunk) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   df64* const st = reinterpret_cast<df64*>(smem_raw);
   const int i = blockIdx.x * 32 + threadIdx.x;
@@ -191,10 +193,10 @@ __global__ void __launch_bounds__(256, kZmarchBlocks) k_df_cells(Box b, LeanCoef
   }
 }
 
-__global__ void __launch_bounds__(256) k_df_faces(Box b, LeanCoef<df64> c, LeanFaceIn<df64> in, df64* __restrict__ Vx,
-                                                  df64* __restrict__ Vy, df64* __restrict__ Vz, df64* __restrict__ Rx,
-                                                  df64* __restrict__ Ry, df64* __restrict__ Rz,
+__global__ void __launch_bounds__(256) k_df_faces(Box b, LeanCoef<df64> c, LeanFaceIn<df64> in, df64* Vx,
+                                                  df64* Vy, df64* Vz, df64* Rx, df64* Ry, df64* Rz,
                                                   unsigned long long* red, int check) {
+  chain_begin();
   double r_v = 0.0;
   df_face_point(b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, blockIdx.x * 32 + threadIdx.x, blockIdx.y * 8 + threadIdx.y,
                 blockIdx.z, check, r_v);
@@ -203,10 +205,10 @@ __global__ void __launch_bounds__(256) k_df_faces(Box b, LeanCoef<df64> c, LeanF
 
 // ------------------------------------------------------------------------------ faces
 __global__ void __launch_bounds__(kPlaneThreads) k_lean_faces(Box b, LeanCoef<double> c, LeanFaceIn<double> in,
-                                                              double* __restrict__ Vx, double* __restrict__ Vy,
-                                                              double* __restrict__ Vz, double* __restrict__ Rx,
-                                                              double* __restrict__ Ry, double* __restrict__ Rz,
-                                                              unsigned long long* red, int check, Plane pl) {
+                                                              double* Vx, double* Vy, double* Vz, double* Rx,
+                                                              double* Ry, double* Rz, unsigned long long* red,
+                                                              int check, Plane pl) {
+  chain_begin();
   int i, j;
   double r_v = 0.0;
   if (plane_point(pl, i, j))
@@ -217,8 +219,9 @@ __global__ void __launch_bounds__(kPlaneThreads) k_lean_faces(Box b, LeanCoef<do
 // ------------------------------------------------------------------------------ Picard
 template <class T>
 __global__ void __launch_bounds__(kPlaneThreads) k_lean_picard(Box b, LeanCoef<T> c, LeanPicardIn<T> in,
-                                                               T* __restrict__ mu, T* __restrict__ eta,
+                                                               T* mu, T* eta,
                                                                unsigned long long* red, Plane pl) {
+  chain_begin();
   int i, j;
   double m = 1.0;
   if (plane_point(pl, i, j)) lean_picard_point(b, c, in, mu, eta, i, j, (int)blockIdx.y, m);
@@ -377,7 +380,8 @@ void lean_cells<double>(cudaStream_t st, Box b, const LeanCoef<double>& c, const
   const dim3 g = plane_grid(pl, 1);
   // the pipe is shared by an SM's blocks: a level takes as long as there are blocks on the SM
   const int zc = march_chunk(g.x, b.nz, kLeanCellChunk, kLeanCellBlocks, sm_count(), 0.15, 0.3);
-  k_lean_cells<<<dim3(g.x, (unsigned)((b.nz + zc - 1) / zc)), kPlaneThreads, 0, st>>>(b, c, in, out, red, check, pl, zc);
+  launch_chained(k_lean_cells, dim3(g.x, (unsigned)((b.nz + zc - 1) / zc)), kPlaneThreads, 0, st, b, c, in, out, red,
+                 check, pl, zc);
 }
 // The double-float form: the wall indices i = nx, j = ny carry stress under a background shear only.
 template <>
@@ -387,26 +391,28 @@ void lean_cells<df64>(cudaStream_t st, Box b, const LeanCoef<df64>& c, const Lea
   cudaFuncSetAttribute(k_df_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const unsigned gx = (b.nx + w + 31) / 32, gy = (b.ny + w + 7) / 8;
   const int zc = march_chunk((long long)gx * gy, b.nz, kLeanZChunk, kZmarchBlocks, sm_count(), 1.0, 1.6);
-  k_df_cells<<<dim3(gx, gy, (unsigned)((b.nz + zc - 1) / zc)), dim3(32, 8, 1), smem, st>>>(b, c, in, out, red, check, zc);
+  launch_chained(k_df_cells, dim3(gx, gy, (unsigned)((b.nz + zc - 1) / zc)), dim3(32, 8, 1), smem, st, b, c, in, out,
+                 red, check, zc);
 }
 template <>
 void lean_faces<df64>(cudaStream_t st, Box b, const LeanCoef<df64>& c, const LeanFaceIn<df64>& in, df64* Vx,
                       df64* Vy, df64* Vz, df64* Rx, df64* Ry, df64* Rz, unsigned long long* red, int check) {
   const dim3 g((unsigned)((b.nx + 31) / 32), (unsigned)((b.ny + 7) / 8), (unsigned)b.nz);
-  k_df_faces<<<g, dim3(32, 8, 1), 0, st>>>(b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, red, check);
+  launch_chained(k_df_faces, g, dim3(32, 8, 1), 0, st, b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, red, check);
 }
 template <>
 void lean_faces<double>(cudaStream_t st, Box b, const LeanCoef<double>& c, const LeanFaceIn<double>& in, double* Vx,
                         double* Vy, double* Vz, double* Rx, double* Ry, double* Rz, unsigned long long* red,
                         int check) {
   const Plane pl = plane_of(b, 0);
-  k_lean_faces<<<plane_grid(pl, b.nz), kPlaneThreads, 0, st>>>(b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, red, check, pl);
+  launch_chained(k_lean_faces, plane_grid(pl, b.nz), kPlaneThreads, 0, st, b, c, in, Vx, Vy, Vz, Rx, Ry, Rz, red,
+                 check, pl);
 }
 template <class T>
 void lean_picard(cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanPicardIn<T>& in, T* mu, T* eta,
                  unsigned long long* red) {
   const Plane pl = plane_of(b, 0);
-  k_lean_picard<T><<<plane_grid(pl, b.nz), kPlaneThreads, 0, st>>>(b, c, in, mu, eta, red, pl);
+  launch_chained(k_lean_picard<T>, plane_grid(pl, b.nz), kPlaneThreads, 0, st, b, c, in, mu, eta, red, pl);
 }
 template <class T>
 void lean_coef(cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanCoefIn<T>& in, const LeanCoefOut<T>& out) {

@@ -168,20 +168,23 @@ __global__ void __launch_bounds__(kPlaneThreads) k_mix_begin(Box b, const double
   block_max_atomic(m, red + RED_MUMAX);
 }
 
-__global__ void __launch_bounds__(kPlaneThreads) k_mix_perm(Box b, LeanCoef<double> c, const double* __restrict__ phi,
-                                                            const double* __restrict__ logk,
-                                                            double* __restrict__ perm, Plane pl) {
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_perm(Box b, LeanCoef<double> c, const double* phi,
+                                                            const double* logk,
+                                                            double* perm, Plane pl) {
+  chain_begin();
   int i, j;
   if (plane_point(pl, i, j)) mix_perm_point(b, c, phi, logk, perm, i, j, (int)blockIdx.y);
 }
 
 __global__ void __launch_bounds__(kPlaneThreads) k_mix_porosity(Box b, LeanCoef<double> c, MixPorosity p, Plane pl) {
+  chain_begin();
   int i, j;
   if (plane_point(pl, i, j)) mix_porosity_point(b, c, p, i, j, (int)blockIdx.y);
 }
 
 __global__ void __launch_bounds__(kPlaneThreads) k_mix_prepare(Box b, LeanCoef<double> c, MixPrepIn in,
                                                                MixPrepOut out, unsigned long long* red, Plane pl) {
+  chain_begin();
   int i, j;
   double r_pt = 0.0, r_pf = 0.0;
   if (plane_point(pl, i, j)) mix_prepare_point(b, c, in, out, i, j, (int)blockIdx.y, r_pt, r_pf);
@@ -191,6 +194,7 @@ __global__ void __launch_bounds__(kPlaneThreads) k_mix_prepare(Box b, LeanCoef<d
 
 __global__ void __launch_bounds__(kPlaneThreads) k_mix_faces(Box b, LeanCoef<double> c, MixFaceIn in, MixFaceOut out,
                                                              unsigned long long* red, Plane pl) {
+  chain_begin();
   int i, j;
   double r_v = 0.0, pic = 1.0;
   if (plane_point(pl, i, j)) mix_faces_point(b, c, in, out, i, j, (int)blockIdx.y, r_v, pic);
@@ -544,6 +548,7 @@ __device__ __forceinline__ void corr_tile(const Box& b, const CorrCoef<float>& c
 __global__ void __launch_bounds__(CorrSingle::threads, CorrSingle::blocks) k_corr_iteration(Box b, CorrCoef<float> c, CorrIn<float> in,
                                                         CorrOut<float> out, unsigned long long* red, int check,
                                                         int zchunk) {
+  chain_begin();
   extern __shared__ __align__(16) float corr_smem[];   // CorrSingle::smem, dynamic (above 48 KB)
   const int k0 = blockIdx.z * zchunk;
   corr_tile<CorrSingle>(b, c, in, out, blockIdx.x, blockIdx.y, k0, min(k0 + zchunk, b.nz), red, check, corr_smem);
@@ -564,6 +569,7 @@ __device__ __forceinline__ void mix_update_point(const Box& b, const MixUpdate& 
 }
 
 __global__ void __launch_bounds__(kPlaneThreads) k_mix_update(Box b, MixUpdate u, Plane pl) {
+  chain_begin();
   int i, j;
   if (plane_point(pl, i, j)) mix_update_point(b, u, i, j, (int)blockIdx.y);
 }
@@ -575,25 +581,25 @@ void mix_begin(cudaStream_t s, Box b, const double* Pt, const double* Pf, const 
 }
 void mix_perm(cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk, double* perm) {
   const Plane pl = plane_of(b, 0);
-  k_mix_perm<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, phi, logk, perm, pl);
+  launch_chained(k_mix_perm, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, phi, logk, perm, pl);
 }
 void mix_prepare(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in, const MixPrepOut& out,
                  unsigned long long* red) {
   const Plane pl = plane_of(b, c.bg_on ? 1 : 0);   // wall edges carry stress under a background shear only
-  k_mix_prepare<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, in, out, red, pl);
+  launch_chained(k_mix_prepare, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, in, out, red, pl);
 }
 void mix_faces(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in, const MixFaceOut& out,
                unsigned long long* red) {
   const Plane pl = plane_of(b, 0);
-  k_mix_faces<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, in, out, red, pl);
+  launch_chained(k_mix_faces, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, in, out, red, pl);
 }
 void mix_porosity(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p) {
   const Plane pl = plane_of(b, 0);
-  k_mix_porosity<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, p, pl);
+  launch_chained(k_mix_porosity, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, p, pl);
 }
 void mix_update(cudaStream_t s, Box b, const MixUpdate& u) {
   const Plane pl = plane_of(b, 0);
-  k_mix_update<<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, u, pl);
+  launch_chained(k_mix_update, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, u, pl);
 }
 void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrIn<float>& in,
                     const CorrOut<float>& out, unsigned long long* red, int check) {
@@ -602,7 +608,8 @@ void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrI
   const int zc = march_chunk((long long)gx * gy, b.nz, kCorrZChunk, CorrSingle::blocks, sm_count(), 3.0, 1.0);
   const dim3 g(gx, gy, (unsigned)((b.nz + zc - 1) / zc));
   cudaFuncSetAttribute(k_corr_iteration, cudaFuncAttributeMaxDynamicSharedMemorySize, CorrSingle::smem);
-  k_corr_iteration<<<g, dim3(32, CorrSingle::rows, 1), CorrSingle::smem, s>>>(b, c, in, out, red, check, zc);
+  launch_chained(k_corr_iteration, g, dim3(32, CorrSingle::rows, 1), CorrSingle::smem, s, b, c, in, out, red, check,
+                 zc);
 }
 
 
@@ -610,6 +617,7 @@ void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrI
 // Level f (fine, n cells per direction) and level c (coarse, ceil(n / 2)), through the weight
 // tables of c.ax (MgAxis).
 __global__ void __launch_bounds__(256) k_mg_coef(MgLevel f, MgLevel c, float dtaupt_fac, float dtauv_fac) {
+  chain_begin();
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
   const int K = blockIdx.z;
   if (I >= c.b.nx || J >= c.b.ny || K >= c.b.nz) return;
@@ -637,6 +645,7 @@ __global__ void __launch_bounds__(256) k_mg_coef(MgLevel f, MgLevel c, float dta
 }
 
 __global__ void __launch_bounds__(256) k_mg_restrict(MgLevel f, MgLevel c, float rho_i) {
+  chain_begin();
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
   const int K = blockIdx.z;
   const Box& B = c.b;
@@ -707,6 +716,7 @@ __global__ void __launch_bounds__(256) k_mg_restrict(MgLevel f, MgLevel c, float
 }
 
 __global__ void __launch_bounds__(256) k_mg_prolong(MgLevel c, int dc, MgLevel f, int df) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
   const Box& B = f.b;
@@ -768,15 +778,15 @@ __global__ void __launch_bounds__(256) k_mg_prolong(MgLevel c, int dc, MgLevel f
 
 void mg_coef(cudaStream_t s, const MgLevel& f, const MgLevel& c, float dtaupt_fac, float dtauv_fac) {
   const dim3 bl(32, 8, 1), g((c.b.nx + 31) / 32, (c.b.ny + 7) / 8, c.b.nz);
-  k_mg_coef<<<g, bl, 0, s>>>(f, c, dtaupt_fac, dtauv_fac);
+  launch_chained(k_mg_coef, g, bl, 0, s, f, c, dtaupt_fac, dtauv_fac);
 }
 void mg_restrict(cudaStream_t s, const MgLevel& f, const MgLevel& c, float rho_i) {
   const dim3 bl(32, 8, 1), g((c.b.nx + 1 + 31) / 32, (c.b.ny + 1 + 7) / 8, c.b.nz + 1);
-  k_mg_restrict<<<g, bl, 0, s>>>(f, c, rho_i);
+  launch_chained(k_mg_restrict, g, bl, 0, s, f, c, rho_i);
 }
 void mg_prolong(cudaStream_t s, const MgLevel& c, int dc, const MgLevel& f, int df) {
   const dim3 bl(32, 8, 1), g((f.b.nx + 1 + 31) / 32, (f.b.ny + 1 + 7) / 8, f.b.nz + 1);
-  k_mg_prolong<<<g, bl, 0, s>>>(c, dc, f, df);
+  launch_chained(k_mg_prolong, g, bl, 0, s, c, dc, f, df);
 }
 
 // ============================================================ batched FP32 ensembles (engine)

@@ -41,6 +41,7 @@ __device__ __forceinline__ RxNew<T> rx_cell(const RxCoef<T>& c, T dtau, T divq, 
 template <class T>
 __global__ void __launch_bounds__(kPlaneThreads) k_rx_iter(Box b, RxCoef<T> c, T dtau, RxIn<T> in, RxOut<T> out,
                                                            unsigned long long* red, int check, Plane pl) {
+  chain_begin();
   int i, j;
   const int k = blockIdx.y;
   double chg = 0.0, kb = 0.0;
@@ -89,6 +90,7 @@ __global__ void __launch_bounds__(kQuadThreads, kIterBlocks) k_rx_iter4(Box b, R
                                                                         RxIn<float> in, RxOut<float> out,
                                                                         unsigned long long* red, int check, Quads qd,
                                                                         int zchunk) {
+  chain_begin();
   int i, j;
   QuadChange chg{0u, 0u, 0u};
   int kb = 0;   // largest k / beta_P (not negative) as its bits; a NaN is the largest
@@ -131,8 +133,9 @@ __global__ void __launch_bounds__(kQuadThreads, kIterBlocks) k_rx_iter4(Box b, R
 }
 
 template <class T>
-__global__ void __launch_bounds__(256) k_rx_kbmax(Box b, RxCoef<T> c, const T* __restrict__ phi,
+__global__ void __launch_bounds__(256) k_rx_kbmax(Box b, RxCoef<T> c, const T* phi,
                                                   unsigned long long* red) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -185,16 +188,16 @@ void rx_iter(cudaStream_t s, Box b, const RxCoef<T>& c, double dtau, const RxIn<
       const Quads qd = quads_of(b);
       int zc;
       const dim3 g = quad_grid(qd, b.nz, kIterBlocks, &zc);
-      k_rx_iter4<<<g, kQuadThreads, 0, s>>>(b, c, (float)dtau, in, out, red, check, qd, zc);
+      launch_chained(k_rx_iter4, g, kQuadThreads, 0, s, b, c, (float)dtau, in, out, red, check, qd, zc);
       return;
     }
   }
   const Plane pl = plane_of(b, 0);
-  k_rx_iter<T><<<plane_grid(pl, b.nz), kPlaneThreads, 0, s>>>(b, c, (T)dtau, in, out, red, check, pl);
+  launch_chained(k_rx_iter<T>, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, (T)dtau, in, out, red, check, pl);
 }
 template <class T>
 void rx_kbmax(cudaStream_t s, Box b, const RxCoef<T>& c, const T* phi, unsigned long long* red) {
-  k_rx_kbmax<T><<<rx_grid(b), dim3(32, 8, 1), 0, s>>>(b, c, phi, red);
+  launch_chained(k_rx_kbmax<T>, rx_grid(b), dim3(32, 8, 1), 0, s, b, c, phi, red);
 }
 template <class T>
 void rx_begin(cudaStream_t s, Box b, const RxCoef<T>& c, const double* Pf, const double* phi, const double* Xs,

@@ -9,10 +9,10 @@
 // 2 x 2 x 2 agglomerations; the restriction takes 8-child means of the iterate and of the
 // residual (g = target - current), the FAS source is f_c = mean(r) - g_c(u0_c), and the
 // correction u_c - u0_c (written by the coarse level's last sweep) comes back by trilinear
-// interpolation (3/4, 1/4 per direction, the neighbour held at the wall). In FP64 and on
-// small FP32 grids the sweeps, the restriction and the right-hand side run one thread per cell, on FP32
-// grids from kQuadCells four cells per thread (rx_quad.cuh); the prolongation has one thread per pair of coarse cells, and a
-// small coarsest grid is swept in one block.
+// interpolation (3/4, 1/4 per direction, the neighbour held at the wall). In FP64 and on small
+// FP32 grids the sweeps, the restriction and the right-hand side run one thread per cell, on FP32 grids
+// from kQuadCells four cells per thread (rx_quad.cuh); the prolongation has one thread per pair of coarse
+// cells, and a small coarsest grid is swept in one block.
 #include "rx_quad.cuh"
 
 namespace pt {
@@ -116,6 +116,7 @@ dim3 grid_of(const Box& b) { return dim3((unsigned)((b.nx + 31) / 32), (unsigned
 template <class T, bool FAS, bool LASTE>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 8 : 5) k_mg_smooth(
     Box b, RxCoef<T> c, T romega, RxIn<T> in, MgSrc<T> f, RxOut<T> out, MgE<T> e0, unsigned long long* red, int check) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(kQuadThreads, kSmoothBlocks) k_mg_smooth4(Box 
                                                                             RxOut<float> out, MgE<float> e0,
                                                                             unsigned long long* red, int check,
                                                                             Quads qd, int zchunk) {
+  chain_begin();
   int i, j;
   QuadChange chg{0u, 0u, 0u};
   if (quad_point(qd, i, j)) {
@@ -204,6 +206,7 @@ constexpr int kRbx = 32, kRby = 4, kRbz = 2;
 template <class T, bool FAS>
 __global__ void __launch_bounds__(kRbx * kRby * kRbz) k_mg_restrict(Box fb, Box cb, RxCoef<T> c, RxIn<T> in,
                                                                     MgSrc<T> f, MgCoarse<T> out) {
+  chain_begin();
   const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
   const int i = blockIdx.x * kRbx + tx, j = blockIdx.y * kRby + ty, k = blockIdx.z * kRbz + tz;
   T v[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};        // Pf, phi, Xs, gP, gphi, gX
@@ -260,6 +263,7 @@ __global__ void __launch_bounds__(kQuadThreads, kRestrictBlocks) k_mg_restrict4(
                                                                                 RxIn<float> in, MgSrc<float> f,
                                                                                 MgCoarse<float> out, QuadRows qr,
                                                                                 int zchunk) {
+  chain_begin();
   const int t = min((int)(blockIdx.x * kQuadThreads + threadIdx.x), qr.n - 2 + (int)(threadIdx.x & 1));
   const bool own = (int)(blockIdx.x * kQuadThreads + threadIdx.x) < qr.n;
   const int odd = t & 1, J = (t >> 1) / qr.per_row, P = (t >> 1) - J * qr.per_row;
@@ -319,6 +323,7 @@ __global__ void __launch_bounds__(kQuadThreads, kRestrictBlocks) k_mg_restrict4(
 
 template <class T>
 __global__ void __launch_bounds__(256) k_mg_coarse_rhs(Box b, RxCoef<T> c, RxIn<T> u0, MgCoarse<T> out) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -333,6 +338,7 @@ __global__ void __launch_bounds__(256) k_mg_coarse_rhs(Box b, RxCoef<T> c, RxIn<
 __global__ void __launch_bounds__(kQuadThreads, kRestrictBlocks) k_mg_coarse_rhs4(Box b, RxCoef<float> c,
                                                                                   RxIn<float> u0, MgCoarse<float> out,
                                                                                   Quads qd, int zchunk) {
+  chain_begin();
   int i, j;
   if (!quad_point(qd, i, j)) return;
   const int k0 = blockIdx.y * zchunk, k1 = min(k0 + zchunk, b.nz);
@@ -376,10 +382,11 @@ constexpr int kProlongThreads = 128;
 template <class T>
 __global__ void __launch_bounds__(kProlongThreads) k_mg_prolong(Box fb, Box cb, MgCorr<T> corr, T* Pf, T* phi, T* Xs,
                                                                 int per_row) {
+  chain_begin();
   const int t = blockIdx.x * kProlongThreads + threadIdx.x, J = t / per_row, P = t - J * per_row, K = blockIdx.y;
   if (J >= cb.ny) return;
   const int field = blockIdx.z;
-  const T* __restrict__ e = field == 0 ? corr.Pf : field == 1 ? corr.phi : corr.Xs;
+  const T* e = field == 0 ? corr.Pf : field == 1 ? corr.phi : corr.Xs;
   T* u = field == 0 ? Pf : field == 1 ? phi : Xs;
   const int lo = max(2 * P - 1, 0), hi = min(2 * P + 2, cb.nx - 1);
   const bool lone = 2 * P + 1 >= cb.nx;
@@ -460,6 +467,7 @@ template <class T>
 __global__ void __launch_bounds__(kCoarsestThreads) k_mg_coarsest(Box b, RxCoef<T> c, T romega, RxIn<T> in0,
                                                                   RxIn<T> in1, MgSrc<T> f, RxOut<T> out0,
                                                                   RxOut<T> out1, MgE<T> e0, int sweeps) {
+  chain_begin();
   const int plane = b.nx * b.ny, n = plane * b.nz;
   for (int s = 0; s < sweeps; ++s) {
     const RxIn<T> in = (s & 1) ? in1 : in0;
@@ -492,7 +500,8 @@ bool mg_coarsest_fits(const Box& b) {
 template <class T>
 void mg_coarsest(cudaStream_t s, Box b, const RxCoef<T>& c, double omega, const RxIn<T>& in0, const RxIn<T>& in1,
                  const MgSrc<T>& fas, const RxOut<T>& out0, const RxOut<T>& out1, const MgE<T>& e0, int sweeps) {
-  k_mg_coarsest<T><<<1, kCoarsestThreads, 0, s>>>(b, c, (T)(1.0 / omega), in0, in1, fas, out0, out1, e0, sweeps);
+  launch_chained(k_mg_coarsest<T>, 1, kCoarsestThreads, 0, s, b, c, (T)(1.0 / omega), in0, in1, fas, out0, out1, e0,
+                 sweeps);
 }
 
 template <class T>
@@ -507,21 +516,24 @@ void mg_smooth(cudaStream_t s, Box b, const RxCoef<T>& c, double omega, const Rx
       int zc;
       const dim3 g = quad_grid(qd, b.nz, kSmoothBlocks, &zc);
       if (!fas)
-        k_mg_smooth4<false, false><<<g, kQuadThreads, 0, s>>>(b, c, romega, in, none, out, noe, red, check, qd, zc);
+        launch_chained(k_mg_smooth4<false, false>, g, kQuadThreads, 0, s, b, c, romega, in, none, out, noe, red,
+                       check, qd, zc);
       else if (!laste)
-        k_mg_smooth4<true, false><<<g, kQuadThreads, 0, s>>>(b, c, romega, in, *fas, out, noe, red, check, qd, zc);
+        launch_chained(k_mg_smooth4<true, false>, g, kQuadThreads, 0, s, b, c, romega, in, *fas, out, noe, red,
+                       check, qd, zc);
       else
-        k_mg_smooth4<true, true><<<g, kQuadThreads, 0, s>>>(b, c, romega, in, *fas, out, *laste, red, check, qd, zc);
+        launch_chained(k_mg_smooth4<true, true>, g, kQuadThreads, 0, s, b, c, romega, in, *fas, out, *laste, red,
+                       check, qd, zc);
       return;
     }
   }
   const dim3 g = grid_of(b), blk(32, 8, 1);
   if (!fas)
-    k_mg_smooth<T, false, false><<<g, blk, 0, s>>>(b, c, romega, in, none, out, noe, red, check);
+    launch_chained(k_mg_smooth<T, false, false>, g, blk, 0, s, b, c, romega, in, none, out, noe, red, check);
   else if (!laste)
-    k_mg_smooth<T, true, false><<<g, blk, 0, s>>>(b, c, romega, in, *fas, out, noe, red, check);
+    launch_chained(k_mg_smooth<T, true, false>, g, blk, 0, s, b, c, romega, in, *fas, out, noe, red, check);
   else
-    k_mg_smooth<T, true, true><<<g, blk, 0, s>>>(b, c, romega, in, *fas, out, *laste, red, check);
+    launch_chained(k_mg_smooth<T, true, true>, g, blk, 0, s, b, c, romega, in, *fas, out, *laste, red, check);
 }
 
 template <class T>
@@ -536,9 +548,9 @@ void mg_restrict(cudaStream_t s, Box fine, Box coarse, const RxCoef<T>& c, const
       const int zc = march_chunk(gx, coarse.nz, kQuadChunk / 2, kRestrictBlocks, sm_count(), 1.0, 0.75);
       const dim3 g(gx, (unsigned)((coarse.nz + zc - 1) / zc), 1);
       if (fas)
-        k_mg_restrict4<true><<<g, kQuadThreads, 0, s>>>(fine, coarse, c, in, *fas, out, qr, zc);
+        launch_chained(k_mg_restrict4<true>, g, kQuadThreads, 0, s, fine, coarse, c, in, *fas, out, qr, zc);
       else
-        k_mg_restrict4<false><<<g, kQuadThreads, 0, s>>>(fine, coarse, c, in, none, out, qr, zc);
+        launch_chained(k_mg_restrict4<false>, g, kQuadThreads, 0, s, fine, coarse, c, in, none, out, qr, zc);
       return;
     }
   }
@@ -546,9 +558,9 @@ void mg_restrict(cudaStream_t s, Box fine, Box coarse, const RxCoef<T>& c, const
                (unsigned)((fine.nz + kRbz - 1) / kRbz));
   const dim3 blk(kRbx, kRby, kRbz);
   if (fas)
-    k_mg_restrict<T, true><<<g, blk, 0, s>>>(fine, coarse, c, in, *fas, out);
+    launch_chained(k_mg_restrict<T, true>, g, blk, 0, s, fine, coarse, c, in, *fas, out);
   else
-    k_mg_restrict<T, false><<<g, blk, 0, s>>>(fine, coarse, c, in, none, out);
+    launch_chained(k_mg_restrict<T, false>, g, blk, 0, s, fine, coarse, c, in, none, out);
 }
 
 template <class T>
@@ -558,18 +570,18 @@ void mg_coarse_rhs(cudaStream_t s, Box coarse, const RxCoef<T>& c, const RxIn<T>
       const Quads qd = quads_of(coarse);
       int zc;
       const dim3 g = quad_grid(qd, coarse.nz, kRestrictBlocks, &zc);
-      k_mg_coarse_rhs4<<<g, kQuadThreads, 0, s>>>(coarse, c, u0, out, qd, zc);
+      launch_chained(k_mg_coarse_rhs4, g, kQuadThreads, 0, s, coarse, c, u0, out, qd, zc);
       return;
     }
   }
-  k_mg_coarse_rhs<T><<<grid_of(coarse), dim3(32, 8, 1), 0, s>>>(coarse, c, u0, out);
+  launch_chained(k_mg_coarse_rhs<T>, grid_of(coarse), dim3(32, 8, 1), 0, s, coarse, c, u0, out);
 }
 
 template <class T>
 void mg_prolong(cudaStream_t s, Box fine, Box coarse, const MgCorr<T>& e, T* Pf, T* phi, T* Xs) {
   const int per_row = (coarse.nx + 1) / 2;
   const dim3 g((unsigned)((per_row * coarse.ny + kProlongThreads - 1) / kProlongThreads), (unsigned)coarse.nz, 3);
-  k_mg_prolong<T><<<g, kProlongThreads, 0, s>>>(fine, coarse, e, Pf, phi, Xs, per_row);
+  launch_chained(k_mg_prolong<T>, g, kProlongThreads, 0, s, fine, coarse, e, Pf, phi, Xs, per_row);
 }
 
 template <class T>
