@@ -210,8 +210,8 @@ LeanCoef<df64> lean_coef_df64(const LeanCoef<double>& L) {
   PT_DF(alpha); PT_DF(alpha_B); PT_DF(bd_rdt_a); PT_DF(beta_n); PT_DF(beta_phi); PT_DF(dt);
   PT_DF(rphi0); PT_DF(k0); PT_DF(k0r3); PT_DF(phi0); PT_DF(drho_g); PT_DF(ifac_pf); PT_DF(rrho_i);
   PT_DF(damp_x); PT_DF(damp_y); PT_DF(damp_z); PT_DF(rdx_r); PT_DF(rdy_r); PT_DF(rdz_r);
-  PT_DF(drho_g_r); PT_DF(rho_i); PT_DF(ebg); PT_DF(mu0); PT_DF(eta0); PT_DF(R_weak);
-  PT_DF(rtau0_2); PT_DF(rmu0); PT_DF(rGdtS); PT_DF(dtaupt_fac); PT_DF(dtauv_fac);
+  PT_DF(drho_g_r); PT_DF(rho_i); PT_DF(ebg); PT_DF(mu0); PT_DF(eta0); PT_DF(eta0_weak);
+  PT_DF(rtau0_2h); PT_DF(rtau0_2s); PT_DF(rmu0); PT_DF(rGdtS); PT_DF(dtaupt_fac); PT_DF(dtauv_fac);
 #undef PT_DF
   F.compaction_on = L.compaction_on;
   F.powerlaw_on = L.powerlaw_on;
@@ -267,8 +267,9 @@ void fill_lean_coef(pt_ctx* c) {
   L.compaction_on = k.compaction_on;
   L.powerlaw_on = k.powerlaw_on;
   L.mu0 = k.mu0; L.eta0 = k.eta0; L.tau0 = k.tau0; L.n_pow = k.n_pow;
-  L.rtau0_2 = 1.0 / (k.tau0 * k.tau0);
-  L.rel_mu = k.rel_mu; L.rel_eta = k.rel_eta; L.R_weak = k.R_weak;
+  L.rtau0_2h = 0.5 / (k.tau0 * k.tau0);
+  L.rtau0_2s = 0.125 * L.rtau0_2h;
+  L.rel_mu = k.rel_mu; L.rel_eta = k.rel_eta; L.eta0_weak = k.eta0 * k.R_weak;
   L.rGdtS = k.rGdtS;
   L.dtaupt_fac = k.dtaupt_fac;
   L.dtauv_fac = k.dtauv_fac;

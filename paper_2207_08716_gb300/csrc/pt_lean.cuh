@@ -11,10 +11,11 @@ namespace pt {
 // The coefficients of (1 - t)^(-1/m) = 1 + t (a + t (b + t c) ...) (root_full)
 struct RootSeries {
   double a, b, c;   // 1/m, (m + 1) / (2 m^2), (m + 1) (2 m + 1) / (6 m^3)
+  float af;         // 1/m
 };
 __host__ __device__ inline RootSeries root_series(int m) {
   const double r = m > 0 ? 1.0 / m : 0.0;
-  return RootSeries{r, 0.5 * r * (1.0 + r), r * (1.0 + r) * (1.0 + 0.5 * r) / 3.0};
+  return RootSeries{r, 0.5 * r * (1.0 + r), r * (1.0 + r) * (1.0 + 0.5 * r) / 3.0, (float)r};
 }
 
 // Per-step scalars in the field type, pre-folded so each kernel multiplies instead of divides.
@@ -38,8 +39,8 @@ struct LeanCoef {
   T ebg;                        // background xy strain rate tau_bg / (2 mu0) (Eqs. 32-33)
   int bg_on;                    // tau_bg != 0: wall xy-edges carry the background stress
   // Picard update and coefficient refresh
-  T mu0, eta0, R_weak;
-  T rtau0_2;                    // 1 / tau0^2
+  T mu0, eta0, eta0_weak;       // eta0_weak = eta0 R_weak
+  T rtau0_2h, rtau0_2s;         // 1 / (2 tau0^2), 1 / (16 tau0^2)
   T rGdtS, dtaupt_fac, dtauv_fac;
   double tau0, n_pow, rel_mu, rel_eta;
   T rmu0;                       // 1 / mu0
@@ -132,7 +133,8 @@ void df64_convert(cudaStream_t st, const DfCopy& cp, int narrays, long long n, b
 // Element-wise application of one device math routine (pt_math_check; codes in porowave_pt.h).
 enum { MATH_RCP_PSEUDO = 0, MATH_RCP_FULL = 1, MATH_EXPM1_POS = 2, MATH_EXPM1_NEG = 3, MATH_DF_ADD = 4,
        MATH_DF_SUB = 5, MATH_DF_MUL = 6, MATH_DF_FMA = 7, MATH_DF_RCP = 8, MATH_DF_SQRT = 9,
-       MATH_DF_ROOT = 10, MATH_DF_EXPM1_POS = 11, MATH_DF_EXPM1_NEG = 12, MATH_COUNT = 13 };
+       MATH_DF_ROOT = 10, MATH_DF_EXPM1_POS = 11, MATH_DF_EXPM1_NEG = 12, MATH_TO_FLOAT = 13,
+       MATH_COUNT = 14 };
 void math_check(cudaStream_t st, int fn, const double* a, const double* b, double* out, long long n);
 
 }  // namespace pt

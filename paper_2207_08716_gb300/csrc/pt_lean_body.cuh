@@ -31,6 +31,19 @@ __device__ inline void expm1_pair(double d, double& em_pos, double& em_neg) {
   }
 }
 
+// The FP64 pipe takes a warp instruction every 16 cycles, in which an SM issues 64 others: conversions
+// between FP64 and FP32 and products with powers of two, which run on it, are done on the integers.
+__device__ inline double scale2(double x, int e) {   // x 2^e, x positive and far inside the normal range
+  return __hiloint2double(__double2hiint(x) + e * 0x100000, __double2loint(x));
+}
+// x to FP32, to nearest even as the conversion rounds; values outside FP32's normal range take that
+__device__ inline float to_float(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), a = hi & 0x7fffffffu;
+  if (a - 0x38100000u >= 0x47f00000u - 0x38100000u) return (float)x;
+  const unsigned t = __funnelshift_l(lo, a - 0x38000000u, 3);     // |x| >> 29, exponent rebased
+  return __uint_as_float((t + (((lo & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29)) | (hi & 0x80000000u));
+}
+
 // max of positive values through their bit patterns (monotone for x > 0)
 __device__ inline double pos_max(double a, double b) {
   const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
@@ -77,15 +90,19 @@ __device__ inline double sqrt_full(double x) {
 
 // x^(1/m) for 3 <= m <= 64 with rx = 1/x: from the FP32 root y (|t| <= 64 2^-20 for
 // t = (x - y^m) / x) by the series above; the first dropped term is below 2^-57. y^m by square and
-// multiply, m is uniform. For m = 10 13 FP64 instructions, where exp(log x / 10) takes some 45.
+// multiply, m is uniform. For m = 10 10 FP64 instructions, where exp(log x / 10) takes some 45.
 // x far from 1 (never near a solution) falls back to the library functions, a NaN stays one.
 __device__ inline double root_full(double x, double rx, int m, const RootSeries& k) {
   const int e2 = (__double2hiint(x) >> 20) - 1023;      // a negative x falls outside too
   if (e2 < -60 || e2 > 60) return exp(k.a * log(x));
   float lg, y0;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"((float)x));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(lg * (float)k.a));
-  const double y = (double)y0;
+  // the seed from x cut to 24 bits
+  const float xf = __uint_as_float(__funnelshift_l((unsigned)__double2loint(x),
+                                                   (unsigned)__double2hiint(x) - 0x38000000u, 3));
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(xf));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(lg * k.af));
+  const unsigned yb = __float_as_uint(y0);              // to FP64 exactly, normal in FP32
+  const double y = __hiloint2double((int)((yb >> 3) + 0x38000000u), (int)(yb << 29));
   int e = m;
   double b = y;
   while (!(e & 1)) {
@@ -309,8 +326,8 @@ __device__ __forceinline__ void lean_cell_level(const Box& b, const LeanCoef<dou
     // porosity in log space (Eq. 22): L = Lo + delta,
     // delta = -[beta_phi ((Pf1 - Pfo) - (Pt1 - Pto)) + dt (Pf1 - Pt1) / eta + dt V.grad(1-phi)/(1-phi)]
     // V.grad(1-phi)/(1-phi) = -(w/2) sum_d rd [v_r (phi_r - phi) + v_l (phi - phi_l)]
-    //                      = -w [sum_d hrd (v_r phi_r - v_l phi_l) - phi divV / 2]
-    const double adv = -w * fma(ph, -0.5 * divV, fma(ax, c.hrdx, fma(ay, c.hrdy, az * c.hrdz)));
+    //                      = -(w/2) [sum_d rd (v_r phi_r - v_l phi_l) - phi divV]
+    const double adv = -scale2(w, -1) * fma(ph, -divV, fma(ax, c.rdx, fma(ay, c.rdy, az * c.rdz)));
     const double dp1 = Pf1 - Pt1;
     const double rate = c.compaction_on ? fma(dp1, ieta, adv) : adv;
     const double delta = -fma(c.beta_phi, dp1 - (Pfo - Pto), c.dt * rate);
@@ -398,18 +415,18 @@ __device__ __forceinline__ void lean_picard_point(const Box& b, const LeanCoef<T
   if (i < b.nx && j < b.ny && k < b.nz) {
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
-    const T axy = T(0.25) * (in.txy[q] + in.txy[q + 1] + in.txy[q + px] + in.txy[q + 1 + px]);
-    const T axz = T(0.25) * (in.txz[q] + in.txz[q + 1] + in.txz[q + pxy] + in.txz[q + 1 + pxy]);
-    const T ayz = T(0.25) * (in.tyz[q] + in.tyz[q + px] + in.tyz[q + pxy] + in.tyz[q + px + pxy]);
+    const T axy = in.txy[q] + in.txy[q + 1] + in.txy[q + px] + in.txy[q + 1 + px];
+    const T axz = in.txz[q] + in.txz[q + 1] + in.txz[q + pxy] + in.txz[q + 1 + pxy];
+    const T ayz = in.tyz[q] + in.tyz[q + px] + in.tyz[q + pxy] + in.tyz[q + px + pxy];
     const T sxx = in.txx[q], syy = in.tyy[q], szz = in.tzz[q];
-    // tau_II^2 = (sxx^2 + syy^2 + szz^2) / 2 + axy^2 + axz^2 + ayz^2 (explicit FMAs: every form
-    // that inlines this body rounds it alike)
-    const T tII2 = fma(T(0.5), fma(sxx, sxx, fma(syy, syy, szz * szz)), fma(axy, axy, fma(axz, axz, ayz * ayz)));
+    // (tau_II / tau0)^2 = N / (2 tau0^2) + A / (16 tau0^2) with N = sxx^2 + syy^2 + szz^2 and A the sum of
+    // the squares of the edges' sums (explicit FMAs: every form that inlines this body rounds it alike)
+    const T N = fma(sxx, sxx, fma(syy, syy, szz * szz)), A = fma(axy, axy, fma(axz, axz, ayz * ayz));
     // Eq. 24: mu* = mu0 / (1 + (tau_II / tau0)^(n-1)); the log-space relaxation
     // exp(rel log mu* + (1 - rel) log mu) is written mu (mu* / mu)^rel (a square root for rel = 1/2)
     T den = T(1.0);
     if (c.powerlaw_on) {
-      const T x2 = tII2 * c.rtau0_2;                               // (tau_II / tau0)^2
+      const T x2 = fma(N, c.rtau0_2h, A * c.rtau0_2s);
       const double p = c.n_pow - 1.0;
       den = p == 2.0 ? T(1.0) + x2 : from_d<T>(1.0 + exp(0.5 * p * log(to_d(x2))));
     }
@@ -417,9 +434,9 @@ __device__ __forceinline__ void lean_picard_point(const Box& b, const LeanCoef<T
     const T D = den * mu_old;
     const T x_mu = c.mu0 * rcp_full(D), rx_mu = D * c.rmu0;          // mu* / mu and its inverse
     const T mu_new = mu_old * relax_pow(x_mu, rx_mu, c.rel_mu, c.root_mu, c.series_mu);
-    const T R = (in.Pf1[q] > in.Pt1[q]) ? c.R_weak : T(1.0);
+    const T eta0R = (in.Pf1[q] > in.Pt1[q]) ? c.eta0_weak : c.eta0;
     // Eq. 26: eta* = eta0 mu / phi R (with the relaxed mu), relaxed the same way
-    const T x_eta = c.eta0 * mu_new * R * rcp_full(in.phi1[q] * eta_old), rx_eta = rcp_full(x_eta);
+    const T x_eta = eta0R * mu_new * rcp_full(in.phi1[q] * eta_old), rx_eta = rcp_full(x_eta);
     m = to_d(abs_max(abs_max(x_mu, rx_mu), abs_max(x_eta, rx_eta)));
     if constexpr (LeanRecompute<T>::value) {
       if (!(x_mu == x_mu && x_eta == x_eta)) m = to_d(x_mu) + to_d(x_eta);   // NaN stays NaN
@@ -442,53 +459,49 @@ __device__ inline T lean_edge_mean_mu_xy(const Box& b, const T* mu, long long q,
   return s * T(n == 4 ? 0.25 : (n == 2 ? 0.5 : 1.0));
 }
 
-// Maxwell stress (Eq. 21) of viscosity m, xi = m rG: tau = tau_o a + M edot with a = xi / (1 + xi),
-// M = 2 m / (1 + xi); for an edge m is given as the sum of its four centres' mu.
-struct Maxwell {
-  double a, M;
-};
-__device__ __forceinline__ Maxwell maxwell(double m, double rG) {
-  const double s = lean_detail::rcp_full(fma(m, rG, 1.0));
-  return Maxwell{1.0 - s, 2.0 * m * s};
-}
-__device__ __forceinline__ Maxwell maxwell4(double sum, double rG) {
-  const double s = lean_detail::rcp_full(fma(sum, 0.25 * rG, 1.0));
-  return Maxwell{1.0 - s, 0.5 * sum * s};
+// Maxwell stress (Eq. 21) of viscosity m, xi = m rG: tau = (tau_o xi + 2 m edot) / (1 + xi), as
+// tau_o + s (2 m edot - tau_o) with s = 1 / (1 + xi).
+__device__ __forceinline__ double maxwell_s(double m, double rG) { return lean_detail::rcp_full(fma(m, rG, 1.0)); }
+__device__ __forceinline__ double maxwell(double s, double m2, double e, double to) {
+  return fma(s, fma(m2, e, -to), to);
 }
 
 // Shear stresses on the three lower edges of (i, j, k), zero on boundary edges unless a background
-// shear is applied (Eqs. 32-33).
+// shear is applied (Eqs. 32-33). An edge's viscosity is the mean of its four centres'.
 __device__ __forceinline__ void stress_edges_point(const Box& b, const LeanCoef<double>& c, const StressIn& in,
                                                    double* __restrict__ txy, double* __restrict__ txz,
                                                    double* __restrict__ tyz, int i, int j, int k) {
+  using lean_detail::scale2;
   if (i > b.nx || j > b.ny || k > b.nz) return;
   const long long q = cidx(b, i, j, k);
   const long long px = b.px, pxy = b.pxy;
   if (k < b.nz) {
     double t = 0.0;
     if (i > 0 && i < b.nx && j > 0 && j < b.ny) {
-      const Maxwell m = maxwell4((in.mu[q - 1 - px] + in.mu[q - px]) + (in.mu[q - 1] + in.mu[q]), c.rGdtS);
+      const double m4 = (in.mu[q - 1 - px] + in.mu[q - px]) + (in.mu[q - 1] + in.mu[q]);
       const double e = fma(in.Vx[q] - in.Vx[q - px], c.hrdy, fma(in.Vy[q] - in.Vy[q - 1], c.hrdx, c.ebg));
-      t = fma(in.txyo[q], m.a, m.M * e);
+      t = maxwell(maxwell_s(scale2(m4, -2), c.rGdtS), scale2(m4, -1), e, in.txyo[q]);
     } else if (c.bg_on) {   // wall edge: background part only
-      const Maxwell m = maxwell(lean_edge_mean_mu_xy(b, in.mu, q, i, j), c.rGdtS);
-      t = fma(in.txyo[q], m.a, m.M * c.ebg);
+      const double m = lean_edge_mean_mu_xy(b, in.mu, q, i, j);
+      t = maxwell(maxwell_s(m, c.rGdtS), scale2(m, 1), c.ebg, in.txyo[q]);
     }
     txy[q] = t;
   }
   if (j < b.ny) {
     double t = 0.0;
     if (i > 0 && i < b.nx && k > 0 && k < b.nz) {
-      const Maxwell m = maxwell4((in.mu[q - 1 - pxy] + in.mu[q - pxy]) + (in.mu[q - 1] + in.mu[q]), c.rGdtS);
-      t = fma(in.txzo[q], m.a, m.M * fma(in.Vx[q] - in.Vx[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - 1]) * c.hrdx));
+      const double m4 = (in.mu[q - 1 - pxy] + in.mu[q - pxy]) + (in.mu[q - 1] + in.mu[q]);
+      const double e = fma(in.Vx[q] - in.Vx[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - 1]) * c.hrdx);
+      t = maxwell(maxwell_s(scale2(m4, -2), c.rGdtS), scale2(m4, -1), e, in.txzo[q]);
     }
     txz[q] = t;
   }
   if (i < b.nx) {
     double t = 0.0;
     if (j > 0 && j < b.ny && k > 0 && k < b.nz) {
-      const Maxwell m = maxwell4((in.mu[q - px - pxy] + in.mu[q - pxy]) + (in.mu[q - px] + in.mu[q]), c.rGdtS);
-      t = fma(in.tyzo[q], m.a, m.M * fma(in.Vy[q] - in.Vy[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - px]) * c.hrdy));
+      const double m4 = (in.mu[q - px - pxy] + in.mu[q - pxy]) + (in.mu[q - px] + in.mu[q]);
+      const double e = fma(in.Vy[q] - in.Vy[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - px]) * c.hrdy);
+      t = maxwell(maxwell_s(scale2(m4, -2), c.rGdtS), scale2(m4, -1), e, in.tyzo[q]);
     }
     tyz[q] = t;
   }

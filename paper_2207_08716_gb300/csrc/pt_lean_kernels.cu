@@ -239,9 +239,8 @@ __global__ void __launch_bounds__(256) k_lean_stresses(Box b, LeanCoef<double> c
   stress_edges_point(b, c, in, out.txy, out.txz, out.tyz, i, j, k);
   if (i >= b.nx || j >= b.ny || k >= b.nz) return;
   const long long q = cidx(b, i, j, k);
-  const double gx = (in.Vx[q + 1] - in.Vx[q]) * c.rdx, gy = (in.Vy[q + b.px] - in.Vy[q]) * c.rdy;
-  const double gz = (in.Vz[q + b.pxy] - in.Vz[q]) * c.rdz;
-  const double divV = gx + gy + gz;
+  const double dvx = in.Vx[q + 1] - in.Vx[q], dvy = in.Vy[q + b.px] - in.Vy[q], dvz = in.Vz[q + b.pxy] - in.Vz[q];
+  const double divV = fma(dvx, c.rdx, fma(dvy, c.rdy, dvz * c.rdz));
   double s3 = divV * (-1.0 / 3.0);
   if (c.beta_n != 0.0) {
     const double Pt = ce.Pt[q], Pf = ce.Pf[q];
@@ -249,10 +248,10 @@ __global__ void __launch_bounds__(256) k_lean_stresses(Box b, LeanCoef<double> c
     const double divVn = fma(Pt - Pf, cc, fma(-c.bd_rdt_a, Pf - ce.Pfo[q], fma(c.bd_rdt, Pt - ce.Pto[q], divV)));
     s3 = fma(c.beta_n, divVn, s3);
   }
-  const Maxwell m = maxwell(in.mu[q], c.rGdtS);
-  out.txx[q] = fma(in.txxo[q], m.a, m.M * (gx + s3));
-  out.tyy[q] = fma(in.tyyo[q], m.a, m.M * (gy + s3));
-  out.tzz[q] = fma(in.tzzo[q], m.a, m.M * (gz + s3));
+  const double s = maxwell_s(in.mu[q], c.rGdtS), m2 = lean_detail::scale2(in.mu[q], 1);
+  out.txx[q] = maxwell(s, m2, fma(dvx, c.rdx, s3), in.txxo[q]);
+  out.tyy[q] = maxwell(s, m2, fma(dvy, c.rdy, s3), in.tyyo[q]);
+  out.tzz[q] = maxwell(s, m2, fma(dvz, c.rdz, s3), in.tzzo[q]);
 }
 void lean_stresses(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c, const StressIn& in,
                    const StressCentre& ce, const StressOut& out) {
@@ -359,6 +358,7 @@ __global__ void k_math_check(int fn, const double* __restrict__ a, const double*
       case MATH_DF_SQRT: r = (double)df_sqrt(df64(x)); break;
       case MATH_DF_ROOT: r = (double)df_root(df64(x), (int)y); break;
       case MATH_DF_EXPM1_POS: expm1_pair(df64(x), dp, dm); r = (double)dp; break;
+      case MATH_TO_FLOAT: r = (double)to_float(x); break;
       case MATH_DF_EXPM1_NEG: expm1_pair(df64(x), dp, dm); r = (double)dm; break;
       default: r = nan(""); break;
     }

@@ -25,8 +25,9 @@ namespace pt {
 // instruction count: coefficients folded on the host (LeanCoef), fused multiply-adds, third-order
 // reciprocals and no division, the porosity by expm1 of its small increment, norms through bit patterns.
 // At 255^3 an outer iteration's phases took 13.0 ms (141 FP64 instructions per cell in k_mix_prepare
-// alone, 137 in the Picard update, 67 at the edges); now 9.3 ms: 118 in k_mix_prepare with the edges, 86 in
-// k_mix_faces with the Picard update, 36 in k_mix_porosity, the pipe at 85 %.
+// alone, 137 in the Picard update, 67 at the edges); now 7.9 ms: 102 in k_mix_prepare with the edges, 81 in
+// k_mix_faces with the Picard update, 36 in k_mix_porosity, the pipe at 84 %. Conversions and products with
+// powers of two moved to the integer units, and fewer products, gave the last 1.2 ms.
 
 // k of the iterate (Eq. 23), read with its neighbours by mix_prepare_point.
 __device__ __forceinline__ void mix_perm_point(const Box& b, const LeanCoef<double>& c, const double* __restrict__ phi,
@@ -66,18 +67,18 @@ __device__ __forceinline__ void mix_prepare_point(const Box& b, const LeanCoef<d
     const double divqD = -fma(sx, c.hrdx2, fma(sy, c.hrdy2, sz * c.hrdz2));
     const double rpf = fma(-dpp, cc, fma(-c.bd_rdt_a, dPt, fma(c.bda_B_rdt, dPf, divqD)));
     // stresses at u (Eq. 21) for the momentum residual and the Picard update
-    const Maxwell m = maxwell(mu, c.rGdtS);
+    const double s = maxwell_s(mu, c.rGdtS), m2 = scale2(mu, 1);
     const double s3 = fma(c.beta_n, divVn, divV * (-1.0 / 3.0));
-    out.txx[q] = fma(in.s.txxo[q], m.a, m.M * fma(dvx, c.rdx, s3));
-    out.tyy[q] = fma(in.s.tyyo[q], m.a, m.M * fma(dvy, c.rdy, s3));
-    out.tzz[q] = fma(in.s.tzzo[q], m.a, m.M * fma(dvz, c.rdz, s3));
+    out.txx[q] = maxwell(s, m2, fma(dvx, c.rdx, s3), in.s.txxo[q]);
+    out.tyy[q] = maxwell(s, m2, fma(dvy, c.rdy, s3), in.s.tyyo[q]);
+    out.tzz[q] = maxwell(s, m2, fma(dvz, c.rdz, s3), in.s.tzzo[q]);
     // right-hand side and frozen coefficients of the correction problem (the iteration derives
     // 1/dtau_Pf from the largest neighbour k and the local-implicit denominators itself)
-    out.r_pt[q] = (float)divVn;
-    out.r_pf[q] = (float)rpf;
-    out.cc[q] = (float)cc;
-    out.perm[q] = (float)kc;
-    out.idtp[q] = (float)rcp_pseudo(c.dtaupt_fac * mu);   // good to 2^-39, kept in FP32
+    out.r_pt[q] = to_float(divVn);
+    out.r_pf[q] = to_float(rpf);
+    out.cc[q] = to_float(cc);
+    out.perm[q] = to_float(kc);
+    out.idtp[q] = to_float(rcp_pseudo(c.dtaupt_fac * mu));   // good to 2^-39, kept in FP32
     r_pt = divVn;
     r_pf = rpf;
   }
@@ -100,26 +101,26 @@ __device__ __forceinline__ void mix_faces_point(const Box& b, const LeanCoef<dou
   if (i > 0) {
     const double F = fma(txx - t.txx[q - 1], c.rdx,
                          fma(t.txy[q + px] - txy, c.rdy, fma(t.txz[q + pxy] - txz, c.rdz, -((Pt - t.Pt1[q - 1]) * c.rdx))));
-    out.rfx[q] = (float)F;
+    out.rfx[q] = to_float(F);
     r_v = F;
   }
   if (j > 0) {
     const double F = fma(t.txy[q + 1] - txy, c.rdx,
                          fma(tyy - t.tyy[q - px], c.rdy, fma(t.tyz[q + pxy] - tyz, c.rdz, -((Pt - t.Pt1[q - px]) * c.rdy))));
-    out.rfy[q] = (float)F;
+    out.rfy[q] = to_float(F);
     r_v = abs_max(r_v, F);
   }
   if (k > 0) {
     const double rog = (0.5 * (t.phi1[q - pxy] + t.phi1[q]) - c.phi0) * c.drho_g;
     const double F = fma(t.txz[q + 1] - txz, c.rdx, fma(t.tyz[q + px] - tyz, c.rdy,
                          fma(tzz - t.tzz[q - pxy], c.rdz, fma(-(Pt - t.Pt1[q - pxy]), c.rdz, -rog))));
-    out.rfz[q] = (float)F;
+    out.rfz[q] = to_float(F);
     r_v = abs_max(r_v, F);
   }
   lean_picard_point(b, c, t, in.mu, in.eta, i, j, k, pic);
   const double mu = in.mu[q];
-  out.mu[q] = (float)mu;
-  out.dtvc[q] = (float)(c.dtauv_fac * rcp_pseudo(mu));
+  out.mu[q] = to_float(mu);
+  out.dtvc[q] = to_float(c.dtauv_fac * rcp_pseudo(mu));
 }
 
 // phi^{k+1} = 1 - (1 - phi_o) exp(delta) at the corrected state, delta = -[beta_phi ((Pf1 - Pfo) -

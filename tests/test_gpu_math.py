@@ -140,3 +140,22 @@ def test_unknown_routine_is_rejected():
     a = torch.ones(4, dtype=torch.float64, device="cuda")
     assert lib.pt_math_check(99, a.data_ptr(), None, a.data_ptr(), 4, None) == N.PT_EINVAL
     assert lib.pt_math_check(DF_ADD, a.data_ptr(), None, a.data_ptr(), 4, None) == N.PT_EINVAL
+
+
+def test_to_float_is_the_conversion():
+    """FP64 to FP32 on the integers (routine 13): the same bits as the conversion, at ties, at the ends of
+    FP32's range and for what lies outside it."""
+    rng = np.random.default_rng(11)
+    x = _loguniform(rng, 1e-37, 1e38, 1 << 18, signed=True)
+    f = x[: 1 << 16].astype(np.float32)
+    up = np.nextafter(f, np.float32(np.inf))
+    tie = 0.5 * (f.astype(np.float64) + up.astype(np.float64))
+    ends = np.array([0.0, -0.0, 1.0, -1.0, 2.0 ** -126, 2.0 ** -127, 2.0 ** -149, 2.0 ** -151, 1e-320, 2.0 ** 128, -2.0 ** 128,
+                     2.0 ** 128 - 2.0 ** 103, 2.0 ** 128 - 2.0 ** 103 - 2.0 ** 75, 3.4028234663852886e38, 1e300, np.inf,
+                     -np.inf, np.nextafter(2.0 ** -126, 0.0)])
+    x = np.concatenate([x, tie, np.nextafter(tie, np.inf), np.nextafter(tie, -np.inf), f.astype(np.float64), ends])
+    with np.errstate(over="ignore", under="ignore"):
+        want = x.astype(np.float32)
+    got = _run(13, x).astype(np.float32)
+    assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
+    assert np.isnan(_run(13, np.array([np.nan]))).all()
