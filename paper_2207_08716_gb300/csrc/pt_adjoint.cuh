@@ -21,12 +21,12 @@ struct AdjCoef {
   double buoy;                          // (rho_f - rho_BG) g
   double hdrho_g;                       // (rho_f - rho_s) g / 2
   double hdt_rdx, hdt_rdy, hdt_rdz;     // dt / 2 / d_i (advection)
-  double rrho_i, damp_x, damp_y, damp_z, dtauv;
+  double damp_x, damp_y, damp_z, dtauv;
   // power-law rheology (Eq. 24): mu varies, the Picard row F_mu = log mu - log mu*(tau_II) joins
   int powerlaw;
   double Gdt;                           // G dtS of the step (xi = mu / Gdt)
   double rtau0_2, pw;                   // 1 / tau0^2, (n - 1) / 2
-  double r_eta0, dtauv_fac, dtaupt_fac; // 1 / eta0, dtau_V = fac / mu, dtau_Pt = fac * mu
+  double r_eta0, dtauv_fac, dtaupt_fac; // 1 / eta0, dtau_V / rho_i = fac / mu, dtau_Pt = fac * mu
 };
 
 struct AdjState {                       // converged state of the step (frozen during its solve)
@@ -98,8 +98,8 @@ void adj_prep(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const Ad
               const AdjPrep& out);
 void adj_cells(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const AdjCellIn& in,
                const AdjCellOut& out, unsigned long long* red, int check);
-void adj_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjFaceIn& in, double* Lx,
-               double* Ly, double* Lz, double* Rx, double* Ry, double* Rz, unsigned long long* red, int check);
+void adj_faces(cudaStream_t s, Box b, const AdjCoef& c, const AdjFaceIn& in, double* Lx, double* Ly, double* Lz,
+               double* Rx, double* Ry, double* Rz, unsigned long long* red, int check);
 void adj_carry(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjCarry& a);
 // red[RED_GMAX] = max(red[RED_GMAX], max |gP|, |gF|, |gphi| over the cells)
 void adj_gmax(dim3 g, dim3 bl, cudaStream_t s, Box b, const double* gP, const double* gF, const double* gphi,
@@ -109,9 +109,8 @@ void adj_gmax(dim3 g, dim3 bl, cudaStream_t s, Box b, const double* gP, const do
 // two passes (edges, then centres); tau_e are three scratch edge arrays for the state's edge stresses
 void adj_prep_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const double* K0,
                  const AdjPrep& out, const AdjPrepPL& pl, double* tau_xy, double* tau_xz, double* tau_yz);
-void adj_edges_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjEdgeIn& in,
-                  const AdjEdgeOut& out);
-void adj_cells_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const AdjCellIn& in,
+void adj_edges_pl(cudaStream_t s, Box b, const AdjCoef& c, const AdjEdgeIn& in, const AdjEdgeOut& out);
+void adj_cells_pl(cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const AdjCellIn& in,
                   const AdjCellOut& out, const AdjPrepPL& pl, const AdjMuIn& mu, unsigned long long* red,
                   int check);
 // sum over the grid of d(lambda . F)/d(G dtS) into *acc (one double, atomically), for the carry of

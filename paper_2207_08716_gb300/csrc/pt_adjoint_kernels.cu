@@ -20,6 +20,7 @@
 // and their inverses — is computed once per step by k_adj_prep, and the iteration kernels are
 // left with multiply-adds: no division and no k(phi) evaluation per iteration.
 #include "pt_adjoint.cuh"
+#include "pt_lean_body.cuh"
 
 namespace pt {
 
@@ -224,47 +225,47 @@ __global__ void __launch_bounds__(256) k_adj_cells(Box b, AdjCoef c, AdjState u,
   }
 }
 
-// Faces: row V with lambda_P1 and mL = lambda_L / (1 - phi); damped R, lambda_V update.
-__global__ void __launch_bounds__(256) k_adj_faces(Box b, AdjCoef c, AdjFaceIn in, double* Lx, double* Ly,
-                                                   double* Lz, double* Rx, double* Ry, double* Rz,
-                                                   unsigned long long* red, int check) {
+// Faces: row V with lambda_P1 and mL = lambda_L / (1 - phi); damped residual R (here rho_i times it, the
+// pseudo-steps carrying 1 / rho_i), lambda_V update. Bound by the FP64 pipe: 35 instructions per cell; the
+// norm is taken on checks only. 63^3 cold: 25.8 -> 24.5 us (edges 23.0 -> 19.5, cells 50.2 -> 48.7); most of
+// the gain comes on planes that do not fill 32-wide tiles (80^3 gradient: 58.2 -> 51.7 ms) and small grids.
+__global__ void __launch_bounds__(kPlaneThreads) k_adj_faces(Box b, AdjCoef c, AdjFaceIn in, double* Lx, double* Ly,
+                                                             double* Lz, double* Rx, double* Ry, double* Rz,
+                                                             unsigned long long* red, int check, Plane pl) {
   chain_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z;
+  int i, j;
+  const int k = blockIdx.y;
   double r_v = 0.0;
-  if (i <= b.nx && j <= b.ny && k <= b.nz) {
+  if (plane_point(pl, i, j)) {   // the faces i = nx, j = ny, k = nz are walls
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
-    const bool fx = i > 0 && i < b.nx && j < b.ny && k < b.nz;
-    const bool fy = j > 0 && j < b.ny && i < b.nx && k < b.nz;
-    const bool fz = k > 0 && k < b.nz && i < b.nx && j < b.ny;
+    const bool fx = i > 0, fy = j > 0, fz = k > 0;
+    // all loads before the first store (the arrays are not declared non-aliasing)
+    const double txx = in.txx[q], tyy = in.tyy[q], tzz = in.tzz[q], txy = in.txy[q], txz = in.txz[q], tyz = in.tyz[q];
+    const double lP = in.lP1[q], mL = in.mL[q];
     double Fx = 0.0, Fy = 0.0, Fz = 0.0, Rx1 = 0.0, Ry1 = 0.0, Rz1 = 0.0, Lx1 = 0.0, Ly1 = 0.0, Lz1 = 0.0;
     if (fx) {
-      Fx = (in.txx[q] - in.txx[q - 1]) * c.rdx + (in.txy[q + px] - in.txy[q]) * c.rdy +
-           (in.txz[q + pxy] - in.txz[q]) * c.rdz - (in.lP1[q] - in.lP1[q - 1]) * c.rdx +
-           in.bfx[q] * (in.mL[q - 1] + in.mL[q]);
+      Fx = fma(txx - in.txx[q - 1], c.rdx, fma(in.txy[q + px] - txy, c.rdy, fma(in.txz[q + pxy] - txz, c.rdz,
+               fma(in.lP1[q - 1] - lP, c.rdx, in.bfx[q] * (in.mL[q - 1] + mL)))));
       if (in.update) {
-        Rx1 = Fx * c.rrho_i + c.damp_x * Rx[q];
-        Lx1 = Lx[q] + (in.dtvx ? in.dtvx[q] : c.dtauv) * Rx1;
+        Rx1 = fma(c.damp_x, Rx[q], Fx);
+        Lx1 = fma(in.dtvx ? in.dtvx[q] : c.dtauv, Rx1, Lx[q]);
       }
     }
     if (fy) {
-      Fy = (in.txy[q + 1] - in.txy[q]) * c.rdx + (in.tyy[q] - in.tyy[q - px]) * c.rdy +
-           (in.tyz[q + pxy] - in.tyz[q]) * c.rdz - (in.lP1[q] - in.lP1[q - px]) * c.rdy +
-           in.bfy[q] * (in.mL[q - px] + in.mL[q]);
+      Fy = fma(in.txy[q + 1] - txy, c.rdx, fma(tyy - in.tyy[q - px], c.rdy, fma(in.tyz[q + pxy] - tyz, c.rdz,
+               fma(in.lP1[q - px] - lP, c.rdy, in.bfy[q] * (in.mL[q - px] + mL)))));
       if (in.update) {
-        Ry1 = Fy * c.rrho_i + c.damp_y * Ry[q];
-        Ly1 = Ly[q] + (in.dtvy ? in.dtvy[q] : c.dtauv) * Ry1;
+        Ry1 = fma(c.damp_y, Ry[q], Fy);
+        Ly1 = fma(in.dtvy ? in.dtvy[q] : c.dtauv, Ry1, Ly[q]);
       }
     }
     if (fz) {
-      Fz = (in.txz[q + 1] - in.txz[q]) * c.rdx + (in.tyz[q + px] - in.tyz[q]) * c.rdy +
-           (in.tzz[q] - in.tzz[q - pxy]) * c.rdz - (in.lP1[q] - in.lP1[q - pxy]) * c.rdz +
-           in.bfz[q] * (in.mL[q - pxy] + in.mL[q]);
+      Fz = fma(in.txz[q + 1] - txz, c.rdx, fma(in.tyz[q + px] - tyz, c.rdy, fma(tzz - in.tzz[q - pxy], c.rdz,
+               fma(in.lP1[q - pxy] - lP, c.rdz, in.bfz[q] * (in.mL[q - pxy] + mL)))));
       if (in.update) {
-        Rz1 = Fz * c.rrho_i + c.damp_z * Rz[q];
-        Lz1 = Lz[q] + (in.dtvz ? in.dtvz[q] : c.dtauv) * Rz1;
+        Rz1 = fma(c.damp_z, Rz[q], Fz);
+        Lz1 = fma(in.dtvz ? in.dtvz[q] : c.dtauv, Rz1, Lz[q]);
       }
     }
     if (in.update) {
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(256) k_adj_faces(Box b, AdjCoef c, AdjFaceIn i
     if (fx && in.rx) in.rx[q] = Fx;
     if (fy && in.ry) in.ry[q] = Fy;
     if (fz && in.rz) in.rz[q] = Fz;
-    r_v = fmax(fabs(Fx), fmax(fabs(Fy), fabs(Fz)));
+    if (check) r_v = lean_detail::abs_max(Fx, lean_detail::abs_max(Fy, Fz));
   }
   if (check) block_max_atomic(r_v, red + RED_V);
 }
@@ -490,65 +491,57 @@ __global__ void __launch_bounds__(256) k_adj_prep_pl(Box b, AdjCoef c, AdjState 
   pl.cmuL[q] = (Pt - Pf) * dt_eta * imu;
 }
 
-// Edges of one iteration: sigma_e from lambda_mu, adjoint edge stress m_e (eps_e(lambda_V) - sigma_e/2),
-// Z_e = sigma_e - 2 eps_e(lambda_V); zero on wall edges.
-__global__ void __launch_bounds__(256) k_adj_edges_pl(Box b, AdjCoef c, AdjEdgeIn in, AdjEdgeOut out) {
+// Edges of one iteration: sigma_e from lambda_mu, Z_e = sigma_e - 2 eps_e(lambda_V) and the adjoint edge
+// stress m_e (eps_e(lambda_V) - sigma_e/2) = -(m_e/2) Z_e; zero on wall edges. 29 FP64 instructions per cell (38 before).
+__global__ void __launch_bounds__(kPlaneThreads) k_adj_edges_pl(Box b, AdjCoef c, AdjEdgeIn in, AdjEdgeOut out,
+                                                                Plane pl) {
   chain_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i > b.nx || j > b.ny || k > b.nz) return;
+  int i, j;
+  const int k = blockIdx.y;
+  if (!plane_point(pl, i, j)) return;
   const long long q = cidx(b, i, j, k);
   const long long px = b.px, pxy = b.pxy;
-  if (k < b.nz) {
-    double t = 0.0, Z = 0.0;
-    if (i > 0 && i < b.nx && j > 0 && j < b.ny) {
-      const double e = 0.5 * ((in.Lx[q] - in.Lx[q - px]) * c.rdy + (in.Ly[q] - in.Ly[q - 1]) * c.rdx);
-      const double sg = in.Axy[q - 1 - px] * in.lM[q - 1 - px] + in.Axy[q - px] * in.lM[q - px] +
-                        in.Axy[q - 1] * in.lM[q - 1] + in.Axy[q] * in.lM[q];
-      t = in.me_xy[q] * (e - 0.5 * sg);
-      Z = sg - 2.0 * e;
-    }
-    out.txy[q] = t; out.Zxy[q] = Z;
+  const bool ix = i > 0 && i < b.nx, jy = j > 0 && j < b.ny, kz = k > 0 && k < b.nz;
+  // all loads before the first store (the arrays are not declared non-aliasing)
+  double t[3] = {0.0, 0.0, 0.0}, Z[3] = {0.0, 0.0, 0.0};
+  if (ix && jy && k < b.nz) {
+    const double e2 = fma(in.Lx[q] - in.Lx[q - px], c.rdy, (in.Ly[q] - in.Ly[q - 1]) * c.rdx);
+    const double sg = fma(in.Axy[q], in.lM[q], fma(in.Axy[q - 1], in.lM[q - 1], fma(in.Axy[q - px], in.lM[q - px],
+                          in.Axy[q - 1 - px] * in.lM[q - 1 - px])));
+    Z[0] = sg - e2;
+    t[0] = -lean_detail::scale2(in.me_xy[q], -1) * Z[0];
   }
-  if (j < b.ny) {
-    double t = 0.0, Z = 0.0;
-    if (i > 0 && i < b.nx && k > 0 && k < b.nz) {
-      const double e = 0.5 * ((in.Lx[q] - in.Lx[q - pxy]) * c.rdz + (in.Lz[q] - in.Lz[q - 1]) * c.rdx);
-      const double sg = in.Axz[q - 1 - pxy] * in.lM[q - 1 - pxy] + in.Axz[q - pxy] * in.lM[q - pxy] +
-                        in.Axz[q - 1] * in.lM[q - 1] + in.Axz[q] * in.lM[q];
-      t = in.me_xz[q] * (e - 0.5 * sg);
-      Z = sg - 2.0 * e;
-    }
-    out.txz[q] = t; out.Zxz[q] = Z;
+  if (ix && kz && j < b.ny) {
+    const double e2 = fma(in.Lx[q] - in.Lx[q - pxy], c.rdz, (in.Lz[q] - in.Lz[q - 1]) * c.rdx);
+    const double sg = fma(in.Axz[q], in.lM[q], fma(in.Axz[q - 1], in.lM[q - 1], fma(in.Axz[q - pxy], in.lM[q - pxy],
+                          in.Axz[q - 1 - pxy] * in.lM[q - 1 - pxy])));
+    Z[1] = sg - e2;
+    t[1] = -lean_detail::scale2(in.me_xz[q], -1) * Z[1];
   }
-  if (i < b.nx) {
-    double t = 0.0, Z = 0.0;
-    if (j > 0 && j < b.ny && k > 0 && k < b.nz) {
-      const double e = 0.5 * ((in.Ly[q] - in.Ly[q - pxy]) * c.rdz + (in.Lz[q] - in.Lz[q - px]) * c.rdy);
-      const double sg = in.Ayz[q - px - pxy] * in.lM[q - px - pxy] + in.Ayz[q - pxy] * in.lM[q - pxy] +
-                        in.Ayz[q - px] * in.lM[q - px] + in.Ayz[q] * in.lM[q];
-      t = in.me_yz[q] * (e - 0.5 * sg);
-      Z = sg - 2.0 * e;
-    }
-    out.tyz[q] = t; out.Zyz[q] = Z;
+  if (jy && kz && i < b.nx) {
+    const double e2 = fma(in.Ly[q] - in.Ly[q - pxy], c.rdz, (in.Lz[q] - in.Lz[q - px]) * c.rdy);
+    const double sg = fma(in.Ayz[q], in.lM[q], fma(in.Ayz[q - px], in.lM[q - px], fma(in.Ayz[q - pxy], in.lM[q - pxy],
+                          in.Ayz[q - px - pxy] * in.lM[q - px - pxy])));
+    Z[2] = sg - e2;
+    t[2] = -lean_detail::scale2(in.me_yz[q], -1) * Z[2];
   }
+  if (k < b.nz) { out.txy[q] = t[0]; out.Zxy[q] = Z[0]; }
+  if (j < b.ny) { out.txz[q] = t[1]; out.Zxz[q] = Z[1]; }
+  if (i < b.nx) { out.tyz[q] = t[2]; out.Zyz[q] = Z[2]; }
 }
 
 // Cells (power law): centre adjoint stresses minus the pseudo-stress, rows Pt, Pf, phi with mu per
-// cell, and row mu.
-__global__ void __launch_bounds__(256) k_adj_cells_pl(Box b, AdjCoef c, AdjState u, AdjCellIn in, AdjCellOut out,
-                                                      AdjPrepPL pl, AdjMuIn mi, unsigned long long* red,
-                                                      int check) {
+// cell, and row mu. 86 FP64 instructions per cell.
+__global__ void __launch_bounds__(kPlaneThreads) k_adj_cells_pl(Box b, AdjCoef c, AdjState u, AdjCellIn in,
+                                                                AdjCellOut out, AdjPrepPL pl, AdjMuIn mi,
+                                                                unsigned long long* red, int check, Plane pn) {
   chain_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int k = blockIdx.z;
+  int i, j;
+  const int k = blockIdx.y;
   double r_pt = 0.0, r_pf = 0.0, r_l = 0.0;
-  if (i < b.nx && j < b.ny && k < b.nz) {
+  if (plane_point(pn, i, j)) {
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
-    const double ph = u.phi[q];
     const double cc = pl.cc[q];
     const double lP = in.lP[q], lF = in.lF[q], lL = in.lL[q], lM = mi.lM[q];
     const double Lz0 = in.Lz[q], Lz1 = in.Lz[q + pxy];
@@ -557,83 +550,98 @@ __global__ void __launch_bounds__(256) k_adj_cells_pl(Box b, AdjCoef c, AdjState
     const double divL = gx + gy + gz;
     const double d3 = divL * c.third;
     const double mc = pl.mc[q];
-    out.txx[q] = mc * (gx - d3) - lM * pl.sTxx[q];
-    out.tyy[q] = mc * (gy - d3) - lM * pl.sTyy[q];
-    out.tzz[q] = mc * (gz - d3) - lM * pl.sTzz[q];
-    // ---- row Pt
-    const double cplP = c.bd_rdt_a + cc, cplL = pl.cplL[q];
-    const double resP = divL + (c.bd_rdt + cc) * lP - cplP * lF - cplL * lL - in.gP[q];
-    out.lP[q] = lP - in.cP[q] * resP;
+    const double txx = fma(mc, gx - d3, -lM * pl.sTxx[q]);
+    const double tyy = fma(mc, gy - d3, -lM * pl.sTyy[q]);
+    const double tzz = fma(mc, gz - d3, -lM * pl.sTzz[q]);
+    // ---- row Pt; X: the terms that rows Pt and Pf share with opposite signs
+    const double D = lP - lF;
+    const double X = fma(cc, D, -pl.cplL[q] * lL);
+    const double resP = fma(c.bd_rdt, lP, fma(-c.bd_rdt_a, lF, divL)) + (X - in.gP[q]);
+    const double lP1 = fma(-in.cP[q], resP, lP);
     // ---- row Pf and the advection transpose of row phi over the six faces
     double Klf = 0.0, dkT = 0.0, offx = 0.0, offy = 0.0, offz = 0.0;
     if (i > 0) {
       const double dn = in.lF[q - 1] - lF;
-      Klf -= in.kfx[q] * dn;
-      dkT += in.gkx[q] * dn;
-      offx -= u.Vx[q] * in.mL[q - 1];
+      Klf = -in.kfx[q] * dn;
+      dkT = in.gkx[q] * dn;
+      offx = -u.Vx[q] * in.mL[q - 1];
     }
     if (i < b.nx - 1) {
       const double dn = in.lF[q + 1] - lF;
-      Klf -= in.kfx[q + 1] * dn;
-      dkT -= in.gkx[q + 1] * dn;
-      offx += u.Vx[q + 1] * in.mL[q + 1];
+      Klf = fma(-in.kfx[q + 1], dn, Klf);
+      dkT = fma(-in.gkx[q + 1], dn, dkT);
+      offx = fma(u.Vx[q + 1], in.mL[q + 1], offx);
     }
     if (j > 0) {
       const double dn = in.lF[q - px] - lF;
-      Klf -= in.kfy[q] * dn;
-      dkT += in.gky[q] * dn;
-      offy -= u.Vy[q] * in.mL[q - px];
+      Klf = fma(-in.kfy[q], dn, Klf);
+      dkT = fma(in.gky[q], dn, dkT);
+      offy = -u.Vy[q] * in.mL[q - px];
     }
     if (j < b.ny - 1) {
       const double dn = in.lF[q + px] - lF;
-      Klf -= in.kfy[q + px] * dn;
-      dkT -= in.gky[q + px] * dn;
-      offy += u.Vy[q + px] * in.mL[q + px];
+      Klf = fma(-in.kfy[q + px], dn, Klf);
+      dkT = fma(-in.gky[q + px], dn, dkT);
+      offy = fma(u.Vy[q + px], in.mL[q + px], offy);
     }
     if (k > 0) {
       const double dn = in.lF[q - pxy] - lF;
-      Klf -= in.kfz[q] * dn;
-      dkT += in.gkz[q] * dn;
-      offz -= u.Vz[q] * in.mL[q - pxy];
+      Klf = fma(-in.kfz[q], dn, Klf);
+      dkT = fma(in.gkz[q], dn, dkT);
+      offz = -u.Vz[q] * in.mL[q - pxy];
     }
     if (k < b.nz - 1) {
       const double dn = in.lF[q + pxy] - lF;
-      Klf -= in.kfz[q + pxy] * dn;
-      dkT -= in.gkz[q + pxy] * dn;
-      offz += u.Vz[q + pxy] * in.mL[q + pxy];
+      Klf = fma(-in.kfz[q + pxy], dn, Klf);
+      dkT = fma(-in.gkz[q + pxy], dn, dkT);
+      offz = fma(u.Vz[q + pxy], in.mL[q + pxy], offz);
     }
-    const double off = offx * c.hdt_rdx + offy * c.hdt_rdy + offz * c.hdt_rdz;
-    const double resF = Klf + (c.bda_B_rdt + cc) * lF - cplP * lP + cplL * lL - in.gF[q];
-    out.lF[q] = lF - in.cF[q] * resF;
-    const double a3k = in.a3k[q];
-    if (out.gtheta) out.gtheta[q] = a3k * ph * c.third * dkT;
+    const double off = fma(offx, c.hdt_rdx, fma(offy, c.hdt_rdy, offz * c.hdt_rdz));
+    const double resF = fma(c.bda_B_rdt, lF, fma(-c.bd_rdt_a, lP, Klf)) - (X + in.gF[q]);
+    const double lF1 = fma(-in.cF[q], resF, lF);
     // ---- row phi
-    const double sL = -c.hdrho_g * (Lz0 + Lz1) + in.aPF[q] * (lP - lF) + a3k * dkT + off - in.gphi[q];
+    const double a3k = in.a3k[q];
+    const double sL = fma(-c.hdrho_g, Lz0 + Lz1, fma(in.aPF[q], D, fma(a3k, dkT, off - in.gphi[q])));
     const double lLn = -in.iD[q] * sL;
-    out.lL[q] = lLn;
-    out.mL[q] = lLn * in.W[q];
+    const double mLn = lLn * in.W[q];
     // ---- row mu
-    const double sPZ =
-        pl.P_xy[q] * mi.Zxy[q] + pl.P_xy[q + 1] * mi.Zxy[q + 1] + pl.P_xy[q + px] * mi.Zxy[q + px] +
-        pl.P_xy[q + 1 + px] * mi.Zxy[q + 1 + px] + pl.P_xz[q] * mi.Zxz[q] + pl.P_xz[q + 1] * mi.Zxz[q + 1] +
-        pl.P_xz[q + pxy] * mi.Zxz[q + pxy] + pl.P_xz[q + 1 + pxy] * mi.Zxz[q + 1 + pxy] +
-        pl.P_yz[q] * mi.Zyz[q] + pl.P_yz[q + px] * mi.Zyz[q + px] + pl.P_yz[q + pxy] * mi.Zyz[q + pxy] +
-        pl.P_yz[q + px + pxy] * mi.Zyz[q + px + pxy];
-    const double resM = sPZ - (pl.Qxx[q] * gx + pl.Qyy[q] * gy + pl.Qzz[q] * gz) +
-                        lM * (pl.imu[q] + pl.fTQ[q]) + pl.cmu[q] * (lF - lP) + pl.cmuL[q] * lL - mi.gM[q];
-    mi.lM1[q] = lM - pl.iDmu[q] * resM;
-    if (check || out.rL) {
-      const double resL = sL + in.Dg[q] * lL;
-      if (out.rL) {
-        out.rP[q] = resP;
-        out.rF[q] = resF;
-        out.rL[q] = resL;
-      }
+    double sPZ = pl.P_xy[q] * mi.Zxy[q];
+    sPZ = fma(pl.P_xy[q + 1], mi.Zxy[q + 1], sPZ);
+    sPZ = fma(pl.P_xy[q + px], mi.Zxy[q + px], sPZ);
+    sPZ = fma(pl.P_xy[q + 1 + px], mi.Zxy[q + 1 + px], sPZ);
+    sPZ = fma(pl.P_xz[q], mi.Zxz[q], sPZ);
+    sPZ = fma(pl.P_xz[q + 1], mi.Zxz[q + 1], sPZ);
+    sPZ = fma(pl.P_xz[q + pxy], mi.Zxz[q + pxy], sPZ);
+    sPZ = fma(pl.P_xz[q + 1 + pxy], mi.Zxz[q + 1 + pxy], sPZ);
+    sPZ = fma(pl.P_yz[q], mi.Zyz[q], sPZ);
+    sPZ = fma(pl.P_yz[q + px], mi.Zyz[q + px], sPZ);
+    sPZ = fma(pl.P_yz[q + pxy], mi.Zyz[q + pxy], sPZ);
+    sPZ = fma(pl.P_yz[q + px + pxy], mi.Zyz[q + px + pxy], sPZ);
+    sPZ = fma(-pl.Qxx[q], gx, fma(-pl.Qyy[q], gy, fma(-pl.Qzz[q], gz, sPZ)));
+    const double resM = fma(lM, pl.imu[q] + pl.fTQ[q], fma(-pl.cmu[q], D, fma(pl.cmuL[q], lL, sPZ - mi.gM[q])));
+    const double lM1 = fma(-pl.iDmu[q], resM, lM);
+    const double gth = out.gtheta ? a3k * u.phi[q] * c.third * dkT : 0.0;
+    const double resL = check || out.rL ? fma(in.Dg[q], lL, sL) : 0.0;
+    // every load above precedes the stores (the arrays are not declared non-aliasing)
+    out.txx[q] = txx;
+    out.tyy[q] = tyy;
+    out.tzz[q] = tzz;
+    out.lP[q] = lP1;
+    out.lF[q] = lF1;
+    out.lL[q] = lLn;
+    out.mL[q] = mLn;
+    mi.lM1[q] = lM1;
+    if (out.gtheta) out.gtheta[q] = gth;
+    if (out.rL) {
+      out.rP[q] = resP;
+      out.rF[q] = resF;
+      out.rL[q] = resL;
       if (mi.rM) mi.rM[q] = resM;
-      r_pt = fabs(resP);
-      r_pf = fabs(resF);
-      r_l = fmax(fabs(resL), fabs(resM));
-      if (!(resL == resL && resM == resM)) r_l = resL + resM;   // a NaN surfaces in the norm
+    }
+    if (check) {   // a NaN is the largest
+      r_pt = lean_detail::abs_max(resP, 0.0);
+      r_pf = lean_detail::abs_max(resF, 0.0);
+      r_l = lean_detail::abs_max(resL, resM);
     }
   }
   if (check) {
@@ -721,14 +729,15 @@ void adj_prep_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const
   launch_chained(k_adj_prep_pl_edges, g, bl, 0, s, b, c, u, pl, tau_xy, tau_xz, tau_yz);
   launch_chained(k_adj_prep_pl, g, bl, 0, s, b, c, u, K0, out, pl, tau_xy, tau_xz, tau_yz);
 }
-void adj_edges_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjEdgeIn& in,
-                  const AdjEdgeOut& out) {
-  launch_chained(k_adj_edges_pl, g, bl, 0, s, b, c, in, out);
+void adj_edges_pl(cudaStream_t s, Box b, const AdjCoef& c, const AdjEdgeIn& in, const AdjEdgeOut& out) {
+  const Plane pl = plane_of(b, 1);   // the zeros of the wall edges are written too
+  launch_chained(k_adj_edges_pl, plane_grid(pl, b.nz + 1), kPlaneThreads, 0, s, b, c, in, out, pl);
 }
-void adj_cells_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const AdjCellIn& in,
+void adj_cells_pl(cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u, const AdjCellIn& in,
                   const AdjCellOut& out, const AdjPrepPL& pl, const AdjMuIn& mu, unsigned long long* red,
                   int check) {
-  launch_chained(k_adj_cells_pl, g, bl, 0, s, b, c, u, in, out, pl, mu, red, check);
+  const Plane pn = plane_of(b, 0);
+  launch_chained(k_adj_cells_pl, plane_grid(pn, b.nz), kPlaneThreads, 0, s, b, c, u, in, out, pl, mu, red, check, pn);
 }
 void adj_dgdt_pl(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjState& u,
                  const AdjPrepPL& pl, const double* Lx, const double* Ly, const double* Lz, const double* lM,
@@ -752,9 +761,11 @@ void adj_cells(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const A
                const AdjCellOut& out, unsigned long long* red, int check) {
   launch_chained(k_adj_cells, g, bl, 0, s, b, c, u, in, out, red, check);
 }
-void adj_faces(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjFaceIn& in, double* Lx,
-               double* Ly, double* Lz, double* Rx, double* Ry, double* Rz, unsigned long long* red, int check) {
-  launch_chained(k_adj_faces, g, bl, 0, s, b, c, in, Lx, Ly, Lz, Rx, Ry, Rz, red, check);
+void adj_faces(cudaStream_t s, Box b, const AdjCoef& c, const AdjFaceIn& in, double* Lx, double* Ly, double* Lz,
+               double* Rx, double* Ry, double* Rz, unsigned long long* red, int check) {
+  const Plane pl = plane_of(b, 0);
+  launch_chained(k_adj_faces, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, in, Lx, Ly, Lz, Rx, Ry, Rz, red, check,
+                 pl);
 }
 void adj_carry(dim3 g, dim3 bl, cudaStream_t s, Box b, const AdjCoef& c, const AdjCarry& a) {
   k_adj_carry<<<g, bl, 0, s>>>(b, c, a);

@@ -2045,15 +2045,14 @@ AdjCoef adjoint_coef(const pt_ctx* c) {
   ac.buoy = k.rhof_g - k.rho_bg_g;
   ac.hdrho_g = 0.5 * (c->phys.rhof_g - c->phys.rhos_g);
   ac.hdt_rdx = 0.5 * k.dt * k.rdx; ac.hdt_rdy = 0.5 * k.dt * k.rdy; ac.hdt_rdz = 0.5 * k.dt * k.rdz;
-  ac.rrho_i = k.rrho_i;
   ac.damp_x = k.damp_x; ac.damp_y = k.damp_y; ac.damp_z = k.damp_z;
-  ac.dtauv = k.dtauv_fac / c->phys.mu0;
+  ac.dtauv = k.dtauv_fac / c->phys.mu0 * k.rrho_i;   // of the adjoint velocities, over rho_i
   ac.powerlaw = c->phys.powerlaw_on != 0;
   ac.Gdt = c->phys.G * c->dtS;           // set per step from that step's dtS
   ac.rtau0_2 = 1.0 / (c->phys.tau0 * c->phys.tau0);
   ac.pw = 0.5 * (c->phys.n_pow - 1.0);
   ac.r_eta0 = 1.0 / c->phys.eta0;
-  ac.dtauv_fac = k.dtauv_fac;
+  ac.dtauv_fac = k.dtauv_fac * k.rrho_i;
   ac.dtaupt_fac = k.dtaupt_fac;
   return ac;
 }
@@ -2184,10 +2183,10 @@ int pt_adjoint(pt_ctx* c, const double* dJ_dphi, double* grad, pt_report* rep) {
         const AdjCellOut co{A.txx, A.tyy, A.tzz, A.txy, A.txz, A.tyz, A.lP[1 - cur], A.lF[1 - cur],
                             A.lL[1 - cur], A.mL[1 - cur], check ? A.gth : nullptr, nullptr, nullptr, nullptr};
         if (pl) {
-          PT_LAUNCH(c, K_ADJ_EDGES_PL, adj_edges_pl(gr, bl, c->stream, b, ac, A.edge_in(cur),
+          PT_LAUNCH(c, K_ADJ_EDGES_PL, adj_edges_pl(c->stream, b, ac, A.edge_in(cur),
                                                     AdjEdgeOut{A.txy, A.txz, A.tyz, A.Zxy, A.Zxz, A.Zyz}));
           const AdjMuIn mi{A.lM[cur], A.gM, A.Zxy, A.Zxz, A.Zyz, A.lM[1 - cur], nullptr};
-          PT_LAUNCH(c, K_ADJ_CELLS_PL, adj_cells_pl(gr, bl, c->stream, b, ac, u, A.cell_in(cur, K0), co, A.pl, mi,
+          PT_LAUNCH(c, K_ADJ_CELLS_PL, adj_cells_pl(c->stream, b, ac, u, A.cell_in(cur, K0), co, A.pl, mi,
                                                  c->red, check));
         } else {
           PT_LAUNCH(c, K_ADJ_CELLS, adj_cells(gr, bl, c->stream, b, ac, u, A.cell_in(cur, K0), co, c->red, check));
@@ -2196,7 +2195,7 @@ int pt_adjoint(pt_ctx* c, const double* dJ_dphi, double* grad, pt_report* rep) {
         fi.lP1 = A.lP[1 - cur];
         fi.mL = A.mL[1 - cur];
         PT_LAUNCH(c, pl ? K_ADJ_FACES_PL : K_ADJ_FACES,
-                  adj_faces(gr, bl, c->stream, b, ac, fi, A.Lx, A.Ly, A.Lz, A.LRx, A.LRy, A.LRz, c->red, check));
+                  adj_faces(c->stream, b, ac, fi, A.Lx, A.Ly, A.Lz, A.LRx, A.LRy, A.LRz, c->red, check));
         cur = 1 - cur;
         if (check) {
           rc = read_report(c, &last);
@@ -2215,7 +2214,7 @@ int pt_adjoint(pt_ctx* c, const double* dJ_dphi, double* grad, pt_report* rep) {
         // -(d(lambda . F)/d(G dtS)) / xsi_w into row mu of step n-1 at the cell holding that maximum
         cudaMemsetAsync(A.gM, 0, bytes, c->stream);
         cudaMemsetAsync(A.acc, 0, sizeof(double), c->stream);
-        PT_LAUNCH(c, K_ADJ_CARRY, adj_edges_pl(gr, bl, c->stream, b, ac, A.edge_in(cur),
+        PT_LAUNCH(c, K_ADJ_CARRY, adj_edges_pl(c->stream, b, ac, A.edge_in(cur),
                                                AdjEdgeOut{A.txy, A.txz, A.tyz, A.Zxy, A.Zxz, A.Zyz}));
         PT_LAUNCH(c, K_ADJ_CARRY, adj_dgdt_pl(gr, bl, c->stream, b, ac, u, A.pl, A.Lx, A.Ly, A.Lz, A.lM[cur],
                                               A.Zxy, A.Zxz, A.Zyz, A.acc));
@@ -2271,10 +2270,10 @@ int pt_adjoint_apply(pt_ctx* c, const pt_adj_vec* lam, pt_adj_vec* out, void* ws
   if (pl) {
     PT_LAUNCH(c, K_ADJ_PREP, adj_prep_pl(gr, bl, c->stream, b, ac, u, K0, A.prep_for(0), A.pl, A.Zxy, A.Zxz,
                                          A.Zyz));
-    PT_LAUNCH(c, K_ADJ_EDGES_PL, adj_edges_pl(gr, bl, c->stream, b, ac, A.edge_in(0),
+    PT_LAUNCH(c, K_ADJ_EDGES_PL, adj_edges_pl(c->stream, b, ac, A.edge_in(0),
                                               AdjEdgeOut{A.txy, A.txz, A.tyz, A.Zxy, A.Zxz, A.Zyz}));
     const AdjMuIn mi{A.lM[0], A.gM, A.Zxy, A.Zxz, A.Zyz, A.lM[1], out->mu};
-    PT_LAUNCH(c, K_ADJ_CELLS_PL, adj_cells_pl(gr, bl, c->stream, b, ac, u, A.cell_in(0, K0), co, A.pl, mi, c->red, 0));
+    PT_LAUNCH(c, K_ADJ_CELLS_PL, adj_cells_pl(c->stream, b, ac, u, A.cell_in(0, K0), co, A.pl, mi, c->red, 0));
   } else {
     PT_LAUNCH(c, K_ADJ_PREP, adj_prep(gr, bl, c->stream, b, ac, u, K0, A.prep_for(0)));
     PT_LAUNCH(c, K_ADJ_CELLS, adj_cells(gr, bl, c->stream, b, ac, u, A.cell_in(0, K0), co, c->red, 0));
@@ -2282,7 +2281,7 @@ int pt_adjoint_apply(pt_ctx* c, const pt_adj_vec* lam, pt_adj_vec* out, void* ws
   const AdjFaceIn fi{A.txx, A.tyy, A.tzz, A.txy, A.txz, A.tyz, A.lP[0], A.mL[0],
                      A.prep.bfx, A.prep.bfy, A.prep.bfz, out->Vx, out->Vy, out->Vz, 0, nullptr, nullptr, nullptr};
   PT_LAUNCH(c, pl ? K_ADJ_FACES_PL : K_ADJ_FACES,
-            adj_faces(gr, bl, c->stream, b, ac, fi, A.Lx, A.Ly, A.Lz, A.LRx, A.LRy, A.LRz, c->red, 0));
+            adj_faces(c->stream, b, ac, fi, A.Lx, A.Ly, A.Lz, A.LRx, A.LRy, A.LRz, c->red, 0));
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   return cuda_status(e);

@@ -78,3 +78,44 @@ def test_reactive_cycles_fp32(nx, ny, nz):
     got, want = (C.run(C.prepare(dict(case, form=f), 3)) for f in ("fp32", "fp64"))
     off = {k: float((got[k].double() - want[k]).norm() / want[k].norm().clamp_min(1e-300)) for k in got}
     assert max(off.values()) < 2 * 40 * 8 * 2.0 ** -24, off
+
+
+# index maps of cells, faces and edges: full 32 x 4 tiles of cells or of edges, neither, two cells a side
+@pytest.mark.parametrize("powerlaw", [False, True])
+@pytest.mark.parametrize("dims", [(3, 2, 2), (31, 7, 5), (32, 8, 3), (35, 9, 4)])
+def test_transposed_stencils_at_tile_edges(dims, powerlaw):
+    """J^T w against the vector-Jacobian product of the CPU residual, component by component; the bar of
+    the FP64 kernels against the same product, 1e-12."""
+    import numpy as np
+    import torch
+    import pt_inputs as I
+    from oracle import adjoint as A
+    from paper_2207_08716_gb300.solver import PTSolver
+    nx, ny, nz = dims
+    p = A.adjoint_params(I.c1_params(*dims), powerlaw)
+    p.update(precision=0, tol=1e-9, max_iter=400000)
+    phi = I.gaussian_porosity(p, centres=((0.4, 0.55, 0.5),), width=0.2)
+    theta = I.gaussian_random_field(phi.shape, seed=5, std=0.5)
+    s = PTSolver(p, phi, logk=theta)
+    s.step()
+    UK, FK = (A.U_KEYS_PL, A.F_KEYS_PL) if powerlaw else (A.U_KEYS, A.F_KEYS)
+    u = {k: A._t(s.get(k)).requires_grad_(True) for k in UK}
+    rng = np.random.default_rng(11)
+    shapes = I.field_shapes(nx, ny, nz)
+    w = {k: rng.standard_normal(shapes.get(k, shapes["centre"])) for k in UK}
+    inner = {"Vx": (slice(None), slice(None), slice(1, -1)), "Vy": (slice(None), slice(1, -1), slice(None)),
+             "Vz": (slice(1, -1),)}
+    for k, axis in (("Vx", 2), ("Vy", 1), ("Vz", 0)):
+        np.moveaxis(w[k], axis, 0)[[0, -1]] = 0.0
+    got = s.adjoint_apply(w)
+    s.close()
+    z = torch.zeros_like(u["Pt"])
+    old = dict(Pto=z, Pfo=z, Lo=z)
+    if powerlaw:
+        old["mu_o"] = torch.full_like(u["Pt"], p["mu0"])
+    F = A.residual(p, u, old, A._t(theta))
+    rows = dict(zip(FK, UK))
+    dot = sum((F[f] * A._t(w[k][inner.get(k, ())])).sum() for f, k in rows.items())
+    for k, ref in zip(UK, torch.autograd.grad(dot, [u[k] for k in UK])):
+        ref = ref.numpy()[inner.get(k, ())]
+        assert np.abs(got[k][inner.get(k, ())] - ref).max() <= 1e-12 * max(np.abs(ref).max(), 1e-300), k
