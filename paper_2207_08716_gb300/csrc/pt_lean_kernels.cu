@@ -30,10 +30,10 @@
 namespace pt {
 
 // ------------------------------------------------------------------------------ cells
-// A thread takes a chunk of levels of its column (lean_cell_level's carried values). 95.2 FP64 instructions
+// A thread takes a chunk of levels of its column (lean_cell_level's carried values). 94.5 FP64 instructions
 // per cell at 191^3 (100.1 before the carried flux, the folded spacings and the shared difference of the
 // new pressures), 1.22 ms a launch against 1.31; the pipe runs at 86 % either way.
-constexpr int kLeanCellChunk = 8, kLeanCellBlocks = 5;
+constexpr int kLeanCellBlocks = 5;
 __global__ void __launch_bounds__(kPlaneThreads, kLeanCellBlocks) k_lean_cells(Box b, LeanCoef<double> c,
                                                                                LeanCellIn<double> in,
                                                                                LeanCellOut<double> out,
@@ -378,8 +378,12 @@ void lean_cells<double>(cudaStream_t st, Box b, const LeanCoef<double>& c, const
                         const LeanCellOut<double>& out, unsigned long long* red, int check) {
   const Plane pl = plane_of(b, c.bg_on ? 1 : 0);
   const dim3 g = plane_grid(pl, 1);
-  // the pipe is shared by an SM's blocks: a level takes as long as there are blocks on the SM
-  const int zc = march_chunk(g.x, b.nz, kLeanCellChunk, kLeanCellBlocks, sm_count(), 0.15, 0.3);
+  // the pipe is shared by an SM's blocks: a level takes as long as there are blocks on the SM. Up to some 30
+  // waves of blocks even SMs count more than the carried level: chunks of 1 or 2 measured 5-7 % faster at
+  // 63^3-80 x 90 x 100 and 1-3 % at 96^3 and 127^3 than up to 8, which are 0.5 % faster from 160^3 on
+  const bool large = (long long)g.x * b.nz > 30LL * kLeanCellBlocks * sm_count();
+  const int zc = large ? march_chunk(g.x, b.nz, 8, kLeanCellBlocks, sm_count(), 0.15, 0.3)
+                       : march_chunk(g.x, b.nz, 2, kLeanCellBlocks, sm_count(), 0.05, 0.6);
   launch_chained(k_lean_cells, dim3(g.x, (unsigned)((b.nz + zc - 1) / zc)), kPlaneThreads, 0, st, b, c, in, out, red,
                  check, pl, zc);
 }
