@@ -606,7 +606,11 @@ void corr_iteration(cudaStream_t s, Box b, const CorrCoef<float>& c, const CorrI
                     const CorrOut<float>& out, unsigned long long* red, int check) {
   // the faces i = nx, j = ny, k = nz are walls: tiles cover the cells and their lower faces
   const unsigned gx = (b.nx + kCorrTX - 1) / kCorrTX, gy = (b.ny + CorrSingle::ty - 1) / CorrSingle::ty;
-  const int zc = march_chunk((long long)gx * gy, b.nz, kCorrZChunk, CorrSingle::blocks, sm_count(), 3.0, 1.0);
+  // grids of a few levels per block slot (up to some 56^3) are latency: two blocks on an SM cost little more
+  // than one (48^3: 1412 -> 1297 us per 120 sweeps with their outer phases)
+  const long long cols = (long long)gx * gy;
+  const double base = cols * b.nz < 4LL * CorrSingle::blocks * sm_count() ? 2.0 : 1.0;
+  const int zc = march_chunk(cols, b.nz, kCorrZChunk, CorrSingle::blocks, sm_count(), 3.0, base);
   const dim3 g(gx, gy, (unsigned)((b.nz + zc - 1) / zc));
   cudaFuncSetAttribute(k_corr_iteration, cudaFuncAttributeMaxDynamicSharedMemorySize, CorrSingle::smem);
   launch_chained(k_corr_iteration, g, dim3(32, CorrSingle::rows, 1), CorrSingle::smem, s, b, c, in, out, red, check,
