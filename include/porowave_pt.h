@@ -314,7 +314,7 @@ int pt_mg_axis_tables(int32_t nf, uint32_t *out, size_t words);
  * ninst independent instances (each its own grid, parameters, fields and numerics), all
  * PT_FP64 or all PT_FP32 (mixing returns PT_EINVAL), advanced together by one persistent engine:
  * one launch per phase covers all instances through a flat work list of (instance, tile) items
- * walked by a persistent grid-stride grid (SMs x resident CTAs), the launch sequence captured
+ * walked by a grid-stride grid (four CTAs per resident slot), the launch sequence captured
  * in one CUDA graph per replay, and every decision (convergence, iteration cap, non-finite
  * norms) taken on the device per instance; the host reads a status table once per replay.
  * FP64 ensembles (the FP64-lean form): 2 nup (or 4 nup) PT iterations per replay; each instance

@@ -36,7 +36,7 @@ struct BatchStatus {
   unsigned long long t_start, t_stop;   // device %globaltimer (ns)
 };
 
-enum { BATCH_CELLS = 0, BATCH_FACES = 1, BATCH_PICARD = 2, BATCH_COEF = 3 };
+enum { BATCH_CELLS = 0, BATCH_FACES = 1, BATCH_PICARD = 2, BATCH_COEF = 3, BATCH_PHASES = 4 };
 
 // Launch `phase` over all active instances with parity `a` (0/1); tile shape bx x by.
 void batch_phase(int bx, int by, int grid, cudaStream_t s, int phase, const BatchInst* inst,
@@ -48,6 +48,6 @@ void batch_converge(cudaStream_t s, const BatchInst* inst, BatchStatus* st, int 
 // Start of a step: all instances active, counters zero, reduction slots clear, start time.
 void batch_start(cudaStream_t s, const BatchInst* inst, BatchStatus* st, int ninst);
 // Resident CTAs per SM of the batched cell kernel for a tile shape (occupancy of the widest phase).
-int batch_blocks_per_sm(int bx, int by);
+int batch_blocks_per_sm(int bx, int by, int phase);
 
 }  // namespace pt

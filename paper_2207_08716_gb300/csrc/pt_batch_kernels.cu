@@ -2,8 +2,8 @@
 //
 // All instances of an ensemble are advanced by one launch per PT phase (cells, faces, Picard,
 // coefficients). The work list is the concatenation of every instance's tiles (bx x by cells of
-// one z-level of its padded box); a persistent grid (SMs x resident CTAs) walks it with a grid
-// stride, so instances of uneven size share the GPU without per-instance launches. Each tile
+// one z-level, wall indices only where they carry stress); a grid of a few CTAs per resident slot walks it
+// with a grid stride, so instances of uneven size share the GPU without per-instance launches. Each tile
 // runs the same per-point code as the single-instance FP64-lean kernels (pt_lean_body.cuh) with
 // its instance's box, coefficients and fields, so a batched instance reproduces its
 // single-instance run bit for bit. Retired instances' tiles return at once.
@@ -36,8 +36,10 @@ template <int BX, int BY, int PHASE>
 __global__ void __launch_bounds__(BX * BY) k_batch_phase(const BatchInst* __restrict__ inst,
                                                          const BatchStatus* __restrict__ st, int ninst,
                                                          long long ntiles, int a, int check) {
+  int m = find_instance(inst, ninst, blockIdx.x);
   for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int m = find_instance(inst, ninst, t);
+    // the instances follow one another along t: one load a tile where a search took some five in a row
+    while (m + 1 < ninst && inst[m + 1].tile_base <= t) ++m;
     if (!st[m].active) {                              // uniform over the CTA: a retired instance's
       // tiles are skipped in one step, to the first tile of the next instance this CTA visits
       const long long next = m + 1 < ninst ? inst[m + 1].tile_base : ntiles;
@@ -176,16 +178,31 @@ void batch_start(cudaStream_t s, const BatchInst* inst, BatchStatus* st, int nin
   k_batch_start<<<(ninst + 127) / 128, 128, 0, s>>>(inst, st, ninst);
 }
 
-int batch_blocks_per_sm(int bx, int by) {
+namespace {
+template <int BX, int BY>
+int phase_blocks(int phase) {
   int n = 0;
   cudaError_t e;
-  if (bx == 32 && by == 4)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_phase<32, 4, BATCH_CELLS>, 128, 0);
-  else if (bx == 64 && by == 4)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_phase<64, 4, BATCH_CELLS>, 256, 0);
-  else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_phase<32, 8, BATCH_CELLS>, 256, 0);
+  switch (phase) {
+    case BATCH_CELLS:
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_phase<BX, BY, BATCH_CELLS>, BX * BY, 0);
+      break;
+    case BATCH_FACES:
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_phase<BX, BY, BATCH_FACES>, BX * BY, 0);
+      break;
+    case BATCH_PICARD:
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_phase<BX, BY, BATCH_PICARD>, BX * BY, 0);
+      break;
+    default: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_phase<BX, BY, BATCH_COEF>, BX * BY, 0); break;
+  }
   return (e == cudaSuccess && n > 0) ? n : 1;
+}
+}  // namespace
+
+int batch_blocks_per_sm(int bx, int by, int phase) {
+  if (bx == 32 && by == 4) return phase_blocks<32, 4>(phase);
+  if (bx == 64 && by == 4) return phase_blocks<64, 4>(phase);
+  return phase_blocks<32, 8>(phase);
 }
 
 }  // namespace pt
