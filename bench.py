@@ -69,23 +69,23 @@ DTYPES = {"fp64": "f64", "fp32": "f32", "fp64-stepwise": "f64", "df64": "df64"}
 # at the capture; when the sources have changed since, the figures are stale and the bench
 # reports them as null (`python bench.py --source-hashes` prints the current hashes).
 KERNEL_SOURCES = {
-    **{k: ("pt_lean_kernels.cu", "pt_lean_body.cuh", "pt_lean.cuh", "df64.cuh", "pt_common.cuh")
+    **{k: ("pt_lean_kernels.cu", "pt_lean_body.cuh", "pt_df_body.cuh", "pt_lean.cuh", "df64.cuh", "pt_common.cuh")
        for k in ("k_lean_cells", "k_lean_faces", "k_lean_picard", "k_lean_coef", "k_lean_cells_df64",
                  "k_lean_faces_df64", "k_lean_picard_df64", "k_lean_coef_df64")},
     "k_centres": ("pt_ref_kernels.cu", "pt_kernels.cuh", "pt_common.cuh"),
-    **{k: ("pt_adjoint_kernels.cu", "pt_adjoint.cuh", "pt_common.cuh")
+    **{k: ("pt_adjoint_kernels.cu", "pt_adjoint.cuh", "pt_lean_body.cuh", "pt_common.cuh")
        for k in ("k_adj_cells", "k_adj_faces", "k_adj_edges_pl", "k_adj_cells_pl", "k_adj_faces_pl")},
     "k_corr_iteration": ("pt_mixed_kernels.cu", "pt_mixed.cuh", "pt_common.cuh"),
-    "k_mg_smooth_fp32": ("rx_mg_kernels.cu", "rx.cuh"),
+    "k_mg_smooth_fp32": ("rx_mg_kernels.cu", "rx_quad.cuh", "rx.cuh", "pt_common.cuh"),
 }
 PROFILED = {
     # profiles/kernels_191_ncu_metrics.md (191^3, every launch of one step of each form)
-    "k_lean_cells": {"src": "847b74c5871329ee", "fp64_inst": 100.2, "fp64_flops": 148.4, "traffic": 310.9},
-    "k_lean_faces": {"src": "847b74c5871329ee", "fp64_inst": 33.1, "fp64_flops": 50.0, "traffic": 180.3},
-    "k_lean_cells_df64": {"src": "847b74c5871329ee", "traffic": 260.0, "thread_inst": 1929.0},
-    "k_lean_faces_df64": {"src": "847b74c5871329ee", "traffic": 164.3, "thread_inst": 724.9},
-    # profiles/k_corr_iteration_fp32_255.md (255^3, one launch)
-    "k_corr_iteration": {"src": "642041b57f4bbbcc", "traffic": 106.3, "thread_inst": 720.8},
+    "k_lean_cells": {"src": "a351ee1fa12c90bf", "fp64_inst": 94.0, "fp64_flops": 139.2, "traffic": 312.1},
+    "k_lean_faces": {"src": "a351ee1fa12c90bf", "fp64_inst": 32.9, "fp64_flops": 49.8, "traffic": 180.3},
+    "k_lean_cells_df64": {"src": "a351ee1fa12c90bf", "traffic": 259.9, "thread_inst": 1383.0},
+    "k_lean_faces_df64": {"src": "a351ee1fa12c90bf", "traffic": 164.3, "thread_inst": 586.5},
+    # profiles/k_corr_iteration_fp32_255.md (255^3, the launches of one step)
+    "k_corr_iteration": {"src": "35544df90342ba89", "traffic": 104.5, "thread_inst": 524.6},
 }
 # The FP64 pipe's nominal issue capacity: 304 thread-instructions per GPU clock (2 per SM; ncu's
 # sm__inst_executed_pipe_fp64 peak on this machine's GB300), 629 G/s at 2.07 GHz.
