@@ -85,7 +85,7 @@ PROFILED = {
     "k_lean_cells_df64": {"src": "a351ee1fa12c90bf", "traffic": 259.9, "thread_inst": 1383.0},
     "k_lean_faces_df64": {"src": "a351ee1fa12c90bf", "traffic": 164.3, "thread_inst": 586.5},
     # profiles/k_corr_iteration_fp32_255.md (255^3, the launches of one step)
-    "k_corr_iteration": {"src": "35544df90342ba89", "traffic": 104.5, "thread_inst": 524.6},
+    "k_corr_iteration": {"src": "8dada89a5e251b16", "traffic": 104.5, "thread_inst": 524.6},
 }
 # The FP64 pipe's nominal issue capacity: 304 thread-instructions per GPU clock (2 per SM; ncu's
 # sm__inst_executed_pipe_fp64 peak on this machine's GB300), 629 G/s at 2.07 GHz.

@@ -126,7 +126,7 @@ void mg_prolong(cudaStream_t s, const MgLevel& c, int dc, const MgLevel& f, int 
 // advance together through one graph-captured launch sequence per replay:
 //   PREP     FP64 residuals at u, stresses, Picard update               (members in MB_PREP)
 //   decide   outer norms: converged / non-finite -> MB_DONE, else weight, inner target -> MB_INNER
-//   INIT     frozen FP32 coefficients and a zero correction             (members starting a solve)
+//   INIT     a zero correction and damped residual                      (members starting a solve)
 //   corr x nup   FP32 correction iterations, norms at the last          (members in MB_INNER)
 //   decide   inner stop (drop reached, or the member's iteration budget spent) -> MB_UPDATE
 //   UPDATE, POROSITY   u <- u + omega delta, FP64 porosity integration  (members in MB_UPDATE)
