@@ -35,15 +35,16 @@ template <class T>
 __device__ inline T rx_bp(const RxCoef<T>& c, T ph) {
   return ph * c.beta_f + c.beta_d - (T(1) + ph) * c.beta_s;
 }
-// 1 / x from the hardware's approximate reciprocal refined by Newton steps r' = r + r (1 - x r),
-// each of which squares the relative error (FP64: ~2^-23 seed, rounding-limited after two). x is
-// 1 - phi, 1 - Xs, beta_P or a Jacobi denominator here: positive and far inside the normal range.
+// 1 / x from the hardware's approximate reciprocal r refined by one third-order step r (1 + e + e^2),
+// e = 1 - x r (FP64: r is good to about 2^-20, so e^3 is below the rounding; three instructions, two Newton
+// steps take four). x is 1 - phi, 1 - Xs, beta_P or a Jacobi denominator here: positive and far inside the
+// normal range.
 // FP32 takes the fast reciprocal-multiply intrinsic (2 ulp).
 __device__ inline double rx_rcp(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 __device__ inline float rx_rcp(float x) { return __fdividef(1.0f, x); }
 // max of the three one-iteration changes; NaN if any is (fmax alone would drop it)

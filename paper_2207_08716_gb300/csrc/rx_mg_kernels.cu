@@ -33,7 +33,8 @@ __device__ __forceinline__ MgEq<T> mg_cell(const RxCoef<T>& c, T romega, T divq,
                                            T phi_o, T Xs_o) {
   const T w = rx_rcp(T(1) - ph), ixs = rx_rcp(T(1) - Xs);
   const T xr = c.beta_x * Pf + c.half_xs;
-  const T xseq = rx_clamp(xr, T(0), c.xs_max);
+  const bool pos = xr > T(0), below = xr < c.xs_max;     // Xs_eq is xr clamped to [0, xs_max]
+  const T xseq = pos ? (below ? xr : c.xs_max) : T(0);
   const T dXs = (xseq - Xs) * c.rtau;
   const T rbp = rx_rcp(rx_bp(c, ph));
   const T src = c.sr_opdx * (T(1) - ph) * ixs;
@@ -42,7 +43,7 @@ __device__ __forceinline__ MgEq<T> mg_cell(const RxCoef<T>& c, T romega, T divq,
   e.R = (-divq - comp + src * dXs) * rbp;
   e.gP = e.R - (Pf - Pf_o) * c.rdt;
   if (DEN) {
-    const T dxs_dpf = (xr > T(0) && xr < c.xs_max) ? c.beta_x : T(0);
+    const T dxs_dpf = pos && below ? c.beta_x : T(0);
     const T a = (w * c.reta - src * dxs_dpf * c.rtau) * rbp;
     e.den = Dk * rbp * romega + c.rdt + a;
   } else {
