@@ -48,7 +48,7 @@ def test_fp32_correction_tiles(nx, ny, nz):
 @pytest.mark.parametrize("nx,ny,nz,shear,logk", [(3, 2, 1, False, False), (31, 7, 5, True, False),
                                                  (32, 8, 17, False, True), (33, 9, 16, True, True),
                                                  (64, 15, 33, False, False), (97, 26, 40, True, False),
-                                                 (130, 50, 21, False, True)])
+                                                 (130, 50, 21, False, True), (150, 147, 149, True, True)])
 def test_fixed_count_steps(form, nx, ny, nz, shear, logk):
     """Three Picard intervals of PT iterations; the FP64-class bar of the oracle comparisons, 1e-10."""
     case = dict(kind="step", form=form, nx=nx, ny=ny, nz=nz, iters=45, shear=shear, logk=logk)
