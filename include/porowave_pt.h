@@ -225,11 +225,12 @@ int pt_peak_arith(int32_t kind, void *sink, int32_t steps, int32_t reps, void *s
  *   PT_MATH_DF_ROOT      double-float a^(1/m), m = (int)b[e] (Newton's m-th root)
  *   PT_MATH_DF_EXPM1_POS/NEG  the split Taylor series in double-float
  *   PT_MATH_TO_FLOAT     a rounded to FP32 on the integer units (to nearest even)
+ *   PT_MATH_HALF         a / 2 on the integer units (|a| >= 2^-1021, infinite or NaN)
  * Returns PT_EINVAL for an unknown code or a missing operand. */
 enum { PT_MATH_RCP_PSEUDO = 0, PT_MATH_RCP_FULL = 1, PT_MATH_EXPM1_POS = 2, PT_MATH_EXPM1_NEG = 3,
        PT_MATH_DF_ADD = 4, PT_MATH_DF_SUB = 5, PT_MATH_DF_MUL = 6, PT_MATH_DF_FMA = 7,
        PT_MATH_DF_RCP = 8, PT_MATH_DF_SQRT = 9, PT_MATH_DF_ROOT = 10, PT_MATH_DF_EXPM1_POS = 11,
-       PT_MATH_DF_EXPM1_NEG = 12, PT_MATH_TO_FLOAT = 13 };
+       PT_MATH_DF_EXPM1_NEG = 12, PT_MATH_TO_FLOAT = 13, PT_MATH_HALF = 14 };
 int pt_math_check(int32_t fn, const double *a, const double *b, double *out, int64_t n, void *stream);
 
 /* ---- Residual norms with no allocation at all -------------------------------------------

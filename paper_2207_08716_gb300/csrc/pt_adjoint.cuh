@@ -40,7 +40,7 @@ struct AdjPrepPL {
   double *Qxx, *Qyy, *Qzz;              // dm/dmu times the state's deviatoric strain rates
   double *sTxx, *sTyy, *sTzz;           // m f tau_ii: centre part of the pseudo-stress per lambda_mu
   double *Axy, *Axz, *Ayz;              // f a_e / 2 per centre (a_e: edge stresses averaged to it)
-  double *me_xy, *me_xz, *me_yz;        // edge moduli
+  double *hme_xy, *hme_xz, *hme_yz;     // halves of the edge moduli
   double *P_xy, *P_xz, *P_yz;           // (dm/dmu)_e eps_e / 4 on edges
   double *iDmu, *cmu, *cmuL;            // 1 / diagonal of row mu; (Pt-Pf) cc / mu; (Pt-Pf) dt phi / (eta0 mu^2)
   double *dtvx, *dtvy, *dtvz;           // velocity pseudo-steps at faces (mean of the two centres')
@@ -49,7 +49,7 @@ struct AdjPrepPL {
 // Edges of one adjoint iteration (power law): pseudo-stress sigma_e from lambda_mu, the edge's
 // adjoint stress m_e (eps_e(lambda_V) - sigma_e / 2) and Z_e = sigma_e - 2 eps_e(lambda_V).
 struct AdjEdgeIn {
-  const double *Lx, *Ly, *Lz, *lM, *Axy, *Axz, *Ayz, *me_xy, *me_xz, *me_yz;
+  const double *Lx, *Ly, *Lz, *lM, *Axy, *Axz, *Ayz, *hme_xy, *hme_xz, *hme_yz;
 };
 struct AdjEdgeOut {
   double *txy, *txz, *tyz, *Zxy, *Zxz, *Zyz;

@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(256) k_adj_prep_pl_edges(Box b, AdjCoef c, Adj
       P = 0.25 * dmodulus(m, c.Gdt) * e;
       t = me * e;
     }
-    pl.me_xy[q] = me; pl.P_xy[q] = P; tau_xy[q] = t;
+    pl.hme_xy[q] = 0.5 * me; pl.P_xy[q] = P; tau_xy[q] = t;
   }
   if (j < b.ny) {
     double me = 0.0, P = 0.0, t = 0.0;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(256) k_adj_prep_pl_edges(Box b, AdjCoef c, Adj
       P = 0.25 * dmodulus(m, c.Gdt) * e;
       t = me * e;
     }
-    pl.me_xz[q] = me; pl.P_xz[q] = P; tau_xz[q] = t;
+    pl.hme_xz[q] = 0.5 * me; pl.P_xz[q] = P; tau_xz[q] = t;
   }
   if (i < b.nx) {
     double me = 0.0, P = 0.0, t = 0.0;
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(256) k_adj_prep_pl_edges(Box b, AdjCoef c, Adj
       P = 0.25 * dmodulus(m, c.Gdt) * e;
       t = me * e;
     }
-    pl.me_yz[q] = me; pl.P_yz[q] = P; tau_yz[q] = t;
+    pl.hme_yz[q] = 0.5 * me; pl.P_yz[q] = P; tau_yz[q] = t;
   }
 }
 
@@ -509,21 +509,21 @@ __global__ void __launch_bounds__(kPlaneThreads) k_adj_edges_pl(Box b, AdjCoef c
     const double sg = fma(in.Axy[q], in.lM[q], fma(in.Axy[q - 1], in.lM[q - 1], fma(in.Axy[q - px], in.lM[q - px],
                           in.Axy[q - 1 - px] * in.lM[q - 1 - px])));
     Z[0] = sg - e2;
-    t[0] = -lean_detail::scale2(in.me_xy[q], -1) * Z[0];
+    t[0] = -in.hme_xy[q] * Z[0];
   }
   if (ix && kz && j < b.ny) {
     const double e2 = fma(in.Lx[q] - in.Lx[q - pxy], c.rdz, (in.Lz[q] - in.Lz[q - 1]) * c.rdx);
     const double sg = fma(in.Axz[q], in.lM[q], fma(in.Axz[q - 1], in.lM[q - 1], fma(in.Axz[q - pxy], in.lM[q - pxy],
                           in.Axz[q - 1 - pxy] * in.lM[q - 1 - pxy])));
     Z[1] = sg - e2;
-    t[1] = -lean_detail::scale2(in.me_xz[q], -1) * Z[1];
+    t[1] = -in.hme_xz[q] * Z[1];
   }
   if (jy && kz && i < b.nx) {
     const double e2 = fma(in.Ly[q] - in.Ly[q - pxy], c.rdz, (in.Lz[q] - in.Lz[q - px]) * c.rdy);
     const double sg = fma(in.Ayz[q], in.lM[q], fma(in.Ayz[q - px], in.lM[q - px], fma(in.Ayz[q - pxy], in.lM[q - pxy],
                           in.Ayz[q - px - pxy] * in.lM[q - px - pxy])));
     Z[2] = sg - e2;
-    t[2] = -lean_detail::scale2(in.me_yz[q], -1) * Z[2];
+    t[2] = -in.hme_yz[q] * Z[2];
   }
   if (k < b.nz) { out.txy[q] = t[0]; out.Zxy[q] = Z[0]; }
   if (j < b.ny) { out.txz[q] = t[1]; out.Zxz[q] = Z[1]; }

@@ -82,6 +82,7 @@ struct pt_ctx {
   double *toa_xx, *toa_yy, *toa_zz, *toa_xy, *toa_xz, *toa_yz, *cm2, *idtp, *ieta;
   double *em2_xy, *em2_xz, *em2_yz, *eb_xy, *eb_xz, *eb_yz, *dtv_x, *dtv_y, *dtv_z, *K0;
   LeanCoef<double> lcoef;
+  StressCoef scoef;
   // double-float path (precision PT_DF64): the lean arrays above hold df64 values; the iterate
   // lives in these df64 arrays between pt_step_begin and the return of each call, the caller's
   // FP64 fields receive it (export) when a call returns
@@ -271,6 +272,8 @@ void fill_lean_coef(pt_ctx* c) {
   L.rtau0_2s = 0.125 * L.rtau0_2h;
   L.rel_mu = k.rel_mu; L.rel_eta = k.rel_eta; L.eta0_weak = k.eta0 * k.R_weak;
   L.rGdtS = k.rGdtS;
+  c->scoef = StressCoef{k.rGdtS, 0.25 * k.rGdtS, 0.25 * k.rdx, 0.25 * k.rdy, 0.25 * k.rdz, 0.5 * k.ebg, 2.0 * k.ebg,
+                        2.0 * k.rdx, 2.0 * k.rdy, 2.0 * k.rdz, 2.0 * k.beta_n, k.bg_on};
   L.dtaupt_fac = k.dtaupt_fac;
   L.dtauv_fac = k.dtauv_fac;
   L.root_mu = relax_root(k.rel_mu);
@@ -707,7 +710,7 @@ int mixed_outer(pt_ctx* c, int n_in, bool early_exit, pt_report* outer, bool* co
                       c->Pt[a], c->Pf[a], c->phi[a], c->eta, c->perm, c->Pto, c->Pfo};
   const MixPrepOut pout{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz,
                         c->m_rpt, c->m_rpf, c->m_cc, c->m_perm, c->m_idtp};
-  PT_LAUNCH(c, K_MIX_PREP, mix_prepare(c->stream, b, k, pin, pout, c->red));
+  PT_LAUNCH(c, K_MIX_PREP, mix_prepare(c->stream, b, k, c->scoef, pin, pout, c->red));
   const MixFaceIn fin{LeanPicardIn<double>{c->s_txx, c->s_tyy, c->s_tzz, c->s_txy, c->s_txz, c->s_tyz, c->phi[a],
                                            c->Pt[a], c->Pf[a]},
                       c->mu, c->eta};
@@ -1119,7 +1122,7 @@ int pt_step_end(pt_ctx* c) {
   if (c->lean || c->mixed) {
     const StressIn si{c->Vx, c->Vy, c->Vz, c->mu, c->txxo, c->tyyo, c->tzzo, c->txyo, c->txzo, c->tyzo};
     PT_LAUNCH(c, K_STRESSES,
-              lean_stresses(grid_dims(b), block_dims(), c->stream, b, c->lcoef, si,
+              lean_stresses(grid_dims(b), block_dims(), c->stream, b, c->lcoef, c->scoef, si,
                             StressCentre{c->Pt[0], c->Pf[0], c->Pto, c->Pfo, c->phi[0], c->eta},
                             StressOut{c->txx, c->tyy, c->tzz, c->txy, c->txz, c->tyz}));
     c->dt_cum += c->num.dt;
@@ -1449,6 +1452,7 @@ void fill_mix_inst(pt_batch* B, int m, long long base, long long cbase) {
   MixBatchInst& I = B->h_minst[m];
   I.b = c->box;
   I.lc = c->lcoef;
+  I.sc = c->scoef;
   I.cc = c->ccoef;
   I.Vx = c->Vx; I.Vy = c->Vy; I.Vz = c->Vz;
   for (int a = 0; a < 2; ++a) {
@@ -2013,7 +2017,7 @@ struct AdjArrays {
     acc = A[72];
   }
   AdjEdgeIn edge_in(int cur) const {
-    return AdjEdgeIn{Lx, Ly, Lz, lM[cur], pl.Axy, pl.Axz, pl.Ayz, pl.me_xy, pl.me_xz, pl.me_yz};
+    return AdjEdgeIn{Lx, Ly, Lz, lM[cur], pl.Axy, pl.Axz, pl.Ayz, pl.hme_xy, pl.hme_xz, pl.hme_yz};
   }
   AdjPrep prep_for(int cur) const {
     AdjPrep p = prep;

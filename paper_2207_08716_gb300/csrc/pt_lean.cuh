@@ -18,6 +18,17 @@ __host__ __device__ inline RootSeries root_series(int m) {
   return RootSeries{r, 0.5 * r * (1.0 + r), r * (1.0 + r) * (1.0 + 0.5 * r) / 3.0, (float)r};
 }
 
+// Scalars of the Maxwell stresses (stress_edges_point, centre_stresses) in which the powers of two of a
+// mean of four viscosities, of 2 mu and of a halved strain rate are folded, always in FP64.
+struct StressCoef {
+  double rG, rG4;               // 1 / (G dtS), and for a sum of four viscosities a quarter of it
+  double qrdx, qrdy, qrdz;      // 1 / (4 d_i): half an edge's strain rate
+  double hebg, tebg;            // half and twice the background xy strain rate (Eqs. 32-33)
+  double trdx, trdy, trdz;      // 2 / d_i: twice a centre's strain rate
+  double tbeta_n;               // 2 beta_n
+  int bg_on;                    // tau_bg != 0: wall xy-edges carry the background stress
+};
+
 // Per-step scalars in the field type, pre-folded so each kernel multiplies instead of divides.
 template <class T>
 struct LeanCoef {
@@ -118,8 +129,8 @@ template <class T>
 void lean_begin(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<T>& c, const LeanBeginIn<T>& in,
                 const LeanBeginOut<T>& out, unsigned long long* red);
 // The stresses of the current state (Eq. 21), centres and edges (end of a step).
-void lean_stresses(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c, const StressIn& in,
-                   const StressCentre& ce, const StressOut& out);
+void lean_stresses(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c, const StressCoef& sc,
+                   const StressIn& in, const StressCentre& ce, const StressOut& out);
 template <class T>
 void lean_k0(dim3 gr, dim3 bl, cudaStream_t st, Box b, double k0r3, const double* logk, T* K0);
 
@@ -134,7 +145,7 @@ void df64_convert(cudaStream_t st, const DfCopy& cp, int narrays, long long n, b
 enum { MATH_RCP_PSEUDO = 0, MATH_RCP_FULL = 1, MATH_EXPM1_POS = 2, MATH_EXPM1_NEG = 3, MATH_DF_ADD = 4,
        MATH_DF_SUB = 5, MATH_DF_MUL = 6, MATH_DF_FMA = 7, MATH_DF_RCP = 8, MATH_DF_SQRT = 9,
        MATH_DF_ROOT = 10, MATH_DF_EXPM1_POS = 11, MATH_DF_EXPM1_NEG = 12, MATH_TO_FLOAT = 13,
-       MATH_COUNT = 14 };
+       MATH_HALF = 14, MATH_COUNT = 15 };
 void math_check(cudaStream_t st, int fn, const double* a, const double* b, double* out, long long n);
 
 }  // namespace pt

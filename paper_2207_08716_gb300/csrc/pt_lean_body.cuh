@@ -32,9 +32,13 @@ __device__ inline void expm1_pair(double d, double& em_pos, double& em_neg) {
 }
 
 // The FP64 pipe takes a warp instruction every 16 cycles, in which an SM issues 64 others: conversions
-// between FP64 and FP32 and products with powers of two, which run on it, are done on the integers.
-__device__ inline double scale2(double x, int e) {   // x 2^e, x positive and far inside the normal range
-  return __hiloint2double(__double2hiint(x) + e * 0x100000, __double2loint(x));
+// between FP64 and FP32 and one halving, which run on it, are done on the integers. (Other powers of two
+// are folded into the coefficients they meet: nothing changes the exponent of a value that may be
+// anything.)
+// x / 2 for |x| >= 2^-1021, infinities and NaN staying what they are
+__device__ inline double half_of(double x) {
+  const int hi = __double2hiint(x);
+  return __hiloint2double((hi & 0x7ff00000) == 0x7ff00000 ? hi : hi - 0x00100000, __double2loint(x));
 }
 // x to FP32, to nearest even as the conversion rounds; values outside FP32's normal range take that
 __device__ inline float to_float(double x) {
@@ -327,7 +331,7 @@ __device__ __forceinline__ void lean_cell_level(const Box& b, const LeanCoef<dou
     // delta = -[beta_phi ((Pf1 - Pfo) - (Pt1 - Pto)) + dt (Pf1 - Pt1) / eta + dt V.grad(1-phi)/(1-phi)]
     // V.grad(1-phi)/(1-phi) = -(w/2) sum_d rd [v_r (phi_r - phi) + v_l (phi - phi_l)]
     //                      = -(w/2) [sum_d rd (v_r phi_r - v_l phi_l) - phi divV]
-    const double adv = -scale2(w, -1) * fma(ph, -divV, fma(ax, c.rdx, fma(ay, c.rdy, az * c.rdz)));
+    const double adv = -half_of(w) * fma(ph, -divV, fma(ax, c.rdx, fma(ay, c.rdy, az * c.rdz)));
     const double dp1 = Pf1 - Pt1;
     const double rate = c.compaction_on ? fma(dp1, ieta, adv) : adv;
     const double delta = -fma(c.beta_phi, dp1 - (Pfo - Pto), c.dt * rate);
@@ -462,16 +466,30 @@ __device__ inline T lean_edge_mean_mu_xy(const Box& b, const T* mu, long long q,
 // Maxwell stress (Eq. 21) of viscosity m, xi = m rG: tau = (tau_o xi + 2 m edot) / (1 + xi), as
 // tau_o + s (2 m edot - tau_o) with s = 1 / (1 + xi).
 __device__ __forceinline__ double maxwell_s(double m, double rG) { return lean_detail::rcp_full(fma(m, rG, 1.0)); }
-__device__ __forceinline__ double maxwell(double s, double m2, double e, double to) {
-  return fma(s, fma(m2, e, -to), to);
+__device__ __forceinline__ double maxwell(double s, double m, double e2, double to) {   // e2 = 2 edot
+  return fma(s, fma(m, e2, -to), to);
+}
+// An edge's stress from the sum of its four centres' viscosities and half its strain rate:
+// xi = (m4 / 4) rG, 2 m edot = m4 (edot / 2)
+__device__ __forceinline__ double edge_stress(const StressCoef& sc, double m4, double he, double to) {
+  return maxwell(maxwell_s(m4, sc.rG4), m4, he, to);
+}
+// The three normal stresses of a centre of viscosity m (Eq. 21): twice the deviatoric strain rate and
+// beta_n times the numerical divergence divVn.
+__device__ __forceinline__ void centre_stresses(const StressCoef& sc, double m, double dvx, double dvy, double dvz,
+                                                double divV, double divVn, double to_xx, double to_yy, double to_zz,
+                                                double& txx, double& tyy, double& tzz) {
+  const double s = maxwell_s(m, sc.rG), s3 = fma(sc.tbeta_n, divVn, divV * (-2.0 / 3.0));
+  txx = maxwell(s, m, fma(dvx, sc.trdx, s3), to_xx);
+  tyy = maxwell(s, m, fma(dvy, sc.trdy, s3), to_yy);
+  tzz = maxwell(s, m, fma(dvz, sc.trdz, s3), to_zz);
 }
 
 // Shear stresses on the three lower edges of (i, j, k), zero on boundary edges unless a background
 // shear is applied (Eqs. 32-33). An edge's viscosity is the mean of its four centres'.
-__device__ __forceinline__ void stress_edges_point(const Box& b, const LeanCoef<double>& c, const StressIn& in,
+__device__ __forceinline__ void stress_edges_point(const Box& b, const StressCoef& sc, const StressIn& in,
                                                    double* __restrict__ txy, double* __restrict__ txz,
                                                    double* __restrict__ tyz, int i, int j, int k) {
-  using lean_detail::scale2;
   if (i > b.nx || j > b.ny || k > b.nz) return;
   const long long q = cidx(b, i, j, k);
   const long long px = b.px, pxy = b.pxy;
@@ -479,11 +497,11 @@ __device__ __forceinline__ void stress_edges_point(const Box& b, const LeanCoef<
     double t = 0.0;
     if (i > 0 && i < b.nx && j > 0 && j < b.ny) {
       const double m4 = (in.mu[q - 1 - px] + in.mu[q - px]) + (in.mu[q - 1] + in.mu[q]);
-      const double e = fma(in.Vx[q] - in.Vx[q - px], c.hrdy, fma(in.Vy[q] - in.Vy[q - 1], c.hrdx, c.ebg));
-      t = maxwell(maxwell_s(scale2(m4, -2), c.rGdtS), scale2(m4, -1), e, in.txyo[q]);
-    } else if (c.bg_on) {   // wall edge: background part only
+      const double he = fma(in.Vx[q] - in.Vx[q - px], sc.qrdy, fma(in.Vy[q] - in.Vy[q - 1], sc.qrdx, sc.hebg));
+      t = edge_stress(sc, m4, he, in.txyo[q]);
+    } else if (sc.bg_on) {   // wall edge: background part only
       const double m = lean_edge_mean_mu_xy(b, in.mu, q, i, j);
-      t = maxwell(maxwell_s(m, c.rGdtS), scale2(m, 1), c.ebg, in.txyo[q]);
+      t = maxwell(maxwell_s(m, sc.rG), m, sc.tebg, in.txyo[q]);
     }
     txy[q] = t;
   }
@@ -491,8 +509,8 @@ __device__ __forceinline__ void stress_edges_point(const Box& b, const LeanCoef<
     double t = 0.0;
     if (i > 0 && i < b.nx && k > 0 && k < b.nz) {
       const double m4 = (in.mu[q - 1 - pxy] + in.mu[q - pxy]) + (in.mu[q - 1] + in.mu[q]);
-      const double e = fma(in.Vx[q] - in.Vx[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - 1]) * c.hrdx);
-      t = maxwell(maxwell_s(scale2(m4, -2), c.rGdtS), scale2(m4, -1), e, in.txzo[q]);
+      const double he = fma(in.Vx[q] - in.Vx[q - pxy], sc.qrdz, (in.Vz[q] - in.Vz[q - 1]) * sc.qrdx);
+      t = edge_stress(sc, m4, he, in.txzo[q]);
     }
     txz[q] = t;
   }
@@ -500,8 +518,8 @@ __device__ __forceinline__ void stress_edges_point(const Box& b, const LeanCoef<
     double t = 0.0;
     if (j > 0 && j < b.ny && k > 0 && k < b.nz) {
       const double m4 = (in.mu[q - px - pxy] + in.mu[q - pxy]) + (in.mu[q - px] + in.mu[q]);
-      const double e = fma(in.Vy[q] - in.Vy[q - pxy], c.hrdz, (in.Vz[q] - in.Vz[q - px]) * c.hrdy);
-      t = maxwell(maxwell_s(scale2(m4, -2), c.rGdtS), scale2(m4, -1), e, in.tyzo[q]);
+      const double he = fma(in.Vy[q] - in.Vy[q - pxy], sc.qrdz, (in.Vz[q] - in.Vz[q - px]) * sc.qrdy);
+      t = edge_stress(sc, m4, he, in.tyzo[q]);
     }
     tyz[q] = t;
   }

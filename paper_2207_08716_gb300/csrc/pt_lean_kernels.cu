@@ -231,31 +231,31 @@ __global__ void __launch_bounds__(kPlaneThreads) k_lean_picard(Box b, LeanCoef<T
 // ---------------------------------------------------------------------- end-of-step stresses
 // One pass over centres and edges with third-order reciprocals (the two step-by-step kernels divide
 // by 1 + xi: 13.2 + 16.2 ms at 511^3).
-__global__ void __launch_bounds__(256) k_lean_stresses(Box b, LeanCoef<double> c, StressIn in, StressCentre ce,
-                                                       StressOut out) {
+__global__ void __launch_bounds__(256) k_lean_stresses(Box b, LeanCoef<double> c, StressCoef sc, StressIn in,
+                                                       StressCentre ce, StressOut out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
-  stress_edges_point(b, c, in, out.txy, out.txz, out.tyz, i, j, k);
+  stress_edges_point(b, sc, in, out.txy, out.txz, out.tyz, i, j, k);
   if (i >= b.nx || j >= b.ny || k >= b.nz) return;
   const long long q = cidx(b, i, j, k);
   const double dvx = in.Vx[q + 1] - in.Vx[q], dvy = in.Vy[q + b.px] - in.Vy[q], dvz = in.Vz[q + b.pxy] - in.Vz[q];
   const double divV = fma(dvx, c.rdx, fma(dvy, c.rdy, dvz * c.rdz));
-  double s3 = divV * (-1.0 / 3.0);
+  double divVn = divV;
   if (c.beta_n != 0.0) {
     const double Pt = ce.Pt[q], Pf = ce.Pf[q];
     const double cc = c.compaction_on ? lean_detail::rcp_full(ce.eta[q] * (1.0 - ce.phi[q])) : 0.0;
-    const double divVn = fma(Pt - Pf, cc, fma(-c.bd_rdt_a, Pf - ce.Pfo[q], fma(c.bd_rdt, Pt - ce.Pto[q], divV)));
-    s3 = fma(c.beta_n, divVn, s3);
+    divVn = fma(Pt - Pf, cc, fma(-c.bd_rdt_a, Pf - ce.Pfo[q], fma(c.bd_rdt, Pt - ce.Pto[q], divV)));
   }
-  const double s = maxwell_s(in.mu[q], c.rGdtS), m2 = lean_detail::scale2(in.mu[q], 1);
-  out.txx[q] = maxwell(s, m2, fma(dvx, c.rdx, s3), in.txxo[q]);
-  out.tyy[q] = maxwell(s, m2, fma(dvy, c.rdy, s3), in.tyyo[q]);
-  out.tzz[q] = maxwell(s, m2, fma(dvz, c.rdz, s3), in.tzzo[q]);
+  double txx, tyy, tzz;
+  centre_stresses(sc, in.mu[q], dvx, dvy, dvz, divV, divVn, in.txxo[q], in.tyyo[q], in.tzzo[q], txx, tyy, tzz);
+  out.txx[q] = txx;
+  out.tyy[q] = tyy;
+  out.tzz[q] = tzz;
 }
-void lean_stresses(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c, const StressIn& in,
-                   const StressCentre& ce, const StressOut& out) {
-  k_lean_stresses<<<gr, bl, 0, st>>>(b, c, in, ce, out);
+void lean_stresses(dim3 gr, dim3 bl, cudaStream_t st, Box b, const LeanCoef<double>& c, const StressCoef& sc,
+                   const StressIn& in, const StressCentre& ce, const StressOut& out) {
+  k_lean_stresses<<<gr, bl, 0, st>>>(b, c, sc, in, ce, out);
 }
 
 // --------------------------------------------------------------------- coefficient refresh
@@ -359,6 +359,7 @@ __global__ void k_math_check(int fn, const double* __restrict__ a, const double*
       case MATH_DF_ROOT: r = (double)df_root(df64(x), (int)y); break;
       case MATH_DF_EXPM1_POS: expm1_pair(df64(x), dp, dm); r = (double)dp; break;
       case MATH_TO_FLOAT: r = (double)to_float(x); break;
+      case MATH_HALF: r = half_of(x); break;
       case MATH_DF_EXPM1_NEG: expm1_pair(df64(x), dp, dm); r = (double)dm; break;
       default: r = nan(""); break;
     }

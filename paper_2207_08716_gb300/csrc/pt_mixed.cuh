@@ -93,8 +93,8 @@ struct MgLevel {
 void mix_begin(cudaStream_t s, Box b, const double* Pt, const double* Pf, const double* phi, const double* mu,
                double* Pto, double* Pfo, double* phio, unsigned long long* red);
 void mix_perm(cudaStream_t s, Box b, const LeanCoef<double>& c, const double* phi, const double* logk, double* perm);
-void mix_prepare(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in, const MixPrepOut& out,
-                 unsigned long long* red);
+void mix_prepare(cudaStream_t s, Box b, const LeanCoef<double>& c, const StressCoef& sc, const MixPrepIn& in,
+                 const MixPrepOut& out, unsigned long long* red);
 void mix_faces(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in, const MixFaceOut& out,
                unsigned long long* red);
 void mix_porosity(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPorosity& p);
@@ -140,6 +140,7 @@ enum { MB_PH_PERM = 0, MB_PH_PREP = 1, MB_PH_FACES = 2, MB_PH_INIT = 3, MB_PH_UP
 struct MixBatchInst {
   Box b;
   LeanCoef<double> lc;                      // FP64 outer phases
+  StressCoef sc;
   CorrCoef<float> cc;                       // FP32 correction iteration
   double *Vx, *Vy, *Vz, *Pt[2], *Pf[2], *phi[2], *mu, *eta, *perm, *Pto, *Pfo, *Lo;   // Lo: phi of the old step
   const double* logk;

@@ -41,11 +41,11 @@ __device__ __forceinline__ void mix_perm_point(const Box& b, const LeanCoef<doub
 
 // (i) FP64 residuals at cell centres, stresses at u (centres and lower edges), and the frozen
 // coefficients of the correction problem (in FP32).
-__device__ __forceinline__ void mix_prepare_point(const Box& b, const LeanCoef<double>& c, const MixPrepIn& in,
-                                                  const MixPrepOut& out, int i, int j, int k, double& r_pt,
-                                                  double& r_pf) {
+__device__ __forceinline__ void mix_prepare_point(const Box& b, const LeanCoef<double>& c, const StressCoef& sc,
+                                                  const MixPrepIn& in, const MixPrepOut& out, int i, int j, int k,
+                                                  double& r_pt, double& r_pf) {
   using namespace lean_detail;
-  stress_edges_point(b, c, in.s, out.txy, out.txz, out.tyz, i, j, k);
+  stress_edges_point(b, sc, in.s, out.txy, out.txz, out.tyz, i, j, k);
   if (i < b.nx && j < b.ny && k < b.nz) {
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
@@ -67,11 +67,11 @@ __device__ __forceinline__ void mix_prepare_point(const Box& b, const LeanCoef<d
     const double divqD = -fma(sx, c.hrdx2, fma(sy, c.hrdy2, sz * c.hrdz2));
     const double rpf = fma(-dpp, cc, fma(-c.bd_rdt_a, dPt, fma(c.bda_B_rdt, dPf, divqD)));
     // stresses at u (Eq. 21) for the momentum residual and the Picard update
-    const double s = maxwell_s(mu, c.rGdtS), m2 = scale2(mu, 1);
-    const double s3 = fma(c.beta_n, divVn, divV * (-1.0 / 3.0));
-    out.txx[q] = maxwell(s, m2, fma(dvx, c.rdx, s3), in.s.txxo[q]);
-    out.tyy[q] = maxwell(s, m2, fma(dvy, c.rdy, s3), in.s.tyyo[q]);
-    out.tzz[q] = maxwell(s, m2, fma(dvz, c.rdz, s3), in.s.tzzo[q]);
+    double txx, tyy, tzz;
+    centre_stresses(sc, mu, dvx, dvy, dvz, divV, divVn, in.s.txxo[q], in.s.tyyo[q], in.s.tzzo[q], txx, tyy, tzz);
+    out.txx[q] = txx;
+    out.tyy[q] = tyy;
+    out.tzz[q] = tzz;
     // right-hand side and frozen coefficients of the correction problem (the iteration derives
     // 1/dtau_Pf from the largest neighbour k and the local-implicit denominators itself)
     out.r_pt[q] = to_float(divVn);
@@ -183,12 +183,13 @@ __global__ void __launch_bounds__(kPlaneThreads) k_mix_porosity(Box b, LeanCoef<
   if (plane_point(pl, i, j)) mix_porosity_point(b, c, p, i, j, (int)blockIdx.y);
 }
 
-__global__ void __launch_bounds__(kPlaneThreads) k_mix_prepare(Box b, LeanCoef<double> c, MixPrepIn in,
-                                                               MixPrepOut out, unsigned long long* red, Plane pl) {
+__global__ void __launch_bounds__(kPlaneThreads) k_mix_prepare(Box b, LeanCoef<double> c, StressCoef sc,
+                                                               MixPrepIn in, MixPrepOut out, unsigned long long* red,
+                                                               Plane pl) {
   chain_begin();
   int i, j;
   double r_pt = 0.0, r_pf = 0.0;
-  if (plane_point(pl, i, j)) mix_prepare_point(b, c, in, out, i, j, (int)blockIdx.y, r_pt, r_pf);
+  if (plane_point(pl, i, j)) mix_prepare_point(b, c, sc, in, out, i, j, (int)blockIdx.y, r_pt, r_pf);
   block_max_atomic(lean_detail::abs_max(r_pt, 0.0), red + RED_PT);
   block_max_atomic(lean_detail::abs_max(r_pf, 0.0), red + RED_PF);
 }
@@ -584,10 +585,10 @@ void mix_perm(cudaStream_t s, Box b, const LeanCoef<double>& c, const double* ph
   const Plane pl = plane_of(b, 0);
   launch_chained(k_mix_perm, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, phi, logk, perm, pl);
 }
-void mix_prepare(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixPrepIn& in, const MixPrepOut& out,
-                 unsigned long long* red) {
+void mix_prepare(cudaStream_t s, Box b, const LeanCoef<double>& c, const StressCoef& sc, const MixPrepIn& in,
+                 const MixPrepOut& out, unsigned long long* red) {
   const Plane pl = plane_of(b, c.bg_on ? 1 : 0);   // wall edges carry stress under a background shear only
-  launch_chained(k_mix_prepare, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, in, out, red, pl);
+  launch_chained(k_mix_prepare, plane_grid(pl, b.nz), kPlaneThreads, 0, s, b, c, sc, in, out, red, pl);
 }
 void mix_faces(cudaStream_t s, Box b, const LeanCoef<double>& c, const MixFaceIn& in, const MixFaceOut& out,
                unsigned long long* red) {
@@ -863,7 +864,7 @@ __global__ void __launch_bounds__(kMbBX * kMbBY) k_mb_points(const MixBatchInst*
                           I.Pt[a], I.Pf[a], I.phi[a], I.eta, I.perm, I.Pto, I.Pfo};
       const MixPrepOut pout{I.s_txx, I.s_tyy, I.s_tzz, I.s_txy, I.s_txz, I.s_tyz, I.rpt, I.rpf, I.ccf, I.kf, I.idtp};
       double r_pt = 0.0, r_pf = 0.0;
-      mix_prepare_point(b, I.lc, pin, pout, i, j, kz, r_pt, r_pf);
+      mix_prepare_point(b, I.lc, I.sc, pin, pout, i, j, kz, r_pt, r_pf);
       block_max_atomic(lean_detail::abs_max(r_pt, 0.0), I.red + RED_PT);
       block_max_atomic(lean_detail::abs_max(r_pf, 0.0), I.red + RED_PF);
     } else if (PHASE == MB_PH_FACES) {
