@@ -153,7 +153,8 @@ __device__ __forceinline__ void df_cells_run(const Box& b, const LeanCoef<df64>&
     col.k_d = in.perm[d];
     col.vx_d = in.Vx[d];
     col.vy_d = in.Vy[d];
-    col.fz = dfu::mul(dfu::add(col.k_d, in.perm[q]), dfu::add(dfu::sub(in.Pf[q], in.Pf[d]), c.buoy_dz));
+    // as df_cell_level forms it, so that both cells of a chunk's boundary take the same flux
+    col.fz = (col.k_d + in.perm[q]) * (dfu::subn(in.Pf[q], in.Pf[d]) + c.buoy_dz);
   }
   const df64* const t3 = st + (threadIdx.y + 1) * kDfW + threadIdx.x + 2;
   const df64* const tp = st + kDfPW + 32 * threadIdx.y + threadIdx.x;
