@@ -216,7 +216,7 @@ int pt_peak_arith(int32_t kind, void *sink, int32_t steps, int32_t reps, void *s
  * elements, device pointers, synchronises `stream`. It exists so that each replacement of a
  * library operation can be compared with CUDA's own function and with its stated error bound:
  *   PT_MATH_RCP_PSEUDO   1/x, approximate FP64 reciprocal + one Newton-Raphson step (~2^-46)
- *   PT_MATH_RCP_FULL     1/x, approximate FP64 reciprocal + two Newton-Raphson steps (rounding)
+ *   PT_MATH_RCP_FULL     1/x, approximate FP64 reciprocal + one third-order step (rounding)
  *   PT_MATH_EXPM1_POS/NEG  expm1(x), expm1(-x) from the split Taylor series of exp (tiers
  *                          |x| <= 2^-20, <= 2^-6; beyond, CUDA's expm1)
  *   PT_MATH_DF_ADD/SUB/MUL   double-float a + b, a - b, a * b (inputs rounded to double-float)
@@ -226,11 +226,16 @@ int pt_peak_arith(int32_t kind, void *sink, int32_t steps, int32_t reps, void *s
  *   PT_MATH_DF_EXPM1_POS/NEG  the split Taylor series in double-float
  *   PT_MATH_TO_FLOAT     a rounded to FP32 on the integer units (to nearest even)
  *   PT_MATH_HALF         a / 2 on the integer units (|a| >= 2^-1021, infinite or NaN)
+ *   PT_MATH_SQRT_FULL    sqrt(a) from the approximate FP64 reciprocal root, third order (rounding)
+ *   PT_MATH_ROOT_FULL    a^(1/m), m = (int)b[e] (FP32 seed and a binomial series; |log2 a| > 60: library)
+ *   PT_MATH_DF_RCP_SUM   double-float 1/(a + b) of the unnormalised sum (approximate FP32 reciprocal,
+ *                        third-order step)
  * Returns PT_EINVAL for an unknown code or a missing operand. */
 enum { PT_MATH_RCP_PSEUDO = 0, PT_MATH_RCP_FULL = 1, PT_MATH_EXPM1_POS = 2, PT_MATH_EXPM1_NEG = 3,
        PT_MATH_DF_ADD = 4, PT_MATH_DF_SUB = 5, PT_MATH_DF_MUL = 6, PT_MATH_DF_FMA = 7,
        PT_MATH_DF_RCP = 8, PT_MATH_DF_SQRT = 9, PT_MATH_DF_ROOT = 10, PT_MATH_DF_EXPM1_POS = 11,
-       PT_MATH_DF_EXPM1_NEG = 12, PT_MATH_TO_FLOAT = 13, PT_MATH_HALF = 14 };
+       PT_MATH_DF_EXPM1_NEG = 12, PT_MATH_TO_FLOAT = 13, PT_MATH_HALF = 14,
+       PT_MATH_SQRT_FULL = 15, PT_MATH_ROOT_FULL = 16, PT_MATH_DF_RCP_SUM = 17 };
 int pt_math_check(int32_t fn, const double *a, const double *b, double *out, int64_t n, void *stream);
 
 /* ---- Residual norms with no allocation at all -------------------------------------------

@@ -1256,7 +1256,8 @@ void pt_destroy(pt_ctx* c) {
 
 int pt_math_check(int32_t fn, const double* a, const double* b, double* out, int64_t n, void* stream) {
   if (fn < 0 || fn >= MATH_COUNT || !a || !out || n < 0) return PT_EINVAL;
-  if ((fn == MATH_DF_ADD || fn == MATH_DF_SUB || fn == MATH_DF_MUL || fn == MATH_DF_FMA || fn == MATH_DF_ROOT) && !b)
+  if ((fn == MATH_DF_ADD || fn == MATH_DF_SUB || fn == MATH_DF_MUL || fn == MATH_DF_FMA || fn == MATH_DF_ROOT ||
+       fn == MATH_ROOT_FULL || fn == MATH_DF_RCP_SUM) && !b)
     return PT_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   math_check(st, fn, a, b, out, (long long)n);

@@ -145,7 +145,7 @@ void df64_convert(cudaStream_t st, const DfCopy& cp, int narrays, long long n, b
 enum { MATH_RCP_PSEUDO = 0, MATH_RCP_FULL = 1, MATH_EXPM1_POS = 2, MATH_EXPM1_NEG = 3, MATH_DF_ADD = 4,
        MATH_DF_SUB = 5, MATH_DF_MUL = 6, MATH_DF_FMA = 7, MATH_DF_RCP = 8, MATH_DF_SQRT = 9,
        MATH_DF_ROOT = 10, MATH_DF_EXPM1_POS = 11, MATH_DF_EXPM1_NEG = 12, MATH_TO_FLOAT = 13,
-       MATH_HALF = 14, MATH_COUNT = 15 };
+       MATH_HALF = 14, MATH_SQRT_FULL = 15, MATH_ROOT_FULL = 16, MATH_DF_RCP_SUM = 17, MATH_COUNT = 18 };
 void math_check(cudaStream_t st, int fn, const double* a, const double* b, double* out, long long n);
 
 }  // namespace pt

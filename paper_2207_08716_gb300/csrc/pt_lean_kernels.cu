@@ -361,6 +361,9 @@ __global__ void k_math_check(int fn, const double* __restrict__ a, const double*
       case MATH_DF_EXPM1_POS: expm1_pair(df64(x), dp, dm); r = (double)dp; break;
       case MATH_TO_FLOAT: r = (double)to_float(x); break;
       case MATH_HALF: r = half_of(x); break;
+      case MATH_SQRT_FULL: r = sqrt_full(x); break;
+      case MATH_ROOT_FULL: r = root_full(x, rcp_full(x), (int)y, root_series((int)y)); break;
+      case MATH_DF_RCP_SUM: r = (double)dfu::rcp(dfu::add(df64(x), df64(y))); break;
       case MATH_DF_EXPM1_NEG: expm1_pair(df64(x), dp, dm); r = (double)dm; break;
       default: r = nan(""); break;
     }
