@@ -78,7 +78,7 @@ __device__ __forceinline__ void mix_prepare_point(const Box& b, const LeanCoef<d
     out.r_pf[q] = to_float(rpf);
     out.cc[q] = to_float(cc);
     out.perm[q] = to_float(kc);
-    out.idtp[q] = to_float(rcp_pseudo(c.dtaupt_fac * mu));   // good to 2^-39, kept in FP32
+    out.idtp[q] = to_float(rcp_full(c.dtaupt_fac * mu));
     r_pt = divVn;
     r_pf = rpf;
   }
@@ -120,7 +120,7 @@ __device__ __forceinline__ void mix_faces_point(const Box& b, const LeanCoef<dou
   lean_picard_point(b, c, t, in.mu, in.eta, i, j, k, pic);
   const double mu = in.mu[q];
   out.mu[q] = to_float(mu);
-  out.dtvc[q] = to_float(c.dtauv_fac * rcp_pseudo(mu));
+  out.dtvc[q] = to_float(c.dtauv_fac * rcp_full(mu));
 }
 
 // phi^{k+1} = 1 - (1 - phi_o) exp(delta) at the corrected state, delta = -[beta_phi ((Pf1 - Pfo) -
