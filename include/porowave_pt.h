@@ -326,14 +326,14 @@ int pt_mg_axis_tables(int32_t nf, uint32_t *out, size_t words);
  * FP64 ensembles (the FP64-lean form): 2 nup (or 4 nup) PT iterations per replay; each instance
  * stops at its own first check with norms < tol (or at its max_iter / a non-finite norm). The
  * first pt_batch_step tunes the tile shape (32x4, 32x8, 64x4) and the iterations per replay.
- * FP32 ensembles (the FP32 + FP64 defect-correction form): a replay runs `rounds` rounds of
- * [FP64 residuals, stresses and Picard update of the instances starting an outer iteration;
+ * FP32 ensembles (the FP32 + FP64 defect-correction form): a replay runs a round of [FP64 residuals, stresses and Picard update of the instances starting an outer iteration;
  * their outer decision (converged, outer weight, inner target); nup FP32 correction iterations
  * of the instances in a correction solve; their inner decision (relative drop reached or budget
  * spent); the FP64 update and porosity integration of the instances ending one], the instances
  * split into contiguous groups whose rounds are parallel branches of the graph. The first
- * pt_batch_step tunes the correction tile depth (32, 64 levels), the CTAs per SM of the
- * correction kernel (3, 4), the rounds per replay (1, 2) and the groups (1, 4, 8, 16).
+ * pt_batch_steps tune the correction tile depth (32, 64 levels) and the groups (1, 4, 8, 16): a
+ * round each, timed on its correction iterations alone, until every configuration has been timed
+ * on the same number of iterations of every instance (see pt_batch_tuner_check).
  * Either way each instance reproduces its single-instance pt_step: the same per-point code and
  * the same decisions in the same order, so the same iteration counts and statuses, and fields
  * equal to rounding (the shared bodies inlined into other kernels may round their multiply-adds
@@ -354,11 +354,18 @@ int pt_batch_step(pt_batch *batch, pt_report *reps, double *time_to_converge_ms)
  * (FP32 ensembles: the correction tile, 30 x 6 faces) and the (correction) iterations per replay. */
 int pt_batch_config(const pt_batch *batch, int32_t *tile_x, int32_t *tile_y,
                     int32_t *iters_per_graph);
-/* FP32 ensembles: the tuned correction tile depth (z levels), CTAs per SM of the correction
- * kernel and number of member groups (contiguous groups of near-equal cells whose rounds are
+/* FP32 ensembles: the tuned correction tile depth (z levels; the fastest so far while steps are
+ * still tuning), resident CTAs per SM of the correction kernel and number of member groups (contiguous groups of near-equal cells whose rounds are
  * parallel branches of the replayed graph); PT_EINVAL for an FP64 ensemble. */
 int pt_batch_config_fp32(const pt_batch *batch, int32_t *tile_z, int32_t *blocks_per_sm,
                          int32_t *groups);
+/* Host-only check of the FP32 ensembles' choice of a configuration (test aid): nrounds rounds of
+ * ninst instances, round r in step step[r], in which instance m runs sweeps[r ninst + m] correction
+ * iterations and configuration k would take ms[r K + k] for them, K = pt_batch_tuner_configs().
+ * Writes the configuration each round runs in, whether that round is timed, and the choice at the end. */
+int32_t pt_batch_tuner_configs(void);
+int pt_batch_tuner_check(int32_t ninst, int32_t nrounds, const int32_t *step, const int32_t *sweeps, const float *ms,
+                         int32_t *config, int32_t *timed, int32_t *best);
 void pt_batch_destroy(pt_batch *batch);
 
 /* ---- Sub-domain (halo-exchange) form (Art. 1 Section 2.2) ----------------------------------

@@ -26,6 +26,7 @@
 #include "pt_adjoint.cuh"
 #include "pt_dd.cuh"
 #include "pt_host.h"
+#include "pt_tuner.h"
 
 using namespace pt;
 
@@ -1305,19 +1306,23 @@ struct pt_batch {
   DDTables tables;
   std::vector<std::array<int, 6>> own;   // per instance: own_lo[3], own_hi[3]
   // FP32 ensembles (every instance PT_FP32): the defect-correction engine of pt_mixed.cuh, its
-  // decisions taken on the device per member; one graph replay = `mult` rounds of nup
-  // correction iterations with the outer phases between them
+  // decisions taken on the device per member; one graph replay = one round of nup correction
+  // iterations between the outer phases
   bool mixed;
   std::vector<MixBatchInst> h_minst;
   MixBatchInst* d_minst;
   MixBatchStatus* d_mst;
   MixBatchStatus* h_mst;
   unsigned long long* d_ired;
-  int zchunk, mult;         // correction tile depth, rounds per replay
+  int zchunk;               // correction tile depth
   int groups;               // members split into this many contiguous groups, each a parallel graph branch
   long long nptiles, nctiles;
   int pgrid, cgrid;
-  int exec_zchunk, exec_mult, exec_groups;
+  int exec_zchunk, exec_groups;
+  bool exec_timed;
+  MixTuner tuner;
+  std::vector<int> ran, sweeps;         // correction iterations of each member: in the step, in a timed round
+  cudaEvent_t tevent[2];                // around a timed replay's correction sweeps
   std::vector<int> gm;                  // group g = members [gm[g], gm[g + 1])
   std::vector<cudaStream_t> gstream;    // capture streams of the branches
   std::vector<cudaEvent_t> gevent;      // fork (0) and one join per branch
@@ -1526,58 +1531,85 @@ void split_mix_groups(pt_batch* B) {
   B->gm.push_back(B->ninst);
 }
 
-// The rounds of one member group on stream `s`: outer phases, nup correction iterations, update.
-void record_mix_group(pt_batch* B, int g, cudaStream_t s) {
-  const int m0 = B->gm[g], m1 = B->gm[g + 1], n = m1 - m0;
-  const MixBatchInst* inst = B->d_minst + m0;
-  MixBatchStatus* st = B->d_mst + m0;
-  const MixBatchInst& first = B->h_minst[m0];
-  const long long p0 = first.tile_base, c0 = first.ctile_base;
-  const long long p1 = m1 < B->ninst ? B->h_minst[m1].tile_base : B->nptiles;
-  const long long c1 = m1 < B->ninst ? B->h_minst[m1].ctile_base : B->nctiles;
-  for (int r = 0; r < B->mult; ++r) {
-    mb_points(B->pgrid, s, MB_PH_PERM, inst, st, n, p0, p1);
-    mb_points(B->pgrid, s, MB_PH_PREP, inst, st, n, p0, p1);
-    mb_points(B->pgrid, s, MB_PH_FACES, inst, st, n, p0, p1);
-    mb_decide_outer(s, inst, st, n);
-    mb_points(B->pgrid, s, MB_PH_INIT, inst, st, n, p0, p1);
-    for (int k = 1; k <= B->nup; ++k) mb_corr(B->cgrid, s, inst, st, n, c0, c1, k, B->nup, B->zchunk);
-    mb_decide_inner(s, inst, st, n, B->nup);
-    mb_points(B->pgrid, s, MB_PH_UPDATE, inst, st, n, p0, p1);
-    mb_points(B->pgrid, s, MB_PH_POROSITY, inst, st, n, p0, p1);
-    mb_finish(s, inst, st, n);
-  }
+// A range of members [m0, m1) with its point tiles [p0, p1) and correction tiles [c0, c1).
+struct MixRange {
+  const MixBatchInst* inst;
+  MixBatchStatus* st;
+  int n;
+  long long p0, p1, c0, c1;
+};
+MixRange mix_range(pt_batch* B, int m0, int m1) {
+  const bool end = m1 == B->ninst;
+  return MixRange{B->d_minst + m0, B->d_mst + m0, m1 - m0,
+                  B->h_minst[m0].tile_base, end ? B->nptiles : B->h_minst[m1].tile_base,
+                  B->h_minst[m0].ctile_base, end ? B->nctiles : B->h_minst[m1].ctile_base};
 }
 
-// One replay: the member groups as parallel branches (they share no data), forked from and
+// The three parts of a round on stream `s`: outer phases, nup correction iterations, update.
+void record_mix_outer(pt_batch* B, const MixRange& r, cudaStream_t s) {
+  mb_points(B->pgrid, s, MB_PH_PERM, r.inst, r.st, r.n, r.p0, r.p1);
+  mb_points(B->pgrid, s, MB_PH_PREP, r.inst, r.st, r.n, r.p0, r.p1);
+  mb_points(B->pgrid, s, MB_PH_FACES, r.inst, r.st, r.n, r.p0, r.p1);
+  mb_decide_outer(s, r.inst, r.st, r.n);
+  mb_points(B->pgrid, s, MB_PH_INIT, r.inst, r.st, r.n, r.p0, r.p1);
+}
+void record_mix_sweeps(pt_batch* B, const MixRange& r, cudaStream_t s) {
+  for (int k = 1; k <= B->nup; ++k) mb_corr(B->cgrid, s, r.inst, r.st, r.n, r.c0, r.c1, k, B->nup, B->zchunk);
+}
+void record_mix_update(pt_batch* B, const MixRange& r, cudaStream_t s) {
+  mb_decide_inner(s, r.inst, r.st, r.n, B->nup);
+  mb_points(B->pgrid, s, MB_PH_UPDATE, r.inst, r.st, r.n, r.p0, r.p1);
+  mb_points(B->pgrid, s, MB_PH_POROSITY, r.inst, r.st, r.n, r.p0, r.p1);
+  mb_finish(s, r.inst, r.st, r.n);
+}
+
+// `part` of every member group, the groups as parallel branches (they share no data), forked from and
 // joined into the batch's stream.
-void record_mix_rounds(pt_batch* B) {
-  split_mix_groups(B);
+template <class F>
+void record_mix_groups(pt_batch* B, F part) {
   const int G = (int)B->gm.size() - 1;
   if (G == 1) {
-    record_mix_group(B, 0, B->stream);
+    part(mix_range(B, 0, B->ninst), B->stream);
     return;
   }
   cudaEventRecord(B->gevent[0], B->stream);
   for (int g = 0; g < G; ++g) {
     cudaStreamWaitEvent(B->gstream[g], B->gevent[0], 0);
-    record_mix_group(B, g, B->gstream[g]);
+    part(mix_range(B, B->gm[g], B->gm[g + 1]), B->gstream[g]);
     cudaEventRecord(B->gevent[1 + g], B->gstream[g]);
   }
   for (int g = 0; g < G; ++g) cudaStreamWaitEvent(B->stream, B->gevent[1 + g], 0);
 }
 
-int build_mix_graph(pt_batch* B) {
-  if (B->exec && B->exec_zchunk == B->zchunk && B->exec_mult == B->mult &&
-      B->exec_groups == B->groups)
-    return PT_OK;
+// One replay: a round of every group; timed, the groups branch for the correction sweeps alone, between
+// the two timing events.
+void record_mix_round(pt_batch* B, bool timed) {
+  split_mix_groups(B);
+  if (!timed) {
+    record_mix_groups(B, [&](const MixRange& r, cudaStream_t s) {
+      record_mix_outer(B, r, s);
+      record_mix_sweeps(B, r, s);
+      record_mix_update(B, r, s);
+    });
+    return;
+  }
+  const MixRange all = mix_range(B, 0, B->ninst);
+  record_mix_outer(B, all, B->stream);
+  cudaEventRecordWithFlags(B->tevent[0], B->stream, cudaEventRecordExternal);
+  record_mix_groups(B, [&](const MixRange& r, cudaStream_t s) { record_mix_sweeps(B, r, s); });
+  cudaEventRecordWithFlags(B->tevent[1], B->stream, cudaEventRecordExternal);
+  record_mix_update(B, all, B->stream);
+}
+
+int build_mix_graph(pt_batch* B, bool timed) {
+  if (B->exec && B->exec_zchunk == B->zchunk && B->exec_groups == B->groups && B->exec_timed == timed) return PT_OK;
   if (B->exec) {
     cudaGraphExecDestroy(B->exec);
     B->exec = nullptr;
   }
   cudaGraph_t g = nullptr;
   if (cudaStreamBeginCapture(B->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return PT_ECUDA;
-  record_mix_rounds(B);
+  record_mix_round(B, timed);
   cudaError_t e = cudaStreamEndCapture(B->stream, &g);
   if (e == cudaSuccess) e = cudaGraphInstantiate(&B->exec, g, 0);
   if (g) cudaGraphDestroy(g);
@@ -1586,8 +1618,8 @@ int build_mix_graph(pt_batch* B) {
     return PT_ECUDA;
   }
   B->exec_zchunk = B->zchunk;
-  B->exec_mult = B->mult;
   B->exec_groups = B->groups;
+  B->exec_timed = timed;
   return PT_OK;
 }
 
@@ -1613,8 +1645,7 @@ struct TunerEvents {
 };
 
 // FP32 ensemble step: every member's step begin (host, as pt_step), then graph replays until
-// every member is done; the first step times one replay of each candidate configuration
-// (correction tile depth, member groups) and keeps the fastest per round.
+// every member is done, in the configuration (correction tile depth, member groups) that the tuner picks.
 int batch_step_mixed(pt_batch* B, pt_report* reps, double* ttc_ms) {
   int rc = PT_OK;
   int cap = 0;
@@ -1624,54 +1655,37 @@ int batch_step_mixed(pt_batch* B, pt_report* reps, double* ttc_ms) {
   }
   if (rc != PT_OK) return rc;
   if (cudaStreamSynchronize(B->stream) != cudaSuccess) return PT_ECUDA;
-  if (upload_mix(B) != cudaSuccess) return PT_ECUDA;
-  mb_start(B->stream, B->d_minst, B->d_mst, B->ninst);
   // every round advances each member that is not done: an outer iteration takes at least one
   // round and at least min(nup, budget) correction iterations, so this many rounds end every member
   const long long max_rounds = 2LL * ((long long)cap / B->nup + 2) + 4;
-  struct Cfg { int zchunk, mult, groups; };
-  const Cfg cands[] = {{64, 1, 1}, {32, 1, 1}, {64, 1, 4}, {32, 1, 4}, {32, 1, 8}, {64, 1, 8}, {64, 1, 16}};
-  const int ncand = B->tuned ? 0 : (int)(sizeof cands / sizeof cands[0]);
-  float best_ms = 1e30f;
-  Cfg best = {B->zchunk, B->mult, B->groups};
   long long rounds = 0;
   int nactive = B->ninst;
-  TunerEvents ev;
-  if (ncand && !ev.create()) return PT_ECUDA;
-  for (int t = 0; t < ncand && nactive > 0 && rounds < max_rounds; ++t) {
-    B->zchunk = cands[t].zchunk;
-    B->mult = cands[t].mult;
-    B->groups = cands[t].groups;
-    if (upload_mix(B) != cudaSuccess) return PT_ECUDA;
-    rc = build_mix_graph(B);
-    if (rc != PT_OK) return rc;
-    cudaEventRecord(ev.e0, B->stream);
-    if (cudaGraphLaunch(B->exec, B->stream) != cudaSuccess) return PT_ECUDA;
-    cudaEventRecord(ev.e1, B->stream);
-    rounds += B->mult;
-    rc = mix_active(B, &nactive);
-    if (rc != PT_OK) return rc;
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, ev.e0, ev.e1);
-    if (ms / B->mult < best_ms) {
-      best_ms = ms / B->mult;
-      best = cands[t];
+  std::fill(B->ran.begin(), B->ran.end(), 0);
+  B->tuner.begin_step();
+  for (; nactive > 0 && rounds < max_rounds; ++rounds) {
+    const bool timed = B->tuner.timing();
+    const MixConfig& cf = kMixConfigs[B->tuner.config()];
+    if (rounds == 0 || cf.zchunk != B->zchunk || cf.groups != B->groups) {
+      B->zchunk = cf.zchunk;
+      B->groups = cf.groups;
+      if (upload_mix(B) != cudaSuccess) return PT_ECUDA;
     }
-  }
-  if (ncand) {
-    B->zchunk = best.zchunk;
-    B->mult = best.mult;
-    B->groups = best.groups;
-    B->tuned = true;
-    if (upload_mix(B) != cudaSuccess) return PT_ECUDA;
-  }
-  rc = build_mix_graph(B);
-  if (rc != PT_OK) return rc;
-  while (nactive > 0 && rounds < max_rounds) {
+    if (rounds == 0) mb_start(B->stream, B->d_minst, B->d_mst, B->ninst);
+    rc = build_mix_graph(B, timed);
+    if (rc != PT_OK) return rc;
     if (cudaGraphLaunch(B->exec, B->stream) != cudaSuccess) return PT_ECUDA;
-    rounds += B->mult;
     rc = mix_active(B, &nactive);
     if (rc != PT_OK) return rc;
+    if (timed) {
+      for (int m = 0; m < B->ninst; ++m) {
+        const int total = B->h_mst[m].iters + B->h_mst[m].inner;
+        B->sweeps[m] = total - B->ran[m];
+        B->ran[m] = total;
+      }
+      float ms = 0.f;
+      if (cudaEventElapsedTime(&ms, B->tevent[0], B->tevent[1]) != cudaSuccess) return PT_ECUDA;
+      B->tuner.timed_round(B->sweeps, ms);
+    }
   }
   if (nactive > 0) return PT_ECUDA;   // cannot happen: see max_rounds
   int any_nc = 0, any_nan = 0;
@@ -1753,12 +1767,18 @@ int pt_batch_init(pt_batch** out, int32_t ninst, const pt_grid* grids, const pt_
   B->h_inst.resize(ninst);
   B->mixed = fp32;
   B->zchunk = 64;
-  B->mult = 1;
   B->groups = 1;
-  B->exec_zchunk = B->exec_mult = B->exec_groups = 0;
+  B->exec_zchunk = B->exec_groups = 0;
+  B->exec_timed = false;
+  B->tevent[0] = B->tevent[1] = nullptr;
   B->h_st = nullptr;
   B->h_mst = nullptr;
-  if (fp32) B->h_minst.resize(ninst);
+  if (fp32) {
+    B->h_minst.resize(ninst);
+    B->ran.resize(ninst);
+    B->sweeps.resize(ninst);
+    B->tuner.reserve(ninst);
+  }
   char* w = (char*)workspace;
   int rc = PT_OK;
   if (fp32) {   // capture streams and events of the parallel member groups (up to 16)
@@ -1768,6 +1788,8 @@ int pt_batch_init(pt_batch** out, int32_t ninst, const pt_grid* grids, const pt_
       if (rc == PT_OK && cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking) != cudaSuccess) rc = PT_ECUDA;
     for (cudaEvent_t& e : B->gevent)
       if (rc == PT_OK && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) rc = PT_ECUDA;
+    for (cudaEvent_t& e : B->tevent)
+      if (rc == PT_OK && cudaEventCreate(&e) != cudaSuccess) rc = PT_ECUDA;
   }
   for (int m = 0; m < ninst && rc == PT_OK; ++m) {
     const size_t s = pt_workspace_size(&grids[m], &nums[m]);
@@ -1795,6 +1817,8 @@ int pt_batch_init(pt_batch** out, int32_t ninst, const pt_grid* grids, const pt_
     for (cudaStream_t q : B->gstream)
       if (q) cudaStreamDestroy(q);
     for (cudaEvent_t e : B->gevent)
+      if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : B->tevent)
       if (e) cudaEventDestroy(e);
     cudaStreamDestroy(B->stream);
     delete B;
@@ -1907,19 +1931,38 @@ int pt_mg_axis_tables(int32_t nf, uint32_t* out, size_t words) {
   return PT_OK;
 }
 
+int32_t pt_batch_tuner_configs(void) { return kMixConfigCount; }
+
+int pt_batch_tuner_check(int32_t ninst, int32_t nrounds, const int32_t* step, const int32_t* sweeps, const float* ms,
+                         int32_t* config, int32_t* timed, int32_t* best) {
+  if (ninst < 1 || nrounds < 0 || !step || !sweeps || !ms || !config || !timed || !best) return PT_EINVAL;
+  MixTuner t;
+  std::vector<int> ran(ninst);
+  for (int r = 0; r < nrounds; ++r) {
+    if (r == 0 || step[r] != step[r - 1]) t.begin_step();
+    config[r] = t.config();
+    timed[r] = t.timing();
+    ran.assign(sweeps + (size_t)r * ninst, sweeps + (size_t)(r + 1) * ninst);
+    if (timed[r]) t.timed_round(ran, ms[(size_t)r * kMixConfigCount + config[r]]);
+  }
+  *best = t.best();
+  return PT_OK;
+}
+
 int pt_batch_config(const pt_batch* B, int32_t* tile_x, int32_t* tile_y, int32_t* ipg) {
   if (!B) return PT_EINVAL;
   if (tile_x) *tile_x = B->mixed ? corr_tile_x() : B->bx;
   if (tile_y) *tile_y = B->mixed ? corr_tile_y() : B->by;
-  if (ipg) *ipg = B->mixed ? B->mult * B->nup : B->ipg;
+  if (ipg) *ipg = B->mixed ? B->nup : B->ipg;
   return PT_OK;
 }
 
 int pt_batch_config_fp32(const pt_batch* B, int32_t* tile_z, int32_t* blocks_per_sm, int32_t* groups) {
   if (!B || !B->mixed) return PT_EINVAL;
-  if (tile_z) *tile_z = B->zchunk;
+  const MixConfig& cf = kMixConfigs[B->tuner.best()];
+  if (tile_z) *tile_z = cf.zchunk;
   if (blocks_per_sm) *blocks_per_sm = mb_corr_blocks_per_sm();
-  if (groups) *groups = std::max(1, std::min(B->groups, B->ninst));
+  if (groups) *groups = std::max(1, std::min(cf.groups, B->ninst));
   return PT_OK;
 }
 
@@ -1933,6 +1976,8 @@ void pt_batch_destroy(pt_batch* B) {
   for (cudaStream_t q : B->gstream)
     if (q) cudaStreamDestroy(q);
   for (cudaEvent_t e : B->gevent)
+    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : B->tevent)
     if (e) cudaEventDestroy(e);
   cudaStreamDestroy(B->stream);
   delete B;

@@ -19,7 +19,7 @@ LIB_PATH = os.path.join(_BUILD, "libpt_gb300.so")
 SOURCES = ("pt_api.cu", "pt_ref_kernels.cu", "pt_lean_kernels.cu", "pt_mixed_kernels.cu",
            "pt_batch_kernels.cu", "pt_adjoint_kernels.cu", "pt_dd_kernels.cu", "pt_static.cu", "pt_peaks.cu",
            "rx_api.cu", "rx_kernels.cu", "rx_mg_kernels.cu")
-HEADERS = ("pt_common.cuh", "pt_host.h", "pt_kernels.cuh", "pt_ref_points.cuh", "pt_lean.cuh", "pt_lean_body.cuh", "pt_df_body.cuh", "df64.cuh", "pt_mixed.cuh", "pt_batch.cuh", "pt_adjoint.cuh", "pt_dd.cuh", "rx.cuh", "rx_quad.cuh")
+HEADERS = ("pt_common.cuh", "pt_host.h", "pt_tuner.h", "pt_kernels.cuh", "pt_ref_points.cuh", "pt_lean.cuh", "pt_lean_body.cuh", "pt_df_body.cuh", "df64.cuh", "pt_mixed.cuh", "pt_batch.cuh", "pt_adjoint.cuh", "pt_dd.cuh", "rx.cuh", "rx_quad.cuh")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 _lock = threading.Lock()
@@ -216,6 +216,9 @@ SIGNATURES = {
     "pt_batch_config_fp32": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                        C.POINTER(C.c_int32)]),
     "pt_mg_axis_words": (C.c_size_t, [C.c_int32]),
+    "pt_batch_tuner_configs": (C.c_int32, []),
+    "pt_batch_tuner_check": (C.c_int, [C.c_int32, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
+                                       C.c_void_p]),
     "pt_mg_axis_tables": (C.c_int, [C.c_int32, C.c_void_p, C.c_size_t]),
     "pt_batch_destroy": (None, [C.c_void_p]),
     "pt_destroy": (None, [C.c_void_p]),
