@@ -98,8 +98,8 @@ inline int sm_count() {
 // double-float and 7.6 instead of 10.6 (its share of the outer phases included) in FP32; from 127^3 cells on
 // the gain is 3 % and less. The previous kernel does not release its successor early: the waiting blocks
 // then land on the SMs in the uneven order in which these have room, which cost the FP64 kernels up to 27 %
-// at 32^3 to 48^3 and double-float 7 % at 383^3. The pointers of a chained kernel are not __restrict__, so
-// that no load moves above the wait.
+// at 32^3 to 48^3 and double-float 7 % at 383^3. The pointers of a chained kernel and of the functions
+// it inlines are not __restrict__, so that no load moves above the wait.
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>
 inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {

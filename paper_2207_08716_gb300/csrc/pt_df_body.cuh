@@ -203,9 +203,7 @@ __device__ __forceinline__ void df_cell_level(const Box& b, const LeanCoef<df64>
 
 // Momentum residual, damped R and velocity update of the three lower faces of the cell (i, j, k).
 __device__ __forceinline__ void df_face_point(const Box& b, const LeanCoef<df64>& c, const LeanFaceIn<df64>& in,
-                                              df64* __restrict__ Vx, df64* __restrict__ Vy, df64* __restrict__ Vz,
-                                              df64* __restrict__ Rx, df64* __restrict__ Ry, df64* __restrict__ Rz,
-                                              int i, int j, int k, int check, double& r_v) {
+                                              df64* Vx, df64* Vy, df64* Vz, df64* Rx, df64* Ry, df64* Rz, int i, int j, int k, int check, double& r_v) {
   using namespace dfu;
   if (i >= b.nx || j >= b.ny || k >= b.nz) return;   // the faces i = nx, j = ny, k = nz are walls
   const long long q = cidx(b, i, j, k);

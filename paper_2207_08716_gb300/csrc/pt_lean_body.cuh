@@ -364,10 +364,8 @@ __device__ __forceinline__ void lean_cell_level(const Box& b, const LeanCoef<dou
 // Momentum residual, damped R and velocity update of the three lower faces of (i, j, k) in FP64; bit d
 // of `mask` includes the face normal to direction d in the residual norm r_v.
 __device__ __forceinline__ void lean_face_point(const Box& b, const LeanCoef<double>& c, const LeanFaceIn<double>& in,
-                                                double* __restrict__ Vx, double* __restrict__ Vy,
-                                                double* __restrict__ Vz, double* __restrict__ Rx,
-                                                double* __restrict__ Ry, double* __restrict__ Rz, int i, int j, int k,
-                                                int check, double& r_v, int mask = 7) {
+                                                double* Vx, double* Vy, double* Vz, double* Rx, double* Ry, double* Rz,
+                                                int i, int j, int k, int check, double& r_v, int mask = 7) {
   if (i < b.nx && j < b.ny && k < b.nz) {   // the faces i = nx, j = ny, k = nz are walls
     const long long q = cidx(b, i, j, k);
     const long long px = b.px, pxy = b.pxy;
@@ -413,7 +411,7 @@ __device__ __forceinline__ void lean_face_point(const Box& b, const LeanCoef<dou
 // taken once per block by the caller (log is monotone).
 template <class T>
 __device__ __forceinline__ void lean_picard_point(const Box& b, const LeanCoef<T>& c, const LeanPicardIn<T>& in,
-                                                  T* __restrict__ mu, T* __restrict__ eta, int i, int j, int k,
+                                                  T* mu, T* eta, int i, int j, int k,
                                                   double& m) {
   using namespace lean_detail;
   if (i < b.nx && j < b.ny && k < b.nz) {
@@ -488,8 +486,7 @@ __device__ __forceinline__ void centre_stresses(const StressCoef& sc, double m, 
 // Shear stresses on the three lower edges of (i, j, k), zero on boundary edges unless a background
 // shear is applied (Eqs. 32-33). An edge's viscosity is the mean of its four centres'.
 __device__ __forceinline__ void stress_edges_point(const Box& b, const StressCoef& sc, const StressIn& in,
-                                                   double* __restrict__ txy, double* __restrict__ txz,
-                                                   double* __restrict__ tyz, int i, int j, int k) {
+                                                   double* txy, double* txz, double* tyz, int i, int j, int k) {
   if (i > b.nx || j > b.ny || k > b.nz) return;
   const long long q = cidx(b, i, j, k);
   const long long px = b.px, pxy = b.pxy;

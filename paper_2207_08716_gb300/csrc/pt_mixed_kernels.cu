@@ -30,9 +30,8 @@ namespace pt {
 // powers of two moved to the integer units, and fewer products, gave the last 1.2 ms.
 
 // k of the iterate (Eq. 23), read with its neighbours by mix_prepare_point.
-__device__ __forceinline__ void mix_perm_point(const Box& b, const LeanCoef<double>& c, const double* __restrict__ phi,
-                                               const double* __restrict__ logk, double* __restrict__ perm, int i,
-                                               int j, int k) {
+__device__ __forceinline__ void mix_perm_point(const Box& b, const LeanCoef<double>& c, const double* phi,
+                                               const double* logk, double* perm, int i, int j, int k) {
   if (i >= b.nx || j >= b.ny || k >= b.nz) return;
   const long long q = cidx(b, i, j, k);
   const double ph = phi[q], k3 = c.k0r3 * ph * ph * ph;

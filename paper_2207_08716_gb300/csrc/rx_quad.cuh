@@ -104,8 +104,8 @@ __device__ __forceinline__ QuadColumn quad_column(const Box& b, const RxCoef<flo
 // twice minus the divergence of the Darcy flux) and, with KD, kd[v] = sum of (k + k_nb) / d^2. Leaves the
 // column at level k + 1.
 template <bool KD>
-__device__ __forceinline__ void quad_level(const Box& b, const RxCoef<float>& c, const float* __restrict__ gPf,
-                                           const float* __restrict__ gphi, int i, int j, int k, QuadColumn& col,
+__device__ __forceinline__ void quad_level(const Box& b, const RxCoef<float>& c, const float* gPf,
+                                           const float* gphi, int i, int j, int k, QuadColumn& col,
                                            float (&Pf)[4], float (&ph)[4], float (&div)[4], float (&kd)[4]) {
   const long long q = cidx(b, i, j, k);
   const long long px = b.px, pxy = b.pxy;
