@@ -87,9 +87,6 @@ __device__ __forceinline__ bool operator<(df64 x, df64 y) { return x.hi < y.hi |
 __device__ __forceinline__ bool operator>(df64 x, df64 y) { return y < x; }
 __device__ __forceinline__ bool operator==(df64 x, df64 y) { return x.hi == y.hi && x.lo == y.lo; }
 
-// x * 2^k for a power of two given as a float (exact, both parts scaled)
-__device__ __forceinline__ df64 scale2(df64 x, float pow2) { return df64(x.hi * pow2, x.lo * pow2); }
-
 // 1 / x: FP32 correctly rounded seed r, then r + r d with d = 1 - x r from the exact product
 // x.hi r = p + q (|d| <= 2^-24, relative error ~2^-46).
 __device__ __forceinline__ df64 df_rcp(df64 x) {

@@ -209,8 +209,8 @@ LeanCoef<df64> lean_coef_df64(const LeanCoef<double>& L) {
 #define PT_DF(x) F.x = df64(L.x)
   PT_DF(rdx); PT_DF(rdy); PT_DF(rdz); PT_DF(hrdx); PT_DF(hrdy); PT_DF(hrdz);
   PT_DF(hrdx2); PT_DF(hrdy2); PT_DF(hrdz2); PT_DF(buoy_dz); PT_DF(bd_rdt); PT_DF(bda_B_rdt);
-  PT_DF(alpha); PT_DF(alpha_B); PT_DF(bd_rdt_a); PT_DF(beta_n); PT_DF(beta_phi); PT_DF(dt);
-  PT_DF(rphi0); PT_DF(k0); PT_DF(k0r3); PT_DF(phi0); PT_DF(drho_g); PT_DF(ifac_pf); PT_DF(rrho_i);
+  PT_DF(bd_rdt_a); PT_DF(beta_n); PT_DF(beta_phi); PT_DF(dt);
+  PT_DF(k0r3); PT_DF(phi0); PT_DF(drho_g); PT_DF(ifac_pf); PT_DF(rrho_i);
   PT_DF(damp_x); PT_DF(damp_y); PT_DF(damp_z); PT_DF(rdx_r); PT_DF(rdy_r); PT_DF(rdz_r);
   PT_DF(drho_g_r); PT_DF(rho_i); PT_DF(ebg); PT_DF(mu0); PT_DF(eta0); PT_DF(eta0_weak);
   PT_DF(rtau0_2h); PT_DF(rtau0_2s); PT_DF(rmu0); PT_DF(rGdtS); PT_DF(dtaupt_fac); PT_DF(dtauv_fac);
@@ -249,14 +249,10 @@ void fill_lean_coef(pt_ctx* c) {
   L.bg_on = k.bg_on;
   L.bd_rdt = k.beta_d * k.rdt;
   L.bda_B_rdt = k.beta_d * k.alpha / k.B * k.rdt;
-  L.alpha = k.alpha;
   L.bd_rdt_a = k.beta_d * k.alpha * k.rdt;
-  L.alpha_B = k.alpha / k.B;
   L.beta_n = k.beta_n;
   L.beta_phi = k.beta_phi;
   L.dt = k.dt;
-  L.rphi0 = k.rphi0;
-  L.k0 = k.k0;
   L.k0r3 = k.k0 * k.rphi0 * k.rphi0 * k.rphi0;
   L.phi0 = k.phi0;
   L.drho_g = p.rhof_g - p.rhos_g;
@@ -512,7 +508,6 @@ void launch_lean_coef(pt_ctx* c) {
 // (momentum, velocities), and on check iterations the Picard update and coefficient refresh.
 void launch_iteration_lean(pt_ctx* c, int check) {
   const Box& b = c->box;
-  const dim3 bl = block_dims(), gr = grid_dims(b);
   const int a = c->cur, n = 1 - c->cur;
   if (check) cudaMemsetAsync(c->red, 0, RED_N * sizeof(unsigned long long), c->stream);
   LeanCellIn<double> ci{c->Vx, c->Vy, c->Vz, c->Pt[a], c->Pf[a], c->phi[a], c->lw[a], c->lperm[a],
@@ -596,7 +591,6 @@ void df_cells(pt_ctx* c, int a, int n, int check) {
 // One PT iteration in double-float: the lean form's kernels on the df64 iterate.
 void launch_iteration_df(pt_ctx* c, int check) {
   const Box& b = c->box;
-  const dim3 bl = block_dims(), gr = grid_dims(b);
   const int a = c->fcur, n = 1 - a;
   if (check) cudaMemsetAsync(c->red, 0, RED_N * sizeof(unsigned long long), c->stream);
   df_cells(c, a, n, check);
@@ -699,7 +693,6 @@ void zero_arrays(void* first, size_t stride, size_t bytes, int count, cudaStream
 // (then no correction is run).
 int mixed_outer(pt_ctx* c, int n_in, bool early_exit, pt_report* outer, bool* converged, int* inner_done) {
   const Box& b = c->box;
-  const dim3 bl = block_dims(), gr = grid_dims(b);
   const int a = c->cur;
   *converged = false;
   *inner_done = 0;

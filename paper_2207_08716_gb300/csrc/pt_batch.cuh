@@ -47,7 +47,7 @@ void batch_phase(int bx, int by, int grid, cudaStream_t s, int phase, const Batc
 void batch_converge(cudaStream_t s, const BatchInst* inst, BatchStatus* st, int ninst, int nup, int coupled);
 // Start of a step: all instances active, counters zero, reduction slots clear, start time.
 void batch_start(cudaStream_t s, const BatchInst* inst, BatchStatus* st, int ninst);
-// Resident CTAs per SM of the batched cell kernel for a tile shape (occupancy of the widest phase).
+// Resident CTAs per SM of a phase's kernel for a tile shape.
 int batch_blocks_per_sm(int bx, int by, int phase);
 
 }  // namespace pt

@@ -37,10 +37,9 @@ struct LeanCoef {
   T hrdx2, hrdy2, hrdz2;        // 1 / (2 dx^2)
   T buoy_dz;                    // (rho_f - rho_BG) g dz
   T bd_rdt, bda_B_rdt;          // beta_d / dt, beta_d alpha / (B dt)
-  T alpha, alpha_B;             // alpha, alpha / B
   T bd_rdt_a;                   // beta_d alpha / dt
   T beta_n, beta_phi, dt;
-  T rphi0, k0, phi0, drho_g;    // 1 / phi0, k0, phi0, (rho_f - rho_s) g
+  T phi0, drho_g;               // phi0, (rho_f - rho_s) g
   T k0r3;                       // k0 / phi0^3
   T ifac_pf;                    // 1 / (cfl_pf h^2 (1 + beta_d B / alpha)): 1/dtau_Pf = kmax * ifac_pf
   T rrho_i, damp_x, damp_y, damp_z;

@@ -53,13 +53,6 @@ __device__ inline double pos_max(double a, double b) {
   const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
   return __longlong_as_double(ia > ib ? ia : ib);
 }
-__device__ inline float pos_max(float a, float b) {
-  const int ia = __float_as_int(a), ib = __float_as_int(b);
-  return __int_as_float(ia > ib ? ia : ib);
-}
-
-template <class T>
-__device__ inline T tabs(T x) { return x < T(0) ? -x : x; }
 
 // 1 / x for the local-implicit pseudo-step denominators (x > 0, far inside the normal range):
 // the hardware's approximate reciprocal refined by one Newton step, r' = r + r (1 - x r), whose
@@ -71,7 +64,6 @@ __device__ inline double rcp_pseudo(double x) {
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   return fma(r, fma(-x, r, 1.0), r);
 }
-__device__ inline float rcp_pseudo(float x) { return __frcp_rn(x); }
 
 // 1 / x to rounding accuracy for the coefficients that set the fixed point (x > 0, normal): one
 // third-order step r (1 + e + e^2), e = 1 - x r, on the hardware's approximate reciprocal r (good to
@@ -123,9 +115,7 @@ __device__ inline double root_full(double x, double rx, int m, const RootSeries&
 }
 
 // ---- the same operations in double-float (PT_DF64): one Newton step from the FP32 seed
-// reaches the format's own rounding (~2^-46), so the pseudo-step and the fixed-point
-// reciprocals are the same function
-__device__ inline df64 rcp_pseudo(df64 x) { return df_rcp(x); }
+// reaches the format's own rounding (~2^-46)
 __device__ inline df64 rcp_full(df64 x) { return df_rcp(x); }
 
 __device__ inline df64 pos_max(df64 a, df64 b) { return a < b ? b : a; }
@@ -152,20 +142,12 @@ __device__ inline df64 df_expm1(df64 d) {
   }
   return df64(expm1((double)d));
 }
-__device__ inline void expm1_pair(df64 d, df64& em_pos, df64& em_neg) {
-  em_pos = df_expm1(d);
-  em_neg = df_expm1(-d);
-}
 
 // conversions between the field type and FP64 (identity for FP64)
 __device__ inline double to_d(double x) { return x; }
 __device__ inline double to_d(df64 x) { return (double)x; }
 template <class T>
 __device__ inline T from_d(double x) { return T(x); }
-
-// a / b: the plain quotient in FP64, the refined reciprocal in double-float
-__device__ inline double tdiv(double a, double b) { return a / b; }
-__device__ inline df64 tdiv(df64 a, df64 b) { return a * df_rcp(b); }
 
 // x^rel of the log-space Picard relaxation (x > 0, rx = 1/x): the square root for rel = 1/2, the
 // m-th root for rel = 1/m (root = m, set on the host), else exp(rel log x) in FP64.

@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(256) k_lean_begin(Box b, LeanCoef<T> c, LeanBe
     out.phio[q] = ph;
     if constexpr (!LeanRecompute<T>::value) {   // the recomputing forms derive these from phi
       const T Eo = T(1.0) - ph;
-      const T iEo = tdiv(T(1.0), Eo);
+      const T iEo = T(1.0) / Eo;
       out.Eo[q] = Eo;
       out.iEo[q] = iEo;
       out.w[q] = iEo;
@@ -345,7 +345,6 @@ __global__ void k_math_check(int fn, const double* __restrict__ a, const double*
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const double x = a[e], y = b ? b[e] : 0.0;
     double r = 0.0, p = 0.0, m = 0.0;
-    df64 dp, dm;
     switch (fn) {
       case MATH_RCP_PSEUDO: r = rcp_pseudo(x); break;
       case MATH_RCP_FULL: r = rcp_full(x); break;
@@ -358,13 +357,13 @@ __global__ void k_math_check(int fn, const double* __restrict__ a, const double*
       case MATH_DF_RCP: r = (double)df_rcp(df64(x)); break;
       case MATH_DF_SQRT: r = (double)df_sqrt(df64(x)); break;
       case MATH_DF_ROOT: r = (double)df_root(df64(x), (int)y); break;
-      case MATH_DF_EXPM1_POS: expm1_pair(df64(x), dp, dm); r = (double)dp; break;
+      case MATH_DF_EXPM1_POS: r = (double)df_expm1(df64(x)); break;
       case MATH_TO_FLOAT: r = (double)to_float(x); break;
       case MATH_HALF: r = half_of(x); break;
       case MATH_SQRT_FULL: r = sqrt_full(x); break;
       case MATH_ROOT_FULL: r = root_full(x, rcp_full(x), (int)y, root_series((int)y)); break;
       case MATH_DF_RCP_SUM: r = (double)dfu::rcp(dfu::add(df64(x), df64(y))); break;
-      case MATH_DF_EXPM1_NEG: expm1_pair(df64(x), dp, dm); r = (double)dm; break;
+      case MATH_DF_EXPM1_NEG: r = (double)df_expm1(-df64(x)); break;
       default: r = nan(""); break;
     }
     out[e] = r;

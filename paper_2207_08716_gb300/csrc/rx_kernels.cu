@@ -3,7 +3,7 @@
 // (FP64: stored with phi; FP32: from phi) with their six neighbours (Darcy flux, k averaged to the
 // faces), phi, Xs and the old step, and writes the next Pf, phi, Xs (FP64: and k(phi')): 6 arrays read
 // and 3 written in FP32, 7 and 4 in FP64 (the rate dPf/dt only on check and final iterations). Divisions
-// are Newton-refined hardware reciprocals (rx_rcp).
+// are refined hardware reciprocals (rx_rcp).
 #include "rx_quad.cuh"
 #include "rx.cuh"
 
