@@ -80,12 +80,12 @@ KERNEL_SOURCES = {
 }
 PROFILED = {
     # profiles/kernels_191_ncu_metrics.md (191^3, every launch of one step of each form)
-    "k_lean_cells": {"src": "a351ee1fa12c90bf", "fp64_inst": 94.0, "fp64_flops": 139.2, "traffic": 312.1},
-    "k_lean_faces": {"src": "a351ee1fa12c90bf", "fp64_inst": 32.9, "fp64_flops": 49.8, "traffic": 180.3},
-    "k_lean_cells_df64": {"src": "a351ee1fa12c90bf", "traffic": 259.9, "thread_inst": 1383.0},
-    "k_lean_faces_df64": {"src": "a351ee1fa12c90bf", "traffic": 164.3, "thread_inst": 586.5},
+    "k_lean_cells": {"src": "d4eb2f6c65e0d57a", "fp64_inst": 94.0, "fp64_flops": 139.2, "traffic": 312.1},
+    "k_lean_faces": {"src": "d4eb2f6c65e0d57a", "fp64_inst": 32.9, "fp64_flops": 49.8, "traffic": 180.3},
+    "k_lean_cells_df64": {"src": "d4eb2f6c65e0d57a", "traffic": 259.9, "thread_inst": 1383.0},
+    "k_lean_faces_df64": {"src": "d4eb2f6c65e0d57a", "traffic": 164.3, "thread_inst": 586.5},
     # profiles/k_corr_iteration_fp32_255.md (255^3, the launches of one step)
-    "k_corr_iteration": {"src": "8dada89a5e251b16", "traffic": 104.5, "thread_inst": 524.6},
+    "k_corr_iteration": {"src": "c991ed0218c6bdf8", "traffic": 104.5, "thread_inst": 524.6},
 }
 # The FP64 pipe's nominal issue capacity: 304 thread-instructions per GPU clock (2 per SM; ncu's
 # sm__inst_executed_pipe_fp64 peak on this machine's GB300), 629 G/s at 2.07 GHz.
@@ -746,14 +746,16 @@ def measure_reactive(args, dev) -> dict:
         iters = args.steps * args.rx_iters
         t_it = t / iters
         hbm, hbm_kind = peaks()
-        kern_gbs = 10 * pbytes * ncell / t_it / 1e9
+        # FP32 reads 6 arrays and writes 3; FP64 reads and writes k(phi) too (the rate, on checks only, not counted)
+        arrays = 9 if pbytes == 4 else 11
+        kern_gbs = arrays * pbytes * ncell / t_it / 1e9
         out[prec] = {"value": 7 * pbytes * ncell / t_it / 1e9, "unit": "GB/s", "t_it_ms": t_it * 1e3,
                      "it_per_s": 1.0 / t_it, "cells": ncell, "grid": [p["nx"], p["ny"], p["nz"]],
                      "gpu_launches": s.launch_count() - l0, "clocks": clk,
                      "roofline": {"kernel": "k_rx_iter (whole step, begin/end and checks included)",
                                   "bound": "hbm", "achieved": kern_gbs, "peak": hbm, "unit": "GB/s",
                                   "frac": kern_gbs / hbm, "traffic": None,
-                                  "algorithmic_bytes_per_cell": 10 * pbytes}}
+                                  "algorithmic_bytes_per_cell": arrays * pbytes}}
         s.close()
         del s
         torch.cuda.empty_cache()

@@ -215,7 +215,7 @@ int pt_peak_arith(int32_t kind, void *sink, int32_t steps, int32_t reps, void *s
  * Applies one device routine of the PT kernels element-wise: out[e] = f(a[e] (, b[e])), n
  * elements, device pointers, synchronises `stream`. It exists so that each replacement of a
  * library operation can be compared with CUDA's own function and with its stated error bound:
- *   PT_MATH_RCP_PSEUDO   1/x, approximate FP64 reciprocal + one Newton-Raphson step (~2^-46)
+ *   PT_MATH_RCP_PSEUDO   1/x, approximate FP64 reciprocal + one Newton-Raphson step (~2^-40)
  *   PT_MATH_RCP_FULL     1/x, approximate FP64 reciprocal + one third-order step (rounding)
  *   PT_MATH_EXPM1_POS/NEG  expm1(x), expm1(-x) from the split Taylor series of exp (tiers
  *                          |x| <= 2^-20, <= 2^-6; beyond, CUDA's expm1)

@@ -25,9 +25,9 @@ namespace pt {
 // instruction count: coefficients folded on the host (LeanCoef), fused multiply-adds, third-order
 // reciprocals and no division, the porosity by expm1 of its small increment, norms through bit patterns.
 // At 255^3 an outer iteration's phases took 13.0 ms (141 FP64 instructions per cell in k_mix_prepare
-// alone, 137 in the Picard update, 67 at the edges); now 7.9 ms: 102 in k_mix_prepare with the edges, 81 in
-// k_mix_faces with the Picard update, 36 in k_mix_porosity, the pipe at 84 %. Conversions and products with
-// powers of two moved to the integer units, and fewer products, gave the last 1.2 ms.
+// alone, 137 in the Picard update, 67 at the edges); now 7.8 ms: 101 in k_mix_prepare with the edges, 83 in
+// k_mix_faces with the Picard update, 36 in k_mix_porosity, the pipe at 82-84 %. Conversions on the integer
+// units, powers of two folded into coefficients and fewer products gave the last 1.2 ms.
 
 // k of the iterate (Eq. 23), read with its neighbours by mix_prepare_point.
 __device__ __forceinline__ void mix_perm_point(const Box& b, const LeanCoef<double>& c, const double* phi,

